@@ -91,41 +91,55 @@ def draw(rng):
 DTYPES = {"bf16": torch.bfloat16, "f32": torch.float32}
 
 
-def _rotations(N, d, first):
-    """Packed rotary table of N tokens from position `first`: one frequency per feature pair, base 10000."""
+def _angles(N, d, first):
+    """cos and sin of N tokens from position `first`: one frequency per feature pair, base 10000."""
     freq = 10000.0 ** (-torch.arange(d // 2, device="cuda", dtype=torch.float32) / (d // 2))
     angle = torch.arange(first, first + N, device="cuda", dtype=torch.float32)[:, None] * freq
-    return la.rope_pack(angle.cos(), angle.sin())
+    return angle.cos(), angle.sin()
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """The tensors of a case, from the seed alone; k0, v0 (x0): the block that has gone before on a stream."""
     gen = torch.Generator(device="cuda").manual_seed(seed)
     dtype = DTYPES[case["dtype"]]
 
     def normal(*shape, scale=1.0):
         return torch.randn(*shape, device="cuda", generator=gen).mul_(scale).to(dtype)
 
-    state = {"case": case}
-    B = case["B"]
+    B, made = case["B"], {}
     if case["op"].startswith("tconv"):
         T, HW, D = case["T"], case["HW"], case["D"]
-        state["x"] = normal(B, T, HW, D)
-        state["taps"] = torch.randn(3, D, device="cuda", generator=gen).mul_(0.25)
+        made["x"] = normal(B, T, HW, D)
+        made["taps"] = torch.randn(3, D, device="cuda", generator=gen).mul_(0.25)
         if case["op"] == "tconv_step":
-            state["cache"] = la.TConvCache(B, HW, D, dtype, "cuda")
-            state["cache"].absorb(normal(B, 1, HW, D))   # a block has gone before
-        return state
-
+            made["x0"] = normal(B, 1, HW, D)
+        return made
     N, H, d = case["N"] * case["blocks"], case["H"], case["d"]
     # queries and keys as the projections of a normalised activation leave them: zero mean, 1/sqrt(d)
     for name, scale in (("q", d ** -0.5), ("k", d ** -0.5), ("v", 1.0)):
         if case["layout"] == "head":
-            state[name] = normal(B, H, N, d, scale=scale).permute(0, 2, 1, 3)
+            made[name] = normal(B, H, N, d, scale=scale).permute(0, 2, 1, 3)
         else:
-            state[name] = normal(B, N, H, d, scale=scale)
+            made[name] = normal(B, N, H, d, scale=scale)
+    if case["op"] != "forward":
+        made["k0"], made["v0"] = normal(B, case["N"], H, d, scale=d ** -0.5), normal(B, case["N"], H, d)
+    return made
+
+
+def prepare(case, seed):
+    made = _inputs(case, seed)
+    state = {"case": case, **{name: made[name] for name in ("x", "taps", "q", "k", "v") if name in made}}
+    B, dtype = case["B"], DTYPES[case["dtype"]]
+    if case["op"].startswith("tconv"):
+        if case["op"] == "tconv_step":
+            state["cache"] = la.TConvCache(B, case["HW"], case["D"], dtype, "cuda")
+            state["cache"].absorb(made["x0"])
+        return state
+
+    N, H, d = case["N"] * case["blocks"], case["H"], case["d"]
     if case["op"] == "forward":
         if case["rope"]:
-            state["table"] = _rotations(N, d, 0)
+            state["table"] = la.rope_pack(*_angles(N, d, 0))
             state["workspace"] = la.new_rope_workspace(state["q"])
         else:
             state["workspace"] = la.new_workspace(state["q"])
@@ -133,13 +147,11 @@ def prepare(case, seed):
     cache = la.BlockLinCache(B, H, d, dtype, "cuda", max_T_b=case["N"],
                              prefill_blocks=case["blocks"] if case["op"] == "prefill" else 0)
     state["cache"] = cache
-    # a block of the same length has gone before
-    k0, v0 = normal(B, case["N"], H, d, scale=d ** -0.5), normal(B, case["N"], H, d)
     if case["rope"]:
-        cache.step_rope(None, k0, v0, _rotations(case["N"], d, 0))
-        state["table"] = _rotations(N, d, case["N"])
+        cache.step_rope(None, made["k0"], made["v0"], la.rope_pack(*_angles(case["N"], d, 0)))
+        state["table"] = la.rope_pack(*_angles(N, d, case["N"]))
     else:
-        cache.step(None, k0, v0)
+        cache.step(None, made["k0"], made["v0"])
     return state
 
 
@@ -189,3 +201,49 @@ def tolerance(case):
     if case["dtype"] == "f32":
         return {"rel": 1e-6, "max": 6e-6}
     return {"rel": 0.012, "max": 0.08} if case["rope"] else {"rel": 7e-3, "max": 0.016}
+
+
+def _rotated(x, cos, sin):
+    """Feature pairs (2p, 2p+1) of x[B, N, H, d] turned by the angles of their token; the table holds fp16 values."""
+    c, s = cos.half().double()[None, :, None], sin.half().double()[None, :, None]
+    a, b = x[..., 0::2], x[..., 1::2]
+    return torch.stack((a * c - b * s, b * c + a * s), dim=-1).flatten(-2)
+
+
+def exact(case, seed):
+    """What `run` returns, from the definitions, in 64 bits."""
+    made = {name: t.double() for name, t in _inputs(case, seed).items()}
+    op = case["op"]
+    if op.startswith("tconv"):
+        x, w = made["x"], made["taps"]
+        y = x + w[1] * x
+        y[:, 1:] += w[0] * x[:, :-1]
+        y[:, :-1] += w[2] * x[:, 1:]
+        if op == "tconv_forward":
+            return y
+        y[:, :1] += w[0] * made["x0"]
+        return y, x[:, -1]
+
+    N, d, rope = case["N"], case["d"], case["rope"]
+
+    def state_of(k, v, first):
+        k = k.relu()
+        turned = _rotated(k, *_angles(k.shape[1], d, first)) if rope else k
+        return torch.einsum("bnhi,bnhj->bhji", turned, v), k.sum(1)
+
+    def read(q, S, z, first):
+        q = q.relu()
+        turned = _rotated(q, *_angles(q.shape[1], d, first)) if rope else q
+        return torch.einsum("bnhi,bhji->bnhj", turned, S) / (torch.einsum("bnhi,bhi->bnh", q, z) + 1e-6)[..., None]
+
+    q, k, v = made["q"], made["k"], made["v"]
+    if op == "forward":
+        return read(q, *state_of(k, v, 0), 0)
+    S, z = state_of(made["k0"], made["v0"], 0)
+    before = torch.cat((S, z[:, :, None]), dim=2)
+    outs = []
+    for first in range(0, N * case["blocks"], N):
+        dS, dz = state_of(k[:, first:first + N], v[:, first:first + N], N + first)
+        S, z = S + dS, z + dz
+        outs.append(read(q[:, first:first + N], S, z, N + first))
+    return torch.cat(outs, dim=1), before if op == "peek" else torch.cat((S, z[:, :, None]), dim=2)
