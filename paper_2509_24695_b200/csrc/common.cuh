@@ -49,6 +49,13 @@ cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* sta
                       float* partials, cudaStream_t stream, const __half2* rope = nullptr);
 cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, cudaStream_t stream,
                       const __half2* rope = nullptr);
+// The same with register-blocked kernels, for rows that can be read in 16-byte pieces (a, b: the tensors of the call).
+// The state comes as *P <= fma_chunks(N) partial states per unit.
+bool fma_tiled_ok(const Problem& p, const void* a, const void* b, const __half2* rope);
+cudaError_t fma_tiled_state_partials(const Problem& p, const void* k, const void* v, float* partials, const __half2* rope,
+                                     int* P, cudaStream_t stream);
+cudaError_t fma_tiled_apply_tokens(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* rope,
+                                   cudaStream_t stream);
 // blk: [B][M][H][(d+1)*d] per-block states -> running states after each block (on top of cache [B][H][..]), cache := last.
 cudaError_t prefix_states(float* blk, float* cache, int B, int M, long long floats_per_batch, cudaStream_t stream);
 cudaError_t rope_pack(const float* cs, const float* sn, long long count, __half2* out, cudaStream_t stream);

@@ -122,6 +122,7 @@ fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* 
   const int u = blockIdx.y;
   if (e >= E) return;
   double sum = accumulate ? (double)state[(long long)u * E + e] : 0.0;
+#pragma unroll 8   // eight loads in flight
   for (int c = 0; c < P; ++c) sum += (double)partials[((long long)u * P + c) * E + e];
   state[(long long)u * E + e] = (float)sum;
 }
@@ -312,8 +313,9 @@ cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* sta
     if (accumulate) return cudaSuccess;
     return cudaMemsetAsync(state_out, 0, sizeof(float) * E * p.units(), stream);
   }
-  const int P = fma_chunks(p.N);
-  cudaError_t e = state_partial_any(p, k, v, P, partials, rope, stream);
+  int P = fma_chunks(p.N);
+  cudaError_t e = fma_tiled_ok(p, k, v, rope) ? fma_tiled_state_partials(p, k, v, partials, rope, &P, stream)
+                                              : state_partial_any(p, k, v, P, partials, rope, stream);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((E + kThreads - 1) / kThreads), p.units());
   fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, accumulate ? 1 : 0);
@@ -324,6 +326,7 @@ cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* sta
 cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, cudaStream_t stream,
                       const __half2* rope) {
   if (p.N == 0) return cudaSuccess;
+  if (fma_tiled_ok(p, q, o, rope)) return fma_tiled_apply_tokens(p, q, state, o, eps, rope, stream);
   return apply_any(p, q, state, o, eps, rope, stream);
 }
 

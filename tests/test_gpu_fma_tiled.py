@@ -1,0 +1,82 @@
+"""The fp32-arithmetic path (fp32 tensors, bf16 head dims outside the tensor-core kernel's) at the edges of its tiles:
+every padding class of the head dim, token counts around the staged tiles and the split over CTAs, and the general
+kernels it shares the path with (rows that cannot be read in 16-byte pieces)."""
+import numpy as np
+import pytest
+
+import synth
+from parity_util import assert_parity_bf16, assert_parity_f32, assert_state_close, to_dev, to_f64
+
+pytestmark = pytest.mark.gpu
+
+EPS = 1e-6
+HEAD_DIMS = {"f32": [4, 12, 32, 36, 64, 80, 84, 100, 112, 116, 128], "bf16": [8, 24, 40, 56, 72, 88, 96, 104, 120]}
+
+
+@pytest.fixture(scope="module")
+def la():
+    import torch
+
+    assert torch.cuda.is_available(), "these tests need a CUDA device"
+    import paper_2509_24695_b200 as la
+
+    la.load_library()
+    return la
+
+
+def gen(B, N, H, d, seed, dtype):
+    return tuple(synth.gauss((B, N, H, d), seed, t, dtype=dtype) for t in (1, 2, 3))
+
+
+def check(dtype, got, ref, what):
+    (assert_parity_bf16 if dtype == "bf16" else assert_parity_f32)(got, ref, what)
+
+
+@pytest.mark.parametrize("dtype,d", [(t, d) for t in HEAD_DIMS for d in HEAD_DIMS[t]])
+@pytest.mark.parametrize("N", [1, 33, 127, 1300])
+def test_tiles(la, orc, dtype, d, N):
+    B, H = 2, 3
+    q, k, v = gen(B, N, H, d, 7000 + N + d, dtype)
+    S, z = orc.state(k, v)
+    st = la.linattn_state(to_dev(k), to_dev(v))
+    assert_state_close(to_f64(st), S, z, 1e-5, f"state N={N} d={d} {dtype}")
+    o = la.linattn_forward(to_dev(q), to_dev(k), to_dev(v), EPS)
+    check(dtype, to_f64(o), orc.forward(q, k, v, EPS), f"forward N={N} d={d} {dtype}")
+    cos, sin = synth.rope_table(1, 1, N, d)
+    table = la.rope_pack(to_dev(cos), to_dev(sin))
+    packed = table.cpu().numpy().astype(np.float64)
+    o = la.linattn_forward_rope(to_dev(q), to_dev(k), to_dev(v), table, EPS)
+    check(dtype, to_f64(o), orc.rope_forward(q, k, v, packed[..., 0], packed[..., 1], EPS), f"rotary N={N} d={d} {dtype}")
+
+
+@pytest.mark.parametrize("dtype,d", [("f32", 112), ("f32", 64), ("bf16", 72)])
+def test_rows_off_the_16_byte_grid(la, orc, dtype, d):
+    """The same values one element further in memory, with head and token strides that are no multiple of 16 bytes,
+    and head-major."""
+    import torch
+
+    B, N, H = 1, 700, 3
+    q, k, v = gen(B, N, H, d, 7100 + d, dtype)
+    ref = orc.forward(q, k, v, EPS)
+
+    def shifted(x):
+        t = to_dev(x)
+        flat = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
+        flat[1:] = t.flatten()
+        return flat[1:].view(t.shape)
+
+    def strided(x):
+        t = torch.zeros((B, N, H, d + 1), dtype=to_dev(x).dtype, device="cuda")[..., :d]
+        return t.copy_(to_dev(x))
+
+    def head_major(x):
+        return to_dev(x).permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+
+    for place in (shifted, strided, head_major):
+        o = la.linattn_forward(place(q), place(k), place(v), EPS, out=torch.empty_like(place(q)))
+        check(dtype, to_f64(o), ref, f"{place.__name__} {dtype} d={d}")
+    # an output off the grid beside inputs on it
+    out = shifted(q) if dtype == "f32" else None
+    if out is not None:
+        o = la.linattn_forward(to_dev(q), to_dev(k), to_dev(v), EPS, out=out)
+        check(dtype, to_f64(o), ref, "shifted output")
