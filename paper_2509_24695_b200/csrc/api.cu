@@ -66,6 +66,8 @@ inline float* partials_of(void* workspace) {
   return reinterpret_cast<float*>(static_cast<char*>(workspace) + LINATTN_WORKSPACE_CTRL_BYTES);
 }
 
+inline WorkspaceCtrl* ctrl_of(void* workspace) { return static_cast<WorkspaceCtrl*>(workspace); }
+
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? LINATTN_OK : LINATTN_ERR_CUDA; }
 
 // state = (accumulate ? base : 0) + state(k, v), then (q non-null) o = apply(q, state).  `base` is the
@@ -82,10 +84,10 @@ int run_passes(const Problem& p, const void* k, const void* v, const void* q, vo
       return LINATTN_ERR_CUDA;
   }
   if (k) {
-    int st = cuda_status(fma_state(p, k, v, state, accumulate, partials_of(workspace), stream));
+    int st = cuda_status(fma_state(p, k, v, state, accumulate, partials_of(workspace), ctrl_of(workspace), stream));
     if (st != LINATTN_OK) return st;
   }
-  if (q) return cuda_status(fma_apply(p, q, state, o, eps, stream));
+  if (q) return cuda_status(fma_apply(p, q, state, o, eps, ctrl_of(workspace), stream));
   return LINATTN_OK;
 }
 
@@ -110,9 +112,9 @@ int run_rope(const Problem& p, const void* q, const void* k, const void* v, void
     if (cudaMemcpyAsync(state, base, state_bytes_of(p), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
       return LINATTN_ERR_CUDA;
   }
-  int st = cuda_status(fma_state(p, k, v, state, accumulate, partials_of(workspace), stream, rope));
+  int st = cuda_status(fma_state(p, k, v, state, accumulate, partials_of(workspace), ctrl_of(workspace), stream, rope));
   if (st != LINATTN_OK || !q) return st;
-  return cuda_status(fma_apply(p, q, state, o, eps, stream, rope));
+  return cuda_status(fma_apply(p, q, state, o, eps, ctrl_of(workspace), stream, rope));
 }
 
 }  // namespace

@@ -46,16 +46,15 @@ inline int fma_chunks(long long N) {
 // state_out = (accumulate ? state_out : 0) + state of tokens [0, N); partials is scratch.
 // rope: Eq. 2 with its rotary factors, table [N][d/2] of (cos, sin) fp16 pairs, one per pair rotation.
 cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* state_out, bool accumulate,
-                      float* partials, cudaStream_t stream, const __half2* rope = nullptr);
-cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, cudaStream_t stream,
+                      float* partials, WorkspaceCtrl* ctrl, cudaStream_t stream, const __half2* rope = nullptr);
+cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, WorkspaceCtrl* ctrl, cudaStream_t stream,
                       const __half2* rope = nullptr);
-// The same with register-blocked kernels, for rows that can be read in 16-byte pieces (a, b: the tensors of the call).
-// The state comes as *P <= fma_chunks(N) partial states per unit.
-bool fma_tiled_ok(const Problem& p, const void* a, const void* b, const __half2* rope);
-cudaError_t fma_tiled_state_partials(const Problem& p, const void* k, const void* v, float* partials, const __half2* rope,
-                                     int* P, cudaStream_t stream);
-cudaError_t fma_tiled_apply_tokens(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* rope,
-                                   cudaStream_t stream);
+// The same on the tensor cores (split_kernels.cu); ctrl: the workspace's control block.
+bool split_ok(const Problem& p, const void* a, const void* b, const __half2* rope);
+cudaError_t split_state_partials(const Problem& p, const void* k, const void* v, float* partials, const __half2* rope, int* P,
+                                 WorkspaceCtrl* ctrl, cudaStream_t stream);
+cudaError_t split_apply(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* rope,
+                        WorkspaceCtrl* ctrl, cudaStream_t stream);
 // blk: [B][M][H][(d+1)*d] per-block states -> running states after each block (on top of cache [B][H][..]), cache := last.
 cudaError_t prefix_states(float* blk, float* cache, int B, int M, long long floats_per_batch, cudaStream_t stream);
 cudaError_t rope_pack(const float* cs, const float* sn, long long count, __half2* out, cudaStream_t stream);

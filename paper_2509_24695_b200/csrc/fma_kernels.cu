@@ -1,8 +1,8 @@
 // Plain fp32-FMA kernels for ReLU linear attention (Eq. 2 / Eq. 3 of the paper).
 //
-// They serve the fp32 I/O path (fp32 in, fp32 arithmetic, fp32 out) and the bf16
-// shapes the tensor-core kernels do not take (head dims other than 32/64/112/128).
-// Any head dim 1..128 and any element strides are accepted.
+// They serve what neither tensor-core path takes: head dims up to 16, and fp32 and odd-head-dim bf16 rows that cannot
+// be read in 16-byte pieces (split_ok in split_kernels.cu).  Any head dim 1..128 and any element strides are accepted.
+// The split-N partial states of both paths are summed here.
 //
 //   fma_state_partial : one CTA per (split-N chunk, unit) accumulates phi(K)^T V and sum phi(K)
 //                       over its token range into registers and writes one partial state.
@@ -307,15 +307,15 @@ cudaError_t rope_pack(const float* cs, const float* sn, long long count, __half2
 }
 
 cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* state_out, bool accumulate,
-                      float* partials, cudaStream_t stream, const __half2* rope) {
+                      float* partials, WorkspaceCtrl* ctrl, cudaStream_t stream, const __half2* rope) {
   const long long E = p.state_elems();
   if (p.N == 0) {
     if (accumulate) return cudaSuccess;
     return cudaMemsetAsync(state_out, 0, sizeof(float) * E * p.units(), stream);
   }
   int P = fma_chunks(p.N);
-  cudaError_t e = fma_tiled_ok(p, k, v, rope) ? fma_tiled_state_partials(p, k, v, partials, rope, &P, stream)
-                                              : state_partial_any(p, k, v, P, partials, rope, stream);
+  cudaError_t e = split_ok(p, k, v, rope) ? split_state_partials(p, k, v, partials, rope, &P, ctrl, stream)
+                                          : state_partial_any(p, k, v, P, partials, rope, stream);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)((E + kThreads - 1) / kThreads), p.units());
   fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, accumulate ? 1 : 0);
@@ -323,10 +323,10 @@ cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* sta
   return cudaGetLastError();
 }
 
-cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, cudaStream_t stream,
+cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, WorkspaceCtrl* ctrl, cudaStream_t stream,
                       const __half2* rope) {
   if (p.N == 0) return cudaSuccess;
-  if (fma_tiled_ok(p, q, o, rope)) return fma_tiled_apply_tokens(p, q, state, o, eps, rope, stream);
+  if (split_ok(p, q, o, rope) && (reinterpret_cast<uintptr_t>(state) & 15) == 0) return split_apply(p, q, state, o, eps, rope, ctrl, stream);
   return apply_any(p, q, state, o, eps, rope, stream);
 }
 

@@ -1,0 +1,666 @@
+// fp32-accurate state and apply passes on the tensor cores: fp32 tensors, and the bf16 head dims the fused kernel
+// (umma_kernels.cu) does not take, wherever rows can be read in 16-byte pieces (split_ok).
+//
+// An fp32 value is the sum of three bf16 values exactly (8 significand bits each, cut off, not rounded, so that the
+// largest finite value stays finite).  A product of two such sums is nine bf16 products; the three smallest are below
+// 2^-24 of the whole and are left out, the other six are exact in the tensor core's fp32 accumulators.  What is left to
+// chance is how they are added up.  The tensor core truncates when it adds into an accumulator (2^-24 on average, always
+// towards zero), so (1) the leading products have accumulators apart from the five small ones, whose additions are
+// 2^-8 below; (2) they are dealt over several accumulators, so that no chain is longer than two or three; and (3) the
+// accumulators are added up in registers, round to nearest, every 64 tokens.  bf16 operands are one part, rotated ones
+// three; S is always three.  z and the denominators are plain fp32 sums.  The results are closer to the exact ones than
+// those of a chain of fp32 multiply-adds (see the figures at the kernels).
+//
+// Operand layouts are those of the fused kernel: 128-byte swizzled rows of 64 features.  Every thread reads its own
+// pieces with private asynchronous copies, rectifies, rotates and splits them, and stores the parts; one thread issues
+// the MMAs of a tile while all of them prepare the next one.  All waits are on this CTA's own MMAs and bounded.
+#include "common.cuh"
+#include "sm100_ptx.cuh"
+
+namespace linattn {
+namespace {
+
+using namespace ptx;
+
+constexpr int kThreads = 512;                // threads that prepare, drain and store; one more warp issues the MMAs
+constexpr int kBlock = kThreads + 32;
+
+template <typename T>
+struct Piece;   // 16 bytes of a row
+template <>
+struct Piece<float> {
+  static constexpr int E = 4;
+  using Tab = uint2;   // the (cos, sin) fp16 pairs of its feature pairs
+};
+template <>
+struct Piece<__nv_bfloat16> {
+  static constexpr int E = 8;
+  using Tab = uint4;
+};
+
+// What both passes know about a shape.  R = ceil(d / 16).
+template <typename T, int R, bool ROPE>
+struct Shape {
+  static constexpr int E = Piece<T>::E;
+  static constexpr int DP = 16 * R;                        // features with padding
+  static constexpr int BOXES = (DP + 63) / 64;
+  static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr int QK_PARTS = F32 || ROPE ? 3 : 1;     // bf16 parts of phi(k), phi(q)
+  static constexpr int V_PARTS = F32 ? 3 : 1;
+  using Tab = typename Piece<T>::Tab;
+};
+
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* smem_dst, const void* src, bool live) {   // not live: zeros
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
+  if (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(live ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ void widen(const uint4& r, float (&x)[4]) {
+  x[0] = __uint_as_float(r.x); x[1] = __uint_as_float(r.y); x[2] = __uint_as_float(r.z); x[3] = __uint_as_float(r.w);
+}
+__device__ __forceinline__ void widen(const uint4& r, float (&x)[8]) {
+  const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { x[2 * i] = __uint_as_float(w[i] << 16); x[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u); }
+}
+
+// (a, b) -> (a c - b s, b c + a s) for every feature pair of the piece
+template <int E>
+__device__ __forceinline__ void rotate(float (&x)[E], const __half2* tab) {
+#pragma unroll
+  for (int e = 0; e < E; e += 2) {
+    const float2 cs = __half22float2(tab[e / 2]);
+    const float a = x[e], b = x[e + 1];
+    x[e] = a * cs.x - b * cs.y;
+    x[e + 1] = b * cs.x + a * cs.y;
+  }
+}
+
+// Byte offset of feature f (a multiple of 4) of row `row` in an operand of boxes of 64 features, `box_bytes` each.
+__device__ __forceinline__ int operand_offset(int row, int f, int box_bytes) {
+  return (f >> 6) * box_bytes + row * 128 + ((((f & 63) >> 3) ^ (row & 7)) << 4) + ((f & 4) << 1);
+}
+
+// The next bf16 part of every value: its upper half; x becomes what is left.  Packed in pairs.
+template <int E>
+__device__ __forceinline__ void take_part(float (&x)[E], uint32_t (&w)[E / 2]) {
+#pragma unroll
+  for (int e = 0; e < E; e += 2) {
+    const uint32_t a = __float_as_uint(x[e]), b = __float_as_uint(x[e + 1]);
+    w[e / 2] = __byte_perm(a, b, 0x7632);
+    x[e] -= __uint_as_float(a & 0xFFFF0000u);
+    x[e + 1] -= __uint_as_float(b & 0xFFFF0000u);
+  }
+}
+__device__ __forceinline__ void store_words(uint8_t* at, const uint32_t (&w)[2]) { *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]); }
+__device__ __forceinline__ void store_words(uint8_t* at, const uint32_t (&w)[4]) { *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]); }
+
+template <int PARTS, int E>
+__device__ __forceinline__ void store_parts(uint8_t* at, int part_bytes, float (&x)[E]) {
+#pragma unroll
+  for (int s = 0; s < PARTS; ++s) {
+    uint32_t w[E / 2];
+    take_part(x, w);
+    store_words(at + s * part_bytes, w);
+  }
+}
+
+__device__ __forceinline__ void tmem_ld_x8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+
+__device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
+  return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
+}
+
+// ---------------------------------------------------------------- state
+template <typename T, int R, bool ROPE>
+struct StateShape : Shape<T, R, ROPE> {
+  using B = Shape<T, R, ROPE>;
+  // tokens of a tile: 64 where two stages of parts and three of raw pieces fit, else 32
+  static constexpr int BYTES_64 = 2 * (B::QK_PARTS + B::V_PARTS) * B::BOXES * 8192 + 3 * 64 * B::DP * (2 * (int)sizeof(T) + (ROPE ? 2 : 0));
+  static constexpr int TOK = BYTES_64 <= 200 * 1024 ? 64 : 32;
+  static constexpr int LANES = kThreads / TOK;               // threads to a row
+  static constexpr int PIECES = (B::DP / B::E + LANES - 1) / LANES;   // 16-byte pieces of a row per thread
+  static constexpr int FLIP = LANES == 8 && PIECES % 2 == 0 ? 1 : 0;
+  static constexpr int BOX = TOK * 128;
+  static constexpr int PART = B::BOXES * BOX;
+  static constexpr int STAGE = (B::QK_PARTS + B::V_PARTS) * PART;
+  static constexpr int RAW_STAGES = 3;
+  static constexpr int TAB = ROPE ? PIECES * kThreads * (int)sizeof(typename B::Tab) : 0;
+  static constexpr int RAW = 2 * PIECES * kThreads * 16 + TAB;
+  static constexpr int Z_BYTES = TOK * B::DP * 4;
+  static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > Z_BYTES ? RAW_STAGES * RAW : Z_BYTES) + 64;   // (barriers last)
+  static constexpr int LEAD = TOK / 32;                      // accumulators of the leading products: chains of two K steps
+  static constexpr bool REST = B::QK_PARTS + B::V_PARTS > 2;
+  static constexpr int ACC = B::DP <= 64 ? 64 : 128;         // TMEM columns between accumulators
+  static constexpr int SET = (LEAD + (REST ? 1 : 0)) * ACC;  // one set collects a tile while the other is drained
+  static constexpr int COLS = 2 * SET <= 128 ? 128 : 2 * SET <= 256 ? 256 : 512;
+  static_assert(2 * SET <= 512, "tensor memory");
+};
+
+// grid (P, units): partial state of the tiles [c * tiles / P, (c + 1) * tiles / P) of one unit, in the library's layout.
+//
+// Measured (32 760 tokens, 20 heads of 112, fp32; floor: 587 MB, 90 us at the copy rate): 192 us with the reduce of the
+// partial states, where the general kernels take 1050 (fp32 pipe at a quarter of its rate, scalar loads) and a register-blocked
+// form of them on packed fp32 FMAs 492.  A tile of 32 tokens takes 1.2 us, most of it instruction issue (splitting and
+// draining) and the latencies of one tile's chain.  Distance from 64 bits, 2-norm: S 1.3e-7 (general kernels 2.9e-7).
+template <typename T, int R, bool ROPE>
+__global__ void __launch_bounds__(kBlock, 1)
+split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, int P, float* __restrict__ partials,
+                   const __half2* __restrict__ tab, WorkspaceCtrl* ctrl) {
+  using S = StateShape<T, R, ROPE>;
+  using Tab = typename S::Tab;
+  constexpr int E = S::E, PIECES = S::PIECES;
+  constexpr uint32_t IDESC = make_idesc_bf16(128, S::DP, true, true);
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align1024(smem_raw);
+  uint8_t* raw = smem + 2 * S::STAGE;
+  uint64_t* done = reinterpret_cast<uint64_t*>(raw + (S::SMEM - 1024 - 2 * S::STAGE - 64));   // [2] the tile's MMAs are complete
+  uint64_t* ready = done + 2;                                                               // [2] the tile's parts are in its stage
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ready + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int d = p.d, u = blockIdx.y, c = blockIdx.x;
+  const long long all = (p.N + S::TOK - 1) / S::TOK;
+  const long long first = c * all / P;
+  const int tiles = (int)((c + 1) * all / P - first);
+
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kThreads); }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  // padded features are never written and must read as zero
+  for (int i = tid; i < 2 * S::STAGE / 16; i += kBlock) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+  if (warp == 0) { tmem_alloc(tmem_holder, S::COLS); tmem_relinquish(); }
+
+  // this thread's row of every tile, and its pieces of it: features feature(0), feature(1), ...  Sixteen neighbouring
+  // 8-byte stores fill one swizzled row of 128 bytes; with eight threads to a row, odd rows take each pair of pieces in
+  // the other order, so that the stores of two neighbouring rows fall into different halves of the banks.
+  const int row = (tid % kThreads) / S::LANES, l = tid % S::LANES;
+  auto feature = [&](int i) { return (l + S::LANES * (S::FLIP ? i ^ (row & 1) : i)) * E; };
+  const long long base = (long long)(u / p.H) * p.sb + (long long)(u % p.H) * p.sh;
+  auto raw_k = [&](int st, int i) { return reinterpret_cast<uint4*>(raw + st * S::RAW) + 2 * i * kThreads + tid; };
+  auto raw_tab = [&](int st, int i) {
+    return reinterpret_cast<Tab*>(raw + st * S::RAW + 2 * PIECES * kThreads * 16) + i * kThreads + tid;
+  };
+  auto issue = [&](int t, int st) {
+    if (t < tiles) {
+      const long long n = (first + t) * S::TOK + row;
+      const bool live = n < p.N;
+      const long long off = base + (live ? n : 0) * p.sn;
+#pragma unroll
+      for (int i = 0; i < PIECES; ++i) {
+        const int f = feature(i);
+        if (f >= d) continue;
+        copy_async<16>(raw_k(st, i), k + off + f, live);
+        copy_async<16>(raw_k(st, i) + kThreads, v + off + f, live);
+        if (ROPE) copy_async<(int)sizeof(Tab)>(raw_tab(st, i), tab + (live ? n : 0) * (d / 2) + f / 2, live);
+      }
+    }
+    copy_commit();   // one group per tile, empty or not
+  };
+  float z[PIECES][E];
+#pragma unroll
+  for (int i = 0; i < PIECES; ++i)
+#pragma unroll
+    for (int e = 0; e < E; ++e) z[i][e] = 0.f;
+  auto convert = [&](int st, uint8_t* stage) {
+    uint4 kr[PIECES], vr[PIECES];   // all reads before the first store: they overlap
+    Tab tb[PIECES];
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) {
+      kr[i] = *raw_k(st, i);
+      vr[i] = *(raw_k(st, i) + kThreads);
+      if (ROPE) tb[i] = *raw_tab(st, i);
+    }
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) {
+      const int f = feature(i);
+      if (f >= d) continue;
+      float x[E];
+      widen(kr[i], x);
+#pragma unroll
+      for (int e = 0; e < E; ++e) { x[e] = fmaxf(x[e], 0.f); z[i][e] += x[e]; }   // phi = ReLU on the keys; z from the plain ones
+      if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
+      uint8_t* at = stage + operand_offset(row, f, S::BOX);
+      store_parts<S::QK_PARTS>(at, S::PART, x);
+      at += S::QK_PARTS * S::PART;
+      if (S::V_PARTS == 1) {
+        *reinterpret_cast<uint4*>(at) = vr[i];
+      } else {
+        widen(vr[i], x);
+        store_parts<S::V_PARTS>(at, S::PART, x);
+      }
+    }
+  };
+
+  const bool worker = warp < kThreads / 32;
+  if (worker) {
+    issue(0, 0);
+    issue(1, 1);
+  }
+  fence_proxy_async_smem();   // the zeros
+  tcgen05_fence_before();
+  __syncthreads();
+  tcgen05_fence_after();
+  const uint32_t tmem = *tmem_holder;
+
+  // accumulator lane = key feature; each of the four warps of a lane quarter takes a quarter of the value features
+  constexpr int COLS = S::DP / 4;
+  const int key = (warp & 3) * 32 + lane;
+  const int col0 = (warp >> 2) * COLS;
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0;
+  float sum[COLS];
+#pragma unroll
+  for (int x = 0; x < COLS; ++x) sum[x] = 0.f;
+  auto drain = [&](int t) {
+    mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
+    __syncwarp();   // tcgen05.ld wants whole warps
+    tcgen05_fence_after();
+    if ((warp & 3) * 32 < d) {
+#pragma unroll
+      for (int g = 0; g < R; ++g) {
+        uint32_t a[S::LEAD + 1][4];
+#pragma unroll
+        for (int s = 0; s < S::LEAD + (S::REST ? 1 : 0); ++s) tmem_ld_x4(trow + (t & 1) * S::SET + s * S::ACC + 4 * g, a[s]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          float add = __uint_as_float(a[0][x]);
+          if (S::LEAD > 1) add += __uint_as_float(a[S::LEAD > 1 ? 1 : 0][x]);
+          if (S::REST) add += __uint_as_float(a[S::LEAD][x]);
+          sum[4 * g + x] += add;
+        }
+      }
+    }
+    tcgen05_fence_before();
+  };
+
+  if (worker) {
+    for (int t = 0; t < tiles; ++t) {
+      // the stage and the accumulators of tile t - 2 are free: this thread has drained it, and the MMA warp waits for all
+      issue(t + 2, (t + 2) % S::RAW_STAGES);
+      copy_wait<2>();
+      convert(t % S::RAW_STAGES, smem + (t & 1) * S::STAGE);
+      fence_proxy_async_smem();
+      mbar_arrive(&ready[t & 1]);
+      if (t > 0) drain(t - 1);
+    }
+    if (tiles > 0) drain(tiles - 1);
+  } else if (lane == 0) {
+    for (int t = 0; t < tiles; ++t) {
+      mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag);
+      tcgen05_fence_after();
+      constexpr uint32_t LBO = S::BOXES > 1 ? S::BOX : 0;   // 64 features: rows 64..127 of the MMA repeat them and are ignored
+      // shared-memory addresses are below 2^18, so an offset of a multiple of 16 bytes is added to a descriptor as it is
+      const uint64_t a0 = make_smem_desc_sw128(smem_u32(smem + (t & 1) * S::STAGE), LBO, 1024), b0 = a0 + S::QK_PARTS * S::PART / 16;
+      const uint32_t set = tmem + (t & 1) * S::SET;
+      auto mma = [&](int kk, int pk, int pv, uint32_t acc, bool add) {
+        umma_bf16(set + acc * S::ACC, a0 + (pk * S::PART + kk * 2048) / 16, b0 + (pv * S::PART + kk * 2048) / 16, IDESC, add ? 1u : 0u);
+      };
+      if (S::REST) {   // smallest first
+        bool add = false;
+#pragma unroll
+        for (int order = 2; order >= 1; --order)
+#pragma unroll
+          for (int pk = order; pk >= 0; --pk) {
+            const int pv = order - pk;
+            if (pk >= S::QK_PARTS || pv >= S::V_PARTS) continue;
+#pragma unroll
+            for (int kk = 0; kk < S::TOK / 16; ++kk) { mma(kk, pk, pv, S::LEAD, add); add = true; }
+          }
+      }
+#pragma unroll
+      for (int kk = 0; kk < S::TOK / 16; ++kk) mma(kk, 0, 0, kk % S::LEAD, kk >= S::LEAD);
+      umma_commit(&done[t & 1]);
+    }
+  }
+  copy_wait<0>();
+  __syncthreads();
+
+  // W[j][i] = S[i][j], W[d][i] = z[i]
+  float* out = partials + ((long long)u * P + c) * p.state_elems();
+  if (worker && key < d) {
+#pragma unroll
+    for (int x = 0; x < COLS; ++x)
+      if (col0 + x < d) out[(long long)(col0 + x) * d + key] = sum[x];
+  }
+  float* zs = reinterpret_cast<float*>(raw);   // [row][d]
+#pragma unroll
+  for (int i = 0; i < PIECES; ++i) {
+    const int f = feature(i);
+    if (!worker || f >= d) continue;
+#pragma unroll
+    for (int e = 0; e < E; ++e) zs[row * d + f + e] = z[i][e];
+  }
+  __syncthreads();
+  if (tid < d) {
+    float zt = 0.f;
+    for (int r = 0; r < S::TOK; ++r) zt += zs[r * d + tid];
+    out[(long long)d * d + tid] = zt;
+  }
+  if (*abort_flag && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
+  if (warp == 0) tmem_dealloc(tmem, S::COLS);
+}
+
+// ---------------------------------------------------------------- apply
+// O^T = S^T phi(Q)^T: the accumulator's lanes are the value features and its columns the tokens of a tile, so that a
+// tile of 64 tokens is enough for a whole MMA and three parts of S, two tiles' three parts and the next tile's raw
+// pieces fit into shared memory together.
+template <typename T, int R, bool ROPE>
+struct ApplyShape : Shape<T, R, ROPE> {
+  using B = Shape<T, R, ROPE>;
+  static constexpr int TOK = 64;
+  static constexpr int LANES = kThreads / TOK;                // threads to a row
+  static constexpr int PIECES = 2 * ((B::DP / B::E + 2 * LANES - 1) / (2 * LANES));   // 16-byte pieces of a row per thread, even
+  static constexpr int SBOX = B::DP * 128, SPART = B::BOXES * SBOX;   // (lanes from DP on read whatever follows and are ignored)
+  static constexpr int S_BYTES = 3 * SPART;
+  static constexpr int QBOX = TOK * 128, QPART = B::BOXES * QBOX, STAGE = B::QK_PARTS * QPART;
+  static constexpr int DEN = 4 * TOK * 4;
+  static constexpr int OVERRUN = 128 * 128 - SBOX;            // of the last part's last box, when less than that follows
+  static constexpr int AFTER = 2 * STAGE + DEN + 64;
+  static constexpr int SMEM = 1024 + S_BYTES + (AFTER > OVERRUN ? AFTER : OVERRUN);
+  static constexpr int LEAD = 3, ACC = TOK, SET = (LEAD + 1) * ACC;   // TMEM columns: two sets of four accumulators
+};
+
+__device__ __forceinline__ void store_value(float* o, float x) { *o = x; }
+__device__ __forceinline__ void store_value(__nv_bfloat16* o, float x) { *o = __float2bfloat16_rn(x); }
+
+// grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
+//
+// Measured as above: 182 us, general kernels 866, register-blocked on packed fp32 FMAs 489; distance from 64 bits 0.9e-7
+// (general kernels 1.6e-7).  bf16, 28 heads of 80: 165 us, general kernels 644.
+template <typename T, int R, bool ROPE>
+__global__ void __launch_bounds__(kBlock, 1)
+split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* __restrict__ o, Problem p, float eps,
+                   const __half2* __restrict__ tab, WorkspaceCtrl* ctrl) {
+  using A = ApplyShape<T, R, ROPE>;
+  using Tab = typename A::Tab;
+  constexpr int E = A::E, PIECES = A::PIECES;
+  constexpr uint32_t IDESC = make_idesc_bf16(128, A::TOK, false, false);
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* s_op = align1024(smem_raw);
+  uint8_t* stages = s_op + A::S_BYTES;
+  float* den = reinterpret_cast<float*>(stages + 2 * A::STAGE);     // [4][TOK] reciprocals of the denominators
+  uint64_t* done = reinterpret_cast<uint64_t*>(den + 4 * A::TOK);   // [2] as in the state kernel
+  uint64_t* ready = done + 2;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ready + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int d = p.d, u = blockIdx.y;
+  const long long all = (p.N + A::TOK - 1) / A::TOK;
+  const long long first = blockIdx.x * all / gridDim.x;
+  const int tiles = (int)((blockIdx.x + 1) * all / gridDim.x - first);
+  const float* W = state + (long long)u * p.state_elems();
+  const long long base = (long long)(u / p.H) * p.sb + (long long)(u % p.H) * p.sh;
+  // this thread's row of every tile, and its pieces of it.  Odd rows take each pair of pieces in the other order, so that
+  // the 8-byte stores of two neighbouring rows fall into different halves of the banks.
+  const int row = (tid % kThreads) / A::LANES, l = tid % A::LANES;
+  auto feature = [&](int i) { return (l + A::LANES * (i ^ (row & 1))) * E; };
+  const bool worker = warp < kThreads / 32;
+  // two tiles' raw pieces are on their way in registers
+  auto fetch = [&](int t, uint4 (&x)[PIECES], Tab (&tb)[PIECES]) {
+    const long long n = (first + t) * A::TOK + row;
+    const bool live = t < tiles && n < p.N;
+    const long long at = live ? n : 0;
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) {
+      x[i] = make_uint4(0, 0, 0, 0);
+      if (live && feature(i) < d) {
+        x[i] = __ldcs(reinterpret_cast<const uint4*>(q + base + at * p.sn + feature(i)));
+        if (ROPE) tb[i] = __ldg(reinterpret_cast<const Tab*>(tab + at * (d / 2) + feature(i) / 2));
+      }
+    }
+  };
+  uint4 x0[PIECES], x1[PIECES];
+  Tab tb0[PIECES], tb1[PIECES];
+  if (worker) {
+    fetch(0, x0, tb0);
+    fetch(1, x1, tb1);
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kThreads); }
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 0) { tmem_alloc(tmem_holder, 512); tmem_relinquish(); }
+  // padded features of both operands read as zero
+  for (int i = tid; i < (A::S_BYTES + 2 * A::STAGE) / 16; i += kBlock) reinterpret_cast<uint4*>(s_op)[i] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  for (int idx = tid; idx < d * (d / 4); idx += kBlock) {
+    const int j = idx / (d / 4), i = (idx - j * (d / 4)) * 4;
+    float x[4];
+    widen(__ldg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
+    store_parts<3>(s_op + operand_offset(j, i, A::SBOX), A::SPART, x);
+  }
+  float z[PIECES][E];
+#pragma unroll
+  for (int i = 0; i < PIECES; ++i)
+#pragma unroll
+    for (int e = 0; e < E; ++e) z[i][e] = feature(i) < d ? W[(long long)d * d + feature(i) + e] : 0.f;
+
+  auto convert = [&](int t, uint4 (&raw)[PIECES], Tab (&tb)[PIECES]) {
+    uint8_t* stage = stages + (t & 1) * A::STAGE;
+    float dn = 0.f;
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) {
+      const int f = feature(i);
+      if (f >= d) continue;
+      float x[E];
+      widen(raw[i], x);
+#pragma unroll
+      for (int e = 0; e < E; ++e) { x[e] = fmaxf(x[e], 0.f); dn = fmaf(x[e], z[i][e], dn); }   // phi = ReLU on the queries
+      if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
+      store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX), A::QPART, x);
+    }
+    dn += __shfl_xor_sync(0xffffffffu, dn, 1);
+    dn += __shfl_xor_sync(0xffffffffu, dn, 2);
+    dn += __shfl_xor_sync(0xffffffffu, dn, 4);
+    if (l == 0) den[(t & 3) * A::TOK + row] = 1.0f / (dn + eps);   // eps added once, after the dot product
+  };
+  fence_proxy_async_smem();   // S and the zeros
+  tcgen05_fence_before();
+  __syncthreads();
+  tcgen05_fence_after();
+  const uint32_t tmem = *tmem_holder;
+
+  // accumulator lane = value feature; each of the four warps of a lane quarter takes a quarter of the tokens
+  const int j = (warp & 3) * 32 + lane, tok0 = (warp >> 2) * 16;
+  auto epilogue = [&](int t) {
+    mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
+    __syncwarp();   // tcgen05.ld wants whole warps
+    tcgen05_fence_after();
+    if ((warp & 3) * 32 < d) {
+      const uint32_t trow = tmem + (t & 1) * A::SET + ((uint32_t)((warp & 3) * 32) << 16) + tok0;
+      const float* rden = den + (t & 3) * A::TOK + tok0;
+      const long long n0 = (first + t) * A::TOK + tok0;
+      const int live = j < d ? (int)min(16ll, p.N - n0) : 0;
+      T* out = o + base + n0 * p.sn + j;
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        uint32_t a[A::LEAD + 1][8];
+#pragma unroll
+        for (int s = 0; s < (R < 3 ? R : A::LEAD); ++s) tmem_ld_x8(trow + s * A::ACC + 8 * g, a[s]);
+        tmem_ld_x8(trow + A::LEAD * A::ACC + 8 * g, a[A::LEAD]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          float num = __uint_as_float(a[0][x]);
+          if (R > 1) num += __uint_as_float(a[1][x]);
+          if (R > 2) num += __uint_as_float(a[2][x]);
+          num += __uint_as_float(a[A::LEAD][x]);
+          if (8 * g + x < live) store_value(out, num * rden[8 * g + x]);
+          out += p.sn;
+        }
+      }
+    }
+    tcgen05_fence_before();
+  };
+  if (worker) {
+    // stage and accumulators of tile t - 2 are free: this thread has been through its epilogue, and the MMA warp waits for all
+    auto step = [&](int t, uint4 (&x)[PIECES], Tab (&tb)[PIECES]) {
+      convert(t, x, tb);
+      fetch(t + 2, x, tb);
+      fence_proxy_async_smem();
+      mbar_arrive(&ready[t & 1]);
+      if (t > 0) epilogue(t - 1);
+    };
+    for (int t = 0; t < tiles; t += 2) {
+      step(t, x0, tb0);
+      if (t + 1 < tiles) step(t + 1, x1, tb1);
+    }
+    if (tiles > 0) epilogue(tiles - 1);
+  } else if (lane == 0) {
+    for (int t = 0; t < tiles; ++t) {
+      mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag);
+      tcgen05_fence_after();
+      const uint64_t a0 = make_smem_desc_sw128(smem_u32(s_op), 16, 1024);   // offsets are added as in the state kernel
+      const uint64_t b0 = make_smem_desc_sw128(smem_u32(stages + (t & 1) * A::STAGE), 16, 1024);
+      const uint32_t set = tmem + (t & 1) * A::SET;
+      auto mma = [&](int kk, int ps, int pq, uint32_t acc, bool add) {
+        umma_bf16(set + acc * A::ACC, a0 + (ps * A::SPART + (kk >> 2) * A::SBOX + (kk & 3) * 32) / 16,
+                  b0 + (pq * A::QPART + (kk >> 2) * A::QBOX + (kk & 3) * 32) / 16, IDESC, add ? 1u : 0u);
+      };
+      bool add = false;
+#pragma unroll
+      for (int order = 2; order >= 1; --order)   // smallest first
+#pragma unroll
+        for (int pq = order; pq >= 0; --pq) {
+          if (pq >= A::QK_PARTS) continue;
+#pragma unroll
+          for (int kk = 0; kk < R; ++kk) { mma(kk, order - pq, pq, A::LEAD, add); add = true; }
+        }
+#pragma unroll
+      for (int kk = 0; kk < R; ++kk) mma(kk, 0, 0, kk % A::LEAD, kk >= A::LEAD);
+      umma_commit(&done[t & 1]);
+    }
+  }
+  __syncthreads();
+  if (*abort_flag && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
+  if (warp == 0) { tcgen05_fence_after(); tmem_dealloc(tmem, 512); }
+}
+
+// ---------------------------------------------------------------- host side
+int sms() {
+  static int cached[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cached[dev]) {
+    int n = 0;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    cached[dev] = n;
+  }
+  return cached[dev];
+}
+
+template <typename K>
+cudaError_t allow_smem(K kernel, int bytes, bool (&done)[64]) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (done[dev]) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done[dev] = true;
+  return e;
+}
+
+// How many pieces a unit's tiles are cut into, up to `most`: the fewest waves of CTAs times what a CTA takes, `fixed`
+// tiles of which it takes whatever its share.
+int pieces(long long tiles, int units, int slots, long long most, double fixed) {
+  const long long few = (4ll * slots + units - 1) / units;   // four waves: beyond that the last one is small anyway
+  if (most > few) most = few;
+  if (most > tiles) most = tiles;
+  long long best = 1;
+  double cost = 0;
+  for (long long c = 1; c <= most; ++c) {
+    const double now = (double)((c * units + slots - 1) / slots) * ((double)((tiles + c - 1) / c) + fixed);
+    if (c == 1 || now < cost) { best = c; cost = now; }
+  }
+  return (int)best;
+}
+
+template <typename T, int R, bool ROPE>
+cudaError_t launch_state(const Problem& p, const void* k, const void* v, float* partials, const __half2* tab, int* P,
+                         WorkspaceCtrl* ctrl, cudaStream_t stream) {
+  using S = StateShape<T, R, ROPE>;
+  static_assert(S::SMEM <= 227 * 1024, "shared memory of the state kernel");
+  static bool done[64] = {false};
+  const cudaError_t e = allow_smem(split_state_kernel<T, R, ROPE>, S::SMEM, done);
+  if (e != cudaSuccess) return e;
+  *P = pieces((p.N + S::TOK - 1) / S::TOK, p.units(), sms(), fma_chunks(p.N), 6.0);
+  split_state_kernel<T, R, ROPE><<<dim3(*P, p.units()), kBlock, S::SMEM, stream>>>((const T*)k, (const T*)v, p, *P, partials,
+                                                                                    tab, ctrl);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+template <typename T, int R, bool ROPE>
+cudaError_t launch_apply(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* tab,
+                         WorkspaceCtrl* ctrl, cudaStream_t stream) {
+  using A = ApplyShape<T, R, ROPE>;
+  static_assert(A::SMEM <= 227 * 1024, "shared memory of the apply kernel");
+  static bool done[64] = {false};
+  const cudaError_t e = allow_smem(split_apply_kernel<T, R, ROPE>, A::SMEM, done);
+  if (e != cudaSuccess) return e;
+  const int C = pieces((p.N + A::TOK - 1) / A::TOK, p.units(), sms(), 1ll << 30, 4.0);
+  split_apply_kernel<T, R, ROPE><<<dim3(C, p.units()), kBlock, A::SMEM, stream>>>((const T*)q, state, (T*)o, p, eps, tab, ctrl);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+#define LINATTN_SPLIT(FN, T, ROPE, ...)              \
+  switch ((p.d + 15) / 16) {                         \
+    case 2: return FN<T, 2, ROPE>(__VA_ARGS__);      \
+    case 3: return FN<T, 3, ROPE>(__VA_ARGS__);      \
+    case 4: return FN<T, 4, ROPE>(__VA_ARGS__);      \
+    case 5: return FN<T, 5, ROPE>(__VA_ARGS__);      \
+    case 6: return FN<T, 6, ROPE>(__VA_ARGS__);      \
+    case 7: return FN<T, 7, ROPE>(__VA_ARGS__);      \
+    default: return FN<T, 8, ROPE>(__VA_ARGS__);     \
+  }
+
+}  // namespace
+
+// These kernels read rows in 16-byte pieces and the rotations of a piece in one load; everything else (odd head dims,
+// unaligned views) takes the general kernels, and so do head dims up to 16, whose tiles are too small for what a tile
+// costs here (2000 tokens: 100 heads of 8 in bf16 71 against 47 us, 140 heads of 16 in fp32 95 against 69 us; from
+// d = 24 on these kernels win at every size measured, 4000 tokens, 70 heads of 32 in fp32: 103 against 135 us).
+bool split_ok(const Problem& p, const void* a, const void* b, const __half2* rope) {
+  const int per = p.dtype == LINATTN_F32 ? 4 : 8;
+  const uintptr_t tab_align = p.dtype == LINATTN_F32 ? 7 : 15;
+  return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0 && p.d > 16 && p.d % per == 0 && p.sb % per == 0 &&
+         p.sn % per == 0 && p.sh % per == 0 && (reinterpret_cast<uintptr_t>(rope) & tab_align) == 0;
+}
+
+cudaError_t split_state_partials(const Problem& p, const void* k, const void* v, float* partials, const __half2* rope, int* P,
+                                 WorkspaceCtrl* ctrl, cudaStream_t stream) {
+  if (p.dtype == LINATTN_F32) {
+    if (rope) { LINATTN_SPLIT(launch_state, float, true, p, k, v, partials, rope, P, ctrl, stream) }
+    LINATTN_SPLIT(launch_state, float, false, p, k, v, partials, rope, P, ctrl, stream)
+  }
+  if (rope) { LINATTN_SPLIT(launch_state, __nv_bfloat16, true, p, k, v, partials, rope, P, ctrl, stream) }
+  LINATTN_SPLIT(launch_state, __nv_bfloat16, false, p, k, v, partials, rope, P, ctrl, stream)
+}
+
+cudaError_t split_apply(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* rope,
+                        WorkspaceCtrl* ctrl, cudaStream_t stream) {
+  if (p.dtype == LINATTN_F32) {
+    if (rope) { LINATTN_SPLIT(launch_apply, float, true, p, q, state, o, eps, rope, ctrl, stream) }
+    LINATTN_SPLIT(launch_apply, float, false, p, q, state, o, eps, rope, ctrl, stream)
+  }
+  if (rope) { LINATTN_SPLIT(launch_apply, __nv_bfloat16, true, p, q, state, o, eps, rope, ctrl, stream) }
+  LINATTN_SPLIT(launch_apply, __nv_bfloat16, false, p, q, state, o, eps, rope, ctrl, stream)
+}
+
+}  // namespace linattn

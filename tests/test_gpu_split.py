@@ -1,6 +1,6 @@
-"""The fp32-arithmetic path (fp32 tensors, bf16 head dims outside the tensor-core kernel's) at the edges of its tiles:
-every padding class of the head dim, token counts around the staged tiles and the split over CTAs, and the general
-kernels it shares the path with (rows that cannot be read in 16-byte pieces)."""
+"""The fp32-accurate path (fp32 tensors, bf16 head dims outside the fused kernel's) at the edges of its tiles: every
+padding class of the head dim, token counts around the staged tiles and the split over CTAs, and the general kernels it
+shares the path with (rows that cannot be read in 16-byte pieces)."""
 import numpy as np
 import pytest
 
@@ -73,7 +73,7 @@ def test_rows_off_the_16_byte_grid(la, orc, dtype, d):
         return to_dev(x).permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
 
     for place in (shifted, strided, head_major):
-        o = la.linattn_forward(place(q), place(k), place(v), EPS, out=torch.empty_like(place(q)))
+        o = la.linattn_forward(place(q), place(k), place(v), EPS, out=place(q))
         check(dtype, to_f64(o), ref, f"{place.__name__} {dtype} d={d}")
     # an output off the grid beside inputs on it
     out = shifted(q) if dtype == "f32" else None
