@@ -29,6 +29,9 @@
 // Head dims 32 and 64 pack four / two heads into one 128-feature operand (the cross-head blocks of the
 // product are ignored / zero); 112 pads to 128 through TMA out-of-bounds zero fill.
 //
+// A unit of few tokens is taken by one CTA from its first token to its last output instead (SOLO): no grid barrier, no
+// record, no reduce, and an ordinary launch.
+//
 // Warp roles (352 threads): warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-5 ReLU
 // pass, warps 6-9 epilogue, warp 10 output stores.  All cross-role synchronisation is by mbarriers
 // with bounded waits, and the grid barrier is bounded too; a wait that runs out raises a CTA-wide
@@ -63,6 +66,11 @@ constexpr int kRowBytes = 128;      // one swizzle row: 64 bf16
 constexpr int kBox = kTileState * kRowBytes;  // 8 KB: one 64-feature box of a state stage
 constexpr int kTmemCols = 512;
 constexpr int kAccStride = 256;     // TMEM columns between the two accumulator buffers
+
+// rotary variant: floats a partial record carries for z: per warp that sums plain phi(k) (the eight ReLU warps, and
+// the four epilogue warps, which take a share of the second K box in the state pass), per feature
+constexpr int kZSlots = 12;
+constexpr int kZParts = kZSlots * 128;
 
 template <int D>
 struct Cfg {
@@ -99,6 +107,13 @@ struct Cfg {
   static constexpr int DEN_BYTES = D == 112 ? 0 : G * APPLY_SLOTS * kTileApply * 4;
   static constexpr size_t SMEM = 1024 + DATA_BYTES + BAR_BYTES;
   static constexpr size_t SMEM_ROPE = SMEM + DEN_BYTES;
+  // lone CTAs (see solo_drain): the slots, then the warps' sums for z and z, then the unit's state as it is in memory
+  static constexpr int SOLO_SLOTS = D == 128 ? 2 : 3;
+  static constexpr int SOLO_STAGE_BYTES = 4 * kBox;            // no "ones"
+  static constexpr int SOLO_Z = S_BYTES + SOLO_SLOTS * SLOT_BYTES, SOLO_STATE = SOLO_Z + (kZSlots + 1) * 128 * 4;
+  static constexpr int SOLO_DATA = (SOLO_STATE + G * (D + 1) * D * 4 + 127) & ~127;
+  static constexpr size_t SMEM_SOLO = 1024 + SOLO_DATA + BAR_BYTES + DEN_BYTES;
+  static_assert(4 * SOLO_STAGE_BYTES <= SOLO_Z && SMEM_SOLO <= 227 * 1024, "shared memory of a lone CTA");
   // rotary variant: 16-byte chunk of a token's table row (d/2 fp16 pairs) that goes with logical chunk lc of box 0 / 1.
   // With packed heads (d = 32, 64) box 1 starts a new head, so both boxes use the same chunk.
   static constexpr bool SAME_TAB = 64 % D == 0;
@@ -198,14 +213,10 @@ struct FusedParams {
   WorkspaceCtrl* ctrl;
   uint8_t* s_image;        // non-null: the reduce also leaves every unit's S operand (bf16 hi + lo, in the shared-memory
                            // layout) here, S_BYTES per unit, and the apply pass fetches it with one bulk copy
+  int write_state;         // lone CTAs: the new state goes to `state` (a launch whose state nobody reads keeps it on chip)
   const uint4* rope;       // rotary variant: [N][d/8] chunks of four (cos, sin) fp16 pairs; null otherwise
   long long N;             // tokens (bound of the rotary table)
 };
-
-// rotary variant: floats a partial record carries for z: per warp that sums plain phi(k) (the eight ReLU warps, and
-// the four epilogue warps, which take a share of the second K box in the state pass), per feature
-constexpr int kZSlots = 12;
-constexpr int kZParts = kZSlots * 128;
 
 // TMA coordinates (feature, head) of 64-element box `box` (0/1) of head group hg
 template <int D>
@@ -245,6 +256,27 @@ __device__ __forceinline__ void relu_pass(uint8_t* box0, uint8_t* box1, int t) {
     for (int i = 0; i < ROWS / 16; ++i) {
       x[i].x = relu_bf16x2(x[i].x); x[i].y = relu_bf16x2(x[i].y); x[i].z = relu_bf16x2(x[i].z); x[i].w = relu_bf16x2(x[i].w);
       *reinterpret_cast<uint4*>(p1 + i * 16 * kRowBytes) = x[i];
+    }
+  }
+}
+
+// The same, adding the plain values up per thread: z[0..3] for its chunk of box 0, z[4..7] for that of box 1.
+__device__ __forceinline__ void unpack_relu8(const uint4& x, float2 (&f)[4]);
+template <int FEAT, int ROWS>
+__device__ __forceinline__ void relu_sum_pass(uint8_t* box0, uint8_t* box1, int t, float2 (&z)[8]) {
+  relu_pass<FEAT, ROWS>(box0, box1, t);
+  const int row0 = t >> 3, pc = t & 7;
+  const int lc = pc ^ (row0 & 7);
+#pragma unroll
+  for (int box = 0; box < 2; ++box) {
+    if (box == 1 && FEAT < 128 && 64 + lc * 8 >= FEAT) break;
+    const uint8_t* p = (box ? box1 : box0) + row0 * kRowBytes + pc * 16;
+#pragma unroll
+    for (int i = 0; i < ROWS / 16; ++i) {
+      float2 f[4];
+      unpack_relu8(*reinterpret_cast<const uint4*>(p + i * 16 * kRowBytes), f);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) z[4 * box + e] = add2(z[4 * box + e], f[e]);
     }
   }
 }
@@ -660,25 +692,166 @@ __device__ __forceinline__ void build_s_operand(uint8_t* s_op, const float* __re
   }
 }
 
+// ---------------------------------------------------------------- lone CTAs
+// With few tokens a unit's whole work is done by ONE CTA (kernel instantiation SOLO): the epilogue turns the drained
+// accumulators into the apply operand in shared memory where it stands, so that there are no partial records, no grid
+// barriers, no reduce and no operand to fetch.  The state MMA has its operands exchanged, A = V^T and B = phi(K), so
+// that an accumulator lane is a row of the apply operand (a value feature) and a thread stores sixteen bytes of it at a
+// time; with lanes as key features, as the partial records want them, the same step took 20 000 cycles instead of
+// 2 500.  z comes from the ReLU warps' fp32 sums, as in the rotary variant.
+__device__ __forceinline__ void split_hi_lo(const float (&x)[8], uint4& hi, uint4& lo) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    h[e] = pack_bf16x2(x[2 * e], x[2 * e + 1]);
+    l[e] = pack_bf16x2(x[2 * e] - __uint_as_float(h[e] << 16), x[2 * e + 1] - __uint_as_float(h[e] & 0xFFFF0000u));
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Accumulator columns [16 * first, 16 * last) of lane quarter wq (key features; lane = value feature): sums of the four
+// accumulators in a fixed order, on top of the old state when accumulating, to the operand and (write_state) back to
+// where the old state is staged: `st`, copied in at the start and out at the end in one piece (a row per lane straight
+// from and to memory took 15 000 cycles, copies of single rows 5 000).  The lanes' rows there are a multiple of 64 bytes
+// apart, so neighbouring lanes take their four 16-byte pieces in different order: bank conflicts two ways at most.
+// Epilogue and ReLU warps share the columns.
+template <int D>
+__device__ __forceinline__ void solo_drain(const FusedParams& p, uint8_t* s_op, float* st, uint32_t tmem_base, int wq, int lane, int first, int last) {
+  using C = Cfg<D>;
+  const int i = wq * 32 + lane, g = i / D, il = i - g * D;    // row of the operand, its head of the group, value feature
+  const bool live = i < C::FEAT && (int)blockIdx.x % p.HG * C::G + g < p.H;
+  float* row = st + (g * (D + 1) + il) * D;
+  const int rot = (D == 112 ? lane >> 1 : lane) & 3;
+  // x[k] <- x[(k + by) & 3]
+  auto turn = [](float4 (&x)[4], int by) {
+    const float4 y[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = by & 1 ? y[(k + 1) & 3] : y[k];
+    const float4 w[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = by & 2 ? w[(k + 2) & 3] : w[k];
+  };
+  const uint32_t trow = tmem_base + ((uint32_t)(wq * 32) << 16);
+#pragma unroll 1
+  for (int cc = first; cc < last && cc * 16 < C::FEAT; ++cc) {
+    const bool own = live && (C::G == 1 || cc * 16 / D == g);   // blocks across heads are zero
+    float4* at = reinterpret_cast<float4*>(row + (C::G == 1 ? cc * 16 : cc * 16 % D));
+    uint32_t r[4][16];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) tmem_ld_x16(trow + a * 128 + cc * 16, r[a]);
+    tmem_ld_wait();
+    float4 val[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      float f[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        f[e] = own ? __uint_as_float(r[0][4 * x + e]) + __uint_as_float(r[1][4 * x + e]) + __uint_as_float(r[2][4 * x + e]) + __uint_as_float(r[3][4 * x + e]) : 0.f;
+      val[x] = make_float4(f[0], f[1], f[2], f[3]);
+    }
+    if (p.accumulate && own) {
+      float4 old[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) old[k] = at[(k + rot) & 3];
+      turn(old, 4 - rot);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) add4(val[x], old[x]);
+    }
+    if (i < C::FEAT) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float x8[8] = {val[2 * c].x, val[2 * c].y, val[2 * c].z, val[2 * c].w, val[2 * c + 1].x, val[2 * c + 1].y, val[2 * c + 1].z, val[2 * c + 1].w};
+        uint4 hi, lo;
+        split_hi_lo(x8, hi, lo);
+        const int lc = cc * 2 + c;
+        uint8_t* dst = s_op + (lc >> 3) * C::SBOX_BYTES + i * kRowBytes + (((lc & 7) ^ (i & 7)) << 4);
+        *reinterpret_cast<uint4*>(dst) = hi;
+        *reinterpret_cast<uint4*>(dst + 2 * C::SBOX_BYTES) = lo;
+      }
+    }
+    if (p.write_state && own) {
+      turn(val, rot);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) at[(k + rot) & 3] = val[k];
+    }
+  }
+}
+
+// ReLU role: leaves a segment's sums of plain phi(k) in the warp's slot of `slots` and clears them: the four lanes of
+// the warp that share a chunk add up in a fixed order, then one of them stores.
+__device__ __forceinline__ void leave_z(float* slots, float2 (&zacc)[8], int tr, int lc, bool box1_live) {
+  const int w = tr >> 5, r = (tr >> 3) & 3;
+  float tot[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) tot[e] = 0.f;
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr) {
+    const int src = (rr << 3) | (lc ^ ((4 * (w & 1) + rr) & 7));
+#pragma unroll
+    for (int e = 0; e < 16; ++e) tot[e] += __shfl_sync(0xffffffffu, (e & 1) ? zacc[e >> 1].y : zacc[e >> 1].x, src);
+  }
+  if (r == 0) {
+    float* zp = slots + w * 128;
+    *reinterpret_cast<float4*>(zp + 8 * lc) = make_float4(tot[0], tot[1], tot[2], tot[3]);
+    *reinterpret_cast<float4*>(zp + 8 * lc + 4) = make_float4(tot[4], tot[5], tot[6], tot[7]);
+    if (box1_live) {
+      *reinterpret_cast<float4*>(zp + 64 + 8 * lc) = make_float4(tot[8], tot[9], tot[10], tot[11]);
+      *reinterpret_cast<float4*>(zp + 64 + 8 * lc + 4) = make_float4(tot[12], tot[13], tot[14], tot[15]);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) zacc[e] = make_float2(0.f, 0.f);
+}
+
+// One feature of the z rows of the apply operand: z in its head's row, zero in the others.
+template <int D>
+__device__ __forceinline__ void put_z(uint8_t* s_op, int f, float z) {
+  using C = Cfg<D>;
+  const __nv_bfloat16 hi = __float2bfloat16_rn(z), lo = __float2bfloat16_rn(z - __bfloat162float(hi));
+#pragma unroll
+  for (int g = 0; g < C::G; ++g) {
+    const int jrow = C::ZROW + g;
+    uint8_t* at = s_op + (f >> 6) * C::SBOX_BYTES + jrow * kRowBytes + ((((f & 63) >> 3) ^ (jrow & 7)) << 4) + (f & 7) * 2;
+    *reinterpret_cast<__nv_bfloat16*>(at) = g == f / D ? hi : __float2bfloat16_rn(0.f);
+    *reinterpret_cast<__nv_bfloat16*>(at + 2 * C::SBOX_BYTES) = g == f / D ? lo : __float2bfloat16_rn(0.f);
+  }
+}
+
+// z of one feature from the sums the warps left in shared memory; the rotary variant's in reduce_image_zrow's association.
+template <bool ROPE>
+__device__ __forceinline__ float sum_z_slots(const float* slots, int f) {
+  auto slot = [&](int w) { return slots[w * 128 + f]; };
+  float tree = (slot(0) + slot(1)) + (slot(2) + slot(3));
+  if (ROPE) {
+    tree += (slot(4) + slot(5)) + (slot(6) + slot(7));
+    if (f >= 64) tree += (slot(8) + slot(9)) + (slot(10) + slot(11));
+  }
+  return tree;
+}
+
 // ============================================================================ the kernel
-template <int D, bool ROPE>
+template <int D, bool ROPE, bool SOLO>
 __global__ void __launch_bounds__(Roles<ROPE>::THREADS, 1)
 umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                   const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, FusedParams p) {
   using C = Cfg<D>;
   using R = Roles<ROPE>;
-  constexpr int NSA = C::STATE_STAGES;
-  constexpr int STAGE = C::STAGE_BYTES;
-  constexpr int NSC = C::APPLY_SLOTS;
+  constexpr int NSA = SOLO ? 4 : C::STATE_STAGES;
+  constexpr int STAGE = SOLO ? C::SOLO_STAGE_BYTES : C::STAGE_BYTES;
+  constexpr int KOFF = SOLO ? 2 * kBox : C::KOFF;
+  constexpr int NSC = SOLO ? C::SOLO_SLOTS : C::APPLY_SLOTS;
+  constexpr int DATA = SOLO ? C::SOLO_DATA : C::DATA_BYTES;
   constexpr int SLOT = C::SLOT_BYTES;
   constexpr int HALF = SLOT / 2;  // one 64-feature box of 128 tokens
-  constexpr uint32_t IDESC_A = make_idesc_bf16(128, C::NSTATE, true, true);
+  constexpr uint32_t IDESC_A = make_idesc_bf16(128, SOLO ? 128 : C::NSTATE, true, true);
+  constexpr int ACCS = SOLO ? 4 : C::STATE_ACCS, ACC_STRIDE = SOLO ? 128 : C::STATE_ACC_STRIDE;
   constexpr uint32_t IDESC_C = make_idesc_bf16(128, C::NAPPLY, false, false);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint8_t* s_op = smem;                    // apply pass: S operand ...
   uint8_t* slots = smem + C::S_BYTES;      // ... and the Q/O slots; the state pass stages cover both
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::DATA_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + DATA);
   // state pass
   uint64_t* a_full = bars;                 // TMA landed
   uint64_t* a_ready = a_full + NSA;        // ReLU pass done
@@ -695,10 +868,17 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   uint64_t* c_tempty = c_tfull + 2;        // [2] accumulator drained
   uint64_t* s_ready = c_tempty + 2;        // S operand of the current segment is in shared memory
   uint64_t* seg_done = s_ready + 1;        // every MMA of the finished segment is complete
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(seg_done + 1);
+  uint64_t* z_left = seg_done + 1;         // lone CTAs: every warp's share of z is in shared memory ...
+  uint64_t* z_done = z_left + 1;           // ... and (rotary) z itself
+  uint64_t* st_full = z_done + 1;          // lone CTAs: the old state is in shared memory
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(st_full + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  float* den_rows = reinterpret_cast<float*>(smem + C::DATA_BYTES + C::BAR_BYTES);   // [NSC][G][128]: rotary variant, every head dim but 112
-  static_assert((3 * NSA + 5 + 4 * NSC + 6) * 8 + 8 <= C::BAR_BYTES, "barrier block too small");
+  float* den_rows = reinterpret_cast<float*>(smem + DATA + C::BAR_BYTES);   // [NSC][G][128]: rotary variant, every head dim but 112
+  static_assert((3 * NSA + 5 + 4 * NSC + 9) * 8 + 8 <= C::BAR_BYTES, "barrier block too small");
+  // lone CTAs: [kZSlots][128] sums of plain phi(k), then z, then the state, behind the stages and the slots
+  float* z_slots = reinterpret_cast<float*>(smem + C::SOLO_Z);
+  float* z_row = z_slots + kZParts;
+  float* st = reinterpret_cast<float*>(smem + C::SOLO_STATE);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Work wa = p.do_state ? work_of(p.sa, blockIdx.x) : work_of(p.sa, 0x7fffffff);
@@ -707,9 +887,9 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   // generation of the grid-barrier word before this launch's first barrier (it cannot move until every CTA, this
   // one included, has arrived): read once, early, so that an arrival needs no answer from memory
   unsigned gen0 = 0;
-  if (threadIdx.x == 0 && p.do_state) gen0 = ld_acquire_gpu(&p.ctrl->barrier[0]) >> 16;
+  if (!SOLO && threadIdx.x == 0 && p.do_state) gen0 = ld_acquire_gpu(&p.ctrl->barrier[0]) >> 16;
   if (threadIdx.x == 0) {
-    if (blockIdx.x == 0 && p.do_state) grid_barrier_preset(p.ctrl);   // for the first grid barrier
+    if (!SOLO && blockIdx.x == 0 && p.do_state) grid_barrier_preset(p.ctrl);   // for the first grid barrier
     for (int s = 0; s < NSA; ++s) { mbar_init(&a_full[s], 1); mbar_init(&a_ready[s], R::RELU_THREADS + (ROPE ? 128 : 0)); mbar_init(&a_empty[s], 1); }
     mbar_init(a_tfull, 1);
     mbar_init(a_tempty, 128);
@@ -720,6 +900,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     for (int b = 0; b < 2; ++b) { mbar_init(&c_tfull[b], 1); mbar_init(&c_tempty[b], 128); }
     mbar_init(s_ready, R::RELU_THREADS + 128);
     mbar_init(seg_done, 128);
+    if (SOLO) { mbar_init(z_left, R::RELU_THREADS + (ROPE ? 128 : 0)); mbar_init(z_done, R::RELU_THREADS); mbar_init(st_full, 1); }
     *abort_flag = 0;
     fence_mbar_init();
     prefetch_tensormap(&map_k);
@@ -727,7 +908,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     prefetch_tensormap(&map_q);
     prefetch_tensormap(&map_o);
   }
-  if (C::ONES_BOX && wa.f1 > wa.f0) {
+  if (!SOLO && C::ONES_BOX && wa.f1 > wa.f0) {
     // the constant "ones" chunk of every stage: value columns 128..191 of B, of which column 128 is 1
     for (int idx = threadIdx.x; idx < NSA * (kBox / 16); idx += R::THREADS) {
       const int s = idx / (kBox / 16), c = idx % (kBox / 16);
@@ -776,10 +957,10 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         mbar_arrive_expect_tx(&a_full[s], 4 * kBox);
         int c0, c1;
         box_coords<D>(0, hg, c0, c1);
-        tma_load_4d(st + C::KOFF, &map_k, &a_full[s], c0, c1, t.tile() * kTileState, b);
+        tma_load_4d(st + KOFF, &map_k, &a_full[s], c0, c1, t.tile() * kTileState, b);
         tma_load_4d(st, &map_v, &a_full[s], c0, c1, t.tile() * kTileState, b);
         box_coords<D>(1, hg, c0, c1);
-        tma_load_4d(st + C::KOFF + kBox, &map_k, &a_full[s], c0, c1, t.tile() * kTileState, b);
+        tma_load_4d(st + KOFF + kBox, &map_k, &a_full[s], c0, c1, t.tile() * kTileState, b);
         tma_load_4d(st + kBox, &map_v, &a_full[s], c0, c1, t.tile() * kTileState, b);
       }
       // Q does not depend on the state: fill the slots as soon as every MMA of this pass is complete (the
@@ -805,10 +986,10 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         const uint32_t st = smem_u32(smem + s * STAGE);
 #pragma unroll
         for (int kk = 0; kk < kTileState / 16; ++kk, ++n_mma) {
-          const uint64_t a = make_smem_desc_sw128(st + C::KOFF + kk * 2048, kBox, 1024);  // phi(K)^T, MN-major
+          const uint64_t a = make_smem_desc_sw128(st + KOFF + kk * 2048, kBox, 1024);  // phi(K)^T, MN-major
           const uint64_t bq = make_smem_desc_sw128(st + kk * 2048, kBox, 1024);           // [V | 1], MN-major
-          const uint32_t d_tmem = tmem_base + (n_mma % C::STATE_ACCS) * C::STATE_ACC_STRIDE;
-          umma_bf16(d_tmem, a, bq, IDESC_A, n_mma < (uint32_t)C::STATE_ACCS ? 0u : 1u);  // first use of each: overwrite
+          const uint32_t d_tmem = tmem_base + (n_mma % ACCS) * ACC_STRIDE;
+          umma_bf16(d_tmem, SOLO ? bq : a, SOLO ? a : bq, IDESC_A, n_mma < (uint32_t)ACCS ? 0u : 1u);  // first use of each: overwrite
         }
         umma_commit(&a_empty[s]);
         if (t.seg_last()) { umma_commit(a_tfull); ++seg; }
@@ -842,6 +1023,36 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         }
       }
     };
+    // lone CTAs: z from the warps' sums, to memory and (plain) into the operand or (rotary) where this role finds it
+    auto finish_z = [&]() {
+      mbar_arrive(z_left);
+      mbar_wait(z_left, 0, abort_flag);             // every warp's sums are in shared memory
+      if (!ROPE) mbar_wait(a_done, 0, abort_flag);  // the operand lies where the stages were
+      const int f = tr, g = f / D, h = ((int)blockIdx.x % p.HG) * C::G + g;
+      if (p.accumulate) mbar_wait(st_full, 0, abort_flag);
+      if (f < C::FEAT) {
+        float z = sum_z_slots<ROPE>(z_slots, f);
+        float* at = st + (g * (D + 1) + D) * D + (f - g * D);
+        if (p.accumulate && h < p.H) z += *at;
+        if (p.write_state) *at = z;
+        if (ROPE) z_row[f] = z;
+        else put_z<D>(s_op, f, z);
+      }
+      if (ROPE) {
+        mbar_arrive(z_done);
+        mbar_wait(z_done, 0, abort_flag);
+      }
+      // this role's share of the drain
+      if (__all_sync(0xffffffffu, mbar_wait(a_tfull, 0, abort_flag))) {
+        tcgen05_fence_after();
+        const int half = tr >> 7;   // (rotary variant: two warps of this role to a lane quarter)
+        if (ROPE) solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 3 + 3 * half, half ? 8 : 6);
+        else solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 4, 8);
+        tcgen05_fence_before();
+      }
+      fence_proxy_async_smem();
+      mbar_arrive(s_ready);
+    };
     if (ROPE) {
       TileWalk t0(wa);
       if (!t0.done()) {
@@ -856,7 +1067,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         TileWalk tn = t;
         tn.next();
         if (!__all_sync(0xffffffffu, mbar_wait(&a_full[s], (it / NSA) & 1, abort_flag))) break;  // leave as a whole warp
-        uint8_t* p0 = st + C::KOFF + row0 * kRowBytes + pc * 16;
+        uint8_t* p0 = st + KOFF + row0 * kRowBytes + pc * 16;
 #pragma unroll
         for (int i = 0; i < kTileState / 32; ++i) {
           float2 f[4];
@@ -877,34 +1088,24 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         fence_proxy_async_smem();
         mbar_arrive(&a_ready[s]);
         if (t.seg_last()) {
-          // leave the segment's sums behind the record: the four lanes of this warp that share a chunk add
-          // up in a fixed order, then one of them stores
-          const int w = tr >> 5, r = (tr >> 3) & 3;
-          float tot[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) tot[e] = 0.f;
-#pragma unroll
-          for (int rr = 0; rr < 4; ++rr) {
-            const int src = (rr << 3) | (lc ^ ((4 * (w & 1) + rr) & 7));
-#pragma unroll
-            for (int e = 0; e < 16; ++e) tot[e] += __shfl_sync(0xffffffffu, (e & 1) ? zacc[e >> 1].y : zacc[e >> 1].x, src);
-          }
-          if (r == 0) {
-            float* zp = p.partials + (size_t)t.record() * (C::G * (D + 1) * D + kZParts) + C::G * (D + 1) * D + w * 128;
-            *reinterpret_cast<float4*>(zp + 8 * lc) = make_float4(tot[0], tot[1], tot[2], tot[3]);
-            *reinterpret_cast<float4*>(zp + 8 * lc + 4) = make_float4(tot[4], tot[5], tot[6], tot[7]);
-            if (box1_live) {
-              *reinterpret_cast<float4*>(zp + 64 + 8 * lc) = make_float4(tot[8], tot[9], tot[10], tot[11]);
-              *reinterpret_cast<float4*>(zp + 64 + 8 * lc + 4) = make_float4(tot[12], tot[13], tot[14], tot[15]);
-            }
-          }
-#pragma unroll
-          for (int e = 0; e < 8; ++e) zacc[e] = make_float2(0.f, 0.f);
+          leave_z(SOLO ? z_slots : p.partials + (size_t)t.record() * (C::G * (D + 1) * D + kZParts) + C::G * (D + 1) * D, zacc, tr, lc, box1_live);
+          if (SOLO) finish_z();
+        }
+        continue;
+      }
+      if (SOLO) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&a_full[s], (it / NSA) & 1, abort_flag))) break;  // leave as a whole warp
+        relu_sum_pass<C::FEAT, kTileState>(st + KOFF, st + KOFF + kBox, tr, zacc);
+        fence_proxy_async_smem();
+        mbar_arrive(&a_ready[s]);
+        if (t.seg_last()) {
+          leave_z(z_slots, zacc, tr, lc, box1_live);
+          finish_z();
         }
         continue;
       }
       if (!mbar_wait(&a_full[s], (it / NSA) & 1, abort_flag)) break;
-      relu_pass<C::FEAT, kTileState>(st + C::KOFF, st + C::KOFF + kBox, tr);
+      relu_pass<C::FEAT, kTileState>(st + KOFF, st + KOFF + kBox, tr);
       if (!C::ONES_BOX && tr < kTileState) {
         // value column 112 := 1 (logical chunk 6 of the second V box, element 0), so z is accumulator column 112
         *reinterpret_cast<uint16_t*>(st + kBox + tr * kRowBytes + ((6 ^ (tr & 7)) << 4)) = 0x3F80u;
@@ -943,7 +1144,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         TileWalk tn = t;
         tn.next();
         if (!__all_sync(0xffffffffu, mbar_wait(&a_full[s], (it / NSA) & 1, abort_flag))) break;  // leave as a whole warp
-        uint8_t* p1 = smem + s * STAGE + C::KOFF + kBox + (32 + row0h) * kRowBytes + pch * 16;
+        uint8_t* p1 = smem + s * STAGE + KOFF + kBox + (32 + row0h) * kRowBytes + pch * 16;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           if (h_live) {
@@ -971,10 +1172,11 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             for (int e = 0; e < 8; ++e) tot[e] += __shfl_sync(0xffffffffu, (e & 1) ? zh[e >> 1].y : zh[e >> 1].x, src);
           }
           if (rq == 0 && h_live) {
-            float* zp = p.partials + (size_t)t.record() * (C::G * (D + 1) * D + kZParts) + C::G * (D + 1) * D + (8 + (te >> 5)) * 128;
+            float* zp = (SOLO ? z_slots : p.partials + (size_t)t.record() * (C::G * (D + 1) * D + kZParts) + C::G * (D + 1) * D) + (8 + (te >> 5)) * 128;
             *reinterpret_cast<float4*>(zp + 64 + 8 * lch) = make_float4(tot[0], tot[1], tot[2], tot[3]);
             *reinterpret_cast<float4*>(zp + 64 + 8 * lch + 4) = make_float4(tot[4], tot[5], tot[6], tot[7]);
           }
+          if (SOLO) mbar_arrive(z_left);
 #pragma unroll
           for (int e = 0; e < 4; ++e) zh[e] = make_float2(0.f, 0.f);
         }
@@ -984,6 +1186,14 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tcgen05_fence_after();
+      if (SOLO) {
+        if (p.accumulate) { mbar_wait(st_full, 0, abort_flag); __syncwarp(); }
+        solo_drain<D>(p, s_op, st, tmem_base, wq, lane, 0, ROPE ? 3 : 4);
+        fence_proxy_async_smem();   // the operand is read by the MMAs of the apply pass
+        tcgen05_fence_before();
+        mbar_arrive(s_ready);
+        continue;
+      }
       const int u = t.unit(), hg = u % p.HG;
       const int h = hg * C::G + g;
       const bool live = i < C::FEAT && h < p.H;
@@ -1034,6 +1244,22 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       mbar_arrive(a_tempty);
       ++seg;
     }
+  } else if (SOLO) {
+    // ------------------------------------------------------------ store warp: the state in, and out again
+    if (lane == 0) {
+      const int b = (int)blockIdx.x / p.HG, h0 = ((int)blockIdx.x % p.HG) * C::G, heads = p.H - h0 < C::G ? p.H - h0 : C::G;
+      const size_t at = (size_t)(b * p.H + h0) * ((D + 1) * D);
+      const uint32_t bytes = heads * (D + 1) * D * 4;
+      if (p.accumulate) {
+        mbar_arrive_expect_tx(st_full, bytes);
+        bulk_load(st, p.state_base + at, bytes, st_full);
+      }
+      if (p.write_state && mbar_wait(s_ready, 0, abort_flag)) {
+        bulk_store(p.state + at, st, bytes);
+        tma_store_commit();
+      }
+    }
+    __syncwarp();
   } else if (C::G == 1 && p.s_image && p.accumulate && p.do_state && (int)blockIdx.x < p.sa.P * p.sa.U) {
     // ------------------------------------------------------------ store warp (idle in this pass)
     // A cached step adds to the old state, which the K, V stream has pushed out of L2 since the last step:
@@ -1050,7 +1276,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   }
 
   // ==================================================================== reduce
-  if (p.do_state) {
+  if (!SOLO && p.do_state) {
     grid_barrier(p.ctrl, abort_flag, p.do_apply != 0, gen0);
     if (!*abort_flag) {
       if (C::G == 1 && p.s_image) reduce_image<D, ROPE>(p);
@@ -1058,7 +1284,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     }
     if (p.do_apply) grid_barrier(p.ctrl, abort_flag, false, gen0 + 1);
   }
-  if (C::G > 1 && wc.f1 > wc.f0) {
+  if (!SOLO && C::G > 1 && wc.f1 > wc.f0) {
     // cross-head blocks of the packed S operand are never written by a head: they must read as zero
     for (int idx = threadIdx.x; idx < C::S_BYTES / 16; idx += R::THREADS)
       *reinterpret_cast<uint4*>(s_op + idx * 16) = make_uint4(0, 0, 0, 0);
@@ -1137,7 +1363,8 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         if (seg > 0) ok = mbar_wait(seg_done, (seg - 1) & 1, abort_flag);
         if (!ok) break;
         const int u = t.unit();
-        if (C::G == 1 && p.s_image) {
+        if (SOLO) {
+        } else if (C::G == 1 && p.s_image) {
           if (tr == 0) {   // the unit's operand image, made by the reduce: one bulk copy
             fence_proxy_async_all();
             mbar_arrive_expect_tx(s_ready, C::S_BYTES);
@@ -1155,7 +1382,12 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             const int f0 = 64 * box + 8 * lc, g = f0 / D, fl = f0 - g * D;
             const int h = (u % p.HG) * C::G + g;
             float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
-            if ((box == 0 || box1_live) && h < p.H) {
+            if (SOLO) {
+              if (box == 0 || box1_live) {
+                a0 = *reinterpret_cast<const float4*>(z_row + f0);
+                a1 = *reinterpret_cast<const float4*>(z_row + f0 + 4);
+              }
+            } else if ((box == 0 || box1_live) && h < p.H) {
               const float4* zrow = reinterpret_cast<const float4*>(p.state + ((size_t)((u / p.HG) * p.H + h) * (D + 1) + D) * D);
               a0 = __ldcg(zrow + fl / 4);
               a1 = __ldcg(zrow + fl / 4 + 1);
@@ -1164,7 +1396,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             zc[4 * box + 2] = make_float2(a1.x, a1.y); zc[4 * box + 3] = make_float2(a1.z, a1.w);
           }
         }
-        if (!(C::G == 1 && p.s_image)) {
+        if (!SOLO && !(C::G == 1 && p.s_image)) {
           fence_proxy_async_smem();
           mbar_arrive(s_ready);
         }
@@ -1247,7 +1479,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     uint32_t it = 0;
     for (TileWalk t(wc); !t.done(); t.next(), ++it) {
       const int s = it % NSC;
-      if (t.seg_first()) {
+      if (!SOLO && t.seg_first()) {
         // this thread has seen the last accumulator of the previous segment complete: S may be rebuilt
         const int u = t.unit();
         if (!(C::G == 1 && p.s_image)) {
@@ -1352,6 +1584,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         for (int par = 0; par < 2; ++par)
           for (int spin = 0; spin < 4096 && !mbar_try_wait(s < NSA ? &a_full[s] : &c_full[s - NSA], par); ++spin)
             __nanosleep(64);
+      for (int spin = 0; SOLO && p.accumulate && spin < 4096 && !mbar_try_wait(st_full, 0); ++spin) __nanosleep(64);
     }
     __syncthreads();
   }
@@ -1414,7 +1647,41 @@ int sm_count() {
   return cached[dev];
 }
 
+// One CTA per unit instead of all CTAs on all units?  A lone CTA takes about 9 us and 1.2 us for every 64 tokens of its
+// unit; the grid takes about 14 us (two grid barriers, the partial records, the reduce and the operand images between the
+// passes) and a time that grows with all units' tokens together.  Measured, d = 112, plain forward / cached step:
+//   20 units:   64 tokens 10.3 / 10.3 us against 18.5 / 20.2, 256: 12.3 / 14.3 against 16.4 / 17.4, 384: 14.7 / 16.4 against
+//               16.8 / 16.9, 512: 18.5 / 18.5 against 17.8 / 18.4;
+//   60 units:  512: 18.5 / 18.5 against 22.5 / 22.6;   140 units: 512: 20.4 / 20.5 against 28.7 / 29.5.
+// The choice depends on the shape alone, so that all calls on one shape (forward, state and apply, step, peek, the
+// token-sharded three) add up in the same order and give the same bits.
+inline bool solo_pays(const Problem& p, int U, int sms) {
+  return U <= sms && (p.N <= 384 || (p.N <= 512 && 3 * U >= sms));
+}
+
 inline int groups_of(int d) { return d == 32 ? 4 : d == 64 ? 2 : 1; }
+
+// Instantiates and launches the kernel: cooperatively when its CTAs wait for one another.
+template <int D, bool ROPE, bool SOLO>
+int launch_kernel(int grid, void** args, cudaStream_t stream) {
+  using C = Cfg<D>;
+  // the opt-in to more than 48 KB of dynamic shared memory is a per-device setting of the kernel
+  static bool attr_set[64] = {false};
+  constexpr size_t kSmem = SOLO ? C::SMEM_SOLO : ROPE ? C::SMEM_ROPE : C::SMEM;
+  const void* kernel = (const void*)umma_fused_kernel<D, ROPE, SOLO>;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LINATTN_ERR_CUDA;
+  if (!attr_set[dev]) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) != cudaSuccess) return LINATTN_ERR_CUDA;
+    attr_set[dev] = true;
+  }
+  const dim3 block(Roles<ROPE>::THREADS);
+  const cudaError_t e = SOLO ? cudaLaunchKernel(kernel, dim3(grid), block, args, kSmem, stream)
+                             : cudaLaunchCooperativeKernel(kernel, dim3(grid), block, args, kSmem, stream);
+  if (e != cudaSuccess) { cudaGetLastError(); return LINATTN_ERR_CUDA; }
+  count_launches(1);
+  return LINATTN_OK;
+}
 
 template <int D, bool ROPE>
 int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStream_t stream) {
@@ -1449,6 +1716,16 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   // a unit switch costs the apply pass about one tile when the S operand comes as an image, two when the CTA
   // builds it from the fp32 state
   fp.sc = make_sched(U, (p.N + kTileApply - 1) / kTileApply, sms, fp.s_image ? 1 : 2);
+  const bool solo = do_state && solo_pays(p, U, sms);
+  if (solo) {
+    fp.sa.U = fp.sc.U = fp.sa.grid = fp.sc.grid = U;
+    fp.sa.P = fp.sc.P = 1;
+    fp.sa.R = fp.sc.R = fp.sa.m = fp.sc.m = 0;
+    fp.sa.Lc = fp.sa.tpu;
+    fp.sc.Lc = fp.sc.tpu;
+    // in a launch that applies, only a cache that takes the block needs the sum in memory
+    fp.write_state = !do_apply || (c.accumulate && fp.state_base == fp.state);
+  }
   int grid = 0;
   if (do_state) grid = fp.sa.grid;
   if (do_apply && fp.sc.grid > grid) grid = fp.sc.grid;
@@ -1464,23 +1741,8 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
     mq = mk; mo = mk;  // never dereferenced
   }
   if (!do_state) { mk = mq; mv = mq; }
-  // the opt-in to more than 48 KB of dynamic shared memory is a per-device setting of the kernel
-  static bool attr_set[64] = {false};
-  constexpr size_t kSmem = ROPE ? C::SMEM_ROPE : C::SMEM;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LINATTN_ERR_CUDA;
-  if (!attr_set[dev]) {
-    if (cudaFuncSetAttribute(umma_fused_kernel<D, ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) !=
-        cudaSuccess)
-      return LINATTN_ERR_CUDA;
-    attr_set[dev] = true;
-  }
   void* args[] = {&mk, &mv, &mq, &mo, &fp};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)umma_fused_kernel<D, ROPE>, dim3(grid), dim3(Roles<ROPE>::THREADS), args,
-                                                    kSmem, stream);
-  if (e != cudaSuccess) { cudaGetLastError(); return LINATTN_ERR_CUDA; }
-  count_launches(1);
-  return LINATTN_OK;
+  return solo ? launch_kernel<D, ROPE, true>(grid, args, stream) : launch_kernel<D, ROPE, false>(grid, args, stream);
 }
 
 }  // namespace
