@@ -15,6 +15,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 __all__ = [
     "LinAttnError", "library_path", "load_library", "state_bytes", "workspace_bytes", "new_workspace",
@@ -65,7 +66,7 @@ def load_library(path: str | None = None):
         p = _build.build()
     lib = ctypes.CDLL(p)
     vp, i64, sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_size_t
-    dp = ctypes.POINTER(_Desc)
+    dp = vp      # descriptors: byref(_Desc) or the packed bytes of one
     szp = ctypes.POINTER(sz)
     f32 = ctypes.c_float
     sig = {
@@ -102,11 +103,11 @@ def load_library(path: str | None = None):
         "blocklin_cache_joint_prefill": ([vp, ctypes.c_int], ctypes.c_int),
         "blocklin_cache_info": ([vp, ctypes.POINTER(i64), ctypes.POINTER(i64), szp], ctypes.c_int),
         "blocklin_cache_destroy": ([vp], ctypes.c_int),
-        "tconv_cache_bytes": ([ctypes.POINTER(_ConvDesc), szp], ctypes.c_int),
-        "tconv_cache_reset": ([ctypes.POINTER(_ConvDesc), vp, vp], ctypes.c_int),
-        "tconv_forward": ([ctypes.POINTER(_ConvDesc), i64, vp, vp, vp, vp], ctypes.c_int),
-        "tconv_block_step": ([ctypes.POINTER(_ConvDesc), i64, vp, vp, vp, vp, ctypes.c_int, vp], ctypes.c_int),
-        "tconv_prefill": ([ctypes.POINTER(_ConvDesc), i64, i64, vp, vp, vp, vp, vp], ctypes.c_int),
+        "tconv_cache_bytes": ([dp, szp], ctypes.c_int),
+        "tconv_cache_reset": ([dp, vp, vp], ctypes.c_int),
+        "tconv_forward": ([dp, i64, vp, vp, vp, vp], ctypes.c_int),
+        "tconv_block_step": ([dp, i64, vp, vp, vp, vp, ctypes.c_int, vp], ctypes.c_int),
+        "tconv_prefill": ([dp, i64, i64, vp, vp, vp, vp, vp], ctypes.c_int),
     }
     for name, (argtypes, restype) in sig.items():
         fn = getattr(lib, name)
@@ -121,38 +122,54 @@ def _check(status: int, where: str):
         raise LinAttnError(status, where)
 
 
-def _torch():
-    import torch
+_torch_module = None
 
-    return torch
+
+def _torch():
+    global _torch_module
+    if _torch_module is None:
+        import torch
+
+        _torch_module = torch
+    return _torch_module
 
 
 def _dtype_code(t) -> int:
     torch = _torch()
-    if t.dtype == torch.bfloat16:
+    dtype = t.dtype
+    if dtype is torch.bfloat16:
         return LINATTN_BF16
-    if t.dtype == torch.float32:
+    if dtype is torch.float32:
         return LINATTN_F32
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    raise TypeError(f"unsupported dtype {dtype}")
 
 
-def _desc_of(t, *same) -> _Desc:
+# The descriptors as the bytes the library reads.  With few tokens a call's time is the time Python takes to make it
+# (a tiny forward: 15.2 us a call with ctypes structures, pointer objects and torch.cuda.current_stream, of which the
+# library's own launch is 2.6), so the calls below look at every tensor once and pass plain integers and bytes.
+_pack_desc = struct.Struct("=4i3q").pack      # _Desc
+_pack_conv = struct.Struct("=4i2q").pack      # _ConvDesc
+
+
+def _desc_of(t, *same) -> bytes:
     """Descriptor for a [B, N, H, d] tensor; every tensor in `same` must share its layout."""
-    if t.dim() != 4 or t.stride(3) != 1 or not t.is_cuda:
+    shape, stride = t.shape, t.stride()
+    if len(shape) != 4 or stride[3] != 1 or not t.is_cuda:
         raise ValueError("expected a CUDA tensor [B, N, H, d] with a contiguous last axis")
+    dtype, device = t.dtype, t.get_device()
     for o in same:
-        if o.shape != t.shape or o.stride() != t.stride() or o.dtype != t.dtype or o.device != t.device:
+        if o.shape != shape or o.stride() != stride or o.dtype is not dtype or o.get_device() != device:
             raise ValueError("q, k, v, o must share shape, strides, dtype and device")
-    B, N, H, d = t.shape
-    return _Desc(B, H, d, _dtype_code(t), t.stride(0), t.stride(1), t.stride(2))
+    return _pack_desc(shape[0], shape[2], shape[3], _dtype_code(t), stride[0], stride[1], stride[2])
 
 
 def _stream(t) -> int:
-    return _torch().cuda.current_stream(t.device).cuda_stream
+    """The current stream of t's device, as torch.cuda.current_stream(t.device).cuda_stream gives it."""
+    return _torch()._C._cuda_getCurrentRawStream(t.get_device())
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def state_bytes(B: int, H: int, d: int) -> int:
@@ -195,7 +212,7 @@ def linattn_forward(q, k, v, eps: float = 1e-6, out=None, workspace=None):
     o = torch.empty_like(q) if out is None else out
     desc = _desc_of(q, k, v, o)
     ws = new_workspace(q) if workspace is None else workspace
-    _check(lib.linattn_forward(ctypes.byref(desc), q.shape[1], _ptr(q), _ptr(k), _ptr(v), _ptr(o), eps,
+    _check(lib.linattn_forward(desc, q.shape[1], _ptr(q), _ptr(k), _ptr(v), _ptr(o), eps,
                                _ptr(ws), ws.numel(), _stream(q)), "linattn_forward")
     return o
 
@@ -236,12 +253,12 @@ def linattn_forward_rope(q, k, v, rope_table, eps: float = 1e-6, out=None, works
     o = torch.empty_like(q) if out is None else out
     desc = _desc_of(q, k, v, o)
     B, N, H, d = q.shape
-    if tuple(rope_table.shape) != (N, d // 2, 2) or rope_table.dtype != torch.float16 or \
+    if rope_table.shape != (N, d // 2, 2) or rope_table.dtype is not torch.float16 or \
             not rope_table.is_contiguous() or rope_table.device != q.device:
         raise ValueError("rope_table must be a contiguous float16 [N, d//2, 2] tensor on the device of q")
     if workspace is None:
         workspace = new_rope_workspace(q)
-    _check(lib.linattn_forward_rope(ctypes.byref(desc), N, _ptr(q), _ptr(k), _ptr(v), _ptr(o), eps, _ptr(rope_table),
+    _check(lib.linattn_forward_rope(desc, N, _ptr(q), _ptr(k), _ptr(v), _ptr(o), eps, _ptr(rope_table),
                                     _ptr(workspace), workspace.numel(), _stream(q)), "linattn_forward_rope")
     return o
 
@@ -292,7 +309,7 @@ def linattn_state(k, v, out=None, workspace=None):
     B, N, H, d = k.shape
     st = torch.empty((B, H, d + 1, d), dtype=torch.float32, device=k.device) if out is None else out
     ws = new_workspace(k) if workspace is None else workspace
-    _check(lib.linattn_state(ctypes.byref(desc), N, _ptr(k), _ptr(v), _ptr(st), _ptr(ws), ws.numel(), _stream(k)),
+    _check(lib.linattn_state(desc, N, _ptr(k), _ptr(v), _ptr(st), _ptr(ws), ws.numel(), _stream(k)),
            "linattn_state")
     return st
 
@@ -314,7 +331,7 @@ def linattn_state_static_scratch(k, v, out):
     B, N, H, d = k.shape
     if tuple(out.shape) != (B, H, d + 1, d) or out.dtype != torch.float32 or not out.is_contiguous():
         raise ValueError("out must be a contiguous float32 [B, H, d+1, d] tensor")
-    _check(lib.linattn_state_static_scratch(ctypes.byref(desc), N, _ptr(k), _ptr(v), _ptr(out), _stream(k)),
+    _check(lib.linattn_state_static_scratch(desc, N, _ptr(k), _ptr(v), _ptr(out), _stream(k)),
            "linattn_state_static_scratch")
     return out
 
@@ -339,7 +356,7 @@ def linattn_apply(q, state, eps: float = 1e-6, out=None, workspace=None):
     if tuple(state.shape) != (B, H, d + 1, d) or state.dtype != torch.float32 or not state.is_contiguous():
         raise ValueError("state must be a contiguous float32 [B, H, d+1, d] tensor")
     ws = new_workspace(q, 0) if workspace is None else workspace
-    _check(lib.linattn_apply(ctypes.byref(desc), N, _ptr(q), _ptr(state), _ptr(o), eps, _ptr(ws), ws.numel(),
+    _check(lib.linattn_apply(desc, N, _ptr(q), _ptr(state), _ptr(o), eps, _ptr(ws), ws.numel(),
                              _stream(q)), "linattn_apply")
     return o
 
@@ -369,6 +386,7 @@ class BlockLinCache:
         if code is None:
             raise TypeError(f"unsupported dtype {dtype}")
         self._desc = _Desc(B, H, d, code, *strides)
+        self._shape, self._dtype, self._strides = (B, H, d), dtype, tuple(strides)
         state_bytes_, nbytes = self.sizes(B, H, d, dtype, max_T_b, prefill_blocks, strides)
         if state is None:
             state = torch.empty((B, H, d + 1, d), dtype=torch.float32, device=device)
@@ -436,7 +454,7 @@ class BlockLinCache:
             _desc_of(k, v)
         self._check_layout(k)
         d = k.shape[3]
-        if tuple(table.shape) != (rows, d // 2, 2) or table.dtype != torch.float16 or not table.is_contiguous() \
+        if table.shape != (rows, d // 2, 2) or table.dtype is not torch.float16 or not table.is_contiguous() \
                 or table.device != k.device:
             raise ValueError("the rotary table must be a contiguous float16 [tokens, d//2, 2] tensor on the blocks' device")
         return o
@@ -505,15 +523,15 @@ class BlockLinCache:
 
     def _check_layout(self, t):
         """The cache's descriptor fixes (B, H, d, dtype, strides); a block must match it."""
-        dsc = self._desc
-        if (t.shape[0], t.shape[2], t.shape[3]) != (dsc.B, dsc.H, dsc.d) or _dtype_code(t) != dsc.dtype:
+        shape = t.shape
+        if (shape[0], shape[2], shape[3]) != self._shape or t.dtype is not self._dtype:
+            _dtype_code(t)   # (a dtype the library does not know is a TypeError)
             raise ValueError("block does not match the cache's (B, H, d, dtype)")
-        want = (dsc.stride_b, dsc.stride_n, dsc.stride_h)
-        if want == (0, 0, 0):
+        if self._strides == (0, 0, 0):
             if not t.is_contiguous():
                 raise ValueError("this cache was created for dense [B, T_b, H, d] blocks")
-        elif t.numel() and tuple(t.stride()[:3]) != want:
-            raise ValueError(f"block strides {tuple(t.stride()[:3])} differ from the cache's {want}")
+        elif t.numel() and t.stride()[:3] != self._strides:
+            raise ValueError(f"block strides {tuple(t.stride()[:3])} differ from the cache's {self._strides}")
 
     def info(self) -> dict:
         b, t, s = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_size_t()
@@ -535,25 +553,29 @@ class BlockLinCache:
 
 # ---- temporal convolution of the Mix-FFN (tconv.h) ----
 
-def _conv_desc_of(x, y=None) -> _ConvDesc:
+def _conv_desc_of(x, y=None) -> bytes:
     """Descriptor for x[B, T, HW, D] (and y): frames, positions and channels dense, any batch stride."""
-    B, T, HW, D = x.shape if x.dim() == 4 else (0, 0, 0, 0)
-    strides = []
-    for t in (x, y):
-        if t is None:
-            strides.append(0)
-            continue
-        if t.dim() != 4 or not t.is_cuda or t.shape != x.shape or t.dtype != x.dtype or t.device != x.device:
-            raise ValueError("expected CUDA tensors [B, T, HW, D] of one shape, dtype and device")
-        if T > 0 and (t.stride(3) != 1 or t.stride(2) != D or (T > 1 and t.stride(1) != HW * D)):
-            raise ValueError("frames, positions and channels must be dense")
-        strides.append(t.stride(0) if B > 1 and T > 0 else 0)
-    return _ConvDesc(B, HW, D, _dtype_code(x), strides[0], strides[1])
+    shape = x.shape
+    if len(shape) != 4 or not x.is_cuda:
+        raise ValueError("expected CUDA tensors [B, T, HW, D] of one shape, dtype and device")
+    if y is not None and (y.shape != shape or y.dtype is not x.dtype or y.get_device() != x.get_device()):
+        raise ValueError("expected CUDA tensors [B, T, HW, D] of one shape, dtype and device")
+    B, T, HW, D = shape
+    batch = [0, 0]
+    if T > 0:
+        for i, t in enumerate((x, y)):
+            if t is None:
+                continue
+            stride = t.stride()
+            if stride[3] != 1 or stride[2] != D or (T > 1 and stride[1] != HW * D):
+                raise ValueError("frames, positions and channels must be dense")
+            if B > 1:
+                batch[i] = stride[0]
+    return _pack_conv(B, HW, D, _dtype_code(x), batch[0], batch[1])
 
 
 def _check_taps(w, D):
-    torch = _torch()
-    if w.dtype != torch.float32 or tuple(w.shape) != (3, D) or not w.is_contiguous() or not w.is_cuda:
+    if w.dtype is not _torch().float32 or w.shape != (3, D) or not w.is_contiguous() or not w.is_cuda:
         raise ValueError("taps must be a contiguous CUDA float32 tensor [3, D]")
 
 
@@ -562,7 +584,7 @@ def tconv_forward(x, w, out=None):
     y = _torch().empty_like(x) if out is None else out
     desc = _conv_desc_of(x, y)
     _check_taps(w, x.shape[3])
-    _check(load_library().tconv_forward(ctypes.byref(desc), x.shape[1], _ptr(x), _ptr(w), _ptr(y), _stream(x)),
+    _check(load_library().tconv_forward(desc, x.shape[1], _ptr(x), _ptr(w), _ptr(y), _stream(x)),
            "tconv_forward")
     return y
 
@@ -585,10 +607,10 @@ class TConvCache:
         B, HW, D = self.frame.shape
         return _ConvDesc(B, HW, D, _dtype_code(self.frame), stride_b, 0)
 
-    def _desc_for(self, x, y=None) -> _ConvDesc:
+    def _desc_for(self, x, y=None) -> bytes:
         d = _conv_desc_of(x, y)
-        if (d.B, d.HW, d.D, d.dtype) != (self.frame.shape[0], self.frame.shape[1], self.frame.shape[2],
-                                         _dtype_code(self.frame)):
+        shape, frame = x.shape, self.frame
+        if frame.shape != (shape[0], shape[2], shape[3]) or x.dtype is not frame.dtype:
             raise ValueError("block does not match the cache's (B, HW, D, dtype)")
         return d
 
@@ -600,15 +622,15 @@ class TConvCache:
         """One block x_blk[B, T_b, HW, D]; commit=False only reads the cache (a denoising step)."""
         y = _torch().empty_like(x_blk) if out is None else out
         d = self._desc_for(x_blk, y)
-        _check_taps(w, d.D)
-        _check(self._lib.tconv_block_step(ctypes.byref(d), x_blk.shape[1], _ptr(x_blk), _ptr(w), _ptr(self.frame),
+        _check_taps(w, x_blk.shape[3])
+        _check(self._lib.tconv_block_step(d, x_blk.shape[1], _ptr(x_blk), _ptr(w), _ptr(self.frame),
                                           _ptr(y), int(commit), _stream(x_blk)), "tconv_block_step")
         return y
 
     def absorb(self, x_blk):
         """Take a block into the cache without computing its output."""
         d = self._desc_for(x_blk)
-        _check(self._lib.tconv_block_step(ctypes.byref(d), x_blk.shape[1], _ptr(x_blk), None, _ptr(self.frame), None, 1,
+        _check(self._lib.tconv_block_step(d, x_blk.shape[1], _ptr(x_blk), None, _ptr(self.frame), None, 1,
                                           _stream(x_blk)), "tconv_block_step")
 
     def prefill(self, x, w, n_blocks: int, out=None):
@@ -618,7 +640,7 @@ class TConvCache:
             raise ValueError("frame count must be n_blocks * T_b")
         y = _torch().empty_like(x) if out is None else out
         d = self._desc_for(x, y)
-        _check_taps(w, d.D)
-        _check(self._lib.tconv_prefill(ctypes.byref(d), n_blocks, T // n_blocks, _ptr(x), _ptr(w), _ptr(self.frame),
+        _check_taps(w, x.shape[3])
+        _check(self._lib.tconv_prefill(d, n_blocks, T // n_blocks, _ptr(x), _ptr(w), _ptr(self.frame),
                                        _ptr(y), _stream(x)), "tconv_prefill")
         return y
