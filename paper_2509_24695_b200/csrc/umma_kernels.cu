@@ -376,13 +376,12 @@ __device__ __forceinline__ void reduce_elements(const FusedParams& p, int first,
   float4* state4 = reinterpret_cast<float4*>(p.state);
   const float4* src[NE];
   int u_of[NE], r_lo[NE], nrec[NE];
-  bool live[NE], zpart[NE];
+  bool live[NE];
   float4 sum[NE], v[NE][NR];
 #pragma unroll
   for (int k = 0; k < NE; ++k) {
     const int idx = first + k * (int)blockDim.x;
-    live[k] = idx < i1;
-    zpart[k] = false;
+    live[k] = idx < i1 && !(ROPE && idx % E4 >= D * D / 4);   // (rotary variant: z is reduce_z's)
     if (!live[k]) continue;
     sum[k] = p.accumulate ? __ldcg(reinterpret_cast<const float4*>(p.state_base) + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
     const int bh = idx / E4, e = idx - bh * E4;
@@ -397,59 +396,83 @@ __device__ __forceinline__ void reduce_elements(const FusedParams& p, int first,
       ntrail = trailing_cta_of((long long)(u + 1) * s.m - 1, ttot, s.R) - r_lo[k] + 1;
     }
     nrec[k] = ncol + ntrail;
-    zpart[k] = ROPE && e >= D * D / 4;
   }
   auto record_of = [&](int k, int kk) { return kk < ncol ? kk * s.U + u_of[k] : s.P * s.U + r_lo[k] + (kk - ncol) + u_of[k]; };
   int nmax = 0;
 #pragma unroll
   for (int k = 0; k < NE; ++k)
-    if (live[k] && !zpart[k] && nrec[k] > nmax) nmax = nrec[k];
+    if (live[k] && nrec[k] > nmax) nmax = nrec[k];
   for (int k0 = 0; k0 < nmax; k0 += NR) {
 #pragma unroll
     for (int k = 0; k < NE; ++k)
 #pragma unroll
       for (int r = 0; r < NR; ++r)
-        if (live[k] && !zpart[k] && k0 + r < nrec[k]) v[k][r] = __ldcg(src[k] + (size_t)record_of(k, k0 + r) * REC4);
+        if (live[k] && k0 + r < nrec[k]) v[k][r] = __ldcg(src[k] + (size_t)record_of(k, k0 + r) * REC4);
 #pragma unroll
     for (int k = 0; k < NE; ++k)
 #pragma unroll
       for (int r = 0; r < NR; ++r)
-        if (live[k] && !zpart[k] && k0 + r < nrec[k]) add4(sum[k], v[k][r]);
+        if (live[k] && k0 + r < nrec[k]) add4(sum[k], v[k][r]);
   }
 #pragma unroll
   for (int k = 0; k < NE; ++k) {
     if (!live[k]) continue;
     const int idx = first + k * (int)blockDim.x;
-    if (ROPE && zpart[k]) {
-      // rotary variant: z comes from the plain phi(k) sums that the ReLU warps of every segment left
-      // behind the record (per warp, per feature): per warp slot the records in their fixed order, then the
-      // slots as a balanced tree over sixteen, the missing ones zero (the association reduce_image's shuffles give)
-      const int e = idx % E4;
-      const int ft4 = (((idx / E4) % p.H) % C::G) * (D / 4) + (e - D * D / 4);   // float4 of the operand's 128 features
-      const float4* zp = reinterpret_cast<const float4*>(p.partials) + C::G * E4 + ft4;
-      // (one slot after the other: this form only runs when the operand images are not in use, and the
-      // rotary kernel has no registers to spare)
-      const bool upper = ft4 >= 16;   // features 64..: the epilogue warps' slots hold a share too
-      // (computed depth first, a few registers at a time: this form only runs when the operand images are not in
-      // use, and the rotary kernel has no registers to spare)
-      auto slot = [&](int w) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (w < 8 || (w < kZSlots && upper)) {
-#pragma unroll 2
-          for (int kk = 0; kk < nrec[k]; ++kk) add4(a, __ldcg(zp + (size_t)record_of(k, kk) * REC4 + w * 32));
-        }
-        return a;
-      };
-      auto pair = [&](int w) { float4 a = slot(w); add4(a, slot(w + 1)); return a; };
-      auto quad = [&](int w) { float4 a = pair(w); add4(a, pair(w + 2)); return a; };
-      float4 tree = quad(0);
-      add4(tree, quad(4));
-      float4 high = quad(8);
-      add4(high, quad(12));
-      add4(tree, high);
-      add4(sum[k], tree);
-    }
     state4[idx] = sum[k];
+  }
+}
+
+// Rotary variant: z of all units, split evenly over the CTAs, from the plain phi(k) sums that the warps of every segment
+// left behind the record.  Sixteen threads to a float4 of a unit's 128 features, one warp slot each: all of a slot's
+// records in flight together, added in their fixed order; the slots are then added as a balanced tree, the missing ones
+// zero (reduce_image_zrow's association).  One slot after the other in one thread, as before, this was 25 us of the 66 us
+// of a rotary step of 4680 tokens, 35 heads of 64.
+template <int D>
+__device__ __forceinline__ void reduce_z(const FusedParams& p, int ncol) {
+  using C = Cfg<D>;
+  constexpr int E4 = (D + 1) * D / 4, REC4 = C::G * E4 + kZParts / 4, Z4 = C::FEAT / 4, NR = 6;
+  const Sched& s = p.sa;
+  const long long ttot = (long long)s.U * s.m;
+  const int tot = s.U * Z4, me = (int)blockIdx.x;
+  const int i0 = (int)((long long)tot * me / gridDim.x), i1 = (int)((long long)tot * (me + 1) / gridDim.x);
+  const int w = (int)threadIdx.x & 15;
+  for (int first = i0; first < i1; first += (int)blockDim.x / 16) {   // whole warps: the shuffles below stay inside one
+    const int idx = first + (int)threadIdx.x / 16;
+    const int u = idx / Z4, ft4 = idx - u * Z4;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (idx < i1 && (w < 8 || (w < kZSlots && ft4 >= 16))) {   // (features 64..: the epilogue warps' slots hold a share too)
+      int r_lo = 0, nrec = ncol;
+      if (s.m > 0) {
+        r_lo = trailing_cta_of((long long)u * s.m, ttot, s.R);
+        nrec += trailing_cta_of((long long)(u + 1) * s.m - 1, ttot, s.R) - r_lo + 1;
+      }
+      const float4* zp = reinterpret_cast<const float4*>(p.partials) + C::G * E4 + w * 32 + ft4;
+      for (int k0 = 0; k0 < nrec; k0 += NR) {
+        float4 v[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int kk = k0 + r;
+          if (kk < nrec) v[r] = __ldcg(zp + (size_t)(kk < ncol ? kk * s.U + u : s.P * s.U + r_lo + (kk - ncol) + u) * REC4);
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (k0 + r < nrec) add4(acc, v[r]);
+      }
+    }
+#pragma unroll
+    for (int st = 1; st < 16; st *= 2) {
+      float4 o;
+      o.x = __shfl_xor_sync(0xffffffffu, acc.x, st); o.y = __shfl_xor_sync(0xffffffffu, acc.y, st);
+      o.z = __shfl_xor_sync(0xffffffffu, acc.z, st); o.w = __shfl_xor_sync(0xffffffffu, acc.w, st);
+      add4(acc, o);
+    }
+    const int g = ft4 * 4 / D, h = (u % p.HG) * C::G + g;
+    if (idx < i1 && w == 0 && h < p.H) {
+      const size_t e4 = ((size_t)((u / p.HG) * p.H + h) * (D + 1) + D) * (D / 4) + (ft4 - g * (D / 4));
+      float4 sum = p.accumulate ? __ldcg(reinterpret_cast<const float4*>(p.state_base) + e4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      add4(sum, acc);
+      reinterpret_cast<float4*>(p.state)[e4] = sum;
+    }
   }
 }
 
@@ -462,6 +485,7 @@ __device__ void reduce_slice(const FusedParams& p) {
   const int i0 = me * per + (me < rem ? me : rem);
   const int i1 = i0 + per + (me < rem ? 1 : 0);
   const int ncol = s.P == 0 ? 0 : (s.P < (s.tpu + s.Lc - 1) / s.Lc ? s.P : (s.tpu + s.Lc - 1) / s.Lc);
+  if (ROPE) reduce_z<D>(p, ncol);
   // few elements per thread: more records per batch; more elements: fewer records each (about 20 loads either way;
   // half as many in the rotary variant, whose 480 threads have 128 registers each)
   if (i1 - i0 <= 2 * (int)blockDim.x) {
@@ -472,6 +496,11 @@ __device__ void reduce_slice(const FusedParams& p) {
       reduce_elements<D, ROPE, 3, ROPE ? 3 : 6>(p, first, i1, ncol);
   }
 }
+
+// The rotary kernel has no registers to spare: with this form inlined the passes of a kernel that never takes it (d = 112,
+// 4680 tokens) were 5 % slower.
+template <int D>
+__device__ __noinline__ void reduce_slice_apart(const FusedParams& p) { reduce_slice<D, true>(p); }
 
 // ---------------------------------------------------------------- reduce, with the S operand as a by-product
 // Fused launches of one-head units (d = 112, 128) with at least one column CTA per unit: the column CTAs of a
@@ -834,7 +863,8 @@ __device__ __forceinline__ float sum_z_slots(const float* slots, int f) {
 template <int D, bool ROPE, bool SOLO>
 __global__ void __launch_bounds__(Roles<ROPE>::THREADS, 1)
 umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                  const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o, FusedParams p) {
+                  const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
+                  const __grid_constant__ FusedParams p) {
   using C = Cfg<D>;
   using R = Roles<ROPE>;
   constexpr int NSA = SOLO ? 4 : C::STATE_STAGES;
@@ -1280,6 +1310,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     grid_barrier(p.ctrl, abort_flag, p.do_apply != 0, gen0);
     if (!*abort_flag) {
       if (C::G == 1 && p.s_image) reduce_image<D, ROPE>(p);
+      else if (ROPE) reduce_slice_apart<D>(p);
       else reduce_slice<D, ROPE>(p);
     }
     if (p.do_apply) grid_barrier(p.ctrl, abort_flag, false, gen0 + 1);
