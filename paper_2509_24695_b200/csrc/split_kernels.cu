@@ -13,7 +13,7 @@
 //
 // Operand layouts are those of the fused kernel: 128-byte swizzled rows of 64 features.  Every thread reads its own
 // pieces with private asynchronous copies, rectifies, rotates and splits them, and stores the parts; one thread issues
-// the MMAs of a tile while all of them prepare the next one.  All waits are on this CTA's own MMAs and bounded.
+// the MMAs, and other warps drain the accumulators.  All waits are on this CTA's own work and bounded.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -22,8 +22,13 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 512;                // threads that prepare, drain and store; one more warp issues the MMAs
-constexpr int kBlock = kThreads + 32;
+// Warp roles: 0..7 prepare tiles (load, rectify, rotate, split), 8..15 drain accumulators (and store), 16 issues the MMAs.
+// The roles only meet at barriers, two tiles apart at most; with all sixteen warps doing both in turn a tile took the sum
+// of the two instead of the longer one.
+constexpr int kPrepare = 256;
+constexpr int kDrain = 256;
+constexpr int kMmaWarp = (kPrepare + kDrain) / 32;
+constexpr int kBlock = kPrepare + kDrain + 32;
 
 template <typename T>
 struct Piece;   // 16 bytes of a row
@@ -49,6 +54,12 @@ struct Shape {
   static constexpr int V_PARTS = F32 ? 3 : 1;
   using Tab = typename Piece<T>::Tab;
 };
+
+// With `lanes` threads to a row, which bit of the piece index odd rows flip, so that the stores of the neighbouring rows of
+// one shared-memory access fall into different banks (8-byte stores of fp32 pieces, 16-byte stores of bf16 ones).
+__host__ __device__ constexpr int flip_of(int E, int lanes, int pieces) {
+  return E == 4 ? (lanes == 8 && pieces % 2 == 0 ? 1 : lanes == 4 && pieces % 4 == 0 ? 2 : 0) : (lanes == 4 && pieces % 2 == 0 ? 1 : 0);
+}
 
 template <int BYTES>
 __device__ __forceinline__ void copy_async(void* smem_dst, const void* src, bool live) {   // not live: zeros
@@ -130,15 +141,15 @@ struct StateShape : Shape<T, R, ROPE> {
   // tokens of a tile: 64 where two stages of parts and three of raw pieces fit, else 32
   static constexpr int BYTES_64 = 2 * (B::QK_PARTS + B::V_PARTS) * B::BOXES * 8192 + 3 * 64 * B::DP * (2 * (int)sizeof(T) + (ROPE ? 2 : 0));
   static constexpr int TOK = BYTES_64 <= 200 * 1024 ? 64 : 32;
-  static constexpr int LANES = kThreads / TOK;               // threads to a row
+  static constexpr int LANES = kPrepare / TOK;               // threads to a row
   static constexpr int PIECES = (B::DP / B::E + LANES - 1) / LANES;   // 16-byte pieces of a row per thread
-  static constexpr int FLIP = LANES == 8 && PIECES % 2 == 0 ? 1 : 0;
+  static constexpr int FLIP = flip_of(B::E, LANES, PIECES);
   static constexpr int BOX = TOK * 128;
   static constexpr int PART = B::BOXES * BOX;
   static constexpr int STAGE = (B::QK_PARTS + B::V_PARTS) * PART;
   static constexpr int RAW_STAGES = 3;
-  static constexpr int TAB = ROPE ? PIECES * kThreads * (int)sizeof(typename B::Tab) : 0;
-  static constexpr int RAW = 2 * PIECES * kThreads * 16 + TAB;
+  static constexpr int TAB = ROPE ? PIECES * kPrepare * (int)sizeof(typename B::Tab) : 0;
+  static constexpr int RAW = 2 * PIECES * kPrepare * 16 + TAB;
   static constexpr int Z_BYTES = TOK * B::DP * 4;
   static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > Z_BYTES ? RAW_STAGES * RAW : Z_BYTES) + 64;   // (barriers last)
   static constexpr int LEAD = TOK / 32;                      // accumulators of the leading products: chains of two K steps
@@ -151,10 +162,11 @@ struct StateShape : Shape<T, R, ROPE> {
 
 // grid (P, units): partial state of the tiles [c * tiles / P, (c + 1) * tiles / P) of one unit, in the library's layout.
 //
-// Measured (32 760 tokens, 20 heads of 112, fp32; floor: 587 MB, 90 us at the copy rate): 192 us with the reduce of the
-// partial states, where the general kernels take 1050 (fp32 pipe at a quarter of its rate, scalar loads) and a register-blocked
-// form of them on packed fp32 FMAs 492.  A tile of 32 tokens takes 1.2 us, most of it instruction issue (splitting and
-// draining) and the latencies of one tile's chain.  Distance from 64 bits, 2-norm: S 1.3e-7 (general kernels 2.9e-7).
+// Measured (32 760 tokens, 20 heads of 112, fp32; floor: 587 MB, 90 us at the copy rate): 176 us with the reduce of the
+// partial states (192 with every warp preparing and draining in turn), where the general kernels take 1050 (fp32 pipe at a
+// quarter of its rate, scalar loads) and a register-blocked form of them on packed fp32 FMAs 492.  A tile of 32 tokens takes
+// 1.1 us, with 190 KB through shared memory (pieces in and out, their parts, 90 KB of MMA operands): two thirds of what it
+// moves in that time.  Distance from 64 bits, 2-norm: S 1.3e-7 (general kernels 2.9e-7).
 template <typename T, int R, bool ROPE>
 __global__ void __launch_bounds__(kBlock, 1)
 split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, int P, float* __restrict__ partials,
@@ -168,7 +180,8 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   uint8_t* raw = smem + 2 * S::STAGE;
   uint64_t* done = reinterpret_cast<uint64_t*>(raw + (S::SMEM - 1024 - 2 * S::STAGE - 64));   // [2] the tile's MMAs are complete
   uint64_t* ready = done + 2;                                                               // [2] the tile's parts are in its stage
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ready + 2);
+  uint64_t* drained = ready + 2;                                                            // [2] its accumulators are read
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drained + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d, u = blockIdx.y, c = blockIdx.x;
@@ -177,7 +190,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   const int tiles = (int)((c + 1) * all / P - first);
 
   if (tid == 0) {
-    for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kThreads); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -185,15 +198,13 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   for (int i = tid; i < 2 * S::STAGE / 16; i += kBlock) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
   if (warp == 0) { tmem_alloc(tmem_holder, S::COLS); tmem_relinquish(); }
 
-  // this thread's row of every tile, and its pieces of it: features feature(0), feature(1), ...  Sixteen neighbouring
-  // 8-byte stores fill one swizzled row of 128 bytes; with eight threads to a row, odd rows take each pair of pieces in
-  // the other order, so that the stores of two neighbouring rows fall into different halves of the banks.
-  const int row = (tid % kThreads) / S::LANES, l = tid % S::LANES;
-  auto feature = [&](int i) { return (l + S::LANES * (S::FLIP ? i ^ (row & 1) : i)) * E; };
+  // preparing: this thread's row of every tile, and its pieces of it, features feature(0), feature(1), ...
+  const int row = (tid % kPrepare) / S::LANES, l = tid % S::LANES;
+  auto feature = [&](int i) { return (l + S::LANES * (i ^ (S::FLIP * (row & 1)))) * E; };
   const long long base = (long long)(u / p.H) * p.sb + (long long)(u % p.H) * p.sh;
-  auto raw_k = [&](int st, int i) { return reinterpret_cast<uint4*>(raw + st * S::RAW) + 2 * i * kThreads + tid; };
+  auto raw_k = [&](int st, int i) { return reinterpret_cast<uint4*>(raw + st * S::RAW) + 2 * i * kPrepare + tid; };
   auto raw_tab = [&](int st, int i) {
-    return reinterpret_cast<Tab*>(raw + st * S::RAW + 2 * PIECES * kThreads * 16) + i * kThreads + tid;
+    return reinterpret_cast<Tab*>(raw + st * S::RAW + 2 * PIECES * kPrepare * 16) + i * kPrepare + tid;
   };
   auto issue = [&](int t, int st) {
     if (t < tiles) {
@@ -205,7 +216,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
         const int f = feature(i);
         if (f >= d) continue;
         copy_async<16>(raw_k(st, i), k + off + f, live);
-        copy_async<16>(raw_k(st, i) + kThreads, v + off + f, live);
+        copy_async<16>(raw_k(st, i) + kPrepare, v + off + f, live);
         if (ROPE) copy_async<(int)sizeof(Tab)>(raw_tab(st, i), tab + (live ? n : 0) * (d / 2) + f / 2, live);
       }
     }
@@ -222,7 +233,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
 #pragma unroll
     for (int i = 0; i < PIECES; ++i) {
       kr[i] = *raw_k(st, i);
-      vr[i] = *(raw_k(st, i) + kThreads);
+      vr[i] = *(raw_k(st, i) + kPrepare);
       if (ROPE) tb[i] = *raw_tab(st, i);
     }
 #pragma unroll
@@ -246,8 +257,8 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
     }
   };
 
-  const bool worker = warp < kThreads / 32;
-  if (worker) {
+  const bool preparing = tid < kPrepare;
+  if (preparing) {
     issue(0, 0);
     issue(1, 1);
   }
@@ -257,50 +268,52 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   tcgen05_fence_after();
   const uint32_t tmem = *tmem_holder;
 
-  // accumulator lane = key feature; each of the four warps of a lane quarter takes a quarter of the value features
-  constexpr int COLS = S::DP / 4;
+  // draining: accumulator lane = key feature; each of the two warps of a lane quarter takes half of the value features
+  constexpr int COLS = S::DP / 2;
   const int key = (warp & 3) * 32 + lane;
-  const int col0 = (warp >> 2) * COLS;
-  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0;
+  const int col0 = ((warp >> 2) & 1) * COLS;
   float sum[COLS];
 #pragma unroll
   for (int x = 0; x < COLS; ++x) sum[x] = 0.f;
-  auto drain = [&](int t) {
-    mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
-    __syncwarp();   // tcgen05.ld wants whole warps
-    tcgen05_fence_after();
-    if ((warp & 3) * 32 < d) {
-#pragma unroll
-      for (int g = 0; g < R; ++g) {
-        uint32_t a[S::LEAD + 1][4];
-#pragma unroll
-        for (int s = 0; s < S::LEAD + (S::REST ? 1 : 0); ++s) tmem_ld_x4(trow + (t & 1) * S::SET + s * S::ACC + 4 * g, a[s]);
-        tmem_ld_wait();
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          float add = __uint_as_float(a[0][x]);
-          if (S::LEAD > 1) add += __uint_as_float(a[S::LEAD > 1 ? 1 : 0][x]);
-          if (S::REST) add += __uint_as_float(a[S::LEAD][x]);
-          sum[4 * g + x] += add;
-        }
-      }
-    }
-    tcgen05_fence_before();
-  };
 
-  if (worker) {
+  if (preparing) {
     for (int t = 0; t < tiles; ++t) {
-      // the stage and the accumulators of tile t - 2 are free: this thread has drained it, and the MMA warp waits for all
       issue(t + 2, (t + 2) % S::RAW_STAGES);
       copy_wait<2>();
+      if (t >= 2) mbar_wait(&done[t & 1], ((t - 2) >> 1) & 1, abort_flag);   // the MMAs that read this stage
       convert(t % S::RAW_STAGES, smem + (t & 1) * S::STAGE);
       fence_proxy_async_smem();
       mbar_arrive(&ready[t & 1]);
-      if (t > 0) drain(t - 1);
     }
-    if (tiles > 0) drain(tiles - 1);
+    copy_wait<0>();
+  } else if (warp < kMmaWarp) {
+    const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0;
+    for (int t = 0; t < tiles; ++t) {
+      mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
+      __syncwarp();   // tcgen05.ld wants whole warps
+      tcgen05_fence_after();
+      if ((warp & 3) * 32 < d) {
+#pragma unroll
+        for (int g = 0; g < R; ++g) {
+          uint32_t a[S::LEAD + 1][8];
+#pragma unroll
+          for (int s = 0; s < S::LEAD + (S::REST ? 1 : 0); ++s) tmem_ld_x8(trow + (t & 1) * S::SET + s * S::ACC + 8 * g, a[s]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            float add = __uint_as_float(a[0][x]);
+            if (S::LEAD > 1) add += __uint_as_float(a[S::LEAD > 1 ? 1 : 0][x]);
+            if (S::REST) add += __uint_as_float(a[S::LEAD][x]);
+            sum[8 * g + x] += add;
+          }
+        }
+      }
+      tcgen05_fence_before();
+      mbar_arrive(&drained[t & 1]);
+    }
   } else if (lane == 0) {
     for (int t = 0; t < tiles; ++t) {
+      if (t >= 2) mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag);
       mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag);
       tcgen05_fence_after();
       constexpr uint32_t LBO = S::BOXES > 1 ? S::BOX : 0;   // 64 features: rows 64..127 of the MMA repeat them and are ignored
@@ -327,12 +340,11 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       umma_commit(&done[t & 1]);
     }
   }
-  copy_wait<0>();
   __syncthreads();
 
   // W[j][i] = S[i][j], W[d][i] = z[i]
   float* out = partials + ((long long)u * P + c) * p.state_elems();
-  if (worker && key < d) {
+  if (!preparing && warp < kMmaWarp && key < d) {
 #pragma unroll
     for (int x = 0; x < COLS; ++x)
       if (col0 + x < d) out[(long long)(col0 + x) * d + key] = sum[x];
@@ -341,7 +353,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
 #pragma unroll
   for (int i = 0; i < PIECES; ++i) {
     const int f = feature(i);
-    if (!worker || f >= d) continue;
+    if (!preparing || f >= d) continue;
 #pragma unroll
     for (int e = 0; e < E; ++e) zs[row * d + f + e] = z[i][e];
   }
@@ -362,17 +374,28 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
 template <typename T, int R, bool ROPE>
 struct ApplyShape : Shape<T, R, ROPE> {
   using B = Shape<T, R, ROPE>;
-  static constexpr int TOK = 64;
-  static constexpr int LANES = kThreads / TOK;                // threads to a row
-  static constexpr int PIECES = 2 * ((B::DP / B::E + 2 * LANES - 1) / (2 * LANES));   // 16-byte pieces of a row per thread, even
+  // One part (bf16): tiles of 128 tokens.  The output is rounded to bf16 there, so one accumulator for the leading products
+  // does; three, for short chains, where the output is fp32.
+  static constexpr int TOK = B::QK_PARTS == 1 ? 128 : 64;
+  static constexpr int LEAD = B::QK_PARTS == 1 ? 1 : 3;
+  static constexpr int LANES = kPrepare / TOK;                // threads to a row
+  static constexpr int ROUND = B::F32 ? 4 : 2;                // (see flip_of)
+  static constexpr int PIECES = ROUND * ((B::DP / B::E + ROUND * LANES - 1) / (ROUND * LANES));   // 16-byte pieces of a row per thread
+  static constexpr int FLIP = flip_of(B::E, LANES, PIECES);
   static constexpr int SBOX = B::DP * 128, SPART = B::BOXES * SBOX;   // (lanes from DP on read whatever follows and are ignored)
   static constexpr int S_BYTES = 3 * SPART;
   static constexpr int QBOX = TOK * 128, QPART = B::BOXES * QBOX, STAGE = B::QK_PARTS * QPART;
-  static constexpr int DEN = 4 * TOK * 4;
+  static constexpr int DEN = (4 * TOK + 128) * 4;
+  static constexpr int FIXED = 1024 + S_BYTES + 2 * STAGE + DEN + 64;
+  // a tile's rotations are staged beside its pieces where there is room (not for fp32 at d > 96: loaded where they are used)
+  static constexpr bool TAB_STAGED = ROPE && FIXED + PIECES * kPrepare * (16 + (int)sizeof(typename B::Tab)) <= 227 * 1024;
+  static constexpr int RAW = PIECES * kPrepare * (16 + (TAB_STAGED ? (int)sizeof(typename B::Tab) : 0));   // one tile as loaded
+  static constexpr int FIT = (227 * 1024 - FIXED) / RAW;
+  static constexpr int RAW_STAGES = FIT < 1 ? 1 : FIT > 3 ? 3 : FIT;
   static constexpr int OVERRUN = 128 * 128 - SBOX;            // of the last part's last box, when less than that follows
-  static constexpr int AFTER = 2 * STAGE + DEN + 64;
-  static constexpr int SMEM = 1024 + S_BYTES + (AFTER > OVERRUN ? AFTER : OVERRUN);
-  static constexpr int LEAD = 3, ACC = TOK, SET = (LEAD + 1) * ACC;   // TMEM columns: two sets of four accumulators
+  static constexpr int SMEM = FIXED + (RAW_STAGES * RAW > OVERRUN ? RAW_STAGES * RAW : OVERRUN);
+  static constexpr int ACC = TOK, SET = (LEAD + 1) * ACC;     // TMEM columns: two sets of accumulators
+  static_assert(2 * SET <= 512, "tensor memory");
 };
 
 __device__ __forceinline__ void store_value(float* o, float x) { *o = x; }
@@ -380,8 +403,9 @@ __device__ __forceinline__ void store_value(__nv_bfloat16* o, float x) { *o = __
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
 //
-// Measured as above: 182 us, general kernels 866, register-blocked on packed fp32 FMAs 489; distance from 64 bits 0.9e-7
-// (general kernels 1.6e-7).  bf16, 28 heads of 80: 165 us, general kernels 644.
+// Measured as above: 185 us (operand reads of the MMAs, 250 of 350 KB a tile through shared memory), general kernels 866,
+// register-blocked on packed fp32 FMAs 489; distance from 64 bits 1.0e-7 (general kernels 1.6e-7).  bf16, 28 heads of 80:
+// 152 us (165 with tiles of 64 tokens and every warp in both roles), general kernels 644.
 template <typename T, int R, bool ROPE>
 __global__ void __launch_bounds__(kBlock, 1)
 split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* __restrict__ o, Problem p, float eps,
@@ -394,10 +418,13 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   uint8_t* s_op = align1024(smem_raw);
   uint8_t* stages = s_op + A::S_BYTES;
   float* den = reinterpret_cast<float*>(stages + 2 * A::STAGE);     // [4][TOK] reciprocals of the denominators
-  uint64_t* done = reinterpret_cast<uint64_t*>(den + 4 * A::TOK);   // [2] as in the state kernel
+  float* zs = den + 4 * A::TOK;                                     // [128] z
+  uint64_t* done = reinterpret_cast<uint64_t*>(zs + 128);           // [2] each, as in the state kernel
   uint64_t* ready = done + 2;
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(ready + 2);
+  uint64_t* drained = ready + 2;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drained + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  uint8_t* raw = reinterpret_cast<uint8_t*>(done) + 64;
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d, u = blockIdx.y;
   const long long all = (p.N + A::TOK - 1) / A::TOK;
@@ -405,39 +432,42 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   const int tiles = (int)((blockIdx.x + 1) * all / gridDim.x - first);
   const float* W = state + (long long)u * p.state_elems();
   const long long base = (long long)(u / p.H) * p.sb + (long long)(u % p.H) * p.sh;
-  // this thread's row of every tile, and its pieces of it.  Odd rows take each pair of pieces in the other order, so that
-  // the 8-byte stores of two neighbouring rows fall into different halves of the banks.
-  const int row = (tid % kThreads) / A::LANES, l = tid % A::LANES;
-  auto feature = [&](int i) { return (l + A::LANES * (i ^ (row & 1))) * E; };
-  const bool worker = warp < kThreads / 32;
-  // two tiles' raw pieces are on their way in registers
-  auto fetch = [&](int t, uint4 (&x)[PIECES], Tab (&tb)[PIECES]) {
-    const long long n = (first + t) * A::TOK + row;
-    const bool live = t < tiles && n < p.N;
-    const long long at = live ? n : 0;
+  // preparing: this thread's row of every tile, and its pieces of it
+  const int row = (tid % kPrepare) / A::LANES, l = tid % A::LANES;
+  auto feature = [&](int i) { return (l + A::LANES * (i ^ (A::FLIP * (row & 1)))) * E; };
+  const bool preparing = tid < kPrepare;
+  auto raw_q = [&](int st, int i) { return reinterpret_cast<uint4*>(raw + st * A::RAW) + i * kPrepare + tid; };
+  auto raw_tab = [&](int st, int i) { return reinterpret_cast<Tab*>(raw + st * A::RAW + PIECES * kPrepare * 16) + i * kPrepare + tid; };
+  auto issue = [&](int t) {
+    if (t < tiles) {
+      const long long n = (first + t) * A::TOK + row;
+      const bool live = n < p.N;
+      const long long at = live ? n : 0;
+      const int st = t % A::RAW_STAGES;
 #pragma unroll
-    for (int i = 0; i < PIECES; ++i) {
-      x[i] = make_uint4(0, 0, 0, 0);
-      if (live && feature(i) < d) {
-        x[i] = __ldcs(reinterpret_cast<const uint4*>(q + base + at * p.sn + feature(i)));
-        if (ROPE) tb[i] = __ldg(reinterpret_cast<const Tab*>(tab + at * (d / 2) + feature(i) / 2));
+      for (int i = 0; i < PIECES; ++i) {
+        const int f = feature(i);
+        if (f >= d) continue;
+        copy_async<16>(raw_q(st, i), q + base + at * p.sn + f, live);
+        if (A::TAB_STAGED) copy_async<(int)sizeof(Tab)>(raw_tab(st, i), tab + at * (d / 2) + f / 2, live);
       }
     }
+    copy_commit();
   };
-  uint4 x0[PIECES], x1[PIECES];
-  Tab tb0[PIECES], tb1[PIECES];
-  if (worker) {
-    fetch(0, x0, tb0);
-    fetch(1, x1, tb1);
+  if (preparing) {
+#pragma unroll
+    for (int t = 0; t < A::RAW_STAGES; ++t) issue(t);
   }
   if (tid == 0) {
-    for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kThreads); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
     *abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 0) { tmem_alloc(tmem_holder, 512); tmem_relinquish(); }
   // padded features of both operands read as zero
-  for (int i = tid; i < (A::S_BYTES + 2 * A::STAGE) / 16; i += kBlock) reinterpret_cast<uint4*>(s_op)[i] = make_uint4(0, 0, 0, 0);
+  if (d < A::DP)
+    for (int i = tid; i < (A::S_BYTES + 2 * A::STAGE) / 16; i += kBlock) reinterpret_cast<uint4*>(s_op)[i] = make_uint4(0, 0, 0, 0);
+  if (tid < 128) zs[tid] = tid < d ? W[(long long)d * d + tid] : 0.f;
   __syncthreads();
   for (int idx = tid; idx < d * (d / 4); idx += kBlock) {
     const int j = idx / (d / 4), i = (idx - j * (d / 4)) * 4;
@@ -445,85 +475,96 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     widen(__ldg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
     store_parts<3>(s_op + operand_offset(j, i, A::SBOX), A::SPART, x);
   }
-  float z[PIECES][E];
-#pragma unroll
-  for (int i = 0; i < PIECES; ++i)
-#pragma unroll
-    for (int e = 0; e < E; ++e) z[i][e] = feature(i) < d ? W[(long long)d * d + feature(i) + e] : 0.f;
-
-  auto convert = [&](int t, uint4 (&raw)[PIECES], Tab (&tb)[PIECES]) {
-    uint8_t* stage = stages + (t & 1) * A::STAGE;
-    float dn = 0.f;
-#pragma unroll
-    for (int i = 0; i < PIECES; ++i) {
-      const int f = feature(i);
-      if (f >= d) continue;
-      float x[E];
-      widen(raw[i], x);
-#pragma unroll
-      for (int e = 0; e < E; ++e) { x[e] = fmaxf(x[e], 0.f); dn = fmaf(x[e], z[i][e], dn); }   // phi = ReLU on the queries
-      if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
-      store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX), A::QPART, x);
-    }
-    dn += __shfl_xor_sync(0xffffffffu, dn, 1);
-    dn += __shfl_xor_sync(0xffffffffu, dn, 2);
-    dn += __shfl_xor_sync(0xffffffffu, dn, 4);
-    if (l == 0) den[(t & 3) * A::TOK + row] = 1.0f / (dn + eps);   // eps added once, after the dot product
-  };
   fence_proxy_async_smem();   // S and the zeros
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem = *tmem_holder;
 
-  // accumulator lane = value feature; each of the four warps of a lane quarter takes a quarter of the tokens
-  const int j = (warp & 3) * 32 + lane, tok0 = (warp >> 2) * 16;
-  auto epilogue = [&](int t) {
-    mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
-    __syncwarp();   // tcgen05.ld wants whole warps
-    tcgen05_fence_after();
-    if ((warp & 3) * 32 < d) {
-      const uint32_t trow = tmem + (t & 1) * A::SET + ((uint32_t)((warp & 3) * 32) << 16) + tok0;
-      const float* rden = den + (t & 3) * A::TOK + tok0;
-      const long long n0 = (first + t) * A::TOK + tok0;
-      const int live = j < d ? (int)min(16ll, p.N - n0) : 0;
-      T* out = o + base + n0 * p.sn + j;
+  if (preparing) {
+    for (int t = 0; t < tiles; ++t) {
+      uint8_t* stage = stages + (t & 1) * A::STAGE;
+      const int st = t % A::RAW_STAGES;
+      uint4 x4[PIECES];   // all reads first, then the tile that takes their place is asked for
+      Tab tb[PIECES];
+      if (ROPE && !A::TAB_STAGED) {
+        const long long n = (first + t) * A::TOK + row;
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        uint32_t a[A::LEAD + 1][8];
-#pragma unroll
-        for (int s = 0; s < (R < 3 ? R : A::LEAD); ++s) tmem_ld_x8(trow + s * A::ACC + 8 * g, a[s]);
-        tmem_ld_x8(trow + A::LEAD * A::ACC + 8 * g, a[A::LEAD]);
-        tmem_ld_wait();
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          float num = __uint_as_float(a[0][x]);
-          if (R > 1) num += __uint_as_float(a[1][x]);
-          if (R > 2) num += __uint_as_float(a[2][x]);
-          num += __uint_as_float(a[A::LEAD][x]);
-          if (8 * g + x < live) store_value(out, num * rden[8 * g + x]);
-          out += p.sn;
-        }
+        for (int i = 0; i < PIECES; ++i)
+          if (feature(i) < d) tb[i] = __ldg(reinterpret_cast<const Tab*>(tab + (n < p.N ? n : 0) * (d / 2) + feature(i) / 2));
       }
-    }
-    tcgen05_fence_before();
-  };
-  if (worker) {
-    // stage and accumulators of tile t - 2 are free: this thread has been through its epilogue, and the MMA warp waits for all
-    auto step = [&](int t, uint4 (&x)[PIECES], Tab (&tb)[PIECES]) {
-      convert(t, x, tb);
-      fetch(t + 2, x, tb);
+      copy_wait<A::RAW_STAGES - 1>();
+#pragma unroll
+      for (int i = 0; i < PIECES; ++i) {
+        x4[i] = *raw_q(st, i);
+        if (A::TAB_STAGED) tb[i] = *raw_tab(st, i);
+      }
+      issue(t + A::RAW_STAGES);
+      if (t >= 2) mbar_wait(&done[t & 1], ((t - 2) >> 1) & 1, abort_flag);   // the MMAs that read this stage
+      float dn = 0.f;
+#pragma unroll
+      for (int i = 0; i < PIECES; ++i) {
+        const int f = feature(i);
+        if (f >= d) continue;
+        float x[E];
+        widen(x4[i], x);
+#pragma unroll
+        for (int e = 0; e < E; e += 4) {
+          const float4 z = *reinterpret_cast<const float4*>(zs + f + e);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x[e + k] = fmaxf(x[e + k], 0.f);   // phi = ReLU on the queries
+          dn = fmaf(x[e], z.x, dn); dn = fmaf(x[e + 1], z.y, dn); dn = fmaf(x[e + 2], z.z, dn); dn = fmaf(x[e + 3], z.w, dn);
+        }
+        if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
+        store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX), A::QPART, x);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int st2 = 1; st2 < A::LANES; st2 *= 2) dn += __shfl_xor_sync(0xffffffffu, dn, st2);
+      if (l == 0) den[(t & 3) * A::TOK + row] = 1.0f / (dn + eps);   // eps added once, after the dot product
       fence_proxy_async_smem();
       mbar_arrive(&ready[t & 1]);
-      if (t > 0) epilogue(t - 1);
-    };
-    for (int t = 0; t < tiles; t += 2) {
-      step(t, x0, tb0);
-      if (t + 1 < tiles) step(t + 1, x1, tb1);
     }
-    if (tiles > 0) epilogue(tiles - 1);
+    copy_wait<0>();
+  } else if (warp < kMmaWarp) {
+    // accumulator lane = value feature; each of the two warps of a lane quarter takes half of the tokens
+    constexpr int HALF = A::TOK / 2;
+    const int j = (warp & 3) * 32 + lane, tok0 = ((warp >> 2) & 1) * HALF;
+    for (int t = 0; t < tiles; ++t) {
+      mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
+      __syncwarp();   // tcgen05.ld wants whole warps
+      tcgen05_fence_after();
+      if ((warp & 3) * 32 < d) {
+        const uint32_t trow = tmem + (t & 1) * A::SET + ((uint32_t)((warp & 3) * 32) << 16) + tok0;
+        const float* rden = den + (t & 3) * A::TOK + tok0;
+        const long long n0 = (first + t) * A::TOK + tok0;
+        const int live = j < d ? (int)min((long long)HALF, p.N - n0) : 0;
+        T* out = o + base + n0 * p.sn + j;
+#pragma unroll
+        for (int g = 0; g < HALF / 8; ++g) {
+          constexpr int LEADS = R < A::LEAD ? R : A::LEAD;
+          uint32_t a[A::LEAD + 1][8];
+#pragma unroll
+          for (int s = 0; s < LEADS; ++s) tmem_ld_x8(trow + s * A::ACC + 8 * g, a[s]);
+          tmem_ld_x8(trow + A::LEAD * A::ACC + 8 * g, a[A::LEAD]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            float num = __uint_as_float(a[0][x]);
+#pragma unroll
+            for (int s = 1; s < LEADS; ++s) num += __uint_as_float(a[s][x]);
+            num += __uint_as_float(a[A::LEAD][x]);
+            if (8 * g + x < live) store_value(out, num * rden[8 * g + x]);
+            out += p.sn;
+          }
+        }
+      }
+      tcgen05_fence_before();
+      mbar_arrive(&drained[t & 1]);
+    }
   } else if (lane == 0) {
     for (int t = 0; t < tiles; ++t) {
+      if (t >= 2) mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag);
       mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag);
       tcgen05_fence_after();
       const uint64_t a0 = make_smem_desc_sw128(smem_u32(s_op), 16, 1024);   // offsets are added as in the state kernel
