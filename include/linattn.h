@@ -29,7 +29,7 @@
  *    token range.
  *  - dtype LINATTN_BF16: Q, K, V, O are bfloat16; products are exact in fp32,
  *    accumulation is fp32, O is rounded to nearest-even once at the store.
- *    dtype LINATTN_F32: fp32 in and out, fp32 arithmetic.
+ *    dtype LINATTN_F32: fp32 in and out, fp32 accuracy (products of three-part bf16 sums, fp32 accumulation).
  *  - A "state" is, per (b, h), a (d+1) x d fp32 matrix W stored row-major,
  *    units ordered [B][H]:   W[j][i] = S[i][j]  for j < d  (i: key feature,
  *    j: value feature),      W[d][i] = z[i].

@@ -37,8 +37,8 @@ int resolve(const linattn_desc* desc, long long N, Problem* out) {
 }
 
 // Alignment rule of the header: 16-byte pointers, strides multiples of 16 bytes.  Enforced for the
-// shapes the tensor-core kernels take (their TMA descriptors need it); the FMA kernels use scalar
-// accesses and only need natural alignment.
+// shapes the fused kernel takes (its TMA descriptors need it); the others choose a kernel by alignment
+// (split_ok) and only need natural alignment.
 int check_alignment(const Problem& p, const void* a, const void* b, const void* c, const void* d) {
   if (!umma_supported(p)) return LINATTN_OK;
   const void* ptrs[4] = {a, b, c, d};
@@ -79,12 +79,8 @@ int run_passes(const Problem& p, const void* k, const void* v, const void* q, vo
     UmmaCall c{k, v, q, o, state, base, accumulate, eps, nullptr};
     return umma_run(p, c, workspace, stream);
   }
-  if (k && accumulate && base && base != state) {
-    if (cudaMemcpyAsync(state, base, state_bytes_of(p), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
-      return LINATTN_ERR_CUDA;
-  }
   if (k) {
-    int st = cuda_status(fma_state(p, k, v, state, accumulate, partials_of(workspace), ctrl_of(workspace), stream));
+    int st = cuda_status(fma_state(p, k, v, state, accumulate ? (base ? base : state) : nullptr, partials_of(workspace), ctrl_of(workspace), stream));
     if (st != LINATTN_OK) return st;
   }
   if (q) return cuda_status(fma_apply(p, q, state, o, eps, ctrl_of(workspace), stream));
@@ -108,11 +104,7 @@ int run_rope(const Problem& p, const void* q, const void* k, const void* v, void
     UmmaCall c{k, v, q, o, state, base, accumulate, eps, rope};
     return umma_run(p, c, workspace, stream);
   }
-  if (accumulate && base && base != state) {
-    if (cudaMemcpyAsync(state, base, state_bytes_of(p), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
-      return LINATTN_ERR_CUDA;
-  }
-  int st = cuda_status(fma_state(p, k, v, state, accumulate, partials_of(workspace), ctrl_of(workspace), stream, rope));
+  int st = cuda_status(fma_state(p, k, v, state, accumulate ? (base ? base : state) : nullptr, partials_of(workspace), ctrl_of(workspace), stream, rope));
   if (st != LINATTN_OK || !q) return st;
   return cuda_status(fma_apply(p, q, state, o, eps, ctrl_of(workspace), stream, rope));
 }
@@ -203,7 +195,7 @@ static int step_rope_impl(blocklin_cache* cache, const Problem& p, const void* q
   if (o_blk && (o_blk == q_blk || o_blk == k_blk || o_blk == v_blk)) return LINATTN_ERR_INVALID_ARG;
   int st = check_alignment(p, q_blk, k_blk, v_blk, o_blk);
   if (st != LINATTN_OK) return st;
-  // the tensor-core kernel fetches the rotations in 16-byte chunks; the FMA kernels pair by pair
+  // the tensor-core kernel fetches the rotations in 16-byte chunks; the others choose by its alignment (split_ok)
   if (reinterpret_cast<uintptr_t>(rope_table_blk) & (umma_rope_supported(p) ? 15u : 3u)) return LINATTN_ERR_BAD_ALIGNMENT;
   if (cache->workspace_bytes < rope_workspace_need(p)) return LINATTN_ERR_WORKSPACE_TOO_SMALL;
   if (p.N == 0) return LINATTN_OK;

@@ -33,7 +33,7 @@ static_assert(sizeof(WorkspaceCtrl) <= LINATTN_WORKSPACE_CTRL_BYTES, "control bl
 void count_launches(int n);
 
 constexpr int kMaxCtas = 256;        // upper bound on the persistent grid (B200 has 148 SMs)
-constexpr int kFmaMaxChunks = 64;    // split-N partials per unit on the FMA path
+constexpr int kFmaMaxChunks = 64;    // split-N partials per unit on the fp32-accurate path
 constexpr int kFmaMinChunkTokens = 512;
 
 inline int fma_chunks(long long N) {
@@ -42,17 +42,18 @@ inline int fma_chunks(long long N) {
   return p > kFmaMaxChunks ? kFmaMaxChunks : (int)p;
 }
 
-// ---- FMA kernels (fp32 I/O path, and bf16 shapes the tensor-core kernels do not take) ----
-// state_out = (accumulate ? state_out : 0) + state of tokens [0, N); partials is scratch.
+// ---- fp32-accurate path (fp32 I/O, and bf16 shapes the fused kernel does not take) ----
+// state_out = (base ? base : 0) + state of tokens [0, N), base may be state_out itself; partials is scratch.
 // rope: Eq. 2 with its rotary factors, table [N][d/2] of (cos, sin) fp16 pairs, one per pair rotation.
-cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* state_out, bool accumulate,
+cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* state_out, const float* base,
                       float* partials, WorkspaceCtrl* ctrl, cudaStream_t stream, const __half2* rope = nullptr);
 cudaError_t fma_apply(const Problem& p, const void* q, const float* state, void* o, float eps, WorkspaceCtrl* ctrl, cudaStream_t stream,
                       const __half2* rope = nullptr);
 // The same on the tensor cores (split_kernels.cu); ctrl: the workspace's control block.
 bool split_ok(const Problem& p, const void* a, const void* b, const __half2* rope);
-cudaError_t split_state_partials(const Problem& p, const void* k, const void* v, float* partials, const __half2* rope, int* P,
-                                 WorkspaceCtrl* ctrl, cudaStream_t stream);
+// *P = 0: `state` is complete ((base ? base : 0) + the tokens' state); otherwise *P partial states per unit are to be summed.
+cudaError_t split_state(const Problem& p, const void* k, const void* v, const float* base, float* state, float* partials,
+                        const __half2* rope, int* P, WorkspaceCtrl* ctrl, cudaStream_t stream);
 cudaError_t split_apply(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* rope,
                         WorkspaceCtrl* ctrl, cudaStream_t stream);
 // blk: [B][M][H][(d+1)*d] per-block states -> running states after each block (on top of cache [B][H][..]), cache := last.

@@ -115,13 +115,13 @@ fma_state_partial(const T* __restrict__ k, const T* __restrict__ v, Problem p, i
   }
 }
 
-// grid (ceil(E/256), units): state[u][e] = (accumulate ? state[u][e] : 0) + sum_c partial[u][c][e], c ascending.
+// grid (ceil(E/256), units): state[u][e] = (base ? base[u][e] : 0) + sum_c partial[u][c][e], c ascending.
 __global__ void __launch_bounds__(kThreads)
-fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* __restrict__ state, int accumulate) {
+fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* state, const float* base) {
   const long long e = (long long)blockIdx.x * kThreads + threadIdx.x;
   const int u = blockIdx.y;
   if (e >= E) return;
-  double sum = accumulate ? (double)state[(long long)u * E + e] : 0.0;
+  double sum = base ? (double)base[(long long)u * E + e] : 0.0;
 #pragma unroll 8   // eight loads in flight
   for (int c = 0; c < P; ++c) sum += (double)partials[((long long)u * P + c) * E + e];
   state[(long long)u * E + e] = (float)sum;
@@ -306,19 +306,20 @@ cudaError_t rope_pack(const float* cs, const float* sn, long long count, __half2
   return cudaGetLastError();
 }
 
-cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* state_out, bool accumulate,
+cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* state_out, const float* base,
                       float* partials, WorkspaceCtrl* ctrl, cudaStream_t stream, const __half2* rope) {
   const long long E = p.state_elems();
+  const size_t bytes = sizeof(float) * E * p.units();
   if (p.N == 0) {
-    if (accumulate) return cudaSuccess;
-    return cudaMemsetAsync(state_out, 0, sizeof(float) * E * p.units(), stream);
+    if (!base) return cudaMemsetAsync(state_out, 0, bytes, stream);
+    return base == state_out ? cudaSuccess : cudaMemcpyAsync(state_out, base, bytes, cudaMemcpyDeviceToDevice, stream);
   }
   int P = fma_chunks(p.N);
-  cudaError_t e = split_ok(p, k, v, rope) ? split_state_partials(p, k, v, partials, rope, &P, ctrl, stream)
+  cudaError_t e = split_ok(p, k, v, rope) ? split_state(p, k, v, base, state_out, partials, rope, &P, ctrl, stream)
                                           : state_partial_any(p, k, v, P, partials, rope, stream);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || P == 0) return e;
   dim3 grid((unsigned)((E + kThreads - 1) / kThreads), p.units());
-  fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, accumulate ? 1 : 0);
+  fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, base);
   count_launches(1);
   return cudaGetLastError();
 }

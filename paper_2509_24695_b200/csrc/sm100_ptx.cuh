@@ -88,6 +88,24 @@ __device__ __forceinline__ void bulk_store(void* gmem_dst, const void* smem_src,
 __device__ __forceinline__ void tcgen05_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tcgen05_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// ---------------------------------------------------------------- thread-block clusters
+// All threads of all CTAs of the cluster meet; what they wrote to shared memory before is seen by all after.
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();   // (.aligned: whole warps)
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Address of `smem` in the shared memory of CTA `rank` of the cluster, and a load through it.
+__device__ __forceinline__ uint32_t cluster_address(const void* smem, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(smem)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float cluster_load(uint32_t address) {
+  float x;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(address) : "memory");
+  return x;
+}
+
 // ---------------------------------------------------------------- TMA (tiled, 4-D; every load lands in this CTA alone)
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");

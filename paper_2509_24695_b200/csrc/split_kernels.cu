@@ -151,7 +151,10 @@ struct StateShape : Shape<T, R, ROPE> {
   static constexpr int TAB = ROPE ? PIECES * kPrepare * (int)sizeof(typename B::Tab) : 0;
   static constexpr int RAW = 2 * PIECES * kPrepare * 16 + TAB;
   static constexpr int Z_BYTES = TOK * B::DP * 4;
-  static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > Z_BYTES ? RAW_STAGES * RAW : Z_BYTES) + 64;   // (barriers last)
+  static constexpr int OWN_BYTES = (B::DP + 1) * B::DP * 4;   // a CTA's state, where its cluster reads it
+  static constexpr int Z_OFF = OWN_BYTES > 2 * STAGE ? OWN_BYTES : 2 * STAGE;
+  static constexpr int TAIL = Z_OFF + Z_BYTES - 2 * STAGE;
+  static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > TAIL ? RAW_STAGES * RAW : TAIL) + 64;   // (barriers last)
   static constexpr int LEAD = TOK / 32;                      // accumulators of the leading products: chains of two K steps
   static constexpr bool REST = B::QK_PARTS + B::V_PARTS > 2;
   static constexpr int ACC = B::DP <= 64 ? 64 : 128;         // TMEM columns between accumulators
@@ -160,7 +163,11 @@ struct StateShape : Shape<T, R, ROPE> {
   static_assert(2 * SET <= 512, "tensor memory");
 };
 
-// grid (P, units): partial state of the tiles [c * tiles / P, (c + 1) * tiles / P) of one unit, in the library's layout.
+// grid (P, units): state of the tiles [c * tiles / P, (c + 1) * tiles / P) of one unit, in the library's layout.  Either
+// every CTA writes a partial state (state null), or the P CTAs of a unit are a cluster and add theirs up, in the order of
+// fma_state_reduce and in 64 bits as there, through distributed shared memory: state = (base ? base : 0) + sum.  No second
+// kernel then, and no partial states, so that P is not bound by their room; but a cluster has to fit into one GPC (8 CTAs
+// of this size at most, and 15 such clusters on the chip), so that large inputs want the other form (launch_state).
 //
 // Measured (32 760 tokens, 20 heads of 112, fp32; floor: 587 MB, 90 us at the copy rate): 176 us with the reduce of the
 // partial states (192 with every warp preparing and draining in turn), where the general kernels take 1050 (fp32 pipe at a
@@ -170,7 +177,7 @@ struct StateShape : Shape<T, R, ROPE> {
 template <typename T, int R, bool ROPE>
 __global__ void __launch_bounds__(kBlock, 1)
 split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, int P, float* __restrict__ partials,
-                   const __half2* __restrict__ tab, WorkspaceCtrl* ctrl) {
+                   const float* base_state, float* state, const __half2* __restrict__ tab, WorkspaceCtrl* ctrl) {
   using S = StateShape<T, R, ROPE>;
   using Tab = typename S::Tab;
   constexpr int E = S::E, PIECES = S::PIECES;
@@ -342,14 +349,15 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   }
   __syncthreads();
 
-  // W[j][i] = S[i][j], W[d][i] = z[i]
-  float* out = partials + ((long long)u * P + c) * p.state_elems();
+  // W[j][i] = S[i][j], W[d][i] = z[i]; z's rows are added up in the raw pieces' room, behind what a cluster's state takes
+  float* own = reinterpret_cast<float*>(smem);
+  float* out = state ? own : partials + ((long long)u * P + c) * p.state_elems();
+  float* zs = reinterpret_cast<float*>(smem + S::Z_OFF);   // [row][d]
   if (!preparing && warp < kMmaWarp && key < d) {
 #pragma unroll
     for (int x = 0; x < COLS; ++x)
-      if (col0 + x < d) out[(long long)(col0 + x) * d + key] = sum[x];
+      if (col0 + x < d) out[(col0 + x) * d + key] = sum[x];
   }
-  float* zs = reinterpret_cast<float*>(raw);   // [row][d]
 #pragma unroll
   for (int i = 0; i < PIECES; ++i) {
     const int f = feature(i);
@@ -361,7 +369,26 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   if (tid < d) {
     float zt = 0.f;
     for (int r = 0; r < S::TOK; ++r) zt += zs[r * d + tid];
-    out[(long long)d * d + tid] = zt;
+    out[d * d + tid] = zt;
+  }
+  if (state) {
+    cluster_sync();
+    const int elems = (int)p.state_elems(), e0 = (int)((long long)c * elems / P), e1 = (int)((long long)(c + 1) * elems / P);
+    const long long at = (long long)u * elems;
+    uint32_t peer[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) peer[r] = cluster_address(own, r < P ? r : 0);
+    for (int e = e0 + tid; e < e1; e += kBlock) {
+      float x[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) x[r] = r < P ? cluster_load(peer[r] + 4 * e) : 0.f;
+      double total = base_state ? (double)base_state[at + e] : 0.0;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < P) total += (double)x[r];
+      state[at + e] = (float)total;
+    }
+    cluster_sync();   // nobody leaves while its state is being read
   }
   if (*abort_flag && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
   if (warp == 0) tmem_dealloc(tmem, S::COLS);
@@ -631,19 +658,63 @@ int pieces(long long tiles, int units, int slots, long long most, double fixed) 
   return (int)best;
 }
 
+// Clusters of c CTAs of `kernel` that fit on the device together (0: none), c = 1..8.
+template <typename K>
+int clusters_at_once(K kernel, int smem, int c, int (&cached)[64][9]) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cached[dev][c]) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)c, 1, 1};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(c); cfg.blockDim = dim3(kBlock); cfg.dynamicSmemBytes = smem;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    cached[dev][c] = n > 0 ? n : -1;
+  }
+  return cached[dev][c] > 0 ? cached[dev][c] : 0;
+}
+
+// *P = 0: the state is complete; otherwise *P partial states per unit are to be summed.
 template <typename T, int R, bool ROPE>
-cudaError_t launch_state(const Problem& p, const void* k, const void* v, float* partials, const __half2* tab, int* P,
-                         WorkspaceCtrl* ctrl, cudaStream_t stream) {
+cudaError_t launch_state(const Problem& p, const void* k, const void* v, const float* base, float* state, float* partials,
+                         const __half2* tab, int* P, WorkspaceCtrl* ctrl, cudaStream_t stream) {
   using S = StateShape<T, R, ROPE>;
   static_assert(S::SMEM <= 227 * 1024, "shared memory of the state kernel");
   static bool done[64] = {false};
-  const cudaError_t e = allow_smem(split_state_kernel<T, R, ROPE>, S::SMEM, done);
+  static int fits[64][9] = {{0}};
+  auto kernel = split_state_kernel<T, R, ROPE>;
+  const cudaError_t e = allow_smem(kernel, S::SMEM, done);
   if (e != cudaSuccess) return e;
-  *P = pieces((p.N + S::TOK - 1) / S::TOK, p.units(), sms(), fma_chunks(p.N), 6.0);
-  split_state_kernel<T, R, ROPE><<<dim3(*P, p.units()), kBlock, S::SMEM, stream>>>((const T*)k, (const T*)v, p, *P, partials,
-                                                                                    tab, ctrl);
+  const long long tiles = (p.N + S::TOK - 1) / S::TOK;
+  // In tiles: a CTA costs six whatever its share, the sum of partial states (a kernel of its own) one more than a cluster's.
+  // Measured, cached step, fp32, 20 heads of 112, cluster against partial states: 300 tokens 24.9 against 33.3 us, 512 29.9
+  // against 43.8, 1200 37.6 against 43.7, 4680 75.9 against 73.9; forward of 3000 tokens, 35 heads of 64: 62.5 against 57.8.
+  *P = pieces(tiles, p.units(), sms(), fma_chunks(p.N), 6.0);
+  const double apart = (double)(((long long)*P * p.units() + sms() - 1) / sms()) * ((double)((tiles + *P - 1) / *P) + 6.0) + 1.0;
+  int together = 0;
+  double cost = apart;
+  for (int c = 1; c <= 8 && c <= tiles; ++c) {
+    const int at_once = clusters_at_once(kernel, S::SMEM, c, fits);
+    if (!at_once) continue;
+    const double now = (double)((p.units() + at_once - 1) / at_once) * ((double)((tiles + c - 1) / c) + 6.0);
+    if (now < cost) { together = c; cost = now; }
+  }
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)(together ? together : 1), 1, 1};
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(together ? together : *P, p.units());
+  cfg.blockDim = dim3(kBlock); cfg.dynamicSmemBytes = S::SMEM; cfg.stream = stream;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  const cudaError_t st = cudaLaunchKernelEx(&cfg, kernel, (const T*)k, (const T*)v, p, together ? together : *P, partials, base,
+                                            together ? state : (float*)nullptr, tab, ctrl);
+  if (st != cudaSuccess) { cudaGetLastError(); return st; }
+  if (together) *P = 0;
   count_launches(1);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 template <typename T, int R, bool ROPE>
@@ -684,14 +755,14 @@ bool split_ok(const Problem& p, const void* a, const void* b, const __half2* rop
          p.sn % per == 0 && p.sh % per == 0 && (reinterpret_cast<uintptr_t>(rope) & tab_align) == 0;
 }
 
-cudaError_t split_state_partials(const Problem& p, const void* k, const void* v, float* partials, const __half2* rope, int* P,
-                                 WorkspaceCtrl* ctrl, cudaStream_t stream) {
+cudaError_t split_state(const Problem& p, const void* k, const void* v, const float* base, float* state, float* partials,
+                        const __half2* rope, int* P, WorkspaceCtrl* ctrl, cudaStream_t stream) {
   if (p.dtype == LINATTN_F32) {
-    if (rope) { LINATTN_SPLIT(launch_state, float, true, p, k, v, partials, rope, P, ctrl, stream) }
-    LINATTN_SPLIT(launch_state, float, false, p, k, v, partials, rope, P, ctrl, stream)
+    if (rope) { LINATTN_SPLIT(launch_state, float, true, p, k, v, base, state, partials, rope, P, ctrl, stream) }
+    LINATTN_SPLIT(launch_state, float, false, p, k, v, base, state, partials, rope, P, ctrl, stream)
   }
-  if (rope) { LINATTN_SPLIT(launch_state, __nv_bfloat16, true, p, k, v, partials, rope, P, ctrl, stream) }
-  LINATTN_SPLIT(launch_state, __nv_bfloat16, false, p, k, v, partials, rope, P, ctrl, stream)
+  if (rope) { LINATTN_SPLIT(launch_state, __nv_bfloat16, true, p, k, v, base, state, partials, rope, P, ctrl, stream) }
+  LINATTN_SPLIT(launch_state, __nv_bfloat16, false, p, k, v, base, state, partials, rope, P, ctrl, stream)
 }
 
 cudaError_t split_apply(const Problem& p, const void* q, const float* state, void* o, float eps, const __half2* rope,

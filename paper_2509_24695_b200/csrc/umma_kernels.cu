@@ -1794,7 +1794,7 @@ size_t umma_partial_bytes(const Problem& p, bool rope) {
 // The rotary variant runs on the tensor cores wherever the plain kernel does.  d = 112, the paper's: the denominators
 // travel in the zero padding of the 112-feature rows; every other head dim: in a small shared-memory array per slot
 // and head of the group.  With packed heads (d = 32, 64) both boxes of a row use the same 16-byte chunk of the
-// rotation table, since box 1 starts a new head.  Everything else takes the FMA kernels.
+// rotation table, since box 1 starts a new head.  Everything else takes the fp32-accurate kernels.
 bool umma_rope_supported(const Problem& p) { return umma_supported(p); }
 
 int umma_run(const Problem& p, const UmmaCall& c, void* workspace, cudaStream_t stream) {

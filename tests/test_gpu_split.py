@@ -80,3 +80,25 @@ def test_rows_off_the_16_byte_grid(la, orc, dtype, d):
     if out is not None:
         o = la.linattn_forward(to_dev(q), to_dev(k), to_dev(v), EPS, out=out)
         check(dtype, to_f64(o), ref, "shifted output")
+
+
+@pytest.mark.parametrize("dtype,d,N", [("f32", 112, 5000), ("bf16", 72, 9000), ("f32", 64, 200), ("bf16", 96, 700)])
+def test_cached_step_and_its_read_only_twin(la, orc, dtype, d, N):
+    """On top of an old state, with the CTAs of a unit as a cluster (few tokens) and with partial states (many)."""
+    import torch
+
+    B, H = 1, 3
+    q, k, v = gen(B, N, H, d, 7200 + N, dtype)
+    k0, v0 = gen(B, 50, H, d, 7300 + N, dtype)[1:]
+    td = torch.float32 if dtype == "f32" else torch.bfloat16
+    cache = la.BlockLinCache(B, H, d, td, "cuda", max_T_b=N, eps=EPS)
+    cache.step(None, to_dev(k0), to_dev(v0))
+    before = cache.state.clone()
+    o_peek = cache.peek(to_dev(q), to_dev(k), to_dev(v))
+    assert torch.equal(cache.state, before)
+    o = cache.step(to_dev(q), to_dev(k), to_dev(v))
+    assert torch.equal(o, o_peek) and cache.status() == 0
+    (S0, z0), (S, z) = orc.state(k0, v0), orc.state(k, v)
+    assert_state_close(to_f64(cache.state), S0 + S, z0 + z, 1e-5, f"cache N={N} d={d} {dtype}")
+    ref = orc.apply_rows(q, S0 + S, z0 + z, EPS, np.arange(N))
+    check(dtype, to_f64(o), ref, f"step N={N} d={d} {dtype}")
