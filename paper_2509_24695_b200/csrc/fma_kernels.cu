@@ -116,15 +116,17 @@ fma_state_partial(const T* __restrict__ k, const T* __restrict__ v, Problem p, i
 }
 
 // grid (ceil(E/256), units): state[u][e] = (base ? base[u][e] : 0) + sum_c partial[u][c][e], c ascending.
+// status (null: not asked): where a timeout of the partial states' kernel is recorded; the state then stays as it was.
 __global__ void __launch_bounds__(kThreads)
-fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* state, const float* base) {
+fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* state, const float* base, const int* status) {
   const long long e = (long long)blockIdx.x * kThreads + threadIdx.x;
   const int u = blockIdx.y;
   if (e >= E) return;
+  const int recorded = status ? *status : LINATTN_OK;
   double sum = base ? (double)base[(long long)u * E + e] : 0.0;
 #pragma unroll 8   // eight loads in flight
   for (int c = 0; c < P; ++c) sum += (double)partials[((long long)u * P + c) * E + e];
-  state[(long long)u * E + e] = (float)sum;
+  if (recorded == LINATTN_OK) state[(long long)u * E + e] = (float)sum;
 }
 
 // grid (ceil(N/64), units).  Thread (tn, tj) owns tokens tn + 16*r (r < 4) and outputs j = tj + 16*c.
@@ -315,11 +317,12 @@ cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* sta
     return base == state_out ? cudaSuccess : cudaMemcpyAsync(state_out, base, bytes, cudaMemcpyDeviceToDevice, stream);
   }
   int P = fma_chunks(p.N);
-  cudaError_t e = split_ok(p, k, v, rope) ? split_state(p, k, v, base, state_out, partials, rope, &P, ctrl, stream)
-                                          : state_partial_any(p, k, v, P, partials, rope, stream);
+  const bool split = split_ok(p, k, v, rope);
+  cudaError_t e = split ? split_state(p, k, v, base, state_out, partials, rope, &P, ctrl, stream)
+                        : state_partial_any(p, k, v, P, partials, rope, stream);
   if (e != cudaSuccess || P == 0) return e;
   dim3 grid((unsigned)((E + kThreads - 1) / kThreads), p.units());
-  fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, base);
+  fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, base, split ? &ctrl->status : nullptr);
   count_launches(1);
   return cudaGetLastError();
 }

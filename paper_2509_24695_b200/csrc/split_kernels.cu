@@ -134,6 +134,14 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~(uintptr_t)1023);
 }
 
+// After a wait that ran out: the MMAs that were issued still read this CTA's shared memory and write its tensor memory.
+// They get a bounded time to finish before either is used for something else (whole CTA).
+__device__ __forceinline__ void let_finish(uint64_t* finished) {
+  if (threadIdx.x == 0)
+    for (int spin = 0; spin < 4096 && !mbar_try_wait(finished, 0); ++spin) __nanosleep(64);
+  __syncthreads();
+}
+
 // ---------------------------------------------------------------- state
 template <typename T, int R, bool ROPE>
 struct StateShape : Shape<T, R, ROPE> {
@@ -188,7 +196,8 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   uint64_t* done = reinterpret_cast<uint64_t*>(raw + (S::SMEM - 1024 - 2 * S::STAGE - 64));   // [2] the tile's MMAs are complete
   uint64_t* ready = done + 2;                                                               // [2] the tile's parts are in its stage
   uint64_t* drained = ready + 2;                                                            // [2] its accumulators are read
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drained + 2);
+  uint64_t* finished = drained + 2;                                                         // every MMA issued is complete
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(finished + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d, u = blockIdx.y, c = blockIdx.x;
@@ -198,6 +207,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
 
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
+    mbar_init(finished, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -287,7 +297,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
     for (int t = 0; t < tiles; ++t) {
       issue(t + 2, (t + 2) % S::RAW_STAGES);
       copy_wait<2>();
-      if (t >= 2) mbar_wait(&done[t & 1], ((t - 2) >> 1) & 1, abort_flag);   // the MMAs that read this stage
+      if (t >= 2 && !mbar_wait(&done[t & 1], ((t - 2) >> 1) & 1, abort_flag)) break;   // the MMAs that read this stage
       convert(t % S::RAW_STAGES, smem + (t & 1) * S::STAGE);
       fence_proxy_async_smem();
       mbar_arrive(&ready[t & 1]);
@@ -296,8 +306,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   } else if (warp < kMmaWarp) {
     const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0;
     for (int t = 0; t < tiles; ++t) {
-      mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
-      __syncwarp();   // tcgen05.ld wants whole warps
+      if (!__all_sync(0xffffffffu, mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag))) break;   // tcgen05.ld wants whole warps
       tcgen05_fence_after();
       if ((warp & 3) * 32 < d) {
 #pragma unroll
@@ -319,9 +328,10 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       mbar_arrive(&drained[t & 1]);
     }
   } else if (lane == 0) {
-    for (int t = 0; t < tiles; ++t) {
-      if (t >= 2) mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag);
-      mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag);
+    int t = 0;
+    for (; t < tiles; ++t) {
+      if (t >= 2 && !mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag)) break;
+      if (!mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag)) break;
       tcgen05_fence_after();
       constexpr uint32_t LBO = S::BOXES > 1 ? S::BOX : 0;   // 64 features: rows 64..127 of the MMA repeat them and are ignored
       // shared-memory addresses are below 2^18, so an offset of a multiple of 16 bytes is added to a descriptor as it is
@@ -346,51 +356,61 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       for (int kk = 0; kk < S::TOK / 16; ++kk) mma(kk, 0, 0, kk % S::LEAD, kk >= S::LEAD);
       umma_commit(&done[t & 1]);
     }
+    if (t > 0) umma_commit(finished); else mbar_arrive(finished);
   }
   __syncthreads();
+  const bool aborted = *abort_flag != 0;
+  if (aborted) let_finish(finished);
 
   // W[j][i] = S[i][j], W[d][i] = z[i]; z's rows are added up in the raw pieces' room, behind what a cluster's state takes
   float* own = reinterpret_cast<float*>(smem);
-  float* out = state ? own : partials + ((long long)u * P + c) * p.state_elems();
-  float* zs = reinterpret_cast<float*>(smem + S::Z_OFF);   // [row][d]
-  if (!preparing && warp < kMmaWarp && key < d) {
+  if (!aborted) {
+    float* out = state ? own : partials + ((long long)u * P + c) * p.state_elems();
+    float* zs = reinterpret_cast<float*>(smem + S::Z_OFF);   // [row][d]
+    if (!preparing && warp < kMmaWarp && key < d) {
 #pragma unroll
-    for (int x = 0; x < COLS; ++x)
-      if (col0 + x < d) out[(col0 + x) * d + key] = sum[x];
-  }
+      for (int x = 0; x < COLS; ++x)
+        if (col0 + x < d) out[(col0 + x) * d + key] = sum[x];
+    }
 #pragma unroll
-  for (int i = 0; i < PIECES; ++i) {
-    const int f = feature(i);
-    if (!preparing || f >= d) continue;
+    for (int i = 0; i < PIECES; ++i) {
+      const int f = feature(i);
+      if (!preparing || f >= d) continue;
 #pragma unroll
-    for (int e = 0; e < E; ++e) zs[row * d + f + e] = z[i][e];
-  }
-  __syncthreads();
-  if (tid < d) {
-    float zt = 0.f;
-    for (int r = 0; r < S::TOK; ++r) zt += zs[r * d + tid];
-    out[d * d + tid] = zt;
+      for (int e = 0; e < E; ++e) zs[row * d + f + e] = z[i][e];
+    }
+    __syncthreads();
+    if (tid < d) {
+      float zt = 0.f;
+      for (int r = 0; r < S::TOK; ++r) zt += zs[r * d + tid];
+      out[d * d + tid] = zt;
+    }
+  } else if (tid == 0) {
+    ctrl->status = LINATTN_ERR_TIMEOUT;   // (a sum of partial states looks at it: fma_state_reduce)
   }
   if (state) {
     cluster_sync();
-    const int elems = (int)p.state_elems(), e0 = (int)((long long)c * elems / P), e1 = (int)((long long)(c + 1) * elems / P);
-    const long long at = (long long)u * elems;
-    uint32_t peer[8];
+    // a CTA that gave up has nothing to add: then the state stays as it was
+    const bool gave_up = lane < P && lane < 8 && __float_as_int(cluster_load(cluster_address((const void*)abort_flag, lane))) != 0;
+    if (!__any_sync(0xffffffffu, gave_up)) {
+      const int elems = (int)p.state_elems(), e0 = (int)((long long)c * elems / P), e1 = (int)((long long)(c + 1) * elems / P);
+      const long long at = (long long)u * elems;
+      uint32_t peer[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) peer[r] = cluster_address(own, r < P ? r : 0);
-    for (int e = e0 + tid; e < e1; e += kBlock) {
-      float x[8];
+      for (int r = 0; r < 8; ++r) peer[r] = cluster_address(own, r < P ? r : 0);
+      for (int e = e0 + tid; e < e1; e += kBlock) {
+        float x[8];
 #pragma unroll
-      for (int r = 0; r < 8; ++r) x[r] = r < P ? cluster_load(peer[r] + 4 * e) : 0.f;
-      double total = base_state ? (double)base_state[at + e] : 0.0;
+        for (int r = 0; r < 8; ++r) x[r] = r < P ? cluster_load(peer[r] + 4 * e) : 0.f;
+        double total = base_state ? (double)base_state[at + e] : 0.0;
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (r < P) total += (double)x[r];
-      state[at + e] = (float)total;
+        for (int r = 0; r < 8; ++r)
+          if (r < P) total += (double)x[r];
+        state[at + e] = (float)total;
+      }
     }
     cluster_sync();   // nobody leaves while its state is being read
   }
-  if (*abort_flag && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
   if (warp == 0) tmem_dealloc(tmem, S::COLS);
 }
 
@@ -449,7 +469,8 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   uint64_t* done = reinterpret_cast<uint64_t*>(zs + 128);           // [2] each, as in the state kernel
   uint64_t* ready = done + 2;
   uint64_t* drained = ready + 2;
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drained + 2);
+  uint64_t* finished = drained + 2;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(finished + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
   uint8_t* raw = reinterpret_cast<uint8_t*>(done) + 64;
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -487,6 +508,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   }
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
+    mbar_init(finished, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -527,7 +549,8 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
         if (A::TAB_STAGED) tb[i] = *raw_tab(st, i);
       }
       issue(t + A::RAW_STAGES);
-      if (t >= 2) mbar_wait(&done[t & 1], ((t - 2) >> 1) & 1, abort_flag);   // the MMAs that read this stage
+      // the MMAs that read this stage (the warps below work as a whole, and leave as a whole)
+      if (t >= 2 && !__all_sync(0xffffffffu, mbar_wait(&done[t & 1], ((t - 2) >> 1) & 1, abort_flag))) break;
       float dn = 0.f;
 #pragma unroll
       for (int i = 0; i < PIECES; ++i) {
@@ -558,8 +581,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     constexpr int HALF = A::TOK / 2;
     const int j = (warp & 3) * 32 + lane, tok0 = ((warp >> 2) & 1) * HALF;
     for (int t = 0; t < tiles; ++t) {
-      mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag);
-      __syncwarp();   // tcgen05.ld wants whole warps
+      if (!__all_sync(0xffffffffu, mbar_wait(&done[t & 1], (t >> 1) & 1, abort_flag))) break;   // tcgen05.ld wants whole warps
       tcgen05_fence_after();
       if ((warp & 3) * 32 < d) {
         const uint32_t trow = tmem + (t & 1) * A::SET + ((uint32_t)((warp & 3) * 32) << 16) + tok0;
@@ -590,9 +612,10 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
       mbar_arrive(&drained[t & 1]);
     }
   } else if (lane == 0) {
-    for (int t = 0; t < tiles; ++t) {
-      if (t >= 2) mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag);
-      mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag);
+    int t = 0;
+    for (; t < tiles; ++t) {
+      if (t >= 2 && !mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag)) break;
+      if (!mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag)) break;
       tcgen05_fence_after();
       const uint64_t a0 = make_smem_desc_sw128(smem_u32(s_op), 16, 1024);   // offsets are added as in the state kernel
       const uint64_t b0 = make_smem_desc_sw128(smem_u32(stages + (t & 1) * A::STAGE), 16, 1024);
@@ -614,9 +637,12 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
       for (int kk = 0; kk < R; ++kk) mma(kk, 0, 0, kk % A::LEAD, kk >= A::LEAD);
       umma_commit(&done[t & 1]);
     }
+    if (t > 0) umma_commit(finished); else mbar_arrive(finished);
   }
   __syncthreads();
-  if (*abort_flag && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
+  const bool aborted = *abort_flag != 0;
+  if (aborted) let_finish(finished);
+  if (aborted && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
   if (warp == 0) { tcgen05_fence_after(); tmem_dealloc(tmem, 512); }
 }
 
