@@ -25,6 +25,7 @@ NVCC_FLAGS = [
     "-O3", "-std=c++17", "-lineinfo",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
     "--expt-relaxed-constexpr",
+    "--diag-error", "2809",   # the result of a [[nodiscard]] function (a bounded wait) is dropped
 ]
 
 

@@ -1053,13 +1053,15 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         }
       }
     };
-    // lone CTAs: z from the warps' sums, to memory and (plain) into the operand or (rotary) where this role finds it
+    // lone CTAs: z from the warps' sums, to memory and (plain) into the operand or (rotary) where this role finds it.
+    // A warp whose wait ran out does not report its share of the operand: then nothing is applied and no state leaves.
     auto finish_z = [&]() {
       mbar_arrive(z_left);
-      mbar_wait(z_left, 0, abort_flag);             // every warp's sums are in shared memory
-      if (!ROPE) mbar_wait(a_done, 0, abort_flag);  // the operand lies where the stages were
+      bool ok = mbar_wait(z_left, 0, abort_flag);               // every warp's sums are in shared memory
+      if (!ROPE) ok = ok && mbar_wait(a_done, 0, abort_flag);   // the operand lies where the stages were
       const int f = tr, g = f / D, h = ((int)blockIdx.x % p.HG) * C::G + g;
-      if (p.accumulate) mbar_wait(st_full, 0, abort_flag);
+      if (p.accumulate) ok = ok && mbar_wait(st_full, 0, abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) return;
       if (f < C::FEAT) {
         float z = sum_z_slots<ROPE>(z_slots, f);
         float* at = st + (g * (D + 1) + D) * D + (f - g * D);
@@ -1070,16 +1072,16 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       }
       if (ROPE) {
         mbar_arrive(z_done);
-        mbar_wait(z_done, 0, abort_flag);
+        ok = mbar_wait(z_done, 0, abort_flag);
       }
       // this role's share of the drain
-      if (__all_sync(0xffffffffu, mbar_wait(a_tfull, 0, abort_flag))) {
-        tcgen05_fence_after();
-        const int half = tr >> 7;   // (rotary variant: two warps of this role to a lane quarter)
-        if (ROPE) solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 3 + 3 * half, half ? 8 : 6);
-        else solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 4, 8);
-        tcgen05_fence_before();
-      }
+      ok = ok && mbar_wait(a_tfull, 0, abort_flag);
+      if (!__all_sync(0xffffffffu, ok)) return;
+      tcgen05_fence_after();
+      const int half = tr >> 7;   // (rotary variant: two warps of this role to a lane quarter)
+      if (ROPE) solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 3 + 3 * half, half ? 8 : 6);
+      else solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 4, 8);
+      tcgen05_fence_before();
       fence_proxy_async_smem();
       mbar_arrive(s_ready);
     };
@@ -1217,7 +1219,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       if (!ok) break;
       tcgen05_fence_after();
       if (SOLO) {
-        if (p.accumulate) { mbar_wait(st_full, 0, abort_flag); __syncwarp(); }
+        if (p.accumulate && !__all_sync(0xffffffffu, mbar_wait(st_full, 0, abort_flag))) break;
         solo_drain<D>(p, s_op, st, tmem_base, wq, lane, 0, ROPE ? 3 : 4);
         fence_proxy_async_smem();   // the operand is read by the MMAs of the apply pass
         tcgen05_fence_before();
