@@ -11,6 +11,11 @@
 // three; S is always three.  z and the denominators are plain fp32 sums.  The results are closer to the exact ones than
 // those of a chain of fp32 multiply-adds (see the figures at the kernels).
 //
+// Parts end where bf16 does: a value below 2^-110 loses up to 2^-134, an infinity has no parts (Inf - Inf), and products of
+// parts end at 2^-149.  So a CTA whose sums are not finite, or so small beside its data that this would show, does its
+// share again by plain fp32 multiply-adds, from memory (state_by_fma, apply_by_fma): the result is theirs, infinities and
+// NaN included.  The bounds are far from what data of one scale give: they are looked at once per CTA or token row.
+//
 // Operand layouts are those of the fused kernel: 128-byte swizzled rows of 64 features.  Every thread reads its own
 // pieces with private asynchronous copies, rectifies, rotates and splits them, and stores the parts; one thread issues
 // the MMAs, and other warps drain the accumulators.  All waits are on this CTA's own work and bounded.
@@ -29,6 +34,8 @@ constexpr int kPrepare = 256;
 constexpr int kDrain = 256;
 constexpr int kMmaWarp = (kPrepare + kDrain) / 32;
 constexpr int kBlock = kPrepare + kDrain + 32;
+// Barriers and flags of a CTA.  (The raw pieces follow: 80 bytes in their place cost bf16 heads of 96 14 % of the apply pass.)
+constexpr int kBarBytes = 128;
 
 template <typename T>
 struct Piece;   // 16 bytes of a row
@@ -113,10 +120,15 @@ __device__ __forceinline__ void take_part(float (&x)[E], uint32_t (&w)[E / 2]) {
 __device__ __forceinline__ void store_words(uint8_t* at, const uint32_t (&w)[2]) { *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]); }
 __device__ __forceinline__ void store_words(uint8_t* at, const uint32_t (&w)[4]) { *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]); }
 
+// left: collects what the last of three parts is taken from; bits in its lower half are lost.
 template <int PARTS, int E>
-__device__ __forceinline__ void store_parts(uint8_t* at, int part_bytes, float (&x)[E]) {
+__device__ __forceinline__ void store_parts(uint8_t* at, int part_bytes, float (&x)[E], uint32_t& left) {
 #pragma unroll
   for (int s = 0; s < PARTS; ++s) {
+    if (s == 2) {
+#pragma unroll
+      for (int e = 0; e < E; e += 2) left |= __float_as_uint(x[e]) | __float_as_uint(x[e + 1]);
+    }
     uint32_t w[E / 2];
     take_part(x, w);
     store_words(at + s * part_bytes, w);
@@ -142,6 +154,98 @@ __device__ __forceinline__ void let_finish(uint64_t* finished) {
   __syncthreads();
 }
 
+// ---------------------------------------------------------------- by plain multiply-adds (whole CTA)
+__device__ __forceinline__ void store_value(float* o, float x) { *o = x; }
+__device__ __forceinline__ void store_value(__nv_bfloat16* o, float x) { *o = __float2bfloat16_rn(x); }
+
+// Feature e of token n, rectified, as the general kernels read it: plain, and with ROPE turned.
+template <typename T, bool ROPE>
+__device__ __forceinline__ void phi_of(const T* row, const __half2* tab, int d, long long n, int e, float& plain, float& turned) {
+  plain = turned = fmaxf((float)row[e], 0.f);
+  if (ROPE) {
+    const float other = fmaxf((float)row[e ^ 1], 0.f);
+    const float2 cs = __half22float2(tab[n * (d / 2) + e / 2]);
+    turned = (e & 1) ? other * cs.y + plain * cs.x : plain * cs.x - other * cs.y;
+  }
+}
+
+// S of tokens [n0, n1) of the unit at k, v: out[j * d + i] = sum of phi(k)_i v_j, token after token.  scratch: 16 KB of shared
+// memory.  32 x 16 threads with a tile of 4 x 8 sums each.
+template <typename T, bool ROPE>
+__device__ __noinline__ void state_by_fma(const T* k, const T* v, const __half2* tab, int d, long long sn, long long n0, long long n1,
+                                          float* scratch, float* out) {
+  constexpr int TOK = 16;
+  float* ks = scratch;
+  float* vs = scratch + TOK * 128;
+  const int tid = (int)threadIdx.x, ti = tid >> 4, tj = tid & 15;
+  float acc[4][8];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int s = 0; s < 8; ++s) acc[r][s] = 0.f;
+  for (long long n = n0; n < n1; n += TOK) {
+    __syncthreads();
+    for (int idx = tid; idx < TOK * 128; idx += kBlock) {
+      const int t = idx >> 7, e = idx & 127;
+      float plain = 0.f, x = 0.f, y = 0.f;
+      if (n + t < n1 && e < d) {
+        phi_of<T, ROPE>(k + (n + t) * sn, tab, d, n + t, e, plain, x);
+        y = (float)v[(n + t) * sn + e];
+      }
+      ks[idx] = x;
+      vs[idx] = y;
+    }
+    __syncthreads();
+    const int live = (int)min((long long)TOK, n1 - n);
+    for (int t = 0; t < live && ti < 32; ++t) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float a = ks[t * 128 + ti + 32 * r];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) acc[r][s] = fmaf(a, vs[t * 128 + tj + 16 * s], acc[r][s]);
+      }
+    }
+  }
+  __syncthreads();   // out may be where the scratch is
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int i = ti + 32 * r, j = tj + 16 * s;
+      if (ti < 32 && i < d && j < d) out[j * d + i] = acc[r][s];
+    }
+}
+
+// Outputs of tokens [n0, n1) of the unit at q, o against the state W.  scratch: (d * d + d + 256 * warps) floats of shared
+// memory.  A warp takes a token.
+template <typename T, bool ROPE>
+__device__ __noinline__ void apply_by_fma(const T* q, const float* W, T* o, const __half2* tab, int d, long long sn, long long n0,
+                                          long long n1, float eps, float* scratch) {
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* ss = scratch;              // S[i][j]
+  float* zs = ss + d * d;           // z
+  float* qs = zs + d + 256 * warp;  // this token's phi(q), turned, then plain
+  float* qp = qs + 128;
+  for (int idx = tid; idx < d * d; idx += kBlock) ss[(idx % d) * d + idx / d] = W[idx];
+  for (int i = tid; i < d; i += kBlock) zs[i] = W[(long long)d * d + i];
+  __syncthreads();
+  for (long long n = n0 + warp; n < n1; n += kBlock / 32) {
+    for (int e = lane; e < d; e += 32) phi_of<T, ROPE>(q + n * sn, tab, d, n, e, qp[e], qs[e]);
+    __syncwarp();
+    float num[4] = {0.f, 0.f, 0.f, 0.f}, den = 0.f;
+    for (int i = 0; i < d; ++i) {
+      den = fmaf(qp[i], zs[i], den);
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+        if (lane + 32 * s < d) num[s] = fmaf(qs[i], ss[i * d + lane + 32 * s], num[s]);
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (lane + 32 * s < d) store_value(o + n * sn + lane + 32 * s, num[s] / (den + eps));
+    __syncwarp();
+  }
+}
+
 // ---------------------------------------------------------------- state
 template <typename T, int R, bool ROPE>
 struct StateShape : Shape<T, R, ROPE> {
@@ -158,17 +262,18 @@ struct StateShape : Shape<T, R, ROPE> {
   static constexpr int RAW_STAGES = 3;
   static constexpr int TAB = ROPE ? PIECES * kPrepare * (int)sizeof(typename B::Tab) : 0;
   static constexpr int RAW = 2 * PIECES * kPrepare * 16 + TAB;
-  static constexpr int Z_BYTES = TOK * B::DP * 4;
+  static constexpr int Z_BYTES = TOK * B::DP * 4 + 1024;      // (and the smallest sums)
   static constexpr int OWN_BYTES = (B::DP + 1) * B::DP * 4;   // a CTA's state, where its cluster reads it
   static constexpr int Z_OFF = OWN_BYTES > 2 * STAGE ? OWN_BYTES : 2 * STAGE;
   static constexpr int TAIL = Z_OFF + Z_BYTES - 2 * STAGE;
-  static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > TAIL ? RAW_STAGES * RAW : TAIL) + 64;   // (barriers last)
+  static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > TAIL ? RAW_STAGES * RAW : TAIL) + kBarBytes;   // (barriers last)
   static constexpr int LEAD = TOK / 32;                      // accumulators of the leading products: chains of two K steps
   static constexpr bool REST = B::QK_PARTS + B::V_PARTS > 2;
   static constexpr int ACC = B::DP <= 64 ? 64 : 128;         // TMEM columns between accumulators
   static constexpr int SET = (LEAD + (REST ? 1 : 0)) * ACC;  // one set collects a tile while the other is drained
   static constexpr int COLS = 2 * SET <= 128 ? 128 : 2 * SET <= 256 ? 256 : 512;
   static_assert(2 * SET <= 512, "tensor memory");
+  static_assert(!REST || SMEM - 1024 - kBarBytes - Z_OFF >= 16384, "scratch of state_by_fma");
 };
 
 // grid (P, units): state of the tiles [c * tiles / P, (c + 1) * tiles / P) of one unit, in the library's layout.  Either
@@ -193,12 +298,13 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint8_t* raw = smem + 2 * S::STAGE;
-  uint64_t* done = reinterpret_cast<uint64_t*>(raw + (S::SMEM - 1024 - 2 * S::STAGE - 64));   // [2] the tile's MMAs are complete
+  uint64_t* done = reinterpret_cast<uint64_t*>(raw + (S::SMEM - 1024 - 2 * S::STAGE - kBarBytes));   // [2] the tile's MMAs are complete
   uint64_t* ready = done + 2;                                                               // [2] the tile's parts are in its stage
   uint64_t* drained = ready + 2;                                                            // [2] its accumulators are read
   uint64_t* finished = drained + 2;                                                         // every MMA issued is complete
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(finished + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  volatile int* odd_flag = abort_flag + 1;   // the parts are not the values
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d, u = blockIdx.y, c = blockIdx.x;
   const long long all = (p.N + S::TOK - 1) / S::TOK;
@@ -208,7 +314,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
     mbar_init(finished, 1);
-    *abort_flag = 0;
+    *abort_flag = *odd_flag = 0;
     fence_mbar_init();
   }
   // padded features are never written and must read as zero
@@ -244,6 +350,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   for (int i = 0; i < PIECES; ++i)
 #pragma unroll
     for (int e = 0; e < E; ++e) z[i][e] = 0.f;
+  uint32_t left = 0;   // (a column of V so small that its sums are zero)
   auto convert = [&](int st, uint8_t* stage) {
     uint4 kr[PIECES], vr[PIECES];   // all reads before the first store: they overlap
     Tab tb[PIECES];
@@ -263,13 +370,14 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       for (int e = 0; e < E; ++e) { x[e] = fmaxf(x[e], 0.f); z[i][e] += x[e]; }   // phi = ReLU on the keys; z from the plain ones
       if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
       uint8_t* at = stage + operand_offset(row, f, S::BOX);
-      store_parts<S::QK_PARTS>(at, S::PART, x);
+      uint32_t unused = 0;
+      store_parts<S::QK_PARTS>(at, S::PART, x, unused);
       at += S::QK_PARTS * S::PART;
       if (S::V_PARTS == 1) {
         *reinterpret_cast<uint4*>(at) = vr[i];
       } else {
         widen(vr[i], x);
-        store_parts<S::V_PARTS>(at, S::PART, x);
+        store_parts<S::V_PARTS>(at, S::PART, x, left);
       }
     }
   };
@@ -303,6 +411,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       mbar_arrive(&ready[t & 1]);
     }
     copy_wait<0>();
+    if (left & 0xFFFFu) *odd_flag = 1;
   } else if (warp < kMmaWarp) {
     const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0;
     for (int t = 0; t < tiles; ++t) {
@@ -367,10 +476,21 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   if (!aborted) {
     float* out = state ? own : partials + ((long long)u * P + c) * p.state_elems();
     float* zs = reinterpret_cast<float*>(smem + S::Z_OFF);   // [row][d]
+    float* least = zs + S::TOK * S::DP;                      // [2][128] smallest sum of a key feature, by half of the columns
     if (!preparing && warp < kMmaWarp && key < d) {
+      uint32_t low = 0xFFFFFFFFu;   // twice the bits less one: zero is the largest
+      float rest = 0.f;             // NaN if a sum is not finite
 #pragma unroll
-      for (int x = 0; x < COLS; ++x)
-        if (col0 + x < d) out[(col0 + x) * d + key] = sum[x];
+      for (int x = 0; x < COLS; ++x) {
+        if (col0 + x >= d) continue;
+        out[(col0 + x) * d + key] = sum[x];
+        if (S::REST) {
+          low = min(low, 2 * __float_as_uint(sum[x]) - 1);
+          rest = fmaf(sum[x], 0.f, rest);
+        }
+      }
+      if (S::REST)   // (a sum that is not finite: 0; nothing but zeros: the largest number)
+        least[(warp >> 2 & 1) * 128 + key] = rest != 0.f ? 0.f : __uint_as_float(low == 0xFFFFFFFFu ? 0x7F7FFFFFu : (low >> 1) + 1);
     }
 #pragma unroll
     for (int i = 0; i < PIECES; ++i) {
@@ -384,6 +504,19 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       float zt = 0.f;
       for (int r = 0; r < S::TOK; ++r) zt += zs[r * d + tid];
       out[d * d + tid] = zt;
+      // Values of V below 2^-104 show in S_ij against z_i = sum of phi(k)_i, values of K in z_i against the tokens, and
+      // what products of parts lack in sums below 2^-100.
+      if (S::REST) {
+        const float low = fminf(least[tid], least[128 + tid]);
+        if (low < fmaxf(zt * 0x1p-104f, 0x1p-100f) || (zt > 0.f && zt < (float)tiles * (S::TOK * 0x1p-104f))) *odd_flag = 1;
+      }
+    }
+    if (S::REST) {   // (one part each: the products are exact)
+      __syncthreads();
+      if (*odd_flag) {
+        const long long n0 = first * S::TOK, n1 = min(p.N, (first + tiles) * S::TOK);
+        state_by_fma<T, ROPE>(k + base, v + base, tab, d, p.sn, n0, n1, zs, out);
+      }
     }
   } else if (tid == 0) {
     ctrl->status = LINATTN_ERR_TIMEOUT;   // (a sum of partial states looks at it: fma_state_reduce)
@@ -433,7 +566,7 @@ struct ApplyShape : Shape<T, R, ROPE> {
   static constexpr int S_BYTES = 3 * SPART;
   static constexpr int QBOX = TOK * 128, QPART = B::BOXES * QBOX, STAGE = B::QK_PARTS * QPART;
   static constexpr int DEN = (4 * TOK + 128) * 4;
-  static constexpr int FIXED = 1024 + S_BYTES + 2 * STAGE + DEN + 64;
+  static constexpr int FIXED = 1024 + S_BYTES + 2 * STAGE + DEN + kBarBytes;
   // a tile's rotations are staged beside its pieces where there is room (not for fp32 at d > 96: loaded where they are used)
   static constexpr bool TAB_STAGED = ROPE && FIXED + PIECES * kPrepare * (16 + (int)sizeof(typename B::Tab)) <= 227 * 1024;
   static constexpr int RAW = PIECES * kPrepare * (16 + (TAB_STAGED ? (int)sizeof(typename B::Tab) : 0));   // one tile as loaded
@@ -444,9 +577,6 @@ struct ApplyShape : Shape<T, R, ROPE> {
   static constexpr int ACC = TOK, SET = (LEAD + 1) * ACC;     // TMEM columns: two sets of accumulators
   static_assert(2 * SET <= 512, "tensor memory");
 };
-
-__device__ __forceinline__ void store_value(float* o, float x) { *o = x; }
-__device__ __forceinline__ void store_value(__nv_bfloat16* o, float x) { *o = __float2bfloat16_rn(x); }
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
 //
@@ -472,7 +602,8 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   uint64_t* finished = drained + 2;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(finished + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  uint8_t* raw = reinterpret_cast<uint8_t*>(done) + 64;
+  volatile int* odd_flag = abort_flag + 1;   // the parts are not the values
+  uint8_t* raw = reinterpret_cast<uint8_t*>(done) + kBarBytes;
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = p.d, u = blockIdx.y;
   const long long all = (p.N + A::TOK - 1) / A::TOK;
@@ -509,7 +640,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
     mbar_init(finished, 1);
-    *abort_flag = 0;
+    *abort_flag = *odd_flag = 0;
     fence_mbar_init();
   }
   if (warp == 0) { tmem_alloc(tmem_holder, 512); tmem_relinquish(); }
@@ -518,12 +649,22 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     for (int i = tid; i < (A::S_BYTES + 2 * A::STAGE) / 16; i += kBlock) reinterpret_cast<uint4*>(s_op)[i] = make_uint4(0, 0, 0, 0);
   if (tid < 128) zs[tid] = tid < d ? W[(long long)d * d + tid] : 0.f;
   __syncthreads();
+  uint32_t least = 0xFFFFFFFFu;   // twice the bits of the smallest |S| 2^38, less one (zero is the largest)
+  float rest = 0.f;               // NaN if one is not finite
   for (int idx = tid; idx < d * (d / 4); idx += kBlock) {
     const int j = idx / (d / 4), i = (idx - j * (d / 4)) * 4;
     float x[4];
     widen(__ldg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
-    store_parts<3>(s_op + operand_offset(j, i, A::SBOX), A::SPART, x);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float y = x[e] * 0x1p38f;
+      least = min(least, 2 * __float_as_uint(y) - 1);
+      rest = fmaf(y, 0.f, rest);
+    }
+    uint32_t unused = 0;
+    store_parts<3>(s_op + operand_offset(j, i, A::SBOX), A::SPART, x, unused);
   }
+  bool odd = rest != 0.f || least < 2 * __float_as_uint(0x1p-37f) - 1;   // |S| from 2^-75 to 2^90
   fence_proxy_async_smem();   // S and the zeros
   tcgen05_fence_before();
   __syncthreads();
@@ -531,6 +672,11 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   const uint32_t tmem = *tmem_holder;
 
   if (preparing) {
+    // denominators from z_max 2^-50 to z_max 2^35: rows of queries from 2^-57 to 2^35, products with S from 2^-132 to 2^125
+    float z_max = 0.f;
+    for (int i = lane; i < d; i += 32) z_max = fmaxf(z_max, fabsf(zs[i]));
+#pragma unroll
+    for (int st = 1; st < 32; st *= 2) z_max = fmaxf(z_max, __shfl_xor_sync(0xffffffffu, z_max, st));
     for (int t = 0; t < tiles; ++t) {
       uint8_t* stage = stages + (t & 1) * A::STAGE;
       const int st = t % A::RAW_STAGES;
@@ -566,11 +712,13 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
           dn = fmaf(x[e], z.x, dn); dn = fmaf(x[e + 1], z.y, dn); dn = fmaf(x[e + 2], z.z, dn); dn = fmaf(x[e + 3], z.w, dn);
         }
         if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
-        store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX), A::QPART, x);
+        uint32_t unused = 0;
+        store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX), A::QPART, x, unused);
       }
       __syncwarp();
 #pragma unroll
       for (int st2 = 1; st2 < A::LANES; st2 *= 2) dn += __shfl_xor_sync(0xffffffffu, dn, st2);
+      odd |= dn != 0.f && !(dn >= z_max * 0x1p-50f && dn <= z_max * 0x1p35f);
       if (l == 0) den[(t & 3) * A::TOK + row] = 1.0f / (dn + eps);   // eps added once, after the dot product
       fence_proxy_async_smem();
       mbar_arrive(&ready[t & 1]);
@@ -639,9 +787,14 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     }
     if (t > 0) umma_commit(finished); else mbar_arrive(finished);
   }
+  if (odd) *odd_flag = 1;
   __syncthreads();
   const bool aborted = *abort_flag != 0;
   if (aborted) let_finish(finished);
+  if (!aborted && *odd_flag) {
+    const long long n0 = first * A::TOK, n1 = min(p.N, (first + tiles) * A::TOK);
+    apply_by_fma<T, ROPE>(q + base, W, o + base, tab, d, p.sn, n0, n1, eps, reinterpret_cast<float*>(s_op));
+  }
   if (aborted && tid == 0) ctrl->status = LINATTN_ERR_TIMEOUT;
   if (warp == 0) { tcgen05_fence_after(); tmem_dealloc(tmem, 512); }
 }

@@ -102,3 +102,81 @@ def test_cached_step_and_its_read_only_twin(la, orc, dtype, d, N):
     assert_state_close(to_f64(cache.state), S0 + S, z0 + z, 1e-5, f"cache N={N} d={d} {dtype}")
     ref = orc.apply_rows(q, S0 + S, z0 + z, EPS, np.arange(N))
     check(dtype, to_f64(o), ref, f"step N={N} d={d} {dtype}")
+
+
+def turned(x, table):
+    """Feature pairs of x[B, N, H, d] turned by the (cos, sin) of their token, table [N, d/2, 2]."""
+    if table is None:
+        return x
+    c, s = table[None, :, None, :, 0], table[None, :, None, :, 1]
+    a, b = x[..., 0::2], x[..., 1::2]
+    return np.stack((a * c - b * s, b * c + a * s), axis=-1).reshape(x.shape)
+
+
+def relative(got, ref):
+    return np.sqrt(((got - ref) ** 2).sum() / (ref ** 2).sum())
+
+
+@pytest.mark.parametrize("dtype,d,rope", [("f32", 112, False), ("f32", 24, False), ("f32", 64, True), ("bf16", 72, True),
+                                          ("bf16", 40, False)])
+@pytest.mark.parametrize("N", [1, 50, 1500])
+def test_infinite_values(la, dtype, d, rope, N):
+    """One infinite value gives infinities in its column of S (and of the outputs, where no two of them meet), as a sum of
+    products does, and nothing anywhere else."""
+    import torch
+
+    B, H, j = 1, 3, 5
+    q, k, v = (to_dev(x) for x in gen(B, N, H, d, 7400 + N + d, dtype))
+    q, k = q.abs() + 0.125, k.abs() + 0.125          # every product with the infinity is one
+    v[0, N // 2, 1, j] = float("inf")
+    table = None
+    if rope:
+        cos, sin = synth.rope_table(1, 1, N, d)
+        table = la.rope_pack(to_dev(cos), to_dev(sin))
+    tab = None if table is None else table.cpu().numpy().astype(np.float64)
+    qn, kn, vn = to_f64(q), to_f64(k), to_f64(v)
+    kt, qt = turned(kn, tab), turned(qn, tab)
+    with np.errstate(invalid="ignore"):
+        S = np.einsum("bnhi,bnhj->bhij", kt, vn)
+        O = np.einsum("bnhi,bhij->bnhj", qt, S) / (np.einsum("bnhi,bhi->bnh", qn, kn.sum(1)) + EPS)[..., None]
+    if rope:
+        cache = la.BlockLinCache(B, H, d, q.dtype, "cuda", max_T_b=N, eps=EPS)
+        o, st = cache.step_rope(q, k, v, table), cache.state
+    else:
+        o, st = la.linattn_forward(q, k, v, EPS), la.linattn_state(k, v)
+    for got, ref, bar in ((to_f64(st)[:, :, :d].swapaxes(-1, -2), S, 1e-5), (to_f64(o), O, 1e-5 if dtype == "f32" else 1e-2)):
+        finite = np.isfinite(ref)
+        assert not finite[..., 1, :, j].any() if got.shape == S.shape else not finite[:, :, 1, j].any()
+        assert np.array_equal(got[~finite], ref[~finite], equal_nan=True)
+        assert np.isfinite(got[finite]).all() and relative(got[finite], ref[finite]) <= bar
+
+
+@pytest.mark.parametrize("d", [24, 64, 112])
+@pytest.mark.parametrize("tensor,scale", [("k", 1e-35), ("v", 1e-36), ("q", 1e-35), ("v", 1e-41), ("kv", 1e-19), ("v", 3e38)])
+def test_tiny_and_huge_values(la, d, tensor, scale):
+    """Values whose low bits no bf16 holds, subnormal ones, sums around the smallest normal number, values next to the largest
+    one.  Bar: a chain of fp32 multiply-adds rounds by up to 2^-24 a step (300 of them, random signs: 5e-7), and by 2^-149 where
+    sums are subnormal (around 1e-41)."""
+    import torch
+
+    B, N, H = 1, 300, 3
+    x = dict(zip("qkv", (to_dev(t) for t in gen(B, N, H, d, 7500 + d, "f32"))))
+    x["q"], x["k"] = x["q"].abs(), x["k"].abs()
+    if scale > 1:   # one term to a sum: half of |v| up to 3.4e38, no overflow
+        x["k"].zero_()
+        x["k"][:, -1] = 0.5
+        x["v"] = x["v"].clamp(-1, 1) * 3.4028e38
+        x["q"] = torch.full_like(x["q"], 1.0 / d)
+    else:
+        for name in tensor:
+            x[name] = x[name] * scale
+    q, k, v = (x[n] for n in "qkv")
+    qn, kn, vn = to_f64(q), to_f64(k), to_f64(v)
+    S, z = np.einsum("bnhi,bnhj->bhij", kn, vn), kn.sum(1)
+    bar = max(2e-6, 300 * 2.0 ** -149 / np.sqrt((S ** 2).mean()))
+    st = la.linattn_state(k, v)
+    assert relative(to_f64(st)[:, :, :d].swapaxes(-1, -2), S) <= bar
+    num = np.einsum("bnhi,bhij->bnhj", qn, to_f64(st)[:, :, :d].swapaxes(-1, -2))
+    O = num / (np.einsum("bnhi,bhi->bnh", qn, z) + EPS)[..., None]
+    bar = max(2e-6, 2.0 ** -149 * (d / np.sqrt((num ** 2).mean()) + 1 / np.sqrt((O ** 2).mean())))
+    assert relative(to_f64(la.linattn_apply(q, st, EPS)), O) <= bar
