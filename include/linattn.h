@@ -29,7 +29,8 @@
  *    token range.
  *  - dtype LINATTN_BF16: Q, K, V, O are bfloat16; products are exact in fp32,
  *    accumulation is fp32, O is rounded to nearest-even once at the store.
- *    dtype LINATTN_F32: fp32 in and out, fp32 accuracy (products of three-part bf16 sums, fp32 accumulation).
+ *    dtype LINATTN_F32: fp32 in and out, fp32 arithmetic: sums of fp32 multiply-adds, or of products of three-part bf16
+ *    values in fp32 accumulators where the head dim and the rows allow (no further from the exact sums).
  *  - A "state" is, per (b, h), a (d+1) x d fp32 matrix W stored row-major,
  *    units ordered [B][H]:   W[j][i] = S[i][j]  for j < d  (i: key feature,
  *    j: value feature),      W[d][i] = z[i].

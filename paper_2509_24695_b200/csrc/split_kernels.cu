@@ -1,18 +1,23 @@
 // fp32-accurate state and apply passes on the tensor cores: fp32 tensors, and the bf16 head dims the fused kernel
 // (umma_kernels.cu) does not take, wherever rows can be read in 16-byte pieces (split_ok).
 //
-// An fp32 value is the sum of three bf16 values exactly (8 significand bits each, cut off, not rounded, so that the
-// largest finite value stays finite).  A product of two such sums is nine bf16 products; the three smallest are below
-// 2^-24 of the whole and are left out, the other six are exact in the tensor core's fp32 accumulators.  What is left to
-// chance is how they are added up.  The tensor core truncates when it adds into an accumulator (2^-24 on average, always
-// towards zero), so (1) the leading products have accumulators apart from the five small ones, whose additions are
-// 2^-8 below; (2) they are dealt over several accumulators, so that no chain is longer than two or three; and (3) the
-// accumulators are added up in registers, round to nearest, every 64 tokens.  bf16 operands are one part, rotated ones
-// three; S is always three.  z and the denominators are plain fp32 sums.  The results are closer to the exact ones than
-// those of a chain of fp32 multiply-adds (see the figures at the kernels).
+// An fp32 value is the sum of three bf16 values exactly: 8 significand bits each, rounded to nearest, so that a value in
+// [2^a, 2^(a+1)) leaves at most 2^(a-8) to the second part and 2^(a-16) to the third, of either sign.  A product of two such
+// sums is nine bf16 products, exact in the tensor core's fp32 accumulators.  Six are taken.  Of the other three two are up
+// to 2^-24 of the product of the leading powers of two each (2^-26 on average, without bias; a multiply-add rounds to 2^-24)
+// and one is below 2^-31; inputs of one tile, where nothing averages out, have the two as well.  (Parts cut off instead of
+// rounded all have the value's sign: then the two reach 2^-21 and add up.  All inputs with eight products: 480p layer,
+// state 173 -> 190 us, apply 183 -> 217.)  What is left to chance is how the products are added up.  The tensor core
+// truncates when it adds into an accumulator (2^-24 on average, always towards zero), so (1) the leading products have
+// accumulators apart from the small ones, whose additions are 2^-8 below; (2) they are dealt over several accumulators, so
+// that no chain is longer than two or three; and (3) the accumulators are added up in registers, round to nearest, every 32
+// to 128 tokens.  bf16 operands are one part, rotated ones three; S is always three.  z and the denominators are plain fp32
+// sums.  Distance from 64 bits (2-norm, S / outputs), against the general kernels' chains of fp32 multiply-adds: normal data
+// 1.0 / 0.5 times theirs at one token, 0.65 / 0.5 at 8, 0.4 / 0.5 at 64 and 0.2 to 0.3 / 0.4 from 512 on; one-sign and
+// log-normal data 1.0 at one token and less than theirs beyond.
 //
-// Parts end where bf16 does: a value below 2^-110 loses up to 2^-134, an infinity has no parts (Inf - Inf), and products of
-// parts end at 2^-149.  So a CTA whose sums are not finite, or so small beside its data that this would show, does its
+// Parts end where bf16 does: a value below 2^-110 loses up to 2^-134, an infinity or a value above 3.396e38 has no parts
+// (Inf - Inf), and products of parts end at 2^-149.  So a CTA whose sums are not finite, or so small beside its data that this would show, does its
 // share again by plain fp32 multiply-adds, from memory (state_by_fma, apply_by_fma): the result is theirs, infinities and
 // NaN included.  The bounds are far from what data of one scale give: they are looked at once per CTA or token row.
 //
@@ -106,15 +111,14 @@ __device__ __forceinline__ int operand_offset(int row, int f, int box_bytes) {
   return (f >> 6) * box_bytes + row * 128 + ((((f & 63) >> 3) ^ (row & 7)) << 4) + ((f & 4) << 1);
 }
 
-// The next bf16 part of every value: its upper half; x becomes what is left.  Packed in pairs.
+// The next bf16 part of every value, rounded to nearest; x becomes what is left.  Packed in pairs.
 template <int E>
 __device__ __forceinline__ void take_part(float (&x)[E], uint32_t (&w)[E / 2]) {
 #pragma unroll
   for (int e = 0; e < E; e += 2) {
-    const uint32_t a = __float_as_uint(x[e]), b = __float_as_uint(x[e + 1]);
-    w[e / 2] = __byte_perm(a, b, 0x7632);
-    x[e] -= __uint_as_float(a & 0xFFFF0000u);
-    x[e + 1] -= __uint_as_float(b & 0xFFFF0000u);
+    w[e / 2] = pack_bf16x2(x[e], x[e + 1]);
+    x[e] -= __uint_as_float(w[e / 2] << 16);
+    x[e + 1] -= __uint_as_float(w[e / 2] & 0xFFFF0000u);
   }
 }
 __device__ __forceinline__ void store_words(uint8_t* at, const uint32_t (&w)[2]) { *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]); }
@@ -452,11 +456,11 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       if (S::REST) {   // smallest first
         bool add = false;
 #pragma unroll
-        for (int order = 2; order >= 1; --order)
+        for (int order = 3; order >= 1; --order)
 #pragma unroll
           for (int pk = order; pk >= 0; --pk) {
             const int pv = order - pk;
-            if (pk >= S::QK_PARTS || pv >= S::V_PARTS) continue;
+            if (pk >= S::QK_PARTS || pv >= S::V_PARTS || (order == 3 && p.N > S::TOK)) continue;
 #pragma unroll
             for (int kk = 0; kk < S::TOK / 16; ++kk) { mma(kk, pk, pv, S::LEAD, add); add = true; }
           }

@@ -180,3 +180,33 @@ def test_tiny_and_huge_values(la, d, tensor, scale):
     O = num / (np.einsum("bnhi,bhi->bnh", qn, z) + EPS)[..., None]
     bar = max(2e-6, 2.0 ** -149 * (d / np.sqrt((num ** 2).mean()) + 1 / np.sqrt((O ** 2).mean())))
     assert relative(to_f64(la.linattn_apply(q, st, EPS)), O) <= bar
+
+
+def spread(kind, shape, seed):
+    """Inputs on which products of parts could lose more than a multiply-add rounds: constants whose second and third parts
+    are as large as they get, values of one sign, log-normal and normal ones."""
+    if kind.startswith("constant"):
+        value = {"constant_cut": 1 + 2.0 ** -7 - 2.0 ** -23, "constant_rounded": 1 + 2.0 ** -8 - 2.0 ** -17, "constant_third": 1 / 3}[kind]
+        return tuple(np.full(shape, value, dtype=np.float32) for _ in range(3))
+    x = tuple(synth.gauss(shape, seed, t, dtype="f32") for t in (1, 2, 3))
+    return x if kind == "normal" else tuple(np.abs(t) + 1 for t in x) if kind == "one_sign" else tuple(np.exp(t) for t in x)
+
+
+@pytest.mark.parametrize("kind", ["constant_cut", "constant_rounded", "constant_third", "one_sign", "log_normal", "normal"])
+@pytest.mark.parametrize("d", [32, 112])
+def test_no_further_from_64_bits_than_multiply_adds(la, kind, d):
+    """Bars on the 2-norm of S and z.  One token: a product rounded to nearest, 2^-24.  More: up to 2^-24 for the products left
+    out, 2^-24 for each of the few sums in registers, random signs: 2^-22.  (Six products of parts cut off: 2^-21 alone.)  O on
+    top of the rounded state: 112 products and a quotient, 2^-21."""
+    for N in (1, 2, 7, 32, 64, 65, 200, 512):
+        q, k, v = spread(kind, (1, N, 3, d), 7600 + N)
+        qn, kn, vn = (x.astype(np.float64) for x in (q, k, v))
+        qn, kn = qn.clip(0), kn.clip(0)
+        st = to_f64(la.linattn_state(to_dev(k), to_dev(v)))
+        S, z = np.einsum("bnhi,bnhj->bhji", kn, vn), kn.sum(1)
+        bar = 1.01 * 2.0 ** -24 if N == 1 else 2.0 ** -22
+        assert relative(st[:, :, :d], S) <= bar, f"S, {N} tokens: {relative(st[:, :, :d], S):.2e}"
+        assert relative(st[:, :, d], z) <= bar, f"z, {N} tokens"
+        O = np.einsum("bnhi,bhji->bnhj", qn, S) / (np.einsum("bnhi,bhi->bnh", qn, z) + EPS)[..., None]
+        o = to_f64(la.linattn_forward(to_dev(q), to_dev(k), to_dev(v), EPS))
+        assert relative(o, O) <= 2.0 ** -21, f"O, {N} tokens: {relative(o, O):.2e}"
