@@ -497,11 +497,6 @@ __device__ void reduce_slice(const FusedParams& p) {
   }
 }
 
-// The rotary kernel has no registers to spare: with this form inlined the passes of a kernel that never takes it (d = 112,
-// 4680 tokens) were 5 % slower.
-template <int D>
-__device__ __noinline__ void reduce_slice_apart(const FusedParams& p) { reduce_slice<D, true>(p); }
-
 // ---------------------------------------------------------------- reduce, with the S operand as a by-product
 // Fused launches of one-head units (d = 112, 128) with at least one column CTA per unit: the column CTAs of a
 // unit share its reduce (part c of P), in 32-byte chunks of a state row, and besides the fp32 state each chunk's
@@ -860,11 +855,15 @@ __device__ __forceinline__ float sum_z_slots(const float* slots, int f) {
 }
 
 // ============================================================================ the kernel
-template <int D, bool ROPE, bool SOLO>
+// SOLO: lone CTAs.  IMAGE: the reduce leaves operand images and the apply pass fetches them (p.s_image).  Both are decided
+// on the host, and each form is a kernel of its own: the rotary one has no registers to spare, and with the slice reduce that
+// it does not take compiled into it (even out of line) a read-only rotary step of 4680 tokens took 45.0 us instead of 43.1.
+template <int D, bool ROPE, bool SOLO, bool IMAGE>
 __global__ void __launch_bounds__(Roles<ROPE>::THREADS, 1)
 umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                   const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
                   const __grid_constant__ FusedParams p) {
+  static_assert(!IMAGE || (Cfg<D>::G == 1 && !SOLO), "operand images are of one-head units in a grid");
   using C = Cfg<D>;
   using R = Roles<ROPE>;
   constexpr int NSA = SOLO ? 4 : C::STATE_STAGES;
@@ -1292,7 +1291,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       }
     }
     __syncwarp();
-  } else if (C::G == 1 && p.s_image && p.accumulate && p.do_state && (int)blockIdx.x < p.sa.P * p.sa.U) {
+  } else if (IMAGE && p.accumulate && p.do_state && (int)blockIdx.x < p.sa.P * p.sa.U) {
     // ------------------------------------------------------------ store warp (idle in this pass)
     // A cached step adds to the old state, which the K, V stream has pushed out of L2 since the last step:
     // once this CTA's loads are all issued, ask for its share of it (reduce_image's split), so that the
@@ -1311,8 +1310,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   if (!SOLO && p.do_state) {
     grid_barrier(p.ctrl, abort_flag, p.do_apply != 0, gen0);
     if (!*abort_flag) {
-      if (C::G == 1 && p.s_image) reduce_image<D, ROPE>(p);
-      else if (ROPE) reduce_slice_apart<D>(p);
+      if constexpr (IMAGE) reduce_image<D, ROPE>(p);
       else reduce_slice<D, ROPE>(p);
     }
     if (p.do_apply) grid_barrier(p.ctrl, abort_flag, false, gen0 + 1);
@@ -1397,7 +1395,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         if (!ok) break;
         const int u = t.unit();
         if (SOLO) {
-        } else if (C::G == 1 && p.s_image) {
+        } else if (IMAGE) {
           if (tr == 0) {   // the unit's operand image, made by the reduce: one bulk copy
             fence_proxy_async_all();
             mbar_arrive_expect_tx(s_ready, C::S_BYTES);
@@ -1429,7 +1427,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             zc[4 * box + 2] = make_float2(a1.x, a1.y); zc[4 * box + 3] = make_float2(a1.z, a1.w);
           }
         }
-        if (!SOLO && !(C::G == 1 && p.s_image)) {
+        if (!SOLO && !IMAGE) {
           fence_proxy_async_smem();
           mbar_arrive(s_ready);
         }
@@ -1515,7 +1513,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       if (!SOLO && t.seg_first()) {
         // this thread has seen the last accumulator of the previous segment complete: S may be rebuilt
         const int u = t.unit();
-        if (!(C::G == 1 && p.s_image)) {
+        if (!IMAGE) {
           build_s_operand<D>(s_op, p.state, u / p.HG, u % p.HG, p.H, R::RELU_THREADS + te, R::RELU_THREADS + 128);
           fence_proxy_async_smem();
         }
@@ -1695,13 +1693,13 @@ inline bool solo_pays(const Problem& p, int U, int sms) {
 inline int groups_of(int d) { return d == 32 ? 4 : d == 64 ? 2 : 1; }
 
 // Instantiates and launches the kernel: cooperatively when its CTAs wait for one another.
-template <int D, bool ROPE, bool SOLO>
+template <int D, bool ROPE, bool SOLO, bool IMAGE>
 int launch_kernel(int grid, void** args, cudaStream_t stream) {
   using C = Cfg<D>;
   // the opt-in to more than 48 KB of dynamic shared memory is a per-device setting of the kernel
   static bool attr_set[64] = {false};
   constexpr size_t kSmem = SOLO ? C::SMEM_SOLO : ROPE ? C::SMEM_ROPE : C::SMEM;
-  const void* kernel = (const void*)umma_fused_kernel<D, ROPE, SOLO>;
+  const void* kernel = (const void*)umma_fused_kernel<D, ROPE, SOLO, IMAGE>;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LINATTN_ERR_CUDA;
   if (!attr_set[dev]) {
@@ -1775,7 +1773,9 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   }
   if (!do_state) { mk = mq; mv = mq; }
   void* args[] = {&mk, &mv, &mq, &mo, &fp};
-  return solo ? launch_kernel<D, ROPE, true>(grid, args, stream) : launch_kernel<D, ROPE, false>(grid, args, stream);
+  if (solo) return launch_kernel<D, ROPE, true, false>(grid, args, stream);
+  if (C::G == 1 && fp.s_image) return launch_kernel<D, ROPE, false, C::G == 1>(grid, args, stream);
+  return launch_kernel<D, ROPE, false, false>(grid, args, stream);
 }
 
 }  // namespace
