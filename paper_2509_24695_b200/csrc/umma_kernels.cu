@@ -735,13 +735,17 @@ __device__ __forceinline__ void split_hi_lo(const float (&x)[8], uint4& hi, uint
 }
 
 // Accumulator columns [16 * first, 16 * last) of lane quarter wq (key features; lane = value feature): sums of the four
-// accumulators in a fixed order, on top of the old state when accumulating, to the operand and (write_state) back to
-// where the old state is staged: `st`, copied in at the start and out at the end in one piece (a row per lane straight
-// from and to memory took 15 000 cycles, copies of single rows 5 000).  The lanes' rows there are a multiple of 64 bytes
-// apart, so neighbouring lanes take their four 16-byte pieces in different order: bank conflicts two ways at most.
-// Epilogue and ReLU warps share the columns.
+// accumulators in a fixed order, added (add) to what is staged at `st`, the old state or the tiles before, and left there
+// (store) and in the operand (operand).  `st` is copied in at the start and out at the end in one piece (a row per lane
+// straight from and to memory took 15 000 cycles, copies of single rows 5 000).  The lanes' rows there are a multiple of 64
+// bytes apart, so neighbouring lanes take their four 16-byte pieces in different order: bank conflicts two ways at most.
+// Every 64-token tile is drained: an accumulator takes one MMA, the tiles are added up round to nearest, as the grid's
+// partial records are.  (One drain at the end made chains of up to eight truncating additions: S of 384 tokens 6.0e-8
+// from 64 bits instead of 4.7e-8, with log-normal values 1.2e-7 instead of 4.8e-8.)  The epilogue drains the tiles, and shares
+// the columns of the last one with the ReLU warps.
 template <int D>
-__device__ __forceinline__ void solo_drain(const FusedParams& p, uint8_t* s_op, float* st, uint32_t tmem_base, int wq, int lane, int first, int last) {
+__device__ __forceinline__ void solo_drain(const FusedParams& p, uint8_t* s_op, float* st, uint32_t tmem_base, int wq, int lane, int first, int last,
+                                           bool add, bool store, bool operand) {
   using C = Cfg<D>;
   const int i = wq * 32 + lane, g = i / D, il = i - g * D;    // row of the operand, its head of the group, value feature
   const bool live = i < C::FEAT && (int)blockIdx.x % p.HG * C::G + g < p.H;
@@ -759,7 +763,15 @@ __device__ __forceinline__ void solo_drain(const FusedParams& p, uint8_t* s_op, 
   const uint32_t trow = tmem_base + ((uint32_t)(wq * 32) << 16);
 #pragma unroll 1
   for (int cc = first; cc < last && cc * 16 < C::FEAT; ++cc) {
-    const bool own = live && (C::G == 1 || cc * 16 / D == g);   // blocks across heads are zero
+    auto chunk = [&](int c) {   // 16-byte chunk c of the columns in the operand's row of this lane
+      const int lc = cc * 2 + c;
+      return s_op + (lc >> 3) * C::SBOX_BYTES + i * kRowBytes + (((lc & 7) ^ (i & 7)) << 4);
+    };
+    if (C::G > 1 && cc * 16 / D != g) {   // blocks across heads are zero (the same for a whole warp)
+#pragma unroll
+      for (int c = 0; c < 4 && operand; ++c) *reinterpret_cast<uint4*>(chunk(c & 1) + (c >> 1) * 2 * C::SBOX_BYTES) = make_uint4(0, 0, 0, 0);
+      continue;
+    }
     float4* at = reinterpret_cast<float4*>(row + (C::G == 1 ? cc * 16 : cc * 16 % D));
     uint32_t r[4][16];
 #pragma unroll
@@ -771,10 +783,10 @@ __device__ __forceinline__ void solo_drain(const FusedParams& p, uint8_t* s_op, 
       float f[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        f[e] = own ? __uint_as_float(r[0][4 * x + e]) + __uint_as_float(r[1][4 * x + e]) + __uint_as_float(r[2][4 * x + e]) + __uint_as_float(r[3][4 * x + e]) : 0.f;
+        f[e] = live ? __uint_as_float(r[0][4 * x + e]) + __uint_as_float(r[1][4 * x + e]) + __uint_as_float(r[2][4 * x + e]) + __uint_as_float(r[3][4 * x + e]) : 0.f;
       val[x] = make_float4(f[0], f[1], f[2], f[3]);
     }
-    if (p.accumulate && own) {
+    if (add && live) {
       float4 old[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) old[k] = at[(k + rot) & 3];
@@ -782,19 +794,17 @@ __device__ __forceinline__ void solo_drain(const FusedParams& p, uint8_t* s_op, 
 #pragma unroll
       for (int x = 0; x < 4; ++x) add4(val[x], old[x]);
     }
-    if (i < C::FEAT) {
+    if (operand && i < C::FEAT) {
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const float x8[8] = {val[2 * c].x, val[2 * c].y, val[2 * c].z, val[2 * c].w, val[2 * c + 1].x, val[2 * c + 1].y, val[2 * c + 1].z, val[2 * c + 1].w};
         uint4 hi, lo;
         split_hi_lo(x8, hi, lo);
-        const int lc = cc * 2 + c;
-        uint8_t* dst = s_op + (lc >> 3) * C::SBOX_BYTES + i * kRowBytes + (((lc & 7) ^ (i & 7)) << 4);
-        *reinterpret_cast<uint4*>(dst) = hi;
-        *reinterpret_cast<uint4*>(dst + 2 * C::SBOX_BYTES) = lo;
+        *reinterpret_cast<uint4*>(chunk(c)) = hi;
+        *reinterpret_cast<uint4*>(chunk(c) + 2 * C::SBOX_BYTES) = lo;
       }
     }
-    if (p.write_state && own) {
+    if (store && live) {
       turn(val, rot);
 #pragma unroll
       for (int k = 0; k < 4; ++k) at[(k + rot) & 3] = val[k];
@@ -1008,7 +1018,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       for (TileWalk t(wa); !t.done() && ok; t.next(), ++it) {
         const int s = it % NSA;
         const bool seg_first = t.seg_first();
-        if (seg_first) { ok = mbar_wait(a_tempty, (seg & 1) ^ 1, abort_flag); n_mma = 0; }
+        if (SOLO || seg_first) { ok = mbar_wait(a_tempty, (seg & 1) ^ 1, abort_flag); n_mma = 0; }
         if (ok) ok = mbar_wait(&a_ready[s], (it / NSA) & 1, abort_flag);
         if (!ok) break;
         tcgen05_fence_after();
@@ -1021,7 +1031,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
           umma_bf16(d_tmem, SOLO ? bq : a, SOLO ? a : bq, IDESC_A, n_mma < (uint32_t)ACCS ? 0u : 1u);  // first use of each: overwrite
         }
         umma_commit(&a_empty[s]);
-        if (t.seg_last()) { umma_commit(a_tfull); ++seg; }
+        if (SOLO || t.seg_last()) { umma_commit(a_tfull); ++seg; }
       }
       if (it > 0) umma_commit(a_done); else mbar_arrive(a_done);
     }
@@ -1067,19 +1077,23 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         if (p.accumulate && h < p.H) z += *at;
         if (p.write_state) *at = z;
         if (ROPE) z_row[f] = z;
-        else put_z<D>(s_op, f, z);
+        else if (p.do_apply) put_z<D>(s_op, f, z);
       }
       if (ROPE) {
         mbar_arrive(z_done);
         ok = mbar_wait(z_done, 0, abort_flag);
       }
       // this role's share of the drain
-      ok = ok && mbar_wait(a_tfull, 0, abort_flag);
+      // (a_done: the last tile's accumulators, and the drain of the tile before it has come to its end; looking for that at
+      // a_tempty makes this thread see what the epilogue left at st)
+      const int tiles = (int)(wa.f1 - wa.f0);
+      ok = ok && mbar_wait(a_done, 0, abort_flag);
+      if (tiles > 1) ok = ok && mbar_wait(a_tempty, tiles & 1, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) return;
       tcgen05_fence_after();
       const int half = tr >> 7;   // (rotary variant: two warps of this role to a lane quarter)
-      if (ROPE) solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 3 + 3 * half, half ? 8 : 6);
-      else solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, 4, 8);
+      const int c0 = ROPE ? 3 + 3 * half : 4, c1 = ROPE && !half ? 6 : 8;
+      solo_drain<D>(p, s_op, st, tmem_base, warp & 3, lane, c0, c1, p.accumulate || tiles > 1, p.write_state, p.do_apply);
       tcgen05_fence_before();
       fence_proxy_async_smem();
       mbar_arrive(s_ready);
@@ -1212,17 +1226,19 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
           for (int e = 0; e < 4; ++e) zh[e] = make_float2(0.f, 0.f);
         }
       }
-      if (!t.seg_last()) continue;
+      if (!SOLO && !t.seg_last()) continue;
       bool ok = mbar_wait(a_tfull, seg & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tcgen05_fence_after();
       if (SOLO) {
-        if (p.accumulate && !__all_sync(0xffffffffu, mbar_wait(st_full, 0, abort_flag))) break;
-        solo_drain<D>(p, s_op, st, tmem_base, wq, lane, 0, ROPE ? 3 : 4);
-        fence_proxy_async_smem();   // the operand is read by the MMAs of the apply pass
+        const bool last = t.seg_last();
+        if (p.accumulate && it == 0 && !__all_sync(0xffffffffu, mbar_wait(st_full, 0, abort_flag))) break;
+        solo_drain<D>(p, s_op, st, tmem_base, wq, lane, 0, !last ? 8 : ROPE ? 3 : 4, p.accumulate || it > 0, !last || p.write_state, last && p.do_apply);
+        if (last) fence_proxy_async_smem();   // the operand is read by the MMAs of the apply pass
         tcgen05_fence_before();
-        mbar_arrive(s_ready);
+        mbar_arrive(last ? s_ready : a_tempty);
+        ++seg;
         continue;
       }
       const int u = t.unit(), hg = u % p.HG;
@@ -1678,16 +1694,25 @@ int sm_count() {
   return cached[dev];
 }
 
-// One CTA per unit instead of all CTAs on all units?  A lone CTA takes about 9 us and 1.2 us for every 64 tokens of its
-// unit; the grid takes about 14 us (two grid barriers, the partial records, the reduce and the operand images between the
-// passes) and a time that grows with all units' tokens together.  Measured, d = 112, plain forward / cached step:
-//   20 units:   64 tokens 10.3 / 10.3 us against 18.5 / 20.2, 256: 12.3 / 14.3 against 16.4 / 17.4, 384: 14.7 / 16.4 against
-//               16.8 / 16.9, 512: 18.5 / 18.5 against 17.8 / 18.4;
-//   60 units:  512: 18.5 / 18.5 against 22.5 / 22.6;   140 units: 512: 20.4 / 20.5 against 28.7 / 29.5.
-// The choice depends on the shape alone, so that all calls on one shape (forward, state and apply, step, peek, the
-// token-sharded three) add up in the same order and give the same bits.
+// One CTA per unit instead of all CTAs on all units?  A lone CTA takes about 6 us and 1.6 (packed heads) to 3 us for every 64
+// tokens of its unit; the grid takes 13 to 15 us (two grid barriers, the partial records, the reduce and the operand images
+// between the passes; 8 to 10 without an apply pass) and a time that grows with all units' tokens together.  Measured, launches
+// back to back, lone CTAs against the grid, in us:
+//                       64 tokens                  128                        192                        256
+//                       forward  step  state       forward  step  state       forward  step  state       forward  step  state
+//   d = 112, 1 unit     7.9/16.1 8.5/17.4 6.5/11.4 10.6/14.8 11.6/15.1 9.0/9.8  14.2/14.0 15.2/14.4 11.7/9.2 17.0/13.9 18.0/14.1 14.3/9.0
+//            20         8.1/17.3 8.9/18.2 6.7/12.1 11.0/16.4 11.7/16.9 9.3/10.7 14.4/15.2 15.3/15.6 12.0/9.8 17.3/15.3 18.1/15.6 14.4/9.6
+//            60         8.4/17.4 9.1/18.3 6.8/12.2 11.0/17.5 12.0/17.9 9.3/11.0 14.6/18.3 15.6/18.7 12.1/11.3 17.4/18.5 18.4/19.1 14.5/11.4
+//            148        10.5/19.4 11.1/19.4 7.5/12.5 12.9/20.2 13.9/20.4 9.8/13.1 15.8/21.6 17.1/21.6 12.5/13.6 18.6/22.5 19.6/22.5 15.1/14.1
+//   d = 128, 18 units   8.5/17.4 9.5/18.2 7.1/13.0 11.3/16.3 12.4/16.8 9.7/10.8 15.1/15.4 16.1/15.8 12.5/10.3 18.0/15.7 19.2/15.9 15.4/9.6
+//   d = 64, 35          8.3/16.2 9.0/16.4 6.4/10.5 10.8/15.5 11.6/15.5 8.7/9.5  13.6/15.7 14.5/15.7 10.8/9.4 16.1/16.3 16.9/16.2 12.9/9.6
+//   d = 32, 1           7.5/13.1 7.9/12.6 5.5/8.0  9.9/12.6 10.2/13.3 7.3/7.7   12.3/13.0 12.7/13.1 9.0/7.7  14.0/13.0 14.5/12.9 10.6/7.7
+// with rotary factors alike at d = 112 and 128 and twice as fast as the grid at d = 32 and 64.  So: up to 128 tokens, and up to 192
+// with packed heads or many units.  (States alone of 129 to 192 tokens with packed heads lose 1 us by that.)  The choice depends
+// on the shape alone, so that all calls on one shape (forward, state and apply, step, peek, the token-sharded three) add up in
+// the same order and give the same bits.
 inline bool solo_pays(const Problem& p, int U, int sms) {
-  return U <= sms && (p.N <= 384 || (p.N <= 512 && 3 * U >= sms));
+  return U <= sms && (p.N <= 128 || (p.N <= 192 && (p.d <= 64 || 3 * U >= 2 * sms)));
 }
 
 inline int groups_of(int d) { return d == 32 ? 4 : d == 64 ? 2 : 1; }
