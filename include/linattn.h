@@ -43,10 +43,12 @@
  *  - Every function returns LINATTN_OK (0) or a negative linattn_status.
  *    Arguments are validated before anything is launched.  Zero tokens is a
  *    successful no-op (linattn_state then writes a zero state; linattn_forward
- *    writes nothing).  Nothing here throws, aborts or traps the device; the
- *    only device-side wait (the grid barrier of the fused kernels) gives up
- *    after a bounded number of polls and records LINATTN_ERR_TIMEOUT in the
- *    workspace, readable with linattn_workspace_status.
+ *    writes nothing).  Nothing here throws, aborts or traps the device.
+ *    Device-side waits on barriers, of a CTA and of the fused kernels' grid, give
+ *    up after about a second and record LINATTN_ERR_TIMEOUT in the workspace,
+ *    readable with linattn_workspace_status.  (The CTAs of a thread-block cluster,
+ *    fp32 and the other head dims, and the allocation of tensor memory wait
+ *    without a limit, on CTAs whose own waits have one.)
  *  - Calls that share a workspace (or a cache) must be ordered on one stream:
  *    two of them in flight at once race on the split-N partials.
  */

@@ -33,6 +33,11 @@ static_assert(sizeof(WorkspaceCtrl) <= LINATTN_WORKSPACE_CTRL_BYTES, "control bl
 void count_launches(int n);
 
 constexpr int kMaxCtas = 256;        // upper bound on the persistent grid (B200 has 148 SMs)
+// CTAs that ask for this much shared memory are alone on their SM (228 KB, 1 KB of it the system's per CTA).  Every kernel
+// whose CTAs wait for one another (grid barriers, clusters) does: the allocation of tensor memory waits for whoever holds
+// it, so CTAs of two such launches sharing two SMs could wait for each other for good.
+constexpr int kSmemAlone = 114 * 1024;
+static_assert(2 * (kSmemAlone + 1024) > 228 * 1024, "alone on an SM");
 constexpr int kFmaMaxChunks = 64;    // split-N partials per unit on the fp32-accurate path
 constexpr int kFmaMinChunkTokens = 512;
 

@@ -23,7 +23,9 @@
 //
 // Operand layouts are those of the fused kernel: 128-byte swizzled rows of 64 features.  Every thread reads its own
 // pieces with private asynchronous copies, rectifies, rotates and splits them, and stores the parts; one thread issues
-// the MMAs, and other warps drain the accumulators.  All waits are on this CTA's own work and bounded.
+// the MMAs, and other warps drain the accumulators.  Waits on barriers are on this CTA's own work and bounded.  Two are not:
+// the CTAs of a cluster meet (cluster_sync; each gets there, since its other waits are bounded), and tensor memory is
+// allocated before it (no other CTA can hold it for good: kSmemAlone).
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -270,7 +272,8 @@ struct StateShape : Shape<T, R, ROPE> {
   static constexpr int OWN_BYTES = (B::DP + 1) * B::DP * 4;   // a CTA's state, where its cluster reads it
   static constexpr int Z_OFF = OWN_BYTES > 2 * STAGE ? OWN_BYTES : 2 * STAGE;
   static constexpr int TAIL = Z_OFF + Z_BYTES - 2 * STAGE;
-  static constexpr int SMEM = 1024 + 2 * STAGE + (RAW_STAGES * RAW > TAIL ? RAW_STAGES * RAW : TAIL) + kBarBytes;   // (barriers last)
+  static constexpr int NEED = 1024 + 2 * STAGE + (RAW_STAGES * RAW > TAIL ? RAW_STAGES * RAW : TAIL) + kBarBytes;
+  static constexpr int SMEM = NEED > kSmemAlone ? NEED : kSmemAlone;   // (barriers last)
   static constexpr int LEAD = TOK / 32;                      // accumulators of the leading products: chains of two K steps
   static constexpr bool REST = B::QK_PARTS + B::V_PARTS > 2;
   static constexpr int ACC = B::DP <= 64 ? 64 : 128;         // TMEM columns between accumulators
@@ -854,7 +857,7 @@ int clusters_at_once(K kernel, int smem, int c, int (&cached)[64][9]) {
     cfg.gridDim = dim3(c); cfg.blockDim = dim3(kBlock); cfg.dynamicSmemBytes = smem;
     cfg.attrs = at; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }   // (asked again next time)
     cached[dev][c] = n > 0 ? n : -1;
   }
   return cached[dev][c] > 0 ? cached[dev][c] : 0;

@@ -4,7 +4,7 @@
 // Both contractions of the method are dense and run on the tensor cores, but the work is HBM-bound
 // (about d/2 FLOP per byte); everything here is organised around keeping TMA loads in flight on every SM.
 //
-// ONE persistent, cooperatively launched kernel runs up to three passes back to back:
+// ONE persistent, cooperatively launched kernel runs up to three passes back to back (units of few tokens apart, see below):
 //
 //   state pass   S = sum_n phi(k_n)^T v_n and z = sum_n phi(k_n)   (Eq. 2 / Eq. 3 state).
 //                A = phi(K)^T and B = [V | 1] are both token-major in memory, i.e. MN-major UMMA
@@ -1724,6 +1724,7 @@ int launch_kernel(int grid, void** args, cudaStream_t stream) {
   // the opt-in to more than 48 KB of dynamic shared memory is a per-device setting of the kernel
   static bool attr_set[64] = {false};
   constexpr size_t kSmem = SOLO ? C::SMEM_SOLO : ROPE ? C::SMEM_ROPE : C::SMEM;
+  static_assert(SOLO || kSmem >= kSmemAlone, "CTAs that wait for one another");
   const void* kernel = (const void*)umma_fused_kernel<D, ROPE, SOLO, IMAGE>;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LINATTN_ERR_CUDA;

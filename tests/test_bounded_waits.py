@@ -35,3 +35,40 @@ def test_the_build_refuses_a_dropped_result(tmp_path, statement, compiles):
     src.write_text('#include "sm100_ptx.cuh"\n__global__ void t(uint64_t* b, volatile int* f) { using namespace linattn::ptx; %s }\n' % statement)
     rc = subprocess.run(["nvcc", *build.NVCC_FLAGS, "-I", CSRC, "-c", str(src), "-o", str(tmp_path / "t.o")], capture_output=True).returncode
     assert (rc == 0) == compiles
+
+
+def struct_text(text, name):
+    """The definition of `name` (with its template head, if any) in a source file."""
+    m = re.search(r"(template <[^\n]*>\n)?(struct|__host__ __device__ constexpr int) %s\b[^;{]*\{" % re.escape(name), text)
+    depth, end = 1, m.end()
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[end], 0)
+        end += 1
+    return text[m.start():end] + ";\n"
+
+
+def test_ctas_that_wait_for_one_another_do_not_share_an_sm(tmp_path):
+    """The CTAs of a cluster (split_state_kernel) and those of a grid with barriers (umma_fused_kernel) wait for one another, and
+    the allocation of tensor memory waits for whoever holds it.  Two such launches sharing two SMs could wait for each other for
+    good, so each CTA has to ask for more than half of an SM's 228 KB of shared memory (1 KB of it the system's, per CTA)."""
+    split = open(os.path.join(CSRC, "split_kernels.cu")).read()
+    umma = open(os.path.join(CSRC, "umma_kernels.cu")).read()
+    common = open(os.path.join(CSRC, "common.cuh")).read()
+    consts = [m.group(0) for src in (common, split, umma) for m in
+              re.finditer(r"^constexpr (?:int|size_t) k\w+ = [^;]*;", src, re.M) if "sizeof" not in m.group(0)]
+    pieces = "".join("template <> struct Piece<%s> { static constexpr int E = %d; using Tab = Bytes<%d>; };\n" % x
+                     for x in (("float", 4, 8), ("__nv_bfloat16", 8, 16)))
+    asks = ["StateShape<%s, %d, %s>::SMEM" % (t, r, rope) for t in ("float", "__nv_bfloat16") for r in range(2, 9) for rope in ("false", "true")]
+    asks += ["(int)Cfg<%d>::%s" % (d, s) for d in (32, 64, 112, 128) for s in ("SMEM", "SMEM_ROPE")]
+    src = tmp_path / "t.cpp"
+    src.write_text("#include <cstddef>\n#include <cstdint>\n#include <cstdio>\n#define __host__\n#define __device__\n"
+                   "template <int N> struct Bytes { char b[N]; };\nstruct __nv_bfloat16 { char b[2]; };\ntemplate <typename T> struct Piece;\n"
+                   + pieces + "\n".join(dict.fromkeys(consts)) + "\n"
+                   + "".join(struct_text(split, n) for n in ("flip_of", "Shape", "StateShape")).replace("};\n;", "};\n")
+                   + struct_text(umma, "Cfg")
+                   + "int main() {\n" + "".join('  printf("%s %%d\\n", %s);\n' % (a.replace(" ", ""), a) for a in asks) + "}\n")
+    subprocess.run(["g++", "-std=c++17", "-o", str(tmp_path / "t"), str(src)], check=True)
+    asked = dict(line.rsplit(" ", 1) for line in subprocess.run([str(tmp_path / "t")], capture_output=True, text=True, check=True).stdout.splitlines())
+    assert len(asked) == len(asks)
+    shared = {name: int(n) for name, n in asked.items() if 2 * (int(n) + 1024) <= 228 * 1024}
+    assert not shared, f"two CTAs fit on an SM: {shared}"
