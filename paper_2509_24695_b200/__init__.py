@@ -47,6 +47,18 @@ class _ConvDesc(ctypes.Structure):
                 ("stride_b", ctypes.c_int64), ("stride_b_y", ctypes.c_int64)]
 
 
+def _descriptor_type(structure):
+    """The type of a descriptor argument: what POINTER(structure) takes, or the packed bytes of one."""
+    pointer, size = ctypes.POINTER(structure), ctypes.sizeof(structure)
+
+    class Descriptor:
+        @staticmethod
+        def from_param(value):
+            return value if type(value) is bytes and len(value) == size else pointer.from_param(value)
+
+    return Descriptor
+
+
 _lib = None
 
 
@@ -66,7 +78,7 @@ def load_library(path: str | None = None):
         p = _build.build()
     lib = ctypes.CDLL(p)
     vp, i64, sz = ctypes.c_void_p, ctypes.c_int64, ctypes.c_size_t
-    dp = vp      # descriptors: byref(_Desc) or the packed bytes of one
+    dp, cp = _descriptor_type(_Desc), _descriptor_type(_ConvDesc)
     szp = ctypes.POINTER(sz)
     f32 = ctypes.c_float
     sig = {
@@ -103,11 +115,11 @@ def load_library(path: str | None = None):
         "blocklin_cache_joint_prefill": ([vp, ctypes.c_int], ctypes.c_int),
         "blocklin_cache_info": ([vp, ctypes.POINTER(i64), ctypes.POINTER(i64), szp], ctypes.c_int),
         "blocklin_cache_destroy": ([vp], ctypes.c_int),
-        "tconv_cache_bytes": ([dp, szp], ctypes.c_int),
-        "tconv_cache_reset": ([dp, vp, vp], ctypes.c_int),
-        "tconv_forward": ([dp, i64, vp, vp, vp, vp], ctypes.c_int),
-        "tconv_block_step": ([dp, i64, vp, vp, vp, vp, ctypes.c_int, vp], ctypes.c_int),
-        "tconv_prefill": ([dp, i64, i64, vp, vp, vp, vp, vp], ctypes.c_int),
+        "tconv_cache_bytes": ([cp, szp], ctypes.c_int),
+        "tconv_cache_reset": ([cp, vp, vp], ctypes.c_int),
+        "tconv_forward": ([cp, i64, vp, vp, vp, vp], ctypes.c_int),
+        "tconv_block_step": ([cp, i64, vp, vp, vp, vp, ctypes.c_int, vp], ctypes.c_int),
+        "tconv_prefill": ([cp, i64, i64, vp, vp, vp, vp, vp], ctypes.c_int),
     }
     for name, (argtypes, restype) in sig.items():
         fn = getattr(lib, name)

@@ -128,3 +128,23 @@ def test_prefill_workspace_size_without_gpu(lib):
     assert lib.blocklin_prefill_workspace_bytes(ctypes.byref(d), 4000, 4680, ctypes.byref(pre)) == -2   # 80 000 units
     assert lib.blocklin_prefill_workspace_bytes(ctypes.byref(d), 0, 4680, ctypes.byref(pre)) == -1
     assert lib.blocklin_prefill_workspace_bytes(ctypes.byref(d), 7, 4680, None) == -1
+
+
+def test_descriptor_arguments(lib):
+    """A descriptor is a _Desc (a _ConvDesc) by reference, or the packed bytes of one: nothing else gets through to be read as one."""
+    import paper_2509_24695_b200 as la
+
+    d, c = la._Desc(1, 2, 112, 0, 0, 0, 0), la._ConvDesc(1, 10, 16, 0, 0, 0)
+    packed, packed_conv = la._pack_desc(1, 2, 112, 0, 0, 0, 0), la._pack_conv(1, 10, 16, 0, 0, 0)
+    n = ctypes.c_size_t()
+    for good in (ctypes.byref(d), packed):
+        assert lib.linattn_state_bytes(good, ctypes.byref(n)) == 0 and n.value == 2 * (112 * 112 + 112) * 4
+    for good in (ctypes.byref(c), packed_conv):
+        assert lib.tconv_cache_bytes(good, ctypes.byref(n)) == 0 and n.value == 10 * 16 * 2
+    address = ctypes.addressof(d)
+    for bad in (address, ctypes.c_void_p(address), ctypes.byref(c), packed_conv, packed[:-1], packed + b"\0", "text", 1.0):
+        with pytest.raises(ctypes.ArgumentError):
+            lib.linattn_state_bytes(bad, ctypes.byref(n))
+    for bad in (address, ctypes.byref(d), packed, b""):
+        with pytest.raises(ctypes.ArgumentError):
+            lib.tconv_cache_bytes(bad, ctypes.byref(n))
