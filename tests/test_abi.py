@@ -148,3 +148,21 @@ def test_descriptor_arguments(lib):
     for bad in (address, ctypes.byref(d), packed, b""):
         with pytest.raises(ctypes.ArgumentError):
             lib.tconv_cache_bytes(bad, ctypes.byref(n))
+
+
+@pytest.mark.parametrize("private_name", [True, False])
+def test_the_stream_of_a_call(monkeypatch, private_name):
+    """The current stream of the tensor's device, also from a torch without the private name that gives it fastest."""
+    import sys
+    import types
+
+    import paper_2509_24695_b200 as la
+
+    fake = types.SimpleNamespace(_C=types.SimpleNamespace(), cuda=types.SimpleNamespace(
+        current_stream=lambda i: types.SimpleNamespace(cuda_stream=0x1000 + i)))
+    if private_name:
+        fake._C._cuda_getCurrentRawStream = lambda i: 0x2000 + i
+    monkeypatch.setitem(sys.modules, "torch", fake)
+    monkeypatch.setattr(la, "_torch_module", None)
+    monkeypatch.setattr(la, "_raw_stream", None, raising=False)
+    assert la._stream(types.SimpleNamespace(get_device=lambda: 3)) == (0x2003 if private_name else 0x1003)
