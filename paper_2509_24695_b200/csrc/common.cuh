@@ -23,7 +23,9 @@ struct Problem {
 // Control block at the start of every workspace.
 struct WorkspaceCtrl {
   int status;            // LINATTN_OK or LINATTN_ERR_TIMEOUT, written by kernels
-  int pad0[15];
+  int gave_up;           // a CTA has no partial state to give (split_state_kernel); fma_state_reduce clears it again
+  int gave_up_seen;      // its blocks that have looked
+  int pad0[13];
   unsigned barrier[16];  // grid-barrier counters of the fused kernels
   unsigned unit_arrivals[960];
 };

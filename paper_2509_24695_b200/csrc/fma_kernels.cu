@@ -116,17 +116,24 @@ fma_state_partial(const T* __restrict__ k, const T* __restrict__ v, Problem p, i
 }
 
 // grid (ceil(E/256), units): state[u][e] = (base ? base[u][e] : 0) + sum_c partial[u][c][e], c ascending.
-// status (null: not asked): where a timeout of the partial states' kernel is recorded; the state then stays as it was.
+// ctrl (null: not asked): where a CTA of the partial states' launch says that it gave up; the state then stays as it was, and
+// the last block to see it takes the word back, so that it holds for this sum alone.  (The status word stays: a state held back
+// on its account would be every later one of that workspace.)
 __global__ void __launch_bounds__(kThreads)
-fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* state, const float* base, const int* status) {
+fma_state_reduce(const float* __restrict__ partials, int P, long long E, float* state, const float* base, WorkspaceCtrl* ctrl) {
   const long long e = (long long)blockIdx.x * kThreads + threadIdx.x;
   const int u = blockIdx.y;
-  if (e >= E) return;
-  const int recorded = status ? *status : LINATTN_OK;
-  double sum = base ? (double)base[(long long)u * E + e] : 0.0;
+  const bool live = e < E;
+  const int gave_up = ctrl ? __ldcg(&ctrl->gave_up) : 0;
+  double sum = base && live ? (double)base[(long long)u * E + e] : 0.0;
 #pragma unroll 8   // eight loads in flight
-  for (int c = 0; c < P; ++c) sum += (double)partials[((long long)u * P + c) * E + e];
-  if (recorded == LINATTN_OK) state[(long long)u * E + e] = (float)sum;
+  for (int c = 0; c < (live ? P : 0); ++c) sum += (double)partials[((long long)u * P + c) * E + e];
+  if (gave_up) {
+    __syncthreads();   // the whole block has looked
+    if (threadIdx.x == 0 && atomicAdd(&ctrl->gave_up_seen, 1) == (int)(gridDim.x * gridDim.y) - 1) ctrl->gave_up_seen = ctrl->gave_up = 0;
+    return;
+  }
+  if (live) state[(long long)u * E + e] = (float)sum;
 }
 
 // grid (ceil(N/64), units).  Thread (tn, tj) owns tokens tn + 16*r (r < 4) and outputs j = tj + 16*c.
@@ -322,7 +329,7 @@ cudaError_t fma_state(const Problem& p, const void* k, const void* v, float* sta
                         : state_partial_any(p, k, v, P, partials, rope, stream);
   if (e != cudaSuccess || P == 0) return e;
   dim3 grid((unsigned)((E + kThreads - 1) / kThreads), p.units());
-  fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, base, split ? &ctrl->status : nullptr);
+  fma_state_reduce<<<grid, kThreads, 0, stream>>>(partials, P, E, state_out, base, split ? ctrl : nullptr);
   count_launches(1);
   return cudaGetLastError();
 }

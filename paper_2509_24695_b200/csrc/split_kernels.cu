@@ -526,7 +526,8 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
       }
     }
   } else if (tid == 0) {
-    ctrl->status = LINATTN_ERR_TIMEOUT;   // (a sum of partial states looks at it: fma_state_reduce)
+    ctrl->status = LINATTN_ERR_TIMEOUT;
+    if (!state) ctrl->gave_up = 1;   // for the sum of partial states
   }
   if (state) {
     cluster_sync();

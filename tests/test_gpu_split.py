@@ -210,3 +210,23 @@ def test_no_further_from_64_bits_than_multiply_adds(la, kind, d):
         O = np.einsum("bnhi,bhji->bnhj", qn, S) / (np.einsum("bnhi,bhi->bnh", qn, z) + EPS)[..., None]
         o = to_f64(la.linattn_forward(to_dev(q), to_dev(k), to_dev(v), EPS))
         assert relative(o, O) <= 2.0 ** -21, f"O, {N} tokens: {relative(o, O):.2e}"
+
+
+def test_a_state_is_held_back_for_its_own_launch_alone(la):
+    """A state stays as it was when a CTA of its own launch gave up (said so in the second word of the control block), and only
+    then: not because the status word still has a timeout from before."""
+    import torch
+
+    q, k, v = (to_dev(x) for x in gen(1, 6000, 20, 112, 7700, "f32"))
+    want = la.linattn_state(k, v)
+    ws = la.new_workspace(k)
+    words = ws[:16].view(torch.int32)
+    out = torch.full_like(want, 7.0)
+    before = la.load_library().linattn_kernel_launches()
+    words[1] = 1
+    la.linattn_state(k, v, out=out, workspace=ws)
+    assert la.load_library().linattn_kernel_launches() == before + 2      # partial states and their sum
+    assert (out == 7.0).all() and words.tolist() == [0, 0, 0, 0]
+    words[0] = -6
+    la.linattn_state(k, v, out=out, workspace=ws)
+    assert torch.equal(out, want) and la.workspace_status(ws) == -6
