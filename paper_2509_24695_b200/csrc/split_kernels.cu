@@ -584,6 +584,8 @@ struct ApplyShape : Shape<T, R, ROPE> {
   static constexpr int SMEM = FIXED + (RAW_STAGES * RAW > OVERRUN ? RAW_STAGES * RAW : OVERRUN);
   static constexpr int ACC = TOK, SET = (LEAD + 1) * ACC;     // TMEM columns: two sets of accumulators
   static_assert(2 * SET <= 512, "tensor memory");
+  // apply_by_fma's room ends before the barriers and flags, which other threads may still be looking at
+  static_assert((B::DP * B::DP + B::DP + 256 * (kBlock + 31) / 32) * 4 <= S_BYTES + 2 * STAGE, "scratch of apply_by_fma");
 };
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
@@ -753,15 +755,20 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
           for (int s = 0; s < LEADS; ++s) tmem_ld_x8(trow + s * A::ACC + 8 * g, a[s]);
           tmem_ld_x8(trow + A::LEAD * A::ACC + 8 * g, a[A::LEAD]);
           tmem_ld_wait();
+          float wild = 0.f;   // NaN if a numerator is not finite: queries where z is zero, which no denominator sees, have no bounds
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
             float num = __uint_as_float(a[0][x]);
 #pragma unroll
             for (int s = 1; s < LEADS; ++s) num += __uint_as_float(a[s][x]);
             num += __uint_as_float(a[A::LEAD][x]);
-            if (8 * g + x < live) store_value(out, num * rden[8 * g + x]);
+            if (8 * g + x < live) {
+              store_value(out, num * rden[8 * g + x]);
+              wild = fmaf(num, 0.f, wild);
+            }
             out += p.sn;
           }
+          if (wild != 0.f) *odd_flag = 1;
         }
       }
       tcgen05_fence_before();

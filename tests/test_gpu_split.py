@@ -230,3 +230,28 @@ def test_a_state_is_held_back_for_its_own_launch_alone(la):
     words[0] = -6
     la.linattn_state(k, v, out=out, workspace=ws)
     assert torch.equal(out, want) and la.workspace_status(ws) == -6
+
+
+@pytest.mark.parametrize("d,rope", [(24, False), (64, True), (112, False)])
+@pytest.mark.parametrize("value", [3.4e38, 3e38, float("inf")])
+def test_queries_that_the_denominator_does_not_see(la, d, rope, value):
+    """Where no key has a feature (or neither of a pair), z and S are zero there: the largest finite queries count for nothing, an
+    infinite one makes its row NaN.  The rows around it stay as they are."""
+    import torch
+
+    B, N, H = 1, 200, 2
+    q, k, v = (to_dev(x) for x in gen(B, N, H, d, 7900 + d, "f32"))
+    k[..., 4:6] = -1.0
+    table = None
+    if rope:
+        cos, sin = synth.rope_table(1, 1, N, d)
+        table = la.rope_pack(to_dev(cos), to_dev(sin))
+    call = (lambda: la.linattn_forward_rope(q, k, v, table, EPS)) if rope else (lambda: la.linattn_forward(q, k, v, EPS))
+    q[..., 4:6] = 0.0
+    want = call()
+    q[0, 100, 1, 4] = value
+    got = call()
+    if value == float("inf"):
+        assert got[0, 100, 1].isnan().all()
+        got[0, 100, 1] = want[0, 100, 1]
+    assert relative(to_f64(got), to_f64(want)) <= 2.0 ** -21
