@@ -232,6 +232,39 @@ def test_a_state_is_held_back_for_its_own_launch_alone(la):
     assert torch.equal(out, want) and la.workspace_status(ws) == -6
 
 
+# launches of a step: state and apply when the CTAs of a unit are a cluster, the sum of partial states between them otherwise
+@pytest.mark.parametrize("dtype,B,N,H,d,rope,launches", [
+    ("f32", 2, 300, 3, 112, True, 2), ("f32", 1, 300, 20, 112, False, 2), ("f32", 2, 200, 80, 64, False, 2),
+    ("bf16", 2, 700, 5, 72, True, 2), ("bf16", 2, 300, 80, 40, True, 2), ("f32", 2, 6000, 10, 112, True, 3),
+    ("f32", 1, 6000, 20, 112, False, 3), ("bf16", 1, 6000, 40, 96, True, 3), ("f32", 2, 900, 100, 32, True, 2)])
+def test_both_sums_of_a_unit(la, dtype, B, N, H, d, rope, launches):
+    """A read-only step and two steps through the cache, by clusters and by partial states, several batch entries, more units than
+    SMs.  Bars on the 2-norm as above: 2^-22 for S and z on top of fp16 tables taken as they are."""
+    q, k, v = (to_dev(x) for x in gen(B, N, H, d, 7800 + N + d, dtype))
+    table = tab = None
+    if rope:
+        cos, sin = synth.rope_table(1, 1, N, d)
+        table = la.rope_pack(to_dev(cos), to_dev(sin))
+        tab = table.cpu().numpy().astype(np.float64)
+    qn, kn, vn = to_f64(q).clip(0), to_f64(k).clip(0), to_f64(v)
+    S = (turned(kn, tab).transpose(0, 2, 3, 1) @ vn.transpose(0, 2, 1, 3)).swapaxes(-1, -2)
+    z = kn.sum(1)
+    cache = la.BlockLinCache(B, H, d, q.dtype, "cuda", max_T_b=N, eps=EPS)
+    for steps in (1, 2):
+        args = (q, k, v, table) if rope else (q, k, v)
+        before = la.load_library().linattn_kernel_launches()
+        peek = cache.peek_rope(*args) if rope else cache.peek(*args)
+        assert la.load_library().linattn_kernel_launches() == before + launches
+        o = cache.step_rope(*args) if rope else cache.step(*args)
+        assert la.load_library().linattn_kernel_launches() == before + 2 * launches
+        st = to_f64(cache.state)
+        assert relative(st[:, :, :d], steps * S) <= 2.0 ** -22 and relative(st[:, :, d], steps * z) <= 2.0 ** -22
+        O = turned(qn, tab).transpose(0, 2, 1, 3) @ (steps * S).swapaxes(-1, -2)
+        O = (O / ((qn.transpose(0, 2, 1, 3) @ (steps * z)[..., None]) + EPS)).transpose(0, 2, 1, 3)
+        assert relative(to_f64(o), O) <= (2.0 ** -21 if dtype == "f32" else 2.0 ** -9) and (o == peek).all()
+    assert cache.status() == 0
+
+
 @pytest.mark.parametrize("d,rope", [(24, False), (64, True), (112, False)])
 @pytest.mark.parametrize("value", [3.4e38, 3e38, float("inf")])
 def test_queries_that_the_denominator_does_not_see(la, d, rope, value):
