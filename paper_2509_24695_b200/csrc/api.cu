@@ -324,7 +324,7 @@ int linattn_forward(const linattn_desc* desc, int64_t N, const void* q, const vo
   if (!aligned16(workspace)) return LINATTN_ERR_BAD_ALIGNMENT;
   if (workspace_bytes < workspace_need(p)) return LINATTN_ERR_WORKSPACE_TOO_SMALL;
   if (N == 0) return LINATTN_OK;
-  // the forward keeps its reduced state in the workspace, after the partials
+  // the reduced state stays in the workspace, after the partials (lone CTAs keep it on chip)
   float* state = reinterpret_cast<float*>(static_cast<char*>(workspace) + state_slot_offset(p));
   return run_passes(p, k, v, q, o, state, false, eps, workspace, (cudaStream_t)stream);
 }
