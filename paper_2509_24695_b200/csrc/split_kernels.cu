@@ -289,11 +289,11 @@ struct StateShape : Shape<T, R, ROPE> {
 // kernel then, and no partial states, so that P is not bound by their room; but a cluster has to fit into one GPC (8 CTAs
 // of this size at most, and 15 such clusters on the chip), so that large inputs want the other form (launch_state).
 //
-// Measured (32 760 tokens, 20 heads of 112, fp32; floor: 587 MB, 90 us at the copy rate): 176 us with the reduce of the
+// Measured (32 760 tokens, 20 heads of 112, fp32; floor: 587 MB, 90 us at the copy rate): 177 us with the reduce of the
 // partial states (192 with every warp preparing and draining in turn), where the general kernels take 1050 (fp32 pipe at a
 // quarter of its rate, scalar loads) and a register-blocked form of them on packed fp32 FMAs 492.  A tile of 32 tokens takes
 // 1.1 us, with 190 KB through shared memory (pieces in and out, their parts, 90 KB of MMA operands): two thirds of what it
-// moves in that time.  Distance from 64 bits, 2-norm: S 1.3e-7 (general kernels 2.9e-7).
+// moves in that time.  (Distance from 64 bits: see the top.)
 template <typename T, int R, bool ROPE>
 __global__ void __launch_bounds__(kBlock, 1)
 split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, int P, float* __restrict__ partials,
@@ -590,8 +590,8 @@ struct ApplyShape : Shape<T, R, ROPE> {
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
 //
-// Measured as above: 185 us (operand reads of the MMAs, 250 of 350 KB a tile through shared memory), general kernels 866,
-// register-blocked on packed fp32 FMAs 489; distance from 64 bits 1.0e-7 (general kernels 1.6e-7).  bf16, 28 heads of 80:
+// Measured as above: 186 us (operand reads of the MMAs, 250 of 350 KB a tile through shared memory), general kernels 866,
+// register-blocked on packed fp32 FMAs 489.  bf16, 28 heads of 80:
 // 152 us (165 with tiles of 64 tokens and every warp in both roles), general kernels 644.
 template <typename T, int R, bool ROPE>
 __global__ void __launch_bounds__(kBlock, 1)
