@@ -239,7 +239,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // .x = lo (low 16 bits), .y = hi
   return *reinterpret_cast<uint32_t*>(&v);
 }
-// Packed fp32 pairs (sm_100 has f32x2 FMA, MUL and ADD): one instruction for two lanes, each lane rounded as the
+// Packed fp32 pairs (sm_100 has f32x2 FMA and ADD): one instruction for two lanes, each lane rounded as the
 // scalar instruction would.
 __device__ __forceinline__ unsigned long long pack_f32x2(float2 a) {
   unsigned long long r;
@@ -254,11 +254,6 @@ __device__ __forceinline__ float2 unpack_f32x2(unsigned long long r) {
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
   unsigned long long d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack_f32x2(a)), "l"(pack_f32x2(b)), "l"(pack_f32x2(c)));
-  return unpack_f32x2(d);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack_f32x2(a)), "l"(pack_f32x2(b)));
   return unpack_f32x2(d);
 }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {

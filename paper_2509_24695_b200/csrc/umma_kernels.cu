@@ -107,6 +107,11 @@ struct Cfg {
   static constexpr int DEN_BYTES = D == 112 ? 0 : G * APPLY_SLOTS * kTileApply * 4;
   static constexpr size_t SMEM = 1024 + DATA_BYTES + BAR_BYTES;
   static constexpr size_t SMEM_ROPE = SMEM + DEN_BYTES;
+  // Rotary variant, state pass of the grid form: the stage holds the rotations of its 64 tokens behind V0 V1 K0 K1.
+  static constexpr int TAB_ROW = 2 * D;                      // d/2 (cos, sin) fp16 pairs
+  static constexpr int ROPE_STAGE_BYTES = 4 * kBox + kTileState * TAB_ROW;
+  static constexpr int ROPE_STAGES = 4;
+  static_assert(ROPE_STAGES * ROPE_STAGE_BYTES <= DATA_BYTES, "stages of the rotary variant");
   // lone CTAs (see solo_drain): the slots, then the warps' sums for z and z, then the unit's state as it is in memory
   static constexpr int SOLO_SLOTS = D == 128 ? 2 : 3;
   static constexpr int SOLO_STAGE_BYTES = 4 * kBox;            // no "ones"
@@ -283,8 +288,7 @@ __device__ __forceinline__ void relu_sum_pass(uint8_t* box0, uint8_t* box1, int 
 
 // Rotary variant: a 16-byte chunk holds four feature pairs; `tab` holds their (cos, sin) as fp16 pairs.
 // (a, b) -> (a c - b s, a s + b c), rounded to bf16.
-// The ReLU role of the rotary variant is bound by instruction issue, so the clamp is done on the packed bf16
-// pairs and the sums, the rotation and the denominators use the packed f32x2 instructions.
+// The clamp is done on the packed bf16 pairs, and the sums and the denominators use the packed f32x2 instructions.
 __device__ __forceinline__ void unpack_relu8(const uint4& x, float2 (&f)[4]) {
   const uint32_t w[4] = {relu_bf16x2(x.x), relu_bf16x2(x.y), relu_bf16x2(x.z), relu_bf16x2(x.w)};
 #pragma unroll
@@ -296,9 +300,8 @@ __device__ __forceinline__ uint4 rotate_pack8(const float2 (&f)[4], const uint4&
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const float2 cs = __half22float2(*reinterpret_cast<const __half2*>(&t[e]));
-    // (a, b) -> (a c - b s, b c + a s) = (-b, a) * (s, s) + (a, b) * (c, c)
-    const float2 r = fma2(make_float2(-f[e].y, f[e].x), make_float2(cs.y, cs.y), mul2(f[e], make_float2(cs.x, cs.x)));
-    o[e] = pack_bf16x2(r.x, r.y);
+    // (scalar: the packed f32x2 forms want the cosine and the sine twice in neighbouring registers, and the pair swapped)
+    o[e] = pack_bf16x2(fmaf(-f[e].y, cs.y, f[e].x * cs.x), fmaf(f[e].x, cs.y, f[e].y * cs.x));
   }
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
@@ -864,6 +867,176 @@ __device__ __forceinline__ float sum_z_slots(const float* slots, int f) {
   return tree;
 }
 
+// x := 16 bytes at `at` if `live`, loaded into the registers x is in: no branch, no copy and no choice, which would wait for
+// the load.
+__device__ __forceinline__ void load_in_place(uint4& x, const uint4* at, bool live) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "setp.ne.b32 p, %5, 0;\n"
+      "@p ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n"
+      "}\n"
+      : "+r"(x.x), "+r"(x.y), "+r"(x.z), "+r"(x.w)
+      : "l"(at), "r"((int)live));
+}
+
+// Rotary variant, state pass: this thread's chunks of the 64 rows of a stage, rows row0 and row0 + 32 of box 0 and row0 of
+// box 1 (the epilogue takes the other half of that): plain values to its sums for z, rotated ones back.  All of them are read
+// before the first is written.  rows_left: tokens from row0 on; rows beyond the last one hold zeros, and no rotations.
+template <int D>
+__device__ __forceinline__ void rope_state_rows(uint8_t* k_boxes, const uint8_t* tab, int row0, int pc, int lc, long long rows_left,
+                                                float2 (&zacc)[8]) {
+  using C = Cfg<D>;
+  uint8_t* p0 = k_boxes + row0 * kRowBytes + pc * 16;
+  const uint8_t* tb = tab + row0 * C::TAB_ROW;
+  uint4 x[3], r[3];   // rows row0 and row0 + 32 of box 0, row0 of box 1
+  x[0] = *reinterpret_cast<const uint4*>(p0);
+  x[1] = *reinterpret_cast<const uint4*>(p0 + 32 * kRowBytes);
+  r[0] = *reinterpret_cast<const uint4*>(tb + C::tab_chunk(0, lc) * 16);
+  r[1] = *reinterpret_cast<const uint4*>(tb + 32 * C::TAB_ROW + C::tab_chunk(0, lc) * 16);
+  // (d = 112: two lanes of eight have zero padding there, and turn it; without them a branch would part the rows' work)
+  x[2] = *reinterpret_cast<const uint4*>(p0 + kBox);
+  r[2] = C::SAME_TAB ? r[0] : *reinterpret_cast<const uint4*>(tb + C::tab_chunk(1, lc) * 16);
+  if (rows_left <= 32) {
+    const uint4 identity = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
+    r[1] = identity;
+    if (rows_left <= 0) r[0] = r[2] = identity;
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    float2 f[4];
+    unpack_relu8(x[i], f);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) zacc[(i == 2 ? 4 : 0) + e] = add2(zacc[(i == 2 ? 4 : 0) + e], f[e]);
+    *reinterpret_cast<uint4*>(i == 2 ? p0 + kBox : p0 + i * 32 * kRowBytes) = rotate_pack8(f, r[i]);
+  }
+}
+
+// Rotary variant, apply pass: this thread's chunks of the 128 rows of a Q tile.  The operand of the numerator is the rotated
+// phi(q); the denominator, plain phi(q) . z, is added up over the eight lanes that share a row and left in the row's zero
+// padding (features 112..) or in `den`, [G][128].  tab0, tab1: the rotations of its rows for the two boxes (the same
+// where box 1 starts a new head); next(i) asks for row i's of the next tile.
+//
+// The rotary apply pass waits for this role (8 warps): alone on an SM it takes 1450 cycles a tile, with rotations that
+// never stall it, where the pass could stream one in 2500.  32 760 tokens, 20 heads of 112, forward: 161 us before the rotations of the
+// state pass came through shared memory (its share 84 -> 66 us) and before this function had no branch, copy or choice
+// between its rows (77 -> 67 us); 720p 340 -> 282 us, 35 heads of 64 145 -> 137, 18 of 128 150 -> 137.  Not taken: rotations in
+// a shared-memory ring beside fewer Q slots (90 to 98 us), sixteen warps of 80 registers (115 us).
+template <int D, class Next>
+__device__ __forceinline__ void rope_apply_rows(uint8_t* sl, float* den, int row0, int pc, int lc, const float2 (&zc)[8],
+                                                const uint4 (&tab0)[kTileApply / 32], const uint4 (&tab1)[kTileApply / 32], Next&& next) {
+  using C = Cfg<D>;
+  constexpr int HALF = C::SLOT_BYTES / 2;
+  uint8_t* p0 = sl + row0 * kRowBytes + pc * 16;
+  constexpr int ROWS = kTileApply / 32;
+  float dens[ROWS];
+#pragma unroll
+  for (int i = 0; i < ROWS; ++i) {
+    uint8_t* c0 = p0 + i * 32 * kRowBytes;
+    const uint4 x0 = *reinterpret_cast<const uint4*>(c0);
+    const uint4 x1 = *reinterpret_cast<const uint4*>(c0 + HALF);
+    float2 f[4];
+    unpack_relu8(x0, f);
+    float2 den2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) den2 = fma2(f[e], zc[e], den2);
+    *reinterpret_cast<uint4*>(c0) = rotate_pack8(f, tab0[i]);
+    float2 den2b = make_float2(0.f, 0.f);   // packed heads: box 1 belongs to other heads than box 0
+    unpack_relu8(x1, f);   // (d = 112: padding is turned too, see rope_state_rows; z is zero there)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (C::G == 1) den2 = fma2(f[e], zc[4 + e], den2);
+      else den2b = fma2(f[e], zc[4 + e], den2b);
+    }
+    *reinterpret_cast<uint4*>(c0 + HALF) = rotate_pack8(f, C::SAME_TAB ? tab0[i] : tab1[i]);
+    next(i);
+    const float dn = dens[i] = den2.x + den2.y;
+    // The eight lanes of a row hold one chunk of each box.  Packed heads: box 1 belongs to other heads, and with d = 32 a
+    // head is four lanes wide; the first exchange hands one box's sum to the partner lane, so that each half of the lanes
+    // reduces one box.
+    if (C::G > 1) {
+      const int row = row0 + 32 * i;
+      const float denb = den2b.x + den2b.y;
+      constexpr int XB = C::G == 2 ? 4 : 2;             // lane bit that picks the box after the exchange
+      const bool second = (pc & XB) != 0;
+      float x = second ? denb : dn;
+      x += __shfl_xor_sync(0xffffffffu, second ? dn : denb, XB);
+      x += __shfl_xor_sync(0xffffffffu, x, 1);
+      if (C::G == 2) x += __shfl_xor_sync(0xffffffffu, x, 2);
+      // d = 64: lane 0 of the row has head 0 (box 0), lane 4 head 1.  d = 32: lanes with the same pc / 4 share
+      // a head, whose place in its box is lc / 4; lanes 0 and 4 have box 0, lanes 2 and 6 box 1
+      if (C::G == 2) {
+        if ((pc & 3) == 0) den[(second ? 1 : 0) * kTileApply + row] = x;
+      } else {
+        if ((pc & 1) == 0) den[((second ? 2 : 0) + (lc >> 2)) * kTileApply + row] = x;
+      }
+    }
+  }
+  if (C::G == 1) {
+    // One head: four rows over eight lanes.  Each exchange hands half of what a lane has to its partner, so that four
+    // shuffles do, not twelve, and lanes 2 i and 2 i + 1 end up with row i.
+    const bool b2 = (pc & 4) != 0, b1 = (pc & 2) != 0;
+    const float a0 = (b2 ? dens[2] : dens[0]) + __shfl_xor_sync(0xffffffffu, b2 ? dens[0] : dens[2], 4);
+    const float a1 = (b2 ? dens[3] : dens[1]) + __shfl_xor_sync(0xffffffffu, b2 ? dens[1] : dens[3], 4);
+    float x = (b1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b1 ? a0 : a1, 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    const int row = row0 + 32 * (pc >> 1);
+    if ((pc & 1) == 0) {
+      if (D == 112) *reinterpret_cast<float*>(sl + HALF + row * kRowBytes + ((6 ^ (row & 7)) << 4)) = x;   // features 112..119: padding
+      else den[row] = x;   // no padding to carry it
+    }
+  }
+}
+
+// Epilogue of an apply tile: lane quarter wq of the accumulator at TMEM column `acc` is divided, rounded and staged in the
+// tile's slot; `tempty` gets the accumulator back as soon as it is read.
+template <int D, bool ROPE>
+__device__ __forceinline__ void apply_epilogue(uint32_t acc, uint8_t* sl, const float* den, int wq, int lane, float eps, uint64_t* tempty) {
+  using C = Cfg<D>;
+  constexpr int HALF = C::SLOT_BYTES / 2;
+  const int r = wq * 32 + lane;   // accumulator lane = token row of the tile
+  const uint32_t trow = acc + ((uint32_t)(wq * 32) << 16);
+  float rinv[C::G];
+  if (ROPE) {
+    // the ReLU warps left phi(q) . z of this row in the row's padding
+    if (D == 112) {
+      rinv[0] = 1.0f / (*reinterpret_cast<const float*>(sl + HALF + r * kRowBytes + ((6 ^ (r & 7)) << 4)) + eps);
+    } else {
+#pragma unroll
+      for (int g = 0; g < C::G; ++g) rinv[g] = 1.0f / (den[g * kTileApply + r] + eps);
+    }
+  } else {
+    uint32_t dn[4];
+    tmem_ld_x4(trow + C::ZROW, dn);
+    tmem_ld_wait();
+#pragma unroll
+    for (int g = 0; g < C::G; ++g) rinv[g] = 1.0f / (__uint_as_float(dn[g]) + eps);  // eps added once, after the dot product
+  }
+#pragma unroll
+  for (int cc = 0; cc < 4; ++cc) {
+    if (cc * 32 >= C::FEAT) break;
+    uint32_t v[32];
+    tmem_ld_x32(trow + cc * 32, v);
+    tmem_ld_wait();
+    if (cc == 3 || (cc + 1) * 32 >= C::FEAT) {  // last read of this accumulator: hand it back to the MMA warp
+      tcgen05_fence_before();
+      mbar_arrive(tempty);
+    }
+    const float ri = rinv[(cc * 32) / D < C::G ? (cc * 32) / D : 0];
+#pragma unroll
+    for (int q4 = 0; q4 < 4; ++q4) {
+      const int lc = cc * 4 + q4;  // logical 16-byte chunk of the 256-byte padded row
+      if (lc * 8 >= C::FEAT) break;
+      uint4 pk;
+      pk.x = pack_bf16x2(__uint_as_float(v[q4 * 8 + 0]) * ri, __uint_as_float(v[q4 * 8 + 1]) * ri);
+      pk.y = pack_bf16x2(__uint_as_float(v[q4 * 8 + 2]) * ri, __uint_as_float(v[q4 * 8 + 3]) * ri);
+      pk.z = pack_bf16x2(__uint_as_float(v[q4 * 8 + 4]) * ri, __uint_as_float(v[q4 * 8 + 5]) * ri);
+      pk.w = pack_bf16x2(__uint_as_float(v[q4 * 8 + 6]) * ri, __uint_as_float(v[q4 * 8 + 7]) * ri);
+      *reinterpret_cast<uint4*>(sl + (lc >> 3) * HALF + r * kRowBytes + (((lc & 7) ^ (r & 7)) << 4)) = pk;
+    }
+  }
+}
+
 // ============================================================================ the kernel
 // SOLO: lone CTAs.  IMAGE: the reduce leaves operand images and the apply pass fetches them (p.s_image).  Both are decided
 // on the host, and each form is a kernel of its own: the rotary one has no registers to spare, and with the slice reduce that
@@ -876,15 +1049,18 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   static_assert(!IMAGE || (Cfg<D>::G == 1 && !SOLO), "operand images are of one-head units in a grid");
   using C = Cfg<D>;
   using R = Roles<ROPE>;
-  constexpr int NSA = SOLO ? 4 : C::STATE_STAGES;
-  constexpr int STAGE = SOLO ? C::SOLO_STAGE_BYTES : C::STAGE_BYTES;
-  constexpr int KOFF = SOLO ? 2 * kBox : C::KOFF;
+  // TAB: the state pass has its rotations in shared memory.  (Lone CTAs have no room for them and fetch them into registers.)
+  constexpr bool TAB = ROPE && !SOLO;
+  constexpr int NSA = SOLO ? 4 : ROPE ? C::ROPE_STAGES : C::STATE_STAGES;
+  constexpr int STAGE = SOLO ? C::SOLO_STAGE_BYTES : ROPE ? C::ROPE_STAGE_BYTES : C::STAGE_BYTES;
+  constexpr int KOFF = SOLO || ROPE ? 2 * kBox : C::KOFF;
+  constexpr int TOFF = 4 * kBox;
   constexpr int NSC = SOLO ? C::SOLO_SLOTS : C::APPLY_SLOTS;
   constexpr int DATA = SOLO ? C::SOLO_DATA : C::DATA_BYTES;
   constexpr int SLOT = C::SLOT_BYTES;
   constexpr int HALF = SLOT / 2;  // one 64-feature box of 128 tokens
-  constexpr uint32_t IDESC_A = make_idesc_bf16(128, SOLO ? 128 : C::NSTATE, true, true);
-  constexpr int ACCS = SOLO ? 4 : C::STATE_ACCS, ACC_STRIDE = SOLO ? 128 : C::STATE_ACC_STRIDE;
+  constexpr uint32_t IDESC_A = make_idesc_bf16(128, SOLO || ROPE ? 128 : C::NSTATE, true, true);
+  constexpr int ACCS = SOLO || ROPE ? 4 : C::STATE_ACCS, ACC_STRIDE = SOLO || ROPE ? 128 : C::STATE_ACC_STRIDE;
   constexpr uint32_t IDESC_C = make_idesc_bf16(128, C::NAPPLY, false, false);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
@@ -947,7 +1123,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     prefetch_tensormap(&map_q);
     prefetch_tensormap(&map_o);
   }
-  if (!SOLO && C::ONES_BOX && wa.f1 > wa.f0) {
+  if (!SOLO && !ROPE && C::ONES_BOX && wa.f1 > wa.f0) {
     // the constant "ones" chunk of every stage: value columns 128..191 of B, of which column 128 is 1
     for (int idx = threadIdx.x; idx < NSA * (kBox / 16); idx += R::THREADS) {
       const int s = idx / (kBox / 16), c = idx % (kBox / 16);
@@ -993,7 +1169,14 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         if (!mbar_wait(&a_empty[s], ((it / NSA) & 1) ^ 1, abort_flag)) break;
         const int u = t.unit(), b = u / p.HG, hg = u % p.HG;
         uint8_t* st = smem + s * STAGE;
-        mbar_arrive_expect_tx(&a_full[s], 4 * kBox);
+        if (TAB) {
+          const long long n = (long long)t.tile() * kTileState, left = p.N - n;
+          const uint32_t bytes = (left < kTileState ? (uint32_t)left : (uint32_t)kTileState) * C::TAB_ROW;
+          mbar_arrive_expect_tx(&a_full[s], 4 * kBox + bytes);
+          bulk_load(st + TOFF, p.rope + n * (D / 8), bytes, &a_full[s]);
+        } else {
+          mbar_arrive_expect_tx(&a_full[s], 4 * kBox);
+        }
         int c0, c1;
         box_coords<D>(0, hg, c0, c1);
         tma_load_4d(st + KOFF, &map_k, &a_full[s], c0, c1, t.tile() * kTileState, b);
@@ -1045,7 +1228,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     float2 zacc[8];  // sums of the plain phi(k) over the segment: features 8*lc.. of box 0, 64 + 8*lc.. of box 1
 #pragma unroll
     for (int e = 0; e < 8; ++e) zacc[e] = make_float2(0.f, 0.f);
-    // The rotations of a row do not depend on K: they are fetched one stage ahead, each register reloaded
+    // Lone CTAs: the rotations of a row do not depend on K; they are fetched one stage ahead, each register reloaded
     // for the next stage right after its use, so that their latency is off the stage's critical path.
     // Of the second K box these warps take the first 32 token rows of a stage; the epilogue warps, idle until the
     // segment's accumulators are complete, take the other 32 (this role is what the pass waits for).
@@ -1098,7 +1281,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       fence_proxy_async_smem();
       mbar_arrive(s_ready);
     };
-    if (ROPE) {
+    if (ROPE && SOLO) {
       TileWalk t0(wa);
       if (!t0.done()) {
 #pragma unroll
@@ -1108,6 +1291,15 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     for (TileWalk t(wa); !t.done(); t.next(), ++it) {
       const int s = it % NSA;
       uint8_t* st = smem + s * STAGE;
+      if (TAB) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&a_full[s], (it / NSA) & 1, abort_flag))) break;  // leave as a whole warp
+        rope_state_rows<D>(st + KOFF, st + TOFF, row0, pc, lc, p.N - (long long)t.tile() * kTileState - row0, zacc);
+        fence_proxy_async_smem();
+        mbar_arrive(&a_ready[s]);
+        if (t.seg_last())
+          leave_z(p.partials + (size_t)t.record() * (C::G * (D + 1) * D + kZParts) + C::G * (D + 1) * D, zacc, tr, lc, box1_live);
+        continue;
+      }
       if (ROPE) {
         TileWalk tn = t;
         tn.next();
@@ -1133,8 +1325,8 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         fence_proxy_async_smem();
         mbar_arrive(&a_ready[s]);
         if (t.seg_last()) {
-          leave_z(SOLO ? z_slots : p.partials + (size_t)t.record() * (C::G * (D + 1) * D + kZParts) + C::G * (D + 1) * D, zacc, tr, lc, box1_live);
-          if (SOLO) finish_z();
+          leave_z(z_slots, zacc, tr, lc, box1_live);
+          finish_z();
         }
         continue;
       }
@@ -1178,7 +1370,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       tabh[j] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
       if (h_live && n < p.N) tabh[j] = __ldg(p.rope + n * (D / 8) + C::tab_chunk(1, lch));
     };
-    if (ROPE) {
+    if (ROPE && SOLO) {
       TileWalk t0(wa);
       if (!t0.done()) { fetch_roth(t0.tile(), 0); fetch_roth(t0.tile(), 1); }
     }
@@ -1190,6 +1382,15 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         tn.next();
         if (!__all_sync(0xffffffffu, mbar_wait(&a_full[s], (it / NSA) & 1, abort_flag))) break;  // leave as a whole warp
         uint8_t* p1 = smem + s * STAGE + KOFF + kBox + (32 + row0h) * kRowBytes + pch * 16;
+        if (TAB) {   // this tile's, from its stage
+          const uint8_t* tb = smem + s * STAGE + TOFF + (32 + row0h) * C::TAB_ROW + C::tab_chunk(1, lch) * 16;
+          const long long rows_left = p.N - (long long)t.tile() * kTileState - 32 - row0h;
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            tabh[j] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
+            if (h_live && rows_left > 16 * j) tabh[j] = *reinterpret_cast<const uint4*>(tb + j * 16 * C::TAB_ROW);
+          }
+        }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           if (h_live) {
@@ -1200,7 +1401,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             for (int e = 0; e < 4; ++e) zh[e] = add2(zh[e], f[e]);
             *c1 = rotate_pack8(f, tabh[j]);
           }
-          if (!tn.done()) fetch_roth(tn.tile(), j);
+          if (SOLO && !tn.done()) fetch_roth(tn.tile(), j);
         }
         fence_proxy_async_smem();
         mbar_arrive(&a_ready[s]);
@@ -1259,9 +1460,9 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
           for (int x = 0; x < 32; ++x) sum[x] = __uint_as_float(r[x]);
         }
 #pragma unroll 1
-        for (int a = 1; a < C::STATE_ACCS; ++a) {
+        for (int a = 1; a < ACCS; ++a) {
           uint32_t r[32];
-          tmem_ld_x32(trow + a * C::STATE_ACC_STRIDE + cc * 32, r);
+          tmem_ld_x32(trow + a * ACC_STRIDE + cc * 32, r);
           tmem_ld_wait();
 #pragma unroll
           for (int x = 0; x < 32; ++x) sum[x] += __uint_as_float(r[x]);
@@ -1385,16 +1586,18 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     float2 zc[8];  // the segment's z at this thread's features (8*lc.. of box 0, 64 + 8*lc.. of box 1)
 #pragma unroll
     for (int e = 0; e < 8; ++e) zc[e] = make_float2(0.f, 0.f);
-    // rotations one tile ahead, as in the state pass
+    // The rotations of the next tile's rows are asked for as soon as this tile's have been used.  Nothing may touch them
+    // before their tile comes, since that waits for the load: not a copy (d = 64, where both boxes use the same: 4000 of the 5700
+    // cycles that this role took a tile), and no choice between what is loaded and something else.  Rows beyond the last token
+    // keep what they have (they are not stored), and the last tile asks for its own once more.
     uint4 tab0[kTileApply / 32], tab1[kTileApply / 32];
+#pragma unroll
+    for (int i = 0; i < kTileApply / 32; ++i) tab0[i] = tab1[i] = make_uint4(0, 0, 0, 0);
     auto fetch_rot = [&](int tile, int i) {
       const long long n = (long long)tile * kTileApply + row0 + 32 * i;
-      tab0[i] = tab1[i] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
-      if (n < p.N) {
-        tab0[i] = __ldg(p.rope + n * (D / 8) + C::tab_chunk(0, lc));
-        if (C::SAME_TAB) tab1[i] = tab0[i];
-        else if (box1_live) tab1[i] = __ldg(p.rope + n * (D / 8) + C::tab_chunk(1, lc));
-      }
+      const uint4* at = p.rope + n * (D / 8);
+      load_in_place(tab0[i], at + C::tab_chunk(0, lc), n < p.N);
+      if (!C::SAME_TAB) load_in_place(tab1[i], at + C::tab_chunk(1, lc), n < p.N);
     };
     if (ROPE) {
       TileWalk t0(wc);
@@ -1456,59 +1659,8 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         TileWalk tn = t;
         tn.next();
         if (!__all_sync(0xffffffffu, mbar_wait(&c_full[s], (it / NSC) & 1, abort_flag))) break;  // leave as a whole warp
-        uint8_t* p0 = sl + row0 * kRowBytes + pc * 16;
-#pragma unroll
-        for (int i = 0; i < kTileApply / 32; ++i) {
-          float2 f[4];
-          uint4* c0 = reinterpret_cast<uint4*>(p0 + i * 32 * kRowBytes);
-          unpack_relu8(*c0, f);
-          float2 den2 = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) den2 = fma2(f[e], zc[e], den2);
-          *c0 = rotate_pack8(f, tab0[i]);
-          uint4* c1 = reinterpret_cast<uint4*>(p0 + HALF + i * 32 * kRowBytes);
-          float2 den2b = make_float2(0.f, 0.f);   // packed heads: box 1 belongs to other heads than box 0
-          if (box1_live) {
-            unpack_relu8(*c1, f);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              if (C::G == 1) den2 = fma2(f[e], zc[4 + e], den2);
-              else den2b = fma2(f[e], zc[4 + e], den2b);
-            }
-            *c1 = rotate_pack8(f, tab1[i]);
-          }
-          float den = den2.x + den2.y;
-          if (!tn.done()) fetch_rot(tn.tile(), i);  // this row's rotations for the next tile
-          // The eight lanes of a row hold one chunk of each box.  One head per operand: add all of it over the eight.
-          // Packed heads: box 1 belongs to other heads, and with d = 32 a head is four lanes wide; the first exchange
-          // hands one box's sum to the partner lane, so that each half of the lanes reduces one box.
-          const int row = row0 + 32 * i;
-          if (C::G == 1) {
-            den += __shfl_xor_sync(0xffffffffu, den, 1);
-            den += __shfl_xor_sync(0xffffffffu, den, 2);
-            den += __shfl_xor_sync(0xffffffffu, den, 4);
-            if (D == 112) {
-              if (lc == 6) *reinterpret_cast<float*>(c1) = den;  // chunk 6 of the second box: features 112..119
-            } else {
-              if (pc == 0) den_rows[s * kTileApply + row] = den;   // no padding to carry it
-            }
-          } else {
-            const float denb = den2b.x + den2b.y;
-            constexpr int XB = C::G == 2 ? 4 : 2;             // lane bit that picks the box after the exchange
-            const bool second = (pc & XB) != 0;
-            float x = second ? denb : den;
-            x += __shfl_xor_sync(0xffffffffu, second ? den : denb, XB);
-            x += __shfl_xor_sync(0xffffffffu, x, 1);
-            if (C::G == 2) x += __shfl_xor_sync(0xffffffffu, x, 2);
-            // d = 64: lane 0 of the row has head 0 (box 0), lane 4 head 1.  d = 32: lanes with the same pc / 4 share
-            // a head, whose place in its box is lc / 4; lanes 0 and 4 have box 0, lanes 2 and 6 box 1
-            if (C::G == 2) {
-              if ((pc & 3) == 0) den_rows[(s * 2 + (second ? 1 : 0)) * kTileApply + row] = x;
-            } else {
-              if ((pc & 1) == 0) den_rows[(s * 4 + (second ? 2 : 0) + (lc >> 2)) * kTileApply + row] = x;
-            }
-          }
-        }
+        const int ahead = tn.done() ? t.tile() : tn.tile();
+        rope_apply_rows<D>(sl, den_rows + s * C::G * kTileApply, row0, pc, lc, zc, tab0, tab1, [&](int i) { fetch_rot(ahead, i); });
         fence_proxy_async_smem();
         mbar_arrive(&c_ready[s]);
         continue;
@@ -1522,7 +1674,6 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     // ------------------------------------------------------------ epilogue: divide, round, stage the O tile
     const int wq = warp & 3;
     const int te = threadIdx.x - R::EPI_THREAD0;
-    const int r = wq * 32 + lane;  // accumulator lane = token row of the tile
     uint32_t it = 0;
     for (TileWalk t(wc); !t.done(); t.next(), ++it) {
       const int s = it % NSC;
@@ -1541,47 +1692,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       if (!ok) break;
       tcgen05_fence_after();
       if (t.seg_last()) mbar_arrive(seg_done);
-      const uint32_t trow = tmem_base + acc * kAccStride + ((uint32_t)(wq * 32) << 16);
-      uint8_t* sl = slots + s * SLOT;
-      float rinv[C::G];
-      if (ROPE) {
-        // the ReLU warps left phi(q) . z of this row in the row's padding
-        if (D == 112) {
-          rinv[0] = 1.0f / (*reinterpret_cast<const float*>(sl + HALF + r * kRowBytes + ((6 ^ (r & 7)) << 4)) + p.eps);
-        } else {
-#pragma unroll
-          for (int g = 0; g < C::G; ++g) rinv[g] = 1.0f / (den_rows[(s * C::G + g) * kTileApply + r] + p.eps);
-        }
-      } else {
-        uint32_t dn[4];
-        tmem_ld_x4(trow + C::ZROW, dn);
-        tmem_ld_wait();
-#pragma unroll
-        for (int g = 0; g < C::G; ++g) rinv[g] = 1.0f / (__uint_as_float(dn[g]) + p.eps);  // eps added once, after the dot product
-      }
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        if (cc * 32 >= C::FEAT) break;
-        uint32_t v[32];
-        tmem_ld_x32(trow + cc * 32, v);
-        tmem_ld_wait();
-        if (cc == 3 || (cc + 1) * 32 >= C::FEAT) {  // last read of this accumulator: hand it back to the MMA warp
-          tcgen05_fence_before();
-          mbar_arrive(&c_tempty[acc]);
-        }
-        const float ri = rinv[(cc * 32) / D < C::G ? (cc * 32) / D : 0];
-#pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-          const int lc = cc * 4 + q4;  // logical 16-byte chunk of the 256-byte padded row
-          if (lc * 8 >= C::FEAT) break;
-          uint4 pk;
-          pk.x = pack_bf16x2(__uint_as_float(v[q4 * 8 + 0]) * ri, __uint_as_float(v[q4 * 8 + 1]) * ri);
-          pk.y = pack_bf16x2(__uint_as_float(v[q4 * 8 + 2]) * ri, __uint_as_float(v[q4 * 8 + 3]) * ri);
-          pk.z = pack_bf16x2(__uint_as_float(v[q4 * 8 + 4]) * ri, __uint_as_float(v[q4 * 8 + 5]) * ri);
-          pk.w = pack_bf16x2(__uint_as_float(v[q4 * 8 + 6]) * ri, __uint_as_float(v[q4 * 8 + 7]) * ri);
-          *reinterpret_cast<uint4*>(sl + (lc >> 3) * HALF + r * kRowBytes + (((lc & 7) ^ (r & 7)) << 4)) = pk;
-        }
-      }
+      apply_epilogue<D, ROPE>(tmem_base + acc * kAccStride, slots + s * SLOT, den_rows + s * C::G * kTileApply, wq, lane, p.eps, &c_tempty[acc]);
       fence_proxy_async_smem();
       mbar_arrive(&c_staged[s]);
     }
