@@ -30,7 +30,7 @@
 // product are ignored / zero); 112 pads to 128 through TMA out-of-bounds zero fill.
 //
 // A unit of few tokens is taken by one CTA from its first token to its last output instead (SOLO): no grid barrier, no
-// record, no reduce, and an ordinary launch.
+// record, no reduce, and an ordinary launch.  Between the two, the CTAs of a unit are a cluster (umma_cluster.cuh).
 //
 // Warp roles (352 threads): warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-5 ReLU
 // pass, warps 6-9 epilogue, warp 10 output stores.  All cross-role synchronisation is by mbarriers
@@ -988,14 +988,16 @@ __device__ __forceinline__ void rope_apply_rows(uint8_t* sl, float* den, int row
   }
 }
 
-// Epilogue of an apply tile: lane quarter wq of the accumulator at TMEM column `acc` is divided, rounded and staged in the
-// tile's slot; `tempty` gets the accumulator back as soon as it is read.
+// Epilogue of an apply tile in slot s: lane quarter wq of accumulator `acc` is divided, rounded and staged in the slot; r:
+// accumulator lane = token row of the tile.  The accumulator is handed back as soon as it is read.  (The arguments are what the
+// callers' loops have at hand: with ready-made addresses instead the 480p step took 2 % longer.)
 template <int D, bool ROPE>
-__device__ __forceinline__ void apply_epilogue(uint32_t acc, uint8_t* sl, const float* den, int wq, int lane, float eps, uint64_t* tempty) {
+__device__ __forceinline__ void apply_epilogue(uint32_t tmem_base, uint32_t acc, uint8_t* slots, int s, const float* den_rows, int wq, int r, float eps,
+                                               uint64_t* c_tempty) {
   using C = Cfg<D>;
-  constexpr int HALF = C::SLOT_BYTES / 2;
-  const int r = wq * 32 + lane;   // accumulator lane = token row of the tile
-  const uint32_t trow = acc + ((uint32_t)(wq * 32) << 16);
+  constexpr int SLOT = C::SLOT_BYTES, HALF = SLOT / 2;
+  const uint32_t trow = tmem_base + acc * kAccStride + ((uint32_t)(wq * 32) << 16);
+  uint8_t* sl = slots + s * SLOT;
   float rinv[C::G];
   if (ROPE) {
     // the ReLU warps left phi(q) . z of this row in the row's padding
@@ -1003,7 +1005,7 @@ __device__ __forceinline__ void apply_epilogue(uint32_t acc, uint8_t* sl, const 
       rinv[0] = 1.0f / (*reinterpret_cast<const float*>(sl + HALF + r * kRowBytes + ((6 ^ (r & 7)) << 4)) + eps);
     } else {
 #pragma unroll
-      for (int g = 0; g < C::G; ++g) rinv[g] = 1.0f / (den[g * kTileApply + r] + eps);
+      for (int g = 0; g < C::G; ++g) rinv[g] = 1.0f / (den_rows[(s * C::G + g) * kTileApply + r] + eps);
     }
   } else {
     uint32_t dn[4];
@@ -1020,7 +1022,7 @@ __device__ __forceinline__ void apply_epilogue(uint32_t acc, uint8_t* sl, const 
     tmem_ld_wait();
     if (cc == 3 || (cc + 1) * 32 >= C::FEAT) {  // last read of this accumulator: hand it back to the MMA warp
       tcgen05_fence_before();
-      mbar_arrive(tempty);
+      mbar_arrive(&c_tempty[acc]);
     }
     const float ri = rinv[(cc * 32) / D < C::G ? (cc * 32) / D : 0];
 #pragma unroll
@@ -1674,6 +1676,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     // ------------------------------------------------------------ epilogue: divide, round, stage the O tile
     const int wq = warp & 3;
     const int te = threadIdx.x - R::EPI_THREAD0;
+    const int r = wq * 32 + lane;  // accumulator lane = token row of the tile
     uint32_t it = 0;
     for (TileWalk t(wc); !t.done(); t.next(), ++it) {
       const int s = it % NSC;
@@ -1692,7 +1695,7 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       if (!ok) break;
       tcgen05_fence_after();
       if (t.seg_last()) mbar_arrive(seg_done);
-      apply_epilogue<D, ROPE>(tmem_base + acc * kAccStride, slots + s * SLOT, den_rows + s * C::G * kTileApply, wq, lane, p.eps, &c_tempty[acc]);
+      apply_epilogue<D, ROPE>(tmem_base, acc, slots, s, den_rows, wq, r, p.eps, c_tempty);
       fence_proxy_async_smem();
       mbar_arrive(&c_staged[s]);
     }
@@ -1752,6 +1755,8 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     tmem_dealloc(tmem_base, kTmemCols);
   }
 }
+
+#include "umma_cluster.cuh"
 
 // ============================================================================ host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1851,6 +1856,94 @@ int launch_kernel(int grid, void** args, cudaStream_t stream) {
   return LINATTN_OK;
 }
 
+// Clusters of c CTAs that are on the device together (0: none).
+template <int D, bool ROPE>
+int clusters_at_once(int c) {
+  using L = ClusterCfg<D, ROPE>;
+  static int cached[64][L::MOST + 1] = {{0}};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cached[dev][c]) {
+    const void* kernel = (const void*)umma_cluster_kernel<D, ROPE>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM) != cudaSuccess) { cudaGetLastError(); return 0; }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {(unsigned)c, 1, 1};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(c); cfg.blockDim = dim3(Roles<ROPE>::THREADS); cfg.dynamicSmemBytes = L::SMEM;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }   // (asked again next time)
+    cached[dev][c] = n > 0 ? n : -1;
+  }
+  return cached[dev][c] > 0 ? cached[dev][c] : 0;
+}
+
+// CTAs of a unit's cluster (0: no clusters): the most that the chip holds at once for all units, where what a cluster saves
+// is more than the SMs it leaves out cost.  These are 28 of 148 with 20, 40 or 60 units (clusters of 6, 3 and 2: 22, 45 and
+// 74 at once), so with n 64-token tiles to a CTA there is an n from which the grid is faster; with rotary factors, whose apply
+// pass streams less per SM, it is larger, with many units too (the grid's reduce grows with them), and heads of 128, whose
+// sums and operand leave two Q slots, lose early.  Read-only step, back to back, clusters against the grid (lone CTAs where
+// they would be taken), us:
+//                        192 tokens   300          600          1200         2400         4680
+//   d = 112,  4 heads    14.8/16.8    14.8/16.8    14.9/16.9    16.9/17.0    19.0/17.2    25.1/19.0
+//            20          14.9/16.9    14.9/17.0    17.0/17.1    19.0/19.2    24.0/23.1    31.7/31.3
+//            40          15.2/18.8    16.9/18.9    19.0/21.1    23.0/25.5    31.3/33.7    49.8/49.8
+//            60          16.4/19.7    18.9/21.0    21.0/24.7    27.2/31.2    41.5/45.0    66.3/64.4
+//   d = 64,  35          14.7/16.8    14.8/17.1    16.9/18.9    19.0/21.0    23.9/23.0    33.3/31.2
+//   d = 128, 18          16.0/17.0    17.2/17.6    19.2/18.8    23.0/19.9    29.6/23.3    41.8/33.2
+//   rotary, 112,  4      16.9/19.0    17.0/19.0    18.1/20.1    20.0/25.2    23.2/26.8    29.3/31.3
+//                20      17.2/19.0    17.7/19.4    19.0/21.1    22.3/24.3    27.5/29.1    38.0/39.6
+//                40      18.9/20.9    19.1/21.2    21.2/25.1    27.2/31.3    39.7/41.5    60.3/58.8
+//                60      18.9/21.2    21.0/23.9    24.9/27.3    33.4/35.7    51.8/51.8    82.5/75.2
+//   rotary, 64,  35      15.8/19.0    17.1/19.4    19.1/21.1    21.1/25.1    27.2/27.9    37.1/39.0
+//   rotary, 128, 18      17.0/20.3    18.9/20.9    21.0/21.2    23.1/25.2    30.3/29.3    43.8/39.6
+// Up to 128 tokens lone CTAs are as fast or faster (14.3 against 14.6, 12.9 against 14.9).  S is as far from 64 bits as the
+// grid's or closer (4680 tokens, 20 heads: 9.0e-8 against 1.20e-7).  The choice depends on the shape alone, as solo_pays does.
+template <int D, bool ROPE>
+int cluster_size(const Problem& p, int U, long long tiles) {
+  if (p.N <= 128) return 0;
+  for (int c = tiles < 8 ? (int)tiles : 8; c >= 2; --c) {
+    if (clusters_at_once<D, ROPE>(c) < U) continue;
+    const int most = ROPE ? (D == 128 ? 4 : c == 2 ? 12 : 13) : D == 128 ? (p.N <= 192 ? 1 : 0) : c <= 3 ? 12 : D == 112 ? 2 : 4;
+    return (tiles + c - 1) / c <= most ? c : 0;
+  }
+  return 0;
+}
+
+template <int D, bool ROPE>
+int launch_cluster(const Problem& p, const UmmaCall& c, int size, int U, void* workspace, cudaStream_t stream) {
+  using C = Cfg<D>;
+  using L = ClusterCfg<D, ROPE>;
+  ClusterParams cp{};
+  cp.H = p.H; cp.HG = (p.H + C::G - 1) / C::G;
+  cp.tiles = (int)((p.N + kTileState - 1) / kTileState);
+  cp.c = size;
+  cp.do_apply = c.q != nullptr; cp.accumulate = c.accumulate ? 1 : 0;
+  cp.state = c.state;
+  cp.state_base = c.state_base ? c.state_base : c.state;
+  // in a launch that applies, only a cache that takes the block needs the sum in memory
+  cp.write_state = !cp.do_apply || (c.accumulate && cp.state_base == cp.state);
+  cp.eps = c.eps;
+  cp.ctrl = static_cast<WorkspaceCtrl*>(workspace);
+  cp.rope = static_cast<const uint4*>(c.rope);
+  cp.N = p.N;
+  CUtensorMap mk, mv, mq, mo;
+  if (!make_map(&mk, p, c.k, C::BOX_D, C::BOX_H, kTileState) || !make_map(&mv, p, c.v, C::BOX_D, C::BOX_H, kTileState)) return LINATTN_ERR_CUDA;
+  mq = mk; mo = mk;   // (never used without queries)
+  if (cp.do_apply && (!make_map(&mq, p, c.q, C::BOX_D, C::BOX_H, kTileState) || !make_map(&mo, p, c.o, C::BOX_D, C::BOX_H, kTileState)))
+    return LINATTN_ERR_CUDA;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)size, 1, 1};
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(size * U); cfg.blockDim = dim3(Roles<ROPE>::THREADS); cfg.dynamicSmemBytes = L::SMEM; cfg.stream = stream;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, umma_cluster_kernel<D, ROPE>, mk, mv, mq, mo, cp) != cudaSuccess) { cudaGetLastError(); return LINATTN_ERR_CUDA; }
+  count_launches(1);
+  return LINATTN_OK;
+}
+
 template <int D, bool ROPE>
 int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStream_t stream) {
   using C = Cfg<D>;
@@ -1860,6 +1953,10 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   FusedParams fp{};
   fp.B = p.B; fp.H = p.H; fp.HG = (p.H + C::G - 1) / C::G;
   const int U = p.B * fp.HG;
+  if (do_state) {
+    const int size = cluster_size<D, ROPE>(p, U, (p.N + kTileState - 1) / kTileState);
+    if (size) return launch_cluster<D, ROPE>(p, c, size, U, workspace, stream);
+  }
   fp.sa = make_sched(U, (p.N + kTileState - 1) / kTileState, sms, 2);
   fp.do_state = do_state; fp.do_apply = do_apply; fp.accumulate = c.accumulate ? 1 : 0;
   fp.state = c.state;
