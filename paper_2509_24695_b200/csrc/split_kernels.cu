@@ -572,7 +572,14 @@ struct ApplyShape : Shape<T, R, ROPE> {
   static constexpr int FLIP = flip_of(B::E, LANES, PIECES);
   static constexpr int SBOX = B::DP * 128, SPART = B::BOXES * SBOX;   // (lanes from DP on read whatever follows and are ignored)
   static constexpr int S_BYTES = 3 * SPART;
-  static constexpr int QBOX = TOK * 128, QPART = B::BOXES * QBOX, STAGE = B::QK_PARTS * QPART;
+  static constexpr int QBOX = TOK * 128, STAGE = B::QK_PARTS * B::BOXES * QBOX;
+  // Three parts of many features: those of a box lie behind one another, so that one MMA takes two of them as 128 columns.  An MMA
+  // costs about as much with 64 columns as with 128, and from d = 97 on their number is what the pass waits for (3750 of 4440 cycles
+  // a tile to issue 42 of them): four a K step instead of six.  32 760 tokens, 20 heads of 112: 187 -> 164 us, forward with
+  // rotary factors 406 -> 393; 18 heads of 128: 179 -> 178.  Smaller heads wait for the draining warps, which read one accumulator more
+  // then (80: 212 -> 210, bf16 with rotary factors 405 -> 412, 64: 220 -> 238, 32: 361 -> 402), and keep six.
+  static constexpr bool STACK = B::QK_PARTS == 3 && R >= 7;
+  static constexpr int QPART = STACK ? QBOX : B::BOXES * QBOX, QBOX_STEP = STACK ? 3 * QBOX : QBOX;
   static constexpr int DEN = (4 * TOK + 128) * 4;
   static constexpr int FIXED = 1024 + S_BYTES + 2 * STAGE + DEN + kBarBytes;
   // a tile's rotations are staged beside its pieces where there is room (not for fp32 at d > 96: loaded where they are used)
@@ -582,15 +589,17 @@ struct ApplyShape : Shape<T, R, ROPE> {
   static constexpr int RAW_STAGES = FIT < 1 ? 1 : FIT > 3 ? 3 : FIT;
   static constexpr int OVERRUN = 128 * 128 - SBOX;            // of the last part's last box, when less than that follows
   static constexpr int SMEM = FIXED + (RAW_STAGES * RAW > OVERRUN ? RAW_STAGES * RAW : OVERRUN);
-  static constexpr int ACC = TOK, SET = (LEAD + 1) * ACC;     // TMEM columns: two sets of accumulators
-  static_assert(2 * SET <= 512, "tensor memory");
+  // TMEM columns: two sets of accumulators.  STACK: two sets of those of the leading products, and one pair for the products of
+  // order one (S0 Q1 + S1 Q0) and two (S0 Q2 + S1 Q1 + S2 Q0).
+  static constexpr int ACC = TOK, SET = (STACK ? LEAD : LEAD + 1) * ACC, REST = 2 * SET;
+  static_assert(2 * SET + (STACK ? 2 * ACC : 0) <= 512, "tensor memory");
   // apply_by_fma's room ends before the barriers and flags, which other threads may still be looking at
   static_assert((B::DP * B::DP + B::DP + 256 * (kBlock + 31) / 32) * 4 <= S_BYTES + 2 * STAGE, "scratch of apply_by_fma");
 };
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
 //
-// Measured as above: 186 us (operand reads of the MMAs, 250 of 350 KB a tile through shared memory), general kernels 866,
+// Measured as above: 164 us (issue of the MMAs, see ApplyShape::STACK), general kernels 866,
 // register-blocked on packed fp32 FMAs 489.  bf16, 28 heads of 80:
 // 152 us (165 with tiles of 64 tokens and every warp in both roles), general kernels 644.
 template <typename T, int R, bool ROPE>
@@ -723,7 +732,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
         }
         if (ROPE) rotate<E>(x, reinterpret_cast<const __half2*>(&tb[i]));
         uint32_t unused = 0;
-        store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX), A::QPART, x, unused);
+        store_parts<A::QK_PARTS>(stage + operand_offset(row, f, A::QBOX_STEP), A::QPART, x, unused);
       }
       __syncwarp();
 #pragma unroll
@@ -743,32 +752,59 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
       tcgen05_fence_after();
       if ((warp & 3) * 32 < d) {
         const uint32_t trow = tmem + (t & 1) * A::SET + ((uint32_t)((warp & 3) * 32) << 16) + tok0;
+        const uint32_t rrow = tmem + A::REST + ((uint32_t)((warp & 3) * 32) << 16) + tok0;
         const float* rden = den + (t & 3) * A::TOK + tok0;
         const long long n0 = (first + t) * A::TOK + tok0;
         const int live = j < d ? (int)min((long long)HALF, p.N - n0) : 0;
         T* out = o + base + n0 * p.sn + j;
-#pragma unroll
-        for (int g = 0; g < HALF / 8; ++g) {
-          constexpr int LEADS = R < A::LEAD ? R : A::LEAD;
-          uint32_t a[A::LEAD + 1][8];
+        constexpr int LEADS = R < A::LEAD ? R : A::LEAD;
+        auto read = [&](int g, float (&num)[8]) {   // numerators of tokens 8 g .. 8 g + 7
+          uint32_t a[A::LEAD + 2][8];
 #pragma unroll
           for (int s = 0; s < LEADS; ++s) tmem_ld_x8(trow + s * A::ACC + 8 * g, a[s]);
-          tmem_ld_x8(trow + A::LEAD * A::ACC + 8 * g, a[A::LEAD]);
+          if (A::STACK) {
+            tmem_ld_x8(rrow + 8 * g, a[A::LEAD]);
+            tmem_ld_x8(rrow + A::ACC + 8 * g, a[A::LEAD + 1]);
+          } else {
+            tmem_ld_x8(trow + A::LEAD * A::ACC + 8 * g, a[A::LEAD]);
+          }
           tmem_ld_wait();
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            num[x] = __uint_as_float(a[0][x]);
+#pragma unroll
+            for (int s = 1; s < LEADS; ++s) num[x] += __uint_as_float(a[s][x]);
+            num[x] += A::STACK ? __uint_as_float(a[A::LEAD + 1][x]) + __uint_as_float(a[A::LEAD][x]) : __uint_as_float(a[A::LEAD][x]);
+          }
+        };
+        auto write = [&](int g, const float (&num)[8]) {
           float wild = 0.f;   // NaN if a numerator is not finite: queries where z is zero, which no denominator sees, have no bounds
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
-            float num = __uint_as_float(a[0][x]);
-#pragma unroll
-            for (int s = 1; s < LEADS; ++s) num += __uint_as_float(a[s][x]);
-            num += __uint_as_float(a[A::LEAD][x]);
             if (8 * g + x < live) {
-              store_value(out, num * rden[8 * g + x]);
-              wild = fmaf(num, 0.f, wild);
+              store_value(out, num[x] * rden[8 * g + x]);
+              wild = fmaf(num[x], 0.f, wild);
             }
             out += p.sn;
           }
           if (wild != 0.f) *odd_flag = 1;
+        };
+        if constexpr (A::STACK) {   // the next tile's MMAs wait for the accumulators: all read, and handed back, before the first is stored
+          float num[HALF / 8][8];
+#pragma unroll
+          for (int g = 0; g < HALF / 8; ++g) read(g, num[g]);
+          tcgen05_fence_before();
+          mbar_arrive(&drained[t & 1]);
+#pragma unroll
+          for (int g = 0; g < HALF / 8; ++g) write(g, num[g]);
+          continue;
+        } else {
+#pragma unroll
+          for (int g = 0; g < HALF / 8; ++g) {
+            float num[8];
+            read(g, num);
+            write(g, num);
+          }
         }
       }
       tcgen05_fence_before();
@@ -776,6 +812,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     }
   } else if (lane == 0) {
     int t = 0;
+    bool issued = false;   // MMAs of a tile that was not completed
     for (; t < tiles; ++t) {
       if (t >= 2 && !mbar_wait(&drained[t & 1], ((t - 2) >> 1) & 1, abort_flag)) break;
       if (!mbar_wait(&ready[t & 1], (t >> 1) & 1, abort_flag)) break;
@@ -783,24 +820,40 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
       const uint64_t a0 = make_smem_desc_sw128(smem_u32(s_op), 16, 1024);   // offsets are added as in the state kernel
       const uint64_t b0 = make_smem_desc_sw128(smem_u32(stages + (t & 1) * A::STAGE), 16, 1024);
       const uint32_t set = tmem + (t & 1) * A::SET;
-      auto mma = [&](int kk, int ps, int pq, uint32_t acc, bool add) {
-        umma_bf16(set + acc * A::ACC, a0 + (ps * A::SPART + (kk >> 2) * A::SBOX + (kk & 3) * 32) / 16,
-                  b0 + (pq * A::QPART + (kk >> 2) * A::QBOX + (kk & 3) * 32) / 16, IDESC, add ? 1u : 0u);
+      auto mma = [&](int kk, int ps, int pq, uint32_t acc, uint32_t idesc, bool add) {
+        umma_bf16(acc, a0 + (ps * A::SPART + (kk >> 2) * A::SBOX + (kk & 3) * 32) / 16,
+                  b0 + (pq * A::QPART + (kk >> 2) * A::QBOX_STEP + (kk & 3) * 32) / 16, idesc, add ? 1u : 0u);
       };
-      bool add = false;
+      if constexpr (A::STACK) {
+        constexpr uint32_t WIDE = make_idesc_bf16(128, 2 * A::TOK, false, false);
 #pragma unroll
-      for (int order = 2; order >= 1; --order)   // smallest first
+        for (int kk = 0; kk < R; ++kk) mma(kk, 0, 0, set + (kk % A::LEAD) * A::ACC, IDESC, kk >= A::LEAD);
+        issued = true;
+        if (t > 0 && !mbar_wait(&drained[(t - 1) & 1], ((t - 1) >> 1) & 1, abort_flag)) break;   // the pair
+        tcgen05_fence_after();
+        const uint32_t rest = tmem + A::REST;
 #pragma unroll
-        for (int pq = order; pq >= 0; --pq) {
-          if (pq >= A::QK_PARTS) continue;
-#pragma unroll
-          for (int kk = 0; kk < R; ++kk) { mma(kk, order - pq, pq, A::LEAD, add); add = true; }
+        for (int kk = 0; kk < R; ++kk) {
+          mma(kk, 0, 1, rest, WIDE, kk > 0);                 // S0 [Q1 | Q2]
+          mma(kk, 1, 0, rest, WIDE, true);                   // S1 [Q0 | Q1]
+          mma(kk, 2, 0, rest + A::ACC, IDESC, true);         // S2 Q0
         }
+      } else {
+        bool add = false;
 #pragma unroll
-      for (int kk = 0; kk < R; ++kk) mma(kk, 0, 0, kk % A::LEAD, kk >= A::LEAD);
+        for (int order = 2; order >= 1; --order)   // smallest first
+#pragma unroll
+          for (int pq = order; pq >= 0; --pq) {
+            if (pq >= A::QK_PARTS) continue;
+#pragma unroll
+            for (int kk = 0; kk < R; ++kk) { mma(kk, order - pq, pq, set + A::LEAD * A::ACC, IDESC, add); add = true; }
+          }
+#pragma unroll
+        for (int kk = 0; kk < R; ++kk) mma(kk, 0, 0, set + (kk % A::LEAD) * A::ACC, IDESC, kk >= A::LEAD);
+      }
       umma_commit(&done[t & 1]);
     }
-    if (t > 0) umma_commit(finished); else mbar_arrive(finished);
+    if (t > 0 || issued) umma_commit(finished); else mbar_arrive(finished);
   }
   if (odd) *odd_flag = 1;
   __syncthreads();
