@@ -164,6 +164,12 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
   const int tr = threadIdx.x - kReluThread0;                       // ReLU role
   const int row0 = tr >> 3, pc = tr & 7, lc = pc ^ (row0 & 7);     // its rows, and the 16-byte chunk it holds of all of them
   const bool box1_live = 64 + lc * 8 < C::FEAT;
+  // z: one thread a feature, in every CTA.  A step writes the new z where the old one is, and the CTAs of a cluster go at their
+  // own pace: the old z is read by the threads that write the new one (rank 0's), and before they send theirs, so that what they
+  // write behind everybody's sums nobody reads.
+  const int zh = hg * C::G + tr / D;
+  const bool z_owned = !L::Z_LANE && rank == 0 && (unsigned)tr < (unsigned)C::FEAT && zh < p.H;   // (a head there is, not padding of the group)
+  auto z_at = [&] { return ((size_t)(b * p.H + hg * C::G + tr / D) * (D + 1) + D) * D + tr % D; };
 
   // ==================================================================== state pass
   if (warp == 0) {
@@ -291,6 +297,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         fence_proxy_async_smem();
       }
     }
+    const float z_old = z_owned && p.accumulate ? __ldcg(p.state_base + z_at()) : 0.f;
     if (!L::Z_LANE && ok) {
       leave_z(z_slots, zacc, tr, lc, box1_live);
       mbar_arrive(z_left);
@@ -298,7 +305,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     }
     cluster_wait();
     if (!L::Z_LANE && ok && tr < 128) {
-      const float z = tr < C::FEAT ? sum_z_slots<ROPE>(z_slots, tr) : 0.f;
+      const float z = z_old + (tr < C::FEAT ? sum_z_slots<ROPE>(z_slots, tr) : 0.f);
       for (int r = 0; r < c; ++r) store_async(cluster_address(z_recv + rank * 128 + tr, r), cluster_address(x_full, r), z);
     }
   } else if (warp < R::STORE_WARP) {
@@ -482,11 +489,6 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         acc[k][1] = __ldcg(reinterpret_cast<const float4*>(p.state_base + at_of[k]) + 1);
       }
     }
-    float z = 0.f;
-    const int zg = ot / D, zh = hg * C::G + zg;   // z: every CTA by itself, one thread a feature
-    const bool z_held = !L::Z_LANE && ot < C::FEAT && zh < p.H;
-    const size_t z_at = ((size_t)(b * p.H + zh) * (D + 1) + D) * D + (ot - zg * D);
-    if (p.accumulate && z_held) z = __ldcg(p.state_base + z_at);
 
     if (__all_sync(0xffffffffu, mbar_wait_cluster(x_full, 0, abort_flag))) {
 #pragma unroll
@@ -512,8 +514,9 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
       }
       if (!L::Z_LANE && ot < C::FEAT) {
-        for (int r = 0; r < c; ++r) z += z_recv[r * 128 + ot];
-        if (rank == 0 && p.write_state && z_held) p.state[z_at] = z;
+        float z = 0.f;
+        for (int r = 0; r < c; ++r) z += z_recv[r * 128 + ot];   // (rank 0's has the old z in it)
+        if (z_owned && p.write_state) p.state[z_at()] = z;
         if (ROPE) z_row[ot] = z;
         else if (p.do_apply) put_z<D>(s_op, ot, z);
       }
