@@ -981,6 +981,7 @@ __device__ __forceinline__ void rope_apply_rows(uint8_t* sl, float* den, int row
     float x = (b1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b1 ? a0 : a1, 2);
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     const int row = row0 + 32 * (pc >> 1);
+    if (D == 112) __syncwarp();   // another lane has turned the padding that this row's goes to, and shuffles do not order its store
     if ((pc & 1) == 0) {
       if (D == 112) *reinterpret_cast<float*>(sl + HALF + row * kRowBytes + ((6 ^ (row & 7)) << 4)) = x;   // features 112..119: padding
       else den[row] = x;   // no padding to carry it
