@@ -39,6 +39,8 @@
 // to the common teardown (TMEM is freed, loads in flight are waited for with a bound).
 #include <cuda.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -1857,30 +1859,31 @@ int launch_kernel(int grid, void** args, cudaStream_t stream) {
   return LINATTN_OK;
 }
 
-// Clusters of c CTAs that are on the device together (0: none).
+// Clusters of c CTAs that are on the device together (0: none), or the error that kept the runtime from saying: a call must not
+// take another form, with other low bits, because this once could not be asked.
 template <int D, bool ROPE>
 int clusters_at_once(int c) {
   using L = ClusterCfg<D, ROPE>;
-  static int cached[64][L::MOST + 1] = {{0}};
+  static std::atomic<int> cached[64][L::MOST + 1];   // by device; one more than the number, 0: not asked yet
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!cached[dev][c]) {
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return LINATTN_ERR_CUDA; }
+  int n = cached[dev][c].load(std::memory_order_relaxed) - 1;
+  if (n < 0) {
     const void* kernel = (const void*)umma_cluster_kernel<D, ROPE>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM) != cudaSuccess) { cudaGetLastError(); return LINATTN_ERR_CUDA; }
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim = {(unsigned)c, 1, 1};
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(c); cfg.blockDim = dim3(Roles<ROPE>::THREADS); cfg.dynamicSmemBytes = L::SMEM;
     cfg.attrs = at; cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }   // (asked again next time)
-    cached[dev][c] = n > 0 ? n : -1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 0) { cudaGetLastError(); return LINATTN_ERR_CUDA; }
+    cached[dev][c].store(n + 1, std::memory_order_relaxed);
   }
-  return cached[dev][c] > 0 ? cached[dev][c] : 0;
+  return n;
 }
 
-// CTAs of a unit's cluster (0: no clusters): the most that the chip holds at once for all units, where what a cluster saves
+// CTAs of a unit's cluster (0: no clusters; or an error): the most that the chip holds at once for all units, where what a cluster saves
 // is more than the SMs it leaves out cost.  These are 28 of 148 with 20, 40 or 60 units (clusters of 6, 3 and 2: 22, 45 and
 // 74 at once), so with n 64-token tiles to a CTA there is an n from which the grid is faster; with rotary factors, whose apply
 // pass streams less per SM, it is larger, with many units too (the grid's reduce grows with them), and heads of 128, whose
@@ -1900,12 +1903,15 @@ int clusters_at_once(int c) {
 //   rotary, 64,  35      15.8/19.0    17.1/19.4    19.1/21.1    21.1/25.1    27.2/27.9    37.1/39.0
 //   rotary, 128, 18      17.0/20.3    18.9/20.9    21.0/21.2    23.1/25.2    30.3/29.3    43.8/39.6
 // Up to 128 tokens lone CTAs are as fast or faster (14.3 against 14.6, 12.9 against 14.9).  S is as far from 64 bits as the
-// grid's or closer (4680 tokens, 20 heads: 9.0e-8 against 1.20e-7).  The choice depends on the shape alone, as solo_pays does.
+// grid's or closer (4680 tokens, 20 heads: 9.0e-8 against 1.20e-7).  The choice depends on the shape and on the device (how its SMs
+// are spread over GPCs), as the grid's split depends on its SM count: all calls on one shape give the same bits on one GPU.
 template <int D, bool ROPE>
 int cluster_size(const Problem& p, int U, long long tiles) {
   if (p.N <= 128) return 0;
   for (int c = tiles < 8 ? (int)tiles : 8; c >= 2; --c) {
-    if (clusters_at_once<D, ROPE>(c) < U) continue;
+    const int at_once = clusters_at_once<D, ROPE>(c);
+    if (at_once < 0) return at_once;
+    if (at_once < U) continue;
     const int most = ROPE ? (D == 128 ? 4 : c == 2 ? 12 : 13) : D == 128 ? (p.N <= 192 ? 1 : 0) : c <= 3 ? 12 : D == 112 ? 2 : 4;
     return (tiles + c - 1) / c <= most ? c : 0;
   }
@@ -1956,6 +1962,7 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   const int U = p.B * fp.HG;
   if (do_state) {
     const int size = cluster_size<D, ROPE>(p, U, (p.N + kTileState - 1) / kTileState);
+    if (size < 0) return size;
     if (size) return launch_cluster<D, ROPE>(p, c, size, U, workspace, stream);
   }
   fp.sa = make_sched(U, (p.N + kTileState - 1) / kTileState, sms, 2);
