@@ -207,8 +207,12 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
       for (; it < n; ++it) {
         const int s = it % NSA, set = it & 1;
         // Plain: two accumulators collect a tile's four K steps while the other two are read, so no chain of the tensor
-        // core's truncating additions is longer than two (a lone tile has all four: one).  Rotary: the keys are rounded to
-        // bf16 behind their rotation, which leaves 2^-9 in S; the tiles go to the four accumulators in turn and are read once.
+        // core's truncating additions is longer than two (a lone tile has all four: one).  Rotary: the accumulators are read
+        // once, behind the last tile; each takes one K step of every tile, so a chain is as long as the CTA has tiles.  (Whole
+        // tiles in turn made chains of four times a quarter of that, rounded up.  2-norm of S against 64 bits with factors that
+        // turn nothing, whole tiles / K steps / the forms without clusters: 192 tokens, 3 heads of 64 5.54e-8 / 4.72e-8 / 4.72e-8;
+        // 1200 tokens, 4 heads of 112 7.71e-8 / 7.38e-8 / 9.03e-8; 4680 tokens, 20 heads 1.305e-7 / 1.303e-7 / 1.209e-7.  Turned
+        // keys are rounded to bf16: 1.6e-3 in all of them.)
         if (!ROPE && it >= 2 && !mbar_wait(&a_tempty[set], ((it - 2) >> 1) & 1, abort_flag)) break;
         if (!mbar_wait(&a_ready[s], (it / NSA) & 1, abort_flag)) break;
         tcgen05_fence_after();
@@ -217,8 +221,8 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         for (int kk = 0; kk < kTileState / 16; ++kk) {
           const uint64_t kd = make_smem_desc_sw128(st + KOFF + kk * 2048, kBox, 1024);   // phi(K), MN-major
           const uint64_t vd = make_smem_desc_sw128(st + kk * 2048, kBox, 1024);          // V^T, MN-major
-          const int acc = ROPE ? it & 3 : n == 1 ? kk : 2 * set + (kk & 1);
-          const bool first = ROPE ? it < 4 && kk == 0 : n == 1 || kk < 2;
+          const int acc = ROPE || n == 1 ? kk : 2 * set + (kk & 1);
+          const bool first = ROPE ? it == 0 : n == 1 || kk < 2;
           umma_bf16(tmem_base + acc * 128, vd, kd, IDESC_A, first ? 0u : 1u);
         }
         umma_commit(&a_empty[s]);
@@ -399,16 +403,13 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 #pragma unroll 1
         for (int cc = 0; cc < D / 16; ++cc) {
           float v[16];
-          const int accs = n < 4 ? n : 4;
+          uint32_t r[4][16];
 #pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            if (a >= accs) break;
-            uint32_t r[16];
-            tmem_ld_x16(trow + a * 128 + cc * 16, r);
-            tmem_ld_wait();
+          for (int a = 0; a < 4; ++a) tmem_ld_x16(trow + a * 128 + cc * 16, r[a]);
+          tmem_ld_wait();
 #pragma unroll
-            for (int x = 0; x < 16; ++x) v[x] = a == 0 ? __uint_as_float(r[x]) : v[x] + __uint_as_float(r[x]);
-          }
+          for (int x = 0; x < 16; ++x)
+            v[x] = ((__uint_as_float(r[0][x]) + __uint_as_float(r[1][x])) + __uint_as_float(r[2][x])) + __uint_as_float(r[3][x]);
           if (j < L::ROWS) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) put(cc * 4 + k, make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]));
