@@ -1903,16 +1903,52 @@ int clusters_at_once(int c) {
 //   rotary, 64,  35      15.8/19.0    17.1/19.4    19.1/21.1    21.1/25.1    27.2/27.9    37.1/39.0
 //   rotary, 128, 18      17.0/20.3    18.9/20.9    21.0/21.2    23.1/25.2    30.3/29.3    43.8/39.6
 // Up to 128 tokens lone CTAs are as fast or faster (14.3 against 14.6, 12.9 against 14.9).  S is as far from 64 bits as the
-// grid's or closer (4680 tokens, 20 heads: 9.0e-8 against 1.20e-7).  The choice depends on the shape and on the device (how its SMs
+// grid's or closer (4680 tokens, 20 heads: 9.0e-8 against 1.20e-7; rotary: see the kernel's MMA issuer).  The choice depends on the shape and on the device (how its SMs
 // are spread over GPCs), as the grid's split depends on its SM count: all calls on one shape give the same bits on one GPU.
+//
+// The fewer SMs the clusters take, the earlier the grid, which takes them all, is ahead: below two thirds of them from nine 64-token
+// tiles to a CTA on (heads of 112), below three quarters from thirteen.  Few units put that off, since a unit's reduce in the grid
+// adds up the records of 148 / units CTAs.  Packed heads, whose grid form is slower, lose at thirteen tiles with 3 to 9 units and
+// rotary factors, and at twelve without and below two thirds.  Read-only step and state alone, from CUDA graphs, clusters against the
+// grid, us:
+//   rotary, 112,  4 units, 12 tiles of 8 CTAs   31.9/32.2  18.5/21.7   13 tiles   34.0/32.9  19.2/21.8
+//                 6        10                   29.3/30.0  17.3/19.7   11         31.3/30.4  18.0/20.5
+//                 8         8                   26.3/26.3  16.0/17.2    9         28.7/27.1  16.7/17.7    13  34.6/30.2  19.6/19.0
+//                12         8                   27.5/28.2  16.8/17.6    9         29.8/28.8  17.4/17.9    12  33.9/32.6  19.6/19.2
+//                16         8         6 CTAs    27.6/27.6  17.1/17.1    9         29.9/28.2  17.7/17.3    13  36.0/34.9  20.2/19.4
+//                18        12         6 CTAs    34.4/34.5  19.9/19.4   13         37.1/35.6  20.7/20.1
+//                26        13         5 CTAs    37.9/39.7  21.0/22.7
+//                33        13         4 CTAs    39.0/40.9  21.5/21.3
+//                35        12         3 CTAs    34.1/33.8  19.7/18.6   13         36.2/34.3  20.6/19.2
+//                46         8         2 CTAs    27.3/27.3  17.7/16.7    9         29.7/27.8  18.4/16.9    12  34.1/31.9  20.5/18.3
+//                50        12         2 CTAs    34.9/38.6  20.8/21.7
+//   d = 112,     46         8         2 CTAs    22.5/22.8  14.8/14.3    9         24.2/23.4  15.5/14.3    12  27.5/26.6  17.5/15.5
+//   rotary, 64,   8        12         8 CTAs    31.0/30.8  15.9/18.5   13         33.4/31.1  16.5/18.8
+//   d = 64,      46        11         2 CTAs    27.3/27.6  16.0/15.0   12         28.8/28.2  16.5/15.1
+//   d = 32,      33         4         4 CTAs    18.3/20.9  10.4/11.9
+//   rotary, 32,  22        13         6 CTAs    36.2/42.4  16.7/21.2
+//   d = 128,     18         1         3 CTAs    13.8/15.7  10.8/10.7
+//   rotary, 128, 18         4         6 CTAs    22.9/25.4  15.6/16.0
+//                26         1         5 CTAs    18.7/20.0  12.8/12.1
+// States alone lose 3 to 6 % on clusters with 27 to 29 and 34 to 37 units of ten to twelve tiles, with 46 to 49 units from six
+// on, and with heads of 128 (129 to 192 tokens; with rotary factors, five CTAs), where the steps are level or gain: one form for all calls.
+// Not taken though clusters would be 7 % ahead: thirteen tiles and more of plain heads of 112 with 38 to 45 and 50 to 74 units; heads
+// of 128 of 193 to 300 tokens (3 %).
 template <int D, bool ROPE>
-int cluster_size(const Problem& p, int U, long long tiles) {
+int cluster_size(const Problem& p, int U, long long tiles, int sms) {
   if (p.N <= 128) return 0;
   for (int c = tiles < 8 ? (int)tiles : 8; c >= 2; --c) {
     const int at_once = clusters_at_once<D, ROPE>(c);
     if (at_once < 0) return at_once;
     if (at_once < U) continue;
-    const int most = ROPE ? (D == 128 ? 4 : c == 2 ? 12 : 13) : D == 128 ? (p.N <= 192 ? 1 : 0) : c <= 3 ? 12 : D == 112 ? 2 : 4;
+    int most = ROPE ? (D == 128 ? 4 : c == 2 ? 12 : 13) : D == 128 ? (p.N <= 192 ? 1 : 0) : c <= 3 ? 12 : D == 112 ? 2 : 4;
+    const int used = U * c;   // SMs
+    int few = most;
+    if (D == 112 && 3 * used < 2 * sms) few = U <= 2 ? 13 : U <= 4 ? 12 : U <= 6 ? 10 : 8;
+    else if (D == 112 && 4 * used <= 3 * sms) few = 12;
+    else if (D <= 64 && ROPE && 2 * used < sms) few = U <= 2 ? 13 : 12;
+    else if (D <= 64 && !ROPE && 3 * used < 2 * sms) few = 11;
+    if (few < most) most = few;
     return (tiles + c - 1) / c <= most ? c : 0;
   }
   return 0;
@@ -1961,7 +1997,7 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   fp.B = p.B; fp.H = p.H; fp.HG = (p.H + C::G - 1) / C::G;
   const int U = p.B * fp.HG;
   if (do_state) {
-    const int size = cluster_size<D, ROPE>(p, U, (p.N + kTileState - 1) / kTileState);
+    const int size = cluster_size<D, ROPE>(p, U, (p.N + kTileState - 1) / kTileState, sms);
     if (size < 0) return size;
     if (size) return launch_cluster<D, ROPE>(p, c, size, U, workspace, stream);
   }
