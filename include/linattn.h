@@ -198,6 +198,11 @@ LINATTN_API int linattn_forward_host(const linattn_desc* desc, int64_t N, const 
 /* Number of CUDA kernels this library has launched in this process so far (all entry points). */
 LINATTN_API uint64_t linattn_kernel_launches(void);
 
+/* Which form the tensor-core kernels take for N tokens of this shape on the current device, for tests and profiles: *ctas = the
+ * CTAs of the thread-block cluster that takes a (batch entry, head group); 0: a lone CTA or the whole grid does, or the
+ * shape is not theirs. */
+LINATTN_API int linattn_cluster_ctas(const linattn_desc* desc, int64_t N, int rope, int* ctas);
+
 /* ---- block-causal form with the constant-memory cache (Eq. 3, Algorithm 1) ---- */
 
 typedef struct blocklin_cache blocklin_cache; /* opaque HOST handle */

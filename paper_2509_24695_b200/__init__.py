@@ -19,7 +19,7 @@ import struct
 
 __all__ = [
     "LinAttnError", "library_path", "load_library", "state_bytes", "workspace_bytes", "new_workspace",
-    "linattn_forward", "linattn_forward_rope", "rope_pack", "new_rope_workspace", "linattn_state", "linattn_apply", "linattn_state_static_scratch", "static_scratch_status", "split_state", "BlockLinCache", "workspace_status", "HostForward", "kernel_launches",
+    "linattn_forward", "linattn_forward_rope", "rope_pack", "new_rope_workspace", "linattn_state", "linattn_apply", "linattn_state_static_scratch", "static_scratch_status", "split_state", "BlockLinCache", "workspace_status", "HostForward", "kernel_launches", "cluster_ctas",
     "tconv_forward", "TConvCache",
 ]
 
@@ -98,6 +98,7 @@ def load_library(path: str | None = None):
         "linattn_forward_host_bytes": ([dp, i64, szp], ctypes.c_int),
         "linattn_forward_host": ([dp, i64, vp, vp, vp, vp, f32, vp, sz, vp], ctypes.c_int),
         "linattn_kernel_launches": ([], ctypes.c_uint64),
+        "linattn_cluster_ctas": ([dp, i64, ctypes.c_int, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
         "blocklin_cache_bytes": ([dp, i64, szp, szp], ctypes.c_int),
         "blocklin_cache_init": ([ctypes.POINTER(vp), dp, f32, vp, sz, vp, sz, vp], ctypes.c_int),
         "blocklin_cache_reset": ([vp, vp], ctypes.c_int),
@@ -281,6 +282,15 @@ def linattn_forward_rope(q, k, v, rope_table, eps: float = 1e-6, out=None, works
 def kernel_launches() -> int:
     """CUDA kernels launched by the library in this process so far."""
     return int(load_library().linattn_kernel_launches())
+
+
+def cluster_ctas(B: int, H: int, d: int, N: int, rope: bool = False) -> int:
+    """CTAs of the thread-block cluster that takes a (batch entry, head group) of a bf16 call on N tokens on the current
+    device; 0: a lone CTA or the whole grid does."""
+    n = ctypes.c_int()
+    desc = _Desc(B, H, d, LINATTN_BF16, 0, 0, 0)
+    _check(load_library().linattn_cluster_ctas(ctypes.byref(desc), N, int(rope), ctypes.byref(n)), "linattn_cluster_ctas")
+    return n.value
 
 
 class HostForward:

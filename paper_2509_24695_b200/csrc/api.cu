@@ -372,6 +372,19 @@ int linattn_forward_rope(const linattn_desc* desc, int64_t N, const void* q, con
 
 uint64_t linattn_kernel_launches(void) { return g_kernel_launches.load(std::memory_order_relaxed); }
 
+int linattn_cluster_ctas(const linattn_desc* desc, int64_t N, int rope, int* ctas) {
+  Problem p;
+  if (!ctas) return LINATTN_ERR_INVALID_ARG;
+  int st = resolve(desc, N, &p);
+  if (st != LINATTN_OK) return st;
+  *ctas = 0;
+  if (!(rope ? umma_rope_supported(p) : umma_supported(p))) return LINATTN_OK;
+  st = umma_cluster_ctas(p, rope != 0);
+  if (st < 0) return st;
+  *ctas = st;
+  return LINATTN_OK;
+}
+
 int linattn_forward_host_bytes(const linattn_desc* desc, int64_t N, size_t* bytes) {
   Problem p;
   if (!bytes) return LINATTN_ERR_INVALID_ARG;

@@ -83,6 +83,8 @@ struct UmmaCall {
 bool umma_supported(const Problem& p);
 size_t umma_partial_bytes(const Problem& p, bool rope = false);
 bool umma_rope_supported(const Problem& p);
+// CTAs of the cluster that takes a unit of this shape (0: a lone CTA or the grid), or an error status.
+int umma_cluster_ctas(const Problem& p, bool rope);
 // Returns LINATTN_OK or an error status.
 int umma_run(const Problem& p, const UmmaCall& call, void* workspace, cudaStream_t stream);
 

@@ -2077,6 +2077,23 @@ size_t umma_partial_bytes(const Problem& p, bool rope) {
 // rotation table, since box 1 starts a new head.  Everything else takes the fp32-accurate kernels.
 bool umma_rope_supported(const Problem& p) { return umma_supported(p); }
 
+template <int D, bool ROPE>
+int cluster_ctas(const Problem& p) {
+  const int sms = sm_count();
+  if (!sms) return LINATTN_ERR_CUDA;
+  return cluster_size<D, ROPE>(p, p.B * ((p.H + Cfg<D>::G - 1) / Cfg<D>::G), (p.N + kTileState - 1) / kTileState, sms);
+}
+
+int umma_cluster_ctas(const Problem& p, bool rope) {
+  switch (p.d) {
+    case 32: return rope ? cluster_ctas<32, true>(p) : cluster_ctas<32, false>(p);
+    case 64: return rope ? cluster_ctas<64, true>(p) : cluster_ctas<64, false>(p);
+    case 112: return rope ? cluster_ctas<112, true>(p) : cluster_ctas<112, false>(p);
+    case 128: return rope ? cluster_ctas<128, true>(p) : cluster_ctas<128, false>(p);
+  }
+  return 0;
+}
+
 int umma_run(const Problem& p, const UmmaCall& c, void* workspace, cudaStream_t stream) {
   if (p.N == 0 || (!c.k && !c.q)) return LINATTN_OK;
   switch (p.d) {

@@ -1,6 +1,7 @@
 """Blocks whose units are taken by thread-block clusters: token counts that split evenly and unevenly over the CTAs, CTAs of
-one 64-token tile and of several (an odd number leaves half an apply tile), clusters of two to eight, head counts that leave a
-packed group partly empty, all modes on one shape with the same bits."""
+one 64-token tile and of several (an odd number leaves half an apply tile; enough of them that stages, accumulators and slots come
+round again), clusters of two to eight, head counts that leave a packed group partly empty, all modes on one shape with the same
+bits; and shapes just behind the line, which the grid takes."""
 import numpy as np
 import pytest
 
@@ -10,8 +11,11 @@ from parity_util import assert_parity_bf16, assert_state_close, to_dev, to_f64
 pytestmark = pytest.mark.gpu
 
 EPS = 1e-6
-SHAPES = [(1, 65, 2, 112), (1, 193, 3, 112), (1, 577, 2, 112), (1, 1025, 5, 112), (2, 700, 10, 112), (2, 130, 37, 112), (1, 2100, 33, 112),
-          (1, 260, 3, 128), (1, 1500, 18, 128), (2, 333, 5, 64), (1, 2000, 35, 64), (1, 257, 6, 32), (2, 900, 70, 32)]
+BOTH = [(1, 193, 3, 112), (1, 577, 2, 112), (2, 700, 10, 112), (2, 130, 37, 112), (1, 600, 26, 112), (1, 500, 33, 112), (1, 2000, 40, 112),
+        (1, 1150, 45, 112), (1, 1536, 60, 112), (1, 150, 18, 128), (2, 192, 22, 128), (2, 333, 5, 64), (1, 2000, 80, 64), (1, 257, 6, 32), (2, 900, 70, 32)]
+ROPE_ALONE = [(1, 1025, 5, 112), (1, 2100, 33, 112), (1, 260, 3, 128), (1, 1500, 18, 128), (1, 2000, 35, 64)]   # plain: the grid
+CASES = [(rope, shape, True) for shape in BOTH for rope in (False, True)]
+CASES += [(rope, shape, rope) for shape in ROPE_ALONE for rope in (False, True)] + [(True, (1, 5000, 7, 112), False), (True, (1, 2500, 34, 112), False)]
 
 
 @pytest.fixture(scope="module")
@@ -29,12 +33,12 @@ def gen(B, N, H, d, seed):
     return tuple(synth.gauss((B, N, H, d), seed, t) for t in (1, 2, 3))
 
 
-@pytest.mark.parametrize("rope", [False, True])
-@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "B%d_N%d_H%d_d%d" % s)
-def test_all_modes(la, orc, shape, rope):
+@pytest.mark.parametrize("rope,shape,clusters", CASES, ids=["%sB%d_N%d_H%d_d%d" % ("rope_" if c[0] else "", *c[1]) for c in CASES])
+def test_all_modes(la, orc, shape, rope, clusters):
     import torch
 
     B, N, H, d = shape
+    assert (la.cluster_ctas(B, H, d, N, rope) >= 2) == clusters
     qn, kn, vn = gen(B, N, H, d, 8300 + N + d)
     q, k, v = (to_dev(x) for x in (qn, kn, vn))
     k0, v0 = gen(B, 40, H, d, 8400 + N + d)[1:]

@@ -1,6 +1,6 @@
 """Small problems, where one CTA takes a whole unit: token counts around the 64-token stages, the 128-token tiles and the
 line behind which the whole grid takes the work, every tensor-core head dim, head counts that leave a packed group partly
-empty, all modes on one shape with the same bits."""
+empty, all modes on one shape with the same bits.  (From 129 tokens on lone CTAs have the calls of too many units for clusters.)"""
 import numpy as np
 import pytest
 
@@ -29,7 +29,8 @@ def gen(B, N, H, d, seed):
 
 @pytest.mark.parametrize("shape", [(1, 64, 3, 112), (2, 65, 2, 112), (1, 129, 3, 112), (1, 384, 2, 112), (1, 385, 2, 112),
                                    (1, 512, 50, 112), (1, 513, 50, 112), (1, 1, 2, 128), (2, 127, 3, 128), (1, 384, 2, 128),
-                                   (1, 63, 3, 64), (2, 300, 5, 64), (1, 128, 5, 32), (2, 383, 6, 32)],
+                                   (1, 63, 3, 64), (2, 300, 5, 64), (1, 128, 5, 32), (2, 383, 6, 32), (1, 129, 149, 64), (2, 192, 150, 32),
+                                   (1, 192, 101, 112)],
                          ids=lambda s: "B%d_N%d_H%d_d%d" % s)
 def test_all_modes(la, orc, shape):
     import torch
@@ -73,7 +74,8 @@ def test_all_modes(la, orc, shape):
 
 
 @pytest.mark.parametrize("rope", [False, True])
-@pytest.mark.parametrize("shape", [(1, 65, 3, 112), (1, 128, 2, 112), (1, 128, 2, 128), (1, 192, 3, 64), (2, 192, 6, 32), (1, 192, 101, 112)],
+@pytest.mark.parametrize("shape", [(1, 65, 3, 112), (1, 128, 2, 112), (1, 128, 2, 128), (1, 192, 3, 64), (2, 192, 6, 32), (1, 192, 101, 112),
+                                   (1, 192, 150, 64), (1, 192, 296, 64), (2, 180, 151, 32)],
                          ids=lambda s: "B%d_N%d_H%d_d%d" % s)
 def test_tiles_are_added_round_to_nearest(la, shape, rope):
     """The tensor core truncates when it adds into an accumulator.  Four steps of sixteen tokens leave 2^24 each; what the later
@@ -105,8 +107,15 @@ def test_tiles_are_added_round_to_nearest(la, shape, rope):
     assert (cache.state[:, :, :d] == float(again)).all() and (cache.state[:, :, d] == 2 * N).all()
 
 
+@pytest.mark.parametrize("N,units,d", [(129, 75, 64), (192, 148, 64), (129, 75, 32), (192, 148, 32), (192, 101, 112), (192, 148, 128), (128, 1, 112)])
+@pytest.mark.parametrize("rope", [False, True])
+def test_no_cluster_takes_these(la, N, units, d, rope):
+    """What the shapes of many units are there for: that many clusters do not fit on the GPU at once."""
+    assert la.cluster_ctas(1, units * {32: 4, 64: 2}.get(d, 1), d, N, rope) == 0
+
+
 @pytest.mark.parametrize("shape", [(1, 63, 3, 64), (2, 128, 2, 112), (1, 129, 3, 112), (1, 192, 5, 64), (1, 193, 5, 64), (2, 191, 6, 32), (1, 128, 2, 128),
-                                   (1, 192, 100, 112)], ids=lambda s: "B%d_N%d_H%d_d%d" % s)
+                                   (1, 192, 100, 112), (1, 192, 150, 64), (2, 130, 151, 32)], ids=lambda s: "B%d_N%d_H%d_d%d" % s)
 def test_rotary_sums_in_the_cache(la, shape):
     """What rotary steps leave in the cache: z, of the plain keys, as exact as without rotary factors; S, of turned keys rounded
     to bf16 (2^-9 each, so 2^-9 of the sums' random part: its 2-norm)."""
