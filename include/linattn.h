@@ -46,9 +46,12 @@
  *    writes nothing).  Nothing here throws, aborts or traps the device.
  *    Device-side waits on barriers, of a CTA and of the fused kernels' grid, give
  *    up after about a second and record LINATTN_ERR_TIMEOUT in the workspace,
- *    readable with linattn_workspace_status.  (The CTAs of a thread-block cluster,
- *    fp32 and the other head dims, and the allocation of tensor memory wait
- *    without a limit, on CTAs whose own waits have one.)
+ *    readable with linattn_workspace_status.  (The barrier of a thread-block
+ *    cluster, in either path, and the allocation of tensor memory wait without a
+ *    limit, on CTAs whose own waits have one.)
+ *  - Where calls are said to give the same bits, that is on one GPU: how a call
+ *    is split depends on the number of its SMs and on how many thread-block
+ *    clusters it holds at once.
  *  - Calls that share a workspace (or a cache) must be ordered on one stream:
  *    two of them in flight at once race on the split-N partials.
  */
@@ -296,10 +299,10 @@ LINATTN_API int blocklin_cache_info(const blocklin_cache* cache, int64_t* blocks
                         size_t* state_bytes);
 
 /* Device-side status of the stream's launches so far.  Launches are asynchronous, so a bounded device-side wait
- * that ran out (Sec. 3.2's step is one cooperative launch with two grid-wide meetings) cannot be reported by the
- * call that enqueued it: this call synchronises `stream` and reports LINATTN_OK or LINATTN_ERR_TIMEOUT through
- * *status.  After a timeout the outputs of that launch are undefined and the workspace's barrier word is left
- * half-counted, so every later launch on this cache would time out as well: call blocklin_cache_reset (or restore
+ * that ran out (Sec. 3.2's step is one launch whose CTAs wait for one another, grid-wide or in clusters) cannot be
+ * reported by the call that enqueued it: this call synchronises `stream` and reports LINATTN_OK or LINATTN_ERR_TIMEOUT through
+ * *status.  After a timeout the outputs of that launch are undefined and the workspace's barrier word may be left
+ * half-counted, so that every later launch on this cache would time out as well: call blocklin_cache_reset (or restore
  * a checkpoint of the state and call linattn_workspace_init on the workspace) before going on. */
 LINATTN_API int blocklin_cache_status(const blocklin_cache* cache, void* stream, int* status);
 

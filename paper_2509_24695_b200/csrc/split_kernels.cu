@@ -574,10 +574,11 @@ struct ApplyShape : Shape<T, R, ROPE> {
   static constexpr int S_BYTES = 3 * SPART;
   static constexpr int QBOX = TOK * 128, STAGE = B::QK_PARTS * B::BOXES * QBOX;
   // Three parts of many features: those of a box lie behind one another, so that one MMA takes two of them as 128 columns.  An MMA
-  // costs about as much with 64 columns as with 128, and from d = 97 on their number is what the pass waits for (3750 of 4440 cycles
-  // a tile to issue 42 of them): four a K step instead of six.  32 760 tokens, 20 heads of 112: 187 -> 164 us, forward with
-  // rotary factors 406 -> 393; 18 heads of 128: 179 -> 178.  Smaller heads wait for the draining warps, which read one accumulator more
-  // then (80: 212 -> 210, bf16 with rotary factors 405 -> 412, 64: 220 -> 238, 32: 361 -> 402), and keep six.
+  // costs about as much with 64 columns as with 128 (87 to 89 cycles here beside the preparing warps, 65 by itself), and from d = 97 on
+  // their number was what the pass waited for (3750 of 4440 cycles a tile to issue 42 of them): four a K step instead of six.
+  // 32 760 tokens, apply pass (range of nine runs): 20 heads of 112 187 (186..198) -> 163 us (161..165), 22 of 100 226 -> 208,
+  // 18 of 128 176 (175..183) -> 160 (158..165); 4680 tokens 41.6 -> 37.5 and 39.5 -> 37.5.  Smaller heads wait for the draining warps, which
+  // read one accumulator more then (80: 212 -> 210, bf16 with rotary factors 405 -> 412, 64: 220 -> 238, 32: 361 -> 402), and keep six.
   static constexpr bool STACK = B::QK_PARTS == 3 && R >= 7;
   static constexpr int QPART = STACK ? QBOX : B::BOXES * QBOX, QBOX_STEP = STACK ? 3 * QBOX : QBOX;
   static constexpr int DEN = (4 * TOK + 128) * 4;
@@ -599,8 +600,10 @@ struct ApplyShape : Shape<T, R, ROPE> {
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
 //
-// Measured as above: 164 us (issue of the MMAs, see ApplyShape::STACK), general kernels 866,
-// register-blocked on packed fp32 FMAs 489.  bf16, 28 heads of 80:
+// Measured as above: 163 us, general kernels 866, register-blocked on packed fp32 FMAs 489.  Stamps, cycles of a 64-token tile's
+// 3830: the accumulators of order one and two are there once, so a tile's 21 MMAs on them follow the reading of the last tile's:
+// read 840, issued 1590, complete 1030 later, 3460 in a chain; beside it the seven leading MMAs (840), the draining warps' stores (2340 of
+// their 3180) and the preparing warps (3380).  d = 128: 4520, of which the MMA warp issues for 3240.  bf16, 28 heads of 80:
 // 152 us (165 with tiles of 64 tokens and every warp in both roles), general kernels 644.
 template <typename T, int R, bool ROPE>
 __global__ void __launch_bounds__(kBlock, 1)

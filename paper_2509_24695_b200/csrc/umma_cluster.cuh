@@ -12,8 +12,8 @@
 // two such barriers take the place of the two grid barriers.  (Stores of 16 bytes a lane: 2300 cycles for the sums, 6200 for the
 // operand; behind a fence of the cluster they took longer still.)
 //
-// A cluster has to fit into one GPC, so only 120 to 135 of the 148 SMs take part, and with many tokens the grid, which uses
-// them all, is faster: cluster_size draws the line.
+// A cluster has to fit into one GPC, so 148 SMs hold 15 to 74 clusters of eight to two CTAs, and with many tokens the grid, which
+// uses all SMs, is faster: cluster_size draws the line.
 
 // Addresses below are bytes behind the 1024-byte aligned start of shared memory.
 template <int D, bool ROPE>

@@ -1827,9 +1827,9 @@ int sm_count() {
 //   d = 64, 35          8.3/16.2 9.0/16.4 6.4/10.5 10.8/15.5 11.6/15.5 8.7/9.5  13.6/15.7 14.5/15.7 10.8/9.4 16.1/16.3 16.9/16.2 12.9/9.6
 //   d = 32, 1           7.5/13.1 7.9/12.6 5.5/8.0  9.9/12.6 10.2/13.3 7.3/7.7   12.3/13.0 12.7/13.1 9.0/7.7  14.0/13.0 14.5/12.9 10.6/7.7
 // with rotary factors alike at d = 112 and 128 and twice as fast as the grid at d = 32 and 64.  So: up to 128 tokens, and up to 192
-// with packed heads or many units.  (States alone of 129 to 192 tokens with packed heads lose 1 us by that.)  The choice depends
-// on the shape alone, so that all calls on one shape (forward, state and apply, step, peek, the token-sharded three) add up in
-// the same order and give the same bits.
+// with packed heads or many units where these are too many for clusters, which are asked for first (cluster_size).  (States alone of
+// 129 to 192 tokens with packed heads lose 1 us by that.)  The choice depends on the shape and the device, not on the call, so that all
+// calls on one shape (forward, state and apply, step, peek, the token-sharded three) add up in the same order and give the same bits.
 inline bool solo_pays(const Problem& p, int U, int sms) {
   return U <= sms && (p.N <= 128 || (p.N <= 192 && (p.d <= 64 || 3 * U >= 2 * sms)));
 }
