@@ -327,6 +327,8 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   // padded features are never written and must read as zero
   for (int i = tid; i < 2 * S::STAGE / 16; i += kBlock) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
   if (warp == 0) { tmem_alloc(tmem_holder, S::COLS); tmem_relinquish(); }
+  let_next_grid_start();
+  wait_for_prior_grids();
 
   // preparing: this thread's row of every tile, and its pieces of it, features feature(0), feature(1), ...
   const int row = (tid % kPrepare) / S::LANES, l = tid % S::LANES;
@@ -655,10 +657,6 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     }
     copy_commit();
   };
-  if (preparing) {
-#pragma unroll
-    for (int t = 0; t < A::RAW_STAGES; ++t) issue(t);
-  }
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
     mbar_init(finished, 1);
@@ -669,14 +667,21 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   // padded features of both operands read as zero
   if (d < A::DP)
     for (int i = tid; i < (A::S_BYTES + 2 * A::STAGE) / 16; i += kBlock) reinterpret_cast<uint4*>(s_op)[i] = make_uint4(0, 0, 0, 0);
-  if (tid < 128) zs[tid] = tid < d ? W[(long long)d * d + tid] : 0.f;
+  let_next_grid_start();
+  wait_for_prior_grids();
+  W = behind_wait(W);
+  if (preparing) {
+#pragma unroll
+    for (int t = 0; t < A::RAW_STAGES; ++t) issue(t);
+  }
+  if (tid < 128) zs[tid] = tid < d ? __ldcg(W + (long long)d * d + tid) : 0.f;
   __syncthreads();
   uint32_t least = 0xFFFFFFFFu;   // twice the bits of the smallest |S| 2^38, less one (zero is the largest)
   float rest = 0.f;               // NaN if one is not finite
   for (int idx = tid; idx < d * (d / 4); idx += kBlock) {
     const int j = idx / (d / 4), i = (idx - j * (d / 4)) * 4;
     float x[4];
-    widen(__ldg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
+    widen(__ldcg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const float y = x[e] * 0x1p38f;
@@ -952,13 +957,14 @@ cudaError_t launch_state(const Problem& p, const void* k, const void* v, const f
     const double now = (double)((p.units() + at_once - 1) / at_once) * ((double)((tiles + c - 1) / c) + 6.0);
     if (now < cost) { together = c; cost = now; }
   }
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim = {(unsigned)(together ? together : 1), 1, 1};
+  at[1] = early_start();
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(together ? together : *P, p.units());
   cfg.blockDim = dim3(kBlock); cfg.dynamicSmemBytes = S::SMEM; cfg.stream = stream;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
   const cudaError_t st = cudaLaunchKernelEx(&cfg, kernel, (const T*)k, (const T*)v, p, together ? together : *P, partials, base,
                                             together ? state : (float*)nullptr, tab, ctrl);
   if (st != cudaSuccess) { cudaGetLastError(); return st; }
@@ -976,9 +982,11 @@ cudaError_t launch_apply(const Problem& p, const void* q, const float* state, vo
   const cudaError_t e = allow_smem(split_apply_kernel<T, R, ROPE>, A::SMEM, done);
   if (e != cudaSuccess) return e;
   const int C = pieces((p.N + A::TOK - 1) / A::TOK, p.units(), sms(), 1ll << 30, 4.0);
-  split_apply_kernel<T, R, ROPE><<<dim3(C, p.units()), kBlock, A::SMEM, stream>>>((const T*)q, state, (T*)o, p, eps, tab, ctrl);
+  const cudaError_t st = launch_early(split_apply_kernel<T, R, ROPE>, dim3(C, p.units()), dim3(kBlock), A::SMEM, stream, (const T*)q, state, (T*)o, p,
+                                      eps, tab, ctrl);
+  if (st != cudaSuccess) { cudaGetLastError(); return st; }
   count_launches(1);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 #define LINATTN_SPLIT(FN, T, ROPE, ...)              \

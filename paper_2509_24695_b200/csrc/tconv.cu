@@ -86,10 +86,14 @@ __global__ void __launch_bounds__(256, kAhead > 1 ? 3 : 4) tconv_kernel(const Tc
   using Pc = Piece<T>;
   using Raw = typename Pc::Raw;
   constexpr int PAIRS = Pc::PAIRS;
+  let_next_grid_start();
+  wait_for_prior_grids();
+  const void *const xs = behind_wait(p.x), *const before = behind_wait(p.cache_in);
+  const float* const taps = behind_wait(p.w);
   const unsigned col = (blockIdx.x * blockDim.x + threadIdx.x) * (2 * PAIRS);   // element within a frame (< 2^31)
   if (col >= p.frame) return;
   const int b = blockIdx.y;
-  const T* x = static_cast<const T*>(p.x) + b * p.sb + col;
+  const T* x = static_cast<const T*>(xs) + b * p.sb + col;
   Raw* cache_out = p.cache_out ? reinterpret_cast<Raw*>(static_cast<T*>(p.cache_out) + b * p.frame + col) : nullptr;
   auto frame_of = [&](long long t) { return __ldcs(reinterpret_cast<const Raw*>(x + t * p.frame)); };
   if (!p.y) {  // absorb only: the cache becomes the last frame
@@ -104,14 +108,14 @@ __global__ void __launch_bounds__(256, kAhead > 1 ? 3 : 4) tconv_kernel(const Tc
   for (int tau = 0; tau < 3; ++tau)
 #pragma unroll
     for (int i = 0; i < PAIRS; i += 2) {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(p.w + tau * p.D + c0 + 2 * i));
+      const float4 a = __ldg(reinterpret_cast<const float4*>(taps + tau * p.D + c0 + 2 * i));
       w[tau][i] = make_float2(a.x, a.y);
       w[tau][i + 1] = make_float2(a.z, a.w);
     }
 
   // frames t-1, t, t+1 as floats (each frame is widened once), frames t+2 .. t+1+kAhead as loaded
   Raw r_prev = Pc::zero(), r_cur, r_nxt = Pc::zero(), raw[kAhead];
-  if (p.cache_in) r_prev = __ldcs(reinterpret_cast<const Raw*>(static_cast<const T*>(p.cache_in) + b * p.frame + col));
+  if (before) r_prev = __ldcs(reinterpret_cast<const Raw*>(static_cast<const T*>(before) + b * p.frame + col));
   r_cur = frame_of(0);
   if (p.T > 1) r_nxt = frame_of(1);
 #pragma unroll
@@ -168,6 +172,9 @@ __global__ void __launch_bounds__(256, kStepCtasPerSm) tconv_step_kernel(const T
   using Raw = typename Pc::Raw;
   constexpr int PAIRS = Pc::PAIRS;
   extern __shared__ uint4 ring_raw[];
+  let_next_grid_start();
+  wait_for_prior_grids();
+  const float* const taps = behind_wait(p.w);
   Raw* ring = reinterpret_cast<Raw*>(ring_raw);   // [stage][segment][thread]
   const int tid = (int)threadIdx.x;
   const int nf = (int)p.T;                        // 1..3 frames
@@ -206,7 +213,7 @@ __global__ void __launch_bounds__(256, kStepCtasPerSm) tconv_step_kernel(const T
     for (int tau = 0; tau < 3; ++tau)
 #pragma unroll
       for (int i = 0; i < PAIRS; i += 2) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(p.w + tau * p.D + c0 + 2 * i));
+        const float4 a = __ldg(reinterpret_cast<const float4*>(taps + tau * p.D + c0 + 2 * i));
         w[tau][i] = make_float2(a.x, a.y);
         w[tau][i + 1] = make_float2(a.z, a.w);
       }
@@ -261,8 +268,7 @@ cudaError_t launch_step(const TconvParams& p, int B, cudaStream_t stream) {
   const int sms = sm_count_of_device();
   if (!sms) return cudaErrorUnknown;
   const int grid = (int)(total < kStepCtasPerSm * sms ? total : kStepCtasPerSm * sms);
-  tconv_step_kernel<T><<<grid, 256, smem, stream>>>(p, (int)tpb, (int)total);
-  return cudaGetLastError();
+  return launch_early(tconv_step_kernel<T>, dim3(grid), dim3(256), smem, stream, p, (int)tpb, (int)total);
 }
 
 int check(const tconv_desc* d, long long T, long long* frame, long long* sb, long long* sby, size_t* esz) {
@@ -317,15 +323,11 @@ int run(const tconv_desc* d, long long T, long long T_b, const void* x, const fl
     e = d->dtype == LINATTN_BF16 ? launch_step<__nv_bfloat16>(p, d->B, (cudaStream_t)stream)
                                  : launch_step<float>(p, d->B, (cudaStream_t)stream);
   } else {
-    if (d->dtype == LINATTN_BF16) {
-      if (few) tconv_kernel<__nv_bfloat16, 1><<<grid, 256, 0, (cudaStream_t)stream>>>(p);
-      else tconv_kernel<__nv_bfloat16, 3><<<grid, 256, 0, (cudaStream_t)stream>>>(p);
-    } else {
-      if (few) tconv_kernel<float, 1><<<grid, 256, 0, (cudaStream_t)stream>>>(p);
-      else tconv_kernel<float, 3><<<grid, 256, 0, (cudaStream_t)stream>>>(p);
-    }
-    e = cudaGetLastError();
+    const auto kernel = d->dtype == LINATTN_BF16 ? (few ? tconv_kernel<__nv_bfloat16, 1> : tconv_kernel<__nv_bfloat16, 3>)
+                                                 : (few ? tconv_kernel<float, 1> : tconv_kernel<float, 3>);
+    e = launch_early(kernel, grid, dim3(256), 0, (cudaStream_t)stream, p);
   }
+  if (e != cudaSuccess) cudaGetLastError();
   count_launches(1);
   return e == cudaSuccess ? LINATTN_OK : LINATTN_ERR_CUDA;
 }

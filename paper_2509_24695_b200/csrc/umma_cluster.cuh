@@ -136,6 +136,8 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     prefetch_tensormap(&map_v);
   }
   if (warp == 1) { tmem_alloc(tmem_holder, kTmemCols); tmem_relinquish(); }
+  let_next_grid_start();
+  wait_for_prior_grids();
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
