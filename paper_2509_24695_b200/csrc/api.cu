@@ -645,6 +645,17 @@ int blocklin_prefill(blocklin_cache* cache, int64_t n_blocks, int64_t T_b, const
       cache->workspace_bytes >= workspace_need(pv)) {
     cudaStream_t s = (cudaStream_t)stream;
     float* blk = reinterpret_cast<float*>(static_cast<char*>(cache->workspace) + state_slot_offset(pv));
+    // with the grid on the tensor cores all three are one launch (see reduce_prefix)
+    const int grid = q && umma_supported(pv) ? umma_takes_grid(pv) : 0;
+    if (grid < 0) return grid;
+    if (grid) {
+      UmmaCall c{k, v, q, o, blk, nullptr, false, cache->eps, nullptr, (int)n_blocks, cache->state};
+      st = umma_run(pv, c, cache->workspace, s);
+      if (st != LINATTN_OK) return st;
+      cache->blocks_seen += n_blocks;
+      cache->tokens_seen += n_blocks * T_b;
+      return LINATTN_OK;
+    }
     st = run_passes(pv, k, v, nullptr, nullptr, blk, false, 0.f, cache->workspace, s);
     if (st != LINATTN_OK) return st;
     if (prefix_states(blk, cache->state, p.B, (int)n_blocks, (long long)p.H * p.state_elems(), s) != cudaSuccess)

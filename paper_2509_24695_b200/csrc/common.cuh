@@ -112,12 +112,16 @@ struct UmmaCall {
   bool accumulate;
   float eps;
   const void* rope;  // rotary variant (Eq. 2 with its rotary factors): packed (cos, sin) fp16 table [N][d/2]; else null
+  int blocks = 0;        // above 1: a prefill, whose batch entries are that many blocks of each entry of `cache` ...
+  float* cache = nullptr;  // ... which is read and written; `state` is room for the blocks' states, and behind the partials
 };
 bool umma_supported(const Problem& p);
 size_t umma_partial_bytes(const Problem& p, bool rope = false);
 bool umma_rope_supported(const Problem& p);
 // CTAs of the cluster that takes a unit of this shape (0: a lone CTA or the grid), or an error status.
 int umma_cluster_ctas(const Problem& p, bool rope);
+// 1: the grid takes this shape's state pass, 0: lone CTAs or clusters do; or an error status.
+int umma_takes_grid(const Problem& p);
 // Returns LINATTN_OK or an error status.
 int umma_run(const Problem& p, const UmmaCall& call, void* workspace, cudaStream_t stream);
 

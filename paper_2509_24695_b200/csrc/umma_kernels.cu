@@ -220,6 +220,8 @@ struct FusedParams {
   WorkspaceCtrl* ctrl;
   uint8_t* s_image;        // non-null: the reduce also leaves every unit's S operand (bf16 hi + lo, in the shared-memory
                            // layout) here, S_BYTES per unit, and the apply pass fetches it with one bulk copy
+  int blocks;              // prefill: batch entry b of K, V, Q, O is block b % blocks of entry b / blocks of the cache
+  float* cache;            // ... [B / blocks][H][(d+1)][d]: the state before the first block, and (written) after the last one
   int write_state;         // lone CTAs: the new state goes to `state` (a launch whose state nobody reads keeps it on chip)
   const uint4* rope;       // rotary variant: [N][d/8] chunks of four (cos, sin) fp16 pairs; null otherwise
   long long N;             // tokens (bound of the rotary table)
@@ -668,6 +670,108 @@ __device__ void reduce_image(const FusedParams& p) {
   fence_proxy_async_all();   // the images are read through the async proxy (bulk copy) after the barrier
 }
 
+// Eight fp32 values as bf16 hi + lo, sixteen bytes each.
+__device__ __forceinline__ void split_hi_lo(const float (&x)[8], uint4& hi, uint4& lo) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    h[e] = pack_bf16x2(x[2 * e], x[2 * e + 1]);
+    l[e] = pack_bf16x2(x[2 * e] - __uint_as_float(h[e] << 16), x[2 * e + 1] - __uint_as_float(h[e] & 0xFFFF0000u));
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// ---------------------------------------------------------------- reduce of a prefill
+// All blocks of a cached sequence in one launch: the state that block m's queries see is the cache's, plus the sums of blocks 0..m
+// (Eq. 3).  A thread takes 32 bytes of a state row of one head of the cache and walks the blocks: it adds a block's records up in
+// their fixed order, adds that to what it has, and leaves the result as the block's operand image (IMAGE) or state.  The records of all
+// blocks make one list, of which NR are in flight together (about 148 / heads of them, however they fall on the blocks).  Same sums in
+// the same order as a state launch, prefix_states and an apply launch, without the gaps between three launches and with the operands made
+// once instead of by every CTA from the states.  Before and after, us: 7 blocks of 4680 tokens, 20 heads of 112 134.9 -> 123.5, of 10800 280 -> 241, of 300
+// 36.9 -> 22.6; 2 entries of 6 blocks of 3040, 35 heads of 64 157 -> 142; 7 blocks of 300, 18 heads of 128 39.0 -> 24.7.
+template <int D, bool IMAGE>
+__device__ __forceinline__ void prefix_slice(const FusedParams& p, int& i0, int& i1) {   // this CTA's share of the cache's 32-byte chunks
+  const long long tot = (long long)(p.B / p.blocks) * p.H * ((D + 1) * D / 8);
+  i0 = (int)(tot * blockIdx.x / gridDim.x);
+  i1 = (int)(tot * (blockIdx.x + 1) / gridDim.x);
+}
+
+template <int D, bool IMAGE>
+__device__ void reduce_prefix(const FusedParams& p) {
+  using C = Cfg<D>;
+  constexpr int CPR = D / 8, PER_HEAD = (D + 1) * CPR, E4 = (D + 1) * D / 4, REC4 = C::G * E4, NR = 8;
+  const Sched& s = p.sa;
+  const long long ttot = (long long)s.U * s.m;
+  const int ncol = s.P == 0 ? 0 : (s.P < (s.tpu + s.Lc - 1) / s.Lc ? s.P : (s.tpu + s.Lc - 1) / s.Lc);
+  int i0, i1;
+  prefix_slice<D, IMAGE>(p, i0, i1);
+  for (int idx = i0 + (int)threadIdx.x; idx < i1; idx += (int)blockDim.x) {
+    const int bh = idx / PER_HEAD, rem = idx - bh * PER_HEAD, j = rem / CPR, c = rem - j * CPR;
+    const int b = bh / p.H, h = bh - b * p.H;
+    const float4* part4 = reinterpret_cast<const float4*>(p.partials) + (size_t)(h % C::G) * E4 + j * (D / 4) + 2 * c;
+    float4* cache4 = reinterpret_cast<float4*>(p.cache) + 2 * (size_t)idx;
+    float4 run0 = __ldcg(cache4), run1 = __ldcg(cache4 + 1);
+    float4 sum0 = make_float4(0.f, 0.f, 0.f, 0.f), sum1 = sum0;
+    // the block whose records come next, its unit, and of its records those that are left
+    int m = -1, u = 0, k = 0, nrec = 0, r_lo = 0;
+    auto next_block = [&] {
+      ++m;
+      u = (b * p.blocks + m) * p.HG + h / C::G;
+      k = 0;
+      nrec = ncol;
+      if (s.m > 0) {
+        r_lo = trailing_cta_of((long long)u * s.m, ttot, s.R);
+        nrec += trailing_cta_of((long long)(u + 1) * s.m - 1, ttot, s.R) - r_lo + 1;
+      }
+    };
+    next_block();
+    int done = 0;   // blocks that are complete
+    while (done < p.blocks) {
+      float4 v[NR][2];
+      uint32_t last = 0;   // bit r: record r ends a block
+      int n = 0;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        if (m < p.blocks) {
+          const float4* src = part4 + (size_t)(k < ncol ? k * s.U + u : s.P * s.U + r_lo + (k - ncol) + u) * REC4;
+          v[r][0] = __ldcg(src);
+          v[r][1] = __ldcg(src + 1);
+          n = r + 1;
+          if (++k == nrec) { last |= 1u << r; next_block(); }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        if (r >= n) break;
+        add4(sum0, v[r][0]);
+        add4(sum1, v[r][1]);
+        if (!(last >> r & 1)) continue;
+        add4(run0, sum0);
+        add4(run1, sum1);
+        sum0 = sum1 = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int bm = b * p.blocks + done++;
+        if (IMAGE) {
+          const float x8[8] = {run0.x, run0.y, run0.z, run0.w, run1.x, run1.y, run1.z, run1.w};
+          uint4 hi, lo;
+          split_hi_lo(x8, hi, lo);
+          const int jrow = j < D ? j : C::ZROW, f = c * 8;   // operand row, first key feature
+          uint8_t* to = p.s_image + (size_t)(bm * p.H + h) * C::S_BYTES + (f >> 6) * C::SBOX_BYTES + jrow * kRowBytes + ((((f & 63) >> 3) ^ (jrow & 7)) << 4);
+          *reinterpret_cast<uint4*>(to) = hi;
+          *reinterpret_cast<uint4*>(to + 2 * C::SBOX_BYTES) = lo;
+        } else {
+          float4* to = reinterpret_cast<float4*>(p.state) + (size_t)(bm * p.H + h) * E4 + j * (D / 4) + 2 * c;
+          to[0] = run0;
+          to[1] = run1;
+        }
+      }
+    }
+    cache4[0] = run0;
+    cache4[1] = run1;
+  }
+  if (IMAGE) fence_proxy_async_all();   // the images are read through the async proxy (bulk copy) after the barrier
+}
+
 // ---------------------------------------------------------------- S operand of the apply pass
 // Builds the B operand of the apply MMA for head group (b, hg) from the fp32 state: for every head
 // of the group, rows = value features (plus one row for z), K = key features, split into bf16 hi + lo.
@@ -728,16 +832,6 @@ __device__ __forceinline__ void build_s_operand(uint8_t* s_op, const float* __re
 // that an accumulator lane is a row of the apply operand (a value feature) and a thread stores sixteen bytes of it at a
 // time; with lanes as key features, as the partial records want them, the same step took 20 000 cycles instead of
 // 2 500.  z comes from the ReLU warps' fp32 sums, as in the rotary variant.
-__device__ __forceinline__ void split_hi_lo(const float (&x)[8], uint4& hi, uint4& lo) {
-  uint32_t h[4], l[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    h[e] = pack_bf16x2(x[2 * e], x[2 * e + 1]);
-    l[e] = pack_bf16x2(x[2 * e] - __uint_as_float(h[e] << 16), x[2 * e + 1] - __uint_as_float(h[e] & 0xFFFF0000u));
-  }
-  hi = make_uint4(h[0], h[1], h[2], h[3]);
-  lo = make_uint4(l[0], l[1], l[2], l[3]);
-}
 
 // Accumulator columns [16 * first, 16 * last) of lane quarter wq (key features; lane = value feature): sums of the four
 // accumulators in a fixed order, added (add) to what is staged at `st`, the old state or the tiles before, and left there
@@ -1046,7 +1140,8 @@ __device__ __forceinline__ void apply_epilogue(uint32_t tmem_base, uint32_t acc,
 // SOLO: lone CTAs.  IMAGE: the reduce leaves operand images and the apply pass fetches them (p.s_image).  Both are decided
 // on the host, and each form is a kernel of its own: the rotary one has no registers to spare, and with the slice reduce that
 // it does not take compiled into it (even out of line) a read-only rotary step of 4680 tokens took 45.0 us instead of 43.1.
-template <int D, bool ROPE, bool SOLO, bool IMAGE>
+// PREFIX: a prefill of several blocks (p.blocks, p.cache), the reduce is reduce_prefix.
+template <int D, bool ROPE, bool SOLO, bool IMAGE, bool PREFIX = false>
 __global__ void __launch_bounds__(Roles<ROPE>::THREADS, 1)
 umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                   const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
@@ -1514,6 +1609,15 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
       }
     }
     __syncwarp();
+  } else if (PREFIX) {
+    // ------------------------------------------------------------ store warp (idle in this pass): the cache into L2, as below
+    if (__all_sync(0xffffffffu, mbar_wait(a_done, 0, abort_flag))) {
+      int i0, i1;
+      prefix_slice<D, IMAGE>(p, i0, i1);
+      const char* base = reinterpret_cast<const char*>(p.cache) + (size_t)i0 * 32;
+      for (int off = lane * 128; off < (i1 - i0) * 32; off += 32 * 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off) : "memory");
+    }
   } else if (IMAGE && p.accumulate && p.do_state && (int)blockIdx.x < p.sa.P * p.sa.U) {
     // ------------------------------------------------------------ store warp (idle in this pass)
     // A cached step adds to the old state, which the K, V stream has pushed out of L2 since the last step:
@@ -1533,7 +1637,8 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   if (!SOLO && p.do_state) {
     grid_barrier(p.ctrl, abort_flag, p.do_apply != 0, gen0);
     if (!*abort_flag) {
-      if constexpr (IMAGE) reduce_image<D, ROPE>(p);
+      if constexpr (PREFIX) reduce_prefix<D, IMAGE>(p);
+      else if constexpr (IMAGE) reduce_image<D, ROPE>(p);
       else reduce_slice<D, ROPE>(p);
     }
     if (p.do_apply) grid_barrier(p.ctrl, abort_flag, false, gen0 + 1);
@@ -1838,14 +1943,14 @@ inline bool solo_pays(const Problem& p, int U, int sms) {
 inline int groups_of(int d) { return d == 32 ? 4 : d == 64 ? 2 : 1; }
 
 // Instantiates and launches the kernel: cooperatively when its CTAs wait for one another.
-template <int D, bool ROPE, bool SOLO, bool IMAGE>
+template <int D, bool ROPE, bool SOLO, bool IMAGE, bool PREFIX = false>
 int launch_kernel(int grid, void** args, cudaStream_t stream) {
   using C = Cfg<D>;
   // the opt-in to more than 48 KB of dynamic shared memory is a per-device setting of the kernel
   static bool attr_set[64] = {false};
   constexpr size_t kSmem = SOLO ? C::SMEM_SOLO : ROPE ? C::SMEM_ROPE : C::SMEM;
   static_assert(SOLO || kSmem >= kSmemAlone, "CTAs that wait for one another");
-  const void* kernel = (const void*)umma_fused_kernel<D, ROPE, SOLO, IMAGE>;
+  const void* kernel = (const void*)umma_fused_kernel<D, ROPE, SOLO, IMAGE, PREFIX>;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LINATTN_ERR_CUDA;
   if (!attr_set[dev]) {
@@ -2006,7 +2111,8 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   FusedParams fp{};
   fp.B = p.B; fp.H = p.H; fp.HG = (p.H + C::G - 1) / C::G;
   const int U = p.B * fp.HG;
-  if (do_state) {
+  const bool prefill = c.blocks > 1;   // (asked for where neither clusters nor lone CTAs take the shape)
+  if (do_state && !prefill) {
     const int size = cluster_size<D, ROPE>(p, U, (p.N + kTileState - 1) / kTileState, sms);
     if (size < 0) return size;
     if (size) return launch_cluster<D, ROPE>(p, c, size, U, workspace, stream);
@@ -2021,12 +2127,16 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   fp.rope = static_cast<const uint4*>(c.rope);
   fp.N = p.N;
   fp.s_image = nullptr;
-  if (do_state && do_apply && C::G == 1 && fp.sa.P >= 1) {
+  fp.blocks = c.blocks;
+  fp.cache = c.cache;
+  if (do_state && do_apply && C::G == 1 && (fp.sa.P >= 1 || prefill)) {
     // The operand images live at the end of the partials area, which is sized for kMaxCtas + U records while a
     // launch writes at most P*U + R + U of them: used when they fit behind the records in use.
     const size_t rec_bytes = ((size_t)p.state_elems() + (ROPE ? kZParts : 0)) * sizeof(float);
     const size_t used = ((size_t)fp.sa.P * U + fp.sa.R + U) * rec_bytes;
-    const size_t total = umma_partial_bytes(p, ROPE), img = (size_t)U * C::S_BYTES;
+    const size_t img = (size_t)U * C::S_BYTES;
+    size_t total = umma_partial_bytes(p, ROPE);
+    if (prefill) total = (size_t)(reinterpret_cast<char*>(c.state) - reinterpret_cast<char*>(fp.partials)) + (size_t)U * p.state_elems() * sizeof(float);   // (the images take the place of the states)
     if (total >= img + 1024) {
       const size_t off = (total - img) & ~(size_t)1023;
       if (off >= used) fp.s_image = reinterpret_cast<uint8_t*>(fp.partials) + off;
@@ -2035,7 +2145,7 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   // a unit switch costs the apply pass about one tile when the S operand comes as an image, two when the CTA
   // builds it from the fp32 state
   fp.sc = make_sched(U, (p.N + kTileApply - 1) / kTileApply, sms, fp.s_image ? 1 : 2);
-  const bool solo = do_state && solo_pays(p, U, sms);
+  const bool solo = do_state && !prefill && solo_pays(p, U, sms);
   if (solo) {
     fp.sa.U = fp.sc.U = fp.sa.grid = fp.sc.grid = U;
     fp.sa.P = fp.sc.P = 1;
@@ -2061,6 +2171,9 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   }
   if (!do_state) { mk = mq; mv = mq; }
   void* args[] = {&mk, &mv, &mq, &mo, &fp};
+  if constexpr (!ROPE) {
+    if (prefill) return C::G == 1 && fp.s_image ? launch_kernel<D, false, false, C::G == 1, true>(grid, args, stream) : launch_kernel<D, false, false, false, true>(grid, args, stream);
+  }
   if (solo) return launch_kernel<D, ROPE, true, false>(grid, args, stream);
   if (C::G == 1 && fp.s_image) return launch_kernel<D, ROPE, false, C::G == 1>(grid, args, stream);
   return launch_kernel<D, ROPE, false, false>(grid, args, stream);
@@ -2092,6 +2205,12 @@ int cluster_ctas(const Problem& p) {
   const int sms = sm_count();
   if (!sms) return LINATTN_ERR_CUDA;
   return cluster_size<D, ROPE>(p, p.B * ((p.H + Cfg<D>::G - 1) / Cfg<D>::G), (p.N + kTileState - 1) / kTileState, sms);
+}
+
+int umma_takes_grid(const Problem& p) {
+  const int n = umma_cluster_ctas(p, false), sms = sm_count(), G = groups_of(p.d);
+  if (n < 0) return n;
+  return sms && n == 0 && !solo_pays(p, p.B * ((p.H + G - 1) / G), sms);
 }
 
 int umma_cluster_ctas(const Problem& p, bool rope) {
