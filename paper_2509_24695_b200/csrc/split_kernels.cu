@@ -633,7 +633,11 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   const long long all = (p.N + A::TOK - 1) / A::TOK;
   const long long first = blockIdx.x * all / gridDim.x;
   const int tiles = (int)((blockIdx.x + 1) * all / gridDim.x - first);
-  const float* W = state + (long long)u * p.state_elems();
+  // (Waited for here and not behind the barriers' and tensor memory's set-up: the first pieces were asked for later then, and with more
+  // registers spilled in the loops the pass took 168 us and not 159; at the start of the kernel without an early start, 161.)
+  let_next_grid_start();
+  wait_for_prior_grids();
+  const float* W = behind_wait(state) + (long long)u * p.state_elems();
   const long long base = (long long)(u / p.H) * p.sb + (long long)(u % p.H) * p.sh;
   // preparing: this thread's row of every tile, and its pieces of it
   const int row = (tid % kPrepare) / A::LANES, l = tid % A::LANES;
@@ -657,6 +661,10 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
     }
     copy_commit();
   };
+  if (preparing) {
+#pragma unroll
+    for (int t = 0; t < A::RAW_STAGES; ++t) issue(t);
+  }
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&done[i], 1); mbar_init(&ready[i], kPrepare); mbar_init(&drained[i], kDrain); }
     mbar_init(finished, 1);
@@ -667,21 +675,14 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   // padded features of both operands read as zero
   if (d < A::DP)
     for (int i = tid; i < (A::S_BYTES + 2 * A::STAGE) / 16; i += kBlock) reinterpret_cast<uint4*>(s_op)[i] = make_uint4(0, 0, 0, 0);
-  let_next_grid_start();
-  wait_for_prior_grids();
-  W = behind_wait(W);
-  if (preparing) {
-#pragma unroll
-    for (int t = 0; t < A::RAW_STAGES; ++t) issue(t);
-  }
-  if (tid < 128) zs[tid] = tid < d ? __ldcg(W + (long long)d * d + tid) : 0.f;
+  if (tid < 128) zs[tid] = tid < d ? W[(long long)d * d + tid] : 0.f;
   __syncthreads();
   uint32_t least = 0xFFFFFFFFu;   // twice the bits of the smallest |S| 2^38, less one (zero is the largest)
   float rest = 0.f;               // NaN if one is not finite
   for (int idx = tid; idx < d * (d / 4); idx += kBlock) {
     const int j = idx / (d / 4), i = (idx - j * (d / 4)) * 4;
     float x[4];
-    widen(__ldcg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
+    widen(__ldg(reinterpret_cast<const uint4*>(W + (long long)j * d + i)), x);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const float y = x[e] * 0x1p38f;
