@@ -645,10 +645,8 @@ int blocklin_prefill(blocklin_cache* cache, int64_t n_blocks, int64_t T_b, const
       cache->workspace_bytes >= workspace_need(pv)) {
     cudaStream_t s = (cudaStream_t)stream;
     float* blk = reinterpret_cast<float*>(static_cast<char*>(cache->workspace) + state_slot_offset(pv));
-    // with the grid on the tensor cores all three are one launch (see reduce_prefix)
-    const int grid = q && umma_supported(pv) ? umma_takes_grid(pv) : 0;
-    if (grid < 0) return grid;
-    if (grid) {
+    // on the tensor cores all three are one launch (see reduce_prefix), but for few heads
+    if (q && umma_supported(pv) && umma_joins_prefill(pv, (int)n_blocks)) {
       UmmaCall c{k, v, q, o, blk, nullptr, false, cache->eps, nullptr, (int)n_blocks, cache->state};
       st = umma_run(pv, c, cache->workspace, s);
       if (st != LINATTN_OK) return st;

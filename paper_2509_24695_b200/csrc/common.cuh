@@ -120,8 +120,8 @@ size_t umma_partial_bytes(const Problem& p, bool rope = false);
 bool umma_rope_supported(const Problem& p);
 // CTAs of the cluster that takes a unit of this shape (0: a lone CTA or the grid), or an error status.
 int umma_cluster_ctas(const Problem& p, bool rope);
-// 1: the grid takes this shape's state pass, 0: lone CTAs or clusters do; or an error status.
-int umma_takes_grid(const Problem& p);
+// Does a prefill of p.B / blocks entries of that many blocks of p.N tokens go in one launch (UmmaCall::blocks)?
+bool umma_joins_prefill(const Problem& p, int blocks);
 // Returns LINATTN_OK or an error status.
 int umma_run(const Problem& p, const UmmaCall& call, void* workspace, cudaStream_t stream);
 

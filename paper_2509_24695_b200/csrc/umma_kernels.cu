@@ -689,7 +689,7 @@ __device__ __forceinline__ void split_hi_lo(const float (&x)[8], uint4& hi, uint
 // blocks make one list, of which NR are in flight together (about 148 / heads of them, however they fall on the blocks).  Same sums in
 // the same order as a state launch, prefix_states and an apply launch, without the gaps between three launches and with the operands made
 // once instead of by every CTA from the states.  Before and after, us: 7 blocks of 4680 tokens, 20 heads of 112 134.9 -> 123.5, of 10800 280 -> 241, of 300
-// 36.9 -> 22.6; 2 entries of 6 blocks of 3040, 35 heads of 64 157 -> 142; 7 blocks of 300, 18 heads of 128 39.0 -> 24.7.
+// 36.9 -> 22.6 (more beside umma_joins_prefill); 2 entries of 6 blocks of 3040, 35 heads of 64 157 -> 142; 7 blocks of 300, 18 heads of 128 39.0 -> 24.7.
 template <int D, bool IMAGE>
 __device__ __forceinline__ void prefix_slice(const FusedParams& p, int& i0, int& i1) {   // this CTA's share of the cache's 32-byte chunks
   const long long tot = (long long)(p.B / p.blocks) * p.H * ((D + 1) * D / 8);
@@ -2111,7 +2111,7 @@ int launch_fused(const Problem& p, const UmmaCall& c, void* workspace, cudaStrea
   FusedParams fp{};
   fp.B = p.B; fp.H = p.H; fp.HG = (p.H + C::G - 1) / C::G;
   const int U = p.B * fp.HG;
-  const bool prefill = c.blocks > 1;   // (asked for where neither clusters nor lone CTAs take the shape)
+  const bool prefill = c.blocks > 1;   // (asked for where it pays, see umma_joins_prefill: always the grid)
   if (do_state && !prefill) {
     const int size = cluster_size<D, ROPE>(p, U, (p.N + kTileState - 1) / kTileState, sms);
     if (size < 0) return size;
@@ -2207,10 +2207,22 @@ int cluster_ctas(const Problem& p) {
   return cluster_size<D, ROPE>(p, p.B * ((p.H + Cfg<D>::G - 1) / Cfg<D>::G), (p.N + kTileState - 1) / kTileState, sms);
 }
 
-int umma_takes_grid(const Problem& p) {
-  const int n = umma_cluster_ctas(p, false), sms = sm_count(), G = groups_of(p.d);
-  if (n < 0) return n;
-  return sms && n == 0 && !solo_pays(p, p.B * ((p.H + G - 1) / G), sms);
+// One launch for all blocks, or a state launch, prefix_states and an apply launch?  A thread of reduce_prefix walks the records of all blocks
+// of its piece, CTAs / head groups of them, eight at a time; from some 70 on that is longer than what it saves.  One launch / three, us:
+//                       tokens a block    64         128        192        300        600        1200       2400
+//   d = 112, 20 groups, 2 blocks          18.6/22.6  18.6/26.7  16.5/25.1  17.1/26.7  18.6/26.9  20.6/28.5  24.0/31.1
+//             2                           18.5/22.6  17.3/26.3  16.5/24.7  16.5/24.9  18.6/24.8  20.6/25.0  22.7/25.7
+//            20         7                 18.6/28.8  18.6/30.8  20.6/32.9  22.8/35.4  31.0/45.3  45.4/59.7  68.7/84.5
+//             2         7                 16.5/24.7  16.9/28.8  18.6/26.8  20.6/28.4  26.8/28.8  27.3/28.3  29.4/31.2   (74 records from 1200)
+//             1         7                 16.1/23.7  16.5/27.7  18.6/26.7  20.6/27.9  26.6/27.8  36.4/27.8  37.0/27.9   (35, 70, 133, 148 from 300)
+//   d = 64,  18         2                 18.6/22.7  16.5/24.7  16.5/24.7  18.5/24.7  20.3/24.7  21.5/28.8  24.7/30.9
+//             2         7                 17.1/22.9  18.5/25.2  18.6/26.8  22.4/26.7  27.0/26.7  28.8/29.3  30.9/28.5
+//   d = 32,   2         7                 16.5/22.6  16.5/24.7  18.6/22.7  20.6/22.6  26.7/23.9  26.8/25.6  28.9/26.8
+//   d = 128, 20         7                 18.6/28.8  20.5/30.9  20.7/37.0  24.8/39.1  35.1/51.7  50.0/66.4  78.4/95.0
+bool umma_joins_prefill(const Problem& p, int blocks) {
+  const int sms = sm_count(), G = groups_of(p.d);
+  const long long groups = (long long)(p.B / blocks) * ((p.H + G - 1) / G), tiles = groups * blocks * ((p.N + kTileState - 1) / kTileState);
+  return sms && (tiles < sms ? tiles : sms) <= 64 * groups;
 }
 
 int umma_cluster_ctas(const Problem& p, bool rope) {

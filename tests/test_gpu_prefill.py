@@ -19,7 +19,7 @@ la = pytest.importorskip("paper_2509_24695_b200")
     (1, 40, 321, 30, 64),
 ])
 def test_prefill_is_its_parts(B, M, T, H, d):
-    assert T > 192 and la.cluster_ctas(B * M, H, d, T) == 0   # the grid
+    assert T > 192 and la.cluster_ctas(B * M, H, d, T) == 0   # the parts' state comes from the grid too: the same order
     gen = torch.Generator(device="cuda").manual_seed(7 * T + M)
     q, k, v = (torch.randn(B, M * T, H, d, device="cuda", generator=gen).bfloat16() for _ in range(3))
     cache = la.BlockLinCache(B, H, d, torch.bfloat16, "cuda", max_T_b=T, prefill_blocks=M)
@@ -40,3 +40,30 @@ def test_prefill_is_its_parts(B, M, T, H, d):
     assert torch.equal(cache.state, run)
     assert torch.equal(got.view(B * M, T, H, d), want)
     assert cache.status() == 0
+
+
+@pytest.mark.parametrize("B,M,T,H,d,launches", [
+    (1, 7, 64, 20, 112, 1),     # blocks that lone CTAs would take
+    (1, 3, 130, 1, 32, 1),
+    (2, 5, 700, 4, 112, 1),     # ... and clusters
+    (1, 2, 33, 3, 128, 1),
+    (1, 9, 1, 2, 64, 1),        # blocks of one token
+    (1, 7, 600, 1, 112, 3),     # 70 records to a piece
+    (1, 7, 1500, 2, 64, 3),
+])
+def test_prefill_of_small_blocks(B, M, T, H, d, launches):
+    """Against the steps, block by block: other forms, so to rounding (both sums of S within 1e-6 of 64 bits, outputs bf16)."""
+    gen = torch.Generator(device="cuda").manual_seed(T + M)
+    q, k, v = (torch.randn(B, M * T, H, d, device="cuda", generator=gen).bfloat16() for _ in range(3))
+    one = la.BlockLinCache(B, H, d, torch.bfloat16, "cuda", max_T_b=T, prefill_blocks=M)
+    steps = la.BlockLinCache(B, H, d, torch.bfloat16, "cuda", max_T_b=T)
+    before = la.kernel_launches()
+    got = one.prefill(q, k, v, M)
+    assert la.kernel_launches() == before + launches
+    cut = lambda t, m: t[:, m * T:(m + 1) * T].contiguous()
+    want = torch.cat([steps.step(cut(q, m), cut(k, m), cut(v, m)) for m in range(M)], dim=1)
+    assert (one.state - steps.state).norm() <= 2e-6 * steps.state.norm()
+    # the same bf16 value, or a neighbour of it where the sums fall on both sides of the middle
+    assert (got.float() - want.float()).abs().max() <= 2 ** -7 * want.float().abs().max()
+    assert (got.float() - want.float()).norm() <= 1e-3 * want.float().norm()
+    assert one.status() == 0
