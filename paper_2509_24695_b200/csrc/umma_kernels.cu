@@ -269,6 +269,31 @@ __device__ __forceinline__ void relu_pass(uint8_t* box0, uint8_t* box1, int t) {
   }
 }
 
+// ReLU of row r of a Q tile on its way to tensor memory: the row's features from the slot to the columns from `at` on (of this lane; a
+// warp's rows are its lane quarter), two to a column, as the MMA wants its A operand there.
+template <int FEAT>
+__device__ __forceinline__ void relu_row_to_tmem(const uint8_t* slot, int half, int r, uint32_t at) {
+  const uint8_t* row = slot + r * kRowBytes;
+#pragma unroll
+  for (int box = 0; box < 2; ++box) {
+    uint32_t w[32];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {   // neighbouring rows have a chunk at different places (swizzle): no bank conflicts
+      if (64 * box + 8 * c >= FEAT) break;
+      const uint4 x = *reinterpret_cast<const uint4*>(row + box * half + ((c ^ (r & 7)) << 4));
+      w[4 * c] = relu_bf16x2(x.x); w[4 * c + 1] = relu_bf16x2(x.y); w[4 * c + 2] = relu_bf16x2(x.z); w[4 * c + 3] = relu_bf16x2(x.w);
+    }
+    if (box == 0 || FEAT == 128) {
+      tmem_st_x32(at + 32 * box, w);
+    } else {
+      static_assert(FEAT == 112 || FEAT == 128, "columns of the second box");
+      tmem_st_x16(at + 32, w);
+      tmem_st_x8(at + 48, w + 16);
+    }
+  }
+  tmem_st_wait();
+}
+
 // The same, adding the plain values up per thread: z[0..3] for its chunk of box 0, z[4..7] for that of box 1.
 __device__ __forceinline__ void unpack_relu8(const uint4& x, float2 (&f)[4]);
 template <int FEAT, int ROWS>
@@ -1151,6 +1176,14 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   using R = Roles<ROPE>;
   // TAB: the state pass has its rotations in shared memory.  (Lone CTAs have no room for them and fetch them into registers.)
   constexpr bool TAB = ROPE && !SOLO;
+  // QT: phi(Q) is an operand in tensor memory, beside the accumulator of its tile.  Of the 260 KB that a tile of 128 rows moves through shared
+  // memory that takes out 84 (the clamped rows back, and both MMAs' reads of them): time where a tile is waited for, power where the
+  // chip is at its cap (1000 W, 1.5 to 1.6 GHz: forwards of 32 760 tokens and more).  Before and after, us: step of 4680 tokens 31.6 -> 30.9, of
+  // 2 x 10800 90.0 -> 89.2, 720p, 35 heads of 64 249.5 -> 246.7, 480p 123.3 -> 122.2; same bits.  (Lone CTAs: their accumulators take
+  // all columns up to the first Q tile.  Rotary: the rotated rows come eight lanes to a row.)
+  constexpr bool QT = !ROPE && !SOLO;
+  constexpr uint32_t QT_COL = 160;         // behind the accumulator's columns
+  static_assert(!QT || (C::NAPPLY <= QT_COL && QT_COL + C::FEAT / 2 <= kAccStride), "columns of tensor memory");
   constexpr int NSA = SOLO ? 4 : ROPE ? C::ROPE_STAGES : C::STATE_STAGES;
   constexpr int STAGE = SOLO ? C::SOLO_STAGE_BYTES : ROPE ? C::ROPE_STAGE_BYTES : C::STAGE_BYTES;
   constexpr int KOFF = SOLO || ROPE ? 2 * kBox : C::KOFF;
@@ -1680,8 +1713,13 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
           const uint64_t a = make_smem_desc_sw128(a0 + koff, 16, 1024);                           // phi(Q), K-major
           const uint64_t bh = make_smem_desc_sw128(b0 + boff, 16, 1024);                          // S hi
           const uint64_t bl = make_smem_desc_sw128(b0 + 2 * C::SBOX_BYTES + boff, 16, 1024);      // S lo
-          umma_bf16(d_tmem, a, bh, IDESC_C, k == 0 ? 0u : 1u);
-          umma_bf16(d_tmem, a, bl, IDESC_C, 1u);
+          if (QT) {
+            umma_bf16_ts(d_tmem, d_tmem + QT_COL + k * 8, bh, IDESC_C, k == 0 ? 0u : 1u);
+            umma_bf16_ts(d_tmem, d_tmem + QT_COL + k * 8, bl, IDESC_C, 1u);
+          } else {
+            umma_bf16(d_tmem, a, bh, IDESC_C, k == 0 ? 0u : 1u);
+            umma_bf16(d_tmem, a, bl, IDESC_C, 1u);
+          }
         }
         umma_commit(&c_tfull[acc]);
       }
@@ -1773,6 +1811,18 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         const int ahead = tn.done() ? t.tile() : tn.tile();
         rope_apply_rows<D>(sl, den_rows + s * C::G * kTileApply, row0, pc, lc, zc, tab0, tab1, [&](int i) { fetch_rot(ahead, i); });
         fence_proxy_async_smem();
+        mbar_arrive(&c_ready[s]);
+        continue;
+      }
+      if (QT) {
+        // (the columns are free when the MMAs of the tile two before, which had them, are complete)
+        bool here = mbar_wait(&c_full[s], (it / NSC) & 1, abort_flag);
+        if (it >= 2) here = here && mbar_wait(&c_tfull[it & 1], ((it - 2) >> 1) & 1, abort_flag);
+        if (!__all_sync(0xffffffffu, here)) break;   // leave as a whole warp
+        const int wq = warp & 3;
+        tcgen05_fence_after();
+        relu_row_to_tmem<C::FEAT>(slots + s * SLOT, HALF, wq * 32 + lane, tmem_base + (it & 1) * kAccStride + QT_COL + ((uint32_t)(wq * 32) << 16));
+        tcgen05_fence_before();
         mbar_arrive(&c_ready[s]);
         continue;
       }
