@@ -130,6 +130,37 @@ def load_library(path: str | None = None):
     return lib
 
 
+# The short way (csrc/binding.cpp): the calls of one layer, on plain tensors.  Each function answers NotImplemented for what it
+# does not take, and the general way below goes on.
+_fast = None
+_FAST_CALLS = ("linattn_forward", "linattn_forward_rope", "blocklin_step", "blocklin_peek", "blocklin_step_rope", "blocklin_peek_rope",
+               "tconv_forward", "tconv_block_step")
+
+
+class _NoBinding:
+    """In the place of the binding where it is not built (another torch than the one it was built against)."""
+
+    @staticmethod
+    def forward(*args):
+        return NotImplemented
+
+    forward_rope = step = conv = forward
+
+
+def _bind(lib):
+    """The short way to `lib`."""
+    global _fast
+    _torch()
+    try:
+        from . import _binding
+    except ImportError:
+        _fast = _NoBinding
+    else:
+        _binding.bind(*(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _FAST_CALLS))
+        _fast = _binding
+    return _fast
+
+
 def _check(status: int, where: str):
     if status != 0:
         raise LinAttnError(status, where)
@@ -223,6 +254,9 @@ def workspace_status(ws) -> int:
 
 def linattn_forward(q, k, v, eps: float = 1e-6, out=None, workspace=None):
     """Bidirectional ReLU linear attention (Eq. 2): returns O with the layout of q."""
+    o = (_fast or _bind(load_library())).forward(q, k, v, eps, out, workspace)
+    if o is not NotImplemented:
+        return o
     torch = _torch()
     lib = load_library()
     o = torch.empty_like(q) if out is None else out
@@ -264,6 +298,9 @@ def new_rope_workspace(like):
 def linattn_forward_rope(q, k, v, rope_table, eps: float = 1e-6, out=None, workspace=None):
     """Eq. 2 with its rotary factors (rotation after the ReLU, numerator only).  rope_table: the float16
     [N, d//2, 2] (cos, sin) table of ``rope_pack``: the rotation of feature pair (2p, 2p+1) of token n."""
+    o = (_fast or _bind(load_library())).forward_rope(q, k, v, rope_table, eps, out, workspace)
+    if o is not NotImplemented:
+        return o
     torch = _torch()
     lib = load_library()
     o = torch.empty_like(q) if out is None else out
@@ -452,11 +489,20 @@ class BlockLinCache:
             nbytes = max(nbytes, pb.value)
         return sb.value, nbytes
 
+    def _short(self, commit, q, k, v, table, out):
+        if self._strides != (0, 0, 0):
+            return NotImplemented
+        B, H, d = self._shape
+        return (_fast or _bind(load_library())).step(commit, self._handle.value, B, H, d, self._desc.dtype, q, k, v, table, out)
+
     def reset(self):
         _check(self._lib.blocklin_cache_reset(self._handle, _stream(self.state)), "blocklin_cache_reset")
 
     def step(self, q, k, v, out=None):
         """cache += state(block); returns the block's output (None when q is None)."""
+        o = self._short(True, q, k, v, None, out)
+        if o is not NotImplemented:
+            return o
         torch = _torch()
         o = None
         if q is not None:
@@ -487,6 +533,9 @@ class BlockLinCache:
     def step_rope(self, q, k, v, rope_table_blk, out=None):
         """``step`` with rotary factors; rope_table_blk: float16 [T_b, d//2, 2] rows of the block's tokens
         (a contiguous slice of the stream's ``rope_pack`` table).  q may be None: absorb only."""
+        o = self._short(True, q, k, v, rope_table_blk, out) if rope_table_blk is not None else NotImplemented
+        if o is not NotImplemented:
+            return o
         o = self._rope_args(q, k, v, rope_table_blk, out, k.shape[1])
         _check(self._lib.blocklin_step_rope(self._handle, k.shape[1], _ptr(q), _ptr(k), _ptr(v), _ptr(o),
                                             _ptr(rope_table_blk), _stream(k)), "blocklin_step_rope")
@@ -496,6 +545,9 @@ class BlockLinCache:
         """``peek`` with rotary factors: the block against the rotary cache plus itself, nothing committed."""
         if q is None:
             raise ValueError("peek_rope needs queries")
+        o = self._short(False, q, k, v, rope_table_blk, out) if rope_table_blk is not None else NotImplemented
+        if o is not NotImplemented:
+            return o
         o = self._rope_args(q, k, v, rope_table_blk, out, k.shape[1])
         _check(self._lib.blocklin_peek_rope(self._handle, k.shape[1], _ptr(q), _ptr(k), _ptr(v), _ptr(o),
                                             _ptr(rope_table_blk), _stream(k)), "blocklin_peek_rope")
@@ -521,6 +573,9 @@ class BlockLinCache:
 
     def peek(self, q, k, v, out=None):
         """Output of the block against cache + state(block) without committing (Algorithm 1's denoising steps)."""
+        o = self._short(False, q, k, v, None, out)
+        if o is not NotImplemented:
+            return o
         torch = _torch()
         o = torch.empty_like(q) if out is None else out
         _desc_of(q, k, v, o)
@@ -606,6 +661,9 @@ def _check_taps(w, D):
 
 def tconv_forward(x, w, out=None):
     """Bidirectional temporal convolution with shortcut over x[B, T, HW, D]; taps w[3, D] float32."""
+    y = (_fast or _bind(load_library())).conv(x, w, out, None, False)
+    if y is not NotImplemented:
+        return y
     y = _torch().empty_like(x) if out is None else out
     desc = _conv_desc_of(x, y)
     _check_taps(w, x.shape[3])
@@ -645,6 +703,9 @@ class TConvCache:
 
     def step(self, x_blk, w, out=None, commit: bool = True):
         """One block x_blk[B, T_b, HW, D]; commit=False only reads the cache (a denoising step)."""
+        y = (_fast or _bind(load_library())).conv(x_blk, w, out, self.frame, bool(commit))
+        if y is not NotImplemented:
+            return y
         y = _torch().empty_like(x_blk) if out is None else out
         d = self._desc_for(x_blk, y)
         _check_taps(w, x_blk.shape[3])
