@@ -603,7 +603,8 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     if (ROPE && n_apply > 0) {
 #pragma unroll
       for (int i = 0; i < kTileApply / 32; ++i) fetch_rot(0, i);
-      ok = __all_sync(0xffffffffu, mbar_wait(s_full, 0, abort_flag));   // (z_row)
+      // z_row is this CTA's own work: it is there with its rows of the operand, before the peers' have come
+      ok = __all_sync(0xffffffffu, mbar_wait(s_staged, 0, abort_flag));
 #pragma unroll
       for (int box = 0; box < 2; ++box) {
         float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
