@@ -537,7 +537,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         if (ROPE) z_row[ot] = z;
         else if (p.do_apply) put_z<D>(s_op, ot, z);
       }
-      fence_proxy_async_all();   // the rows are copied, and read by the MMAs
+      fence_proxy_async_smem();   // the rows are copied, and read by the MMAs
       __syncwarp();
       if (lane == 0) { mbar_arrive(s_full); mbar_arrive(s_staged); }
       if (p.do_apply && warp == 2 && __all_sync(0xffffffffu, mbar_wait(s_staged, 0, abort_flag))) {
@@ -568,7 +568,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0 && n_apply > 0) {
       bool ok = operand;
-      fence_proxy_async_all();
+      fence_proxy_async_smem();
       for (int it = 0; it < n_apply && ok; ++it) {
         const int s = it % NSC, acc = it & 1;
         ok = mbar_wait(&c_tempty[acc], ((it >> 1) & 1) ^ 1, abort_flag) && mbar_wait(&c_ready[s], (it / NSC) & 1, abort_flag);
