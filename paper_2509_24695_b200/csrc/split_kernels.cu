@@ -602,7 +602,7 @@ struct ApplyShape : Shape<T, R, ROPE> {
 
 // grid (C, units): tiles [c * tiles / C, (c + 1) * tiles / C) of one unit.
 //
-// Measured as above: 163 us, general kernels 866, register-blocked on packed fp32 FMAs 489.  Stamps, cycles of a 64-token tile's
+// Measured as above: 159 us (163 before early starts), general kernels 866, register-blocked on packed fp32 FMAs 489.  Stamps, cycles of a 64-token tile's
 // 3830: the accumulators of order one and two are there once, so a tile's 21 MMAs on them follow the reading of the last tile's:
 // read 840, issued 1590, complete 1030 later, 3460 in a chain; beside it the seven leading MMAs (840), the draining warps' stores (2340 of
 // their 3180) and the preparing warps (3380).  d = 128: 4520, of which the MMA warp issues for 3240.  bf16, 28 heads of 80:
@@ -948,6 +948,7 @@ cudaError_t launch_state(const Problem& p, const void* k, const void* v, const f
   // In tiles: a CTA costs six whatever its share, the sum of partial states (a kernel of its own) one more than a cluster's.
   // Measured, cached step, fp32, 20 heads of 112, cluster against partial states: 300 tokens 24.9 against 33.3 us, 512 29.9
   // against 43.8, 1200 37.6 against 43.7, 4680 75.9 against 73.9; forward of 3000 tokens, 35 heads of 64: 62.5 against 57.8.
+  // (Without early starts, which take 2 us off a call of either.)
   *P = pieces(tiles, p.units(), sms(), fma_chunks(p.N), 6.0);
   const double apart = (double)(((long long)*P * p.units() + sms() - 1) / sms()) * ((double)((tiles + *P - 1) / *P) + 6.0) + 1.0;
   int together = 0;

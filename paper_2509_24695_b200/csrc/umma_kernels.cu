@@ -21,7 +21,10 @@
 //                bf16 hi + lo parts (two MMAs per K step, so S keeps ~16 mantissa bits), with z as an
 //                extra row of B so the denominator is one more accumulator column.  B comes into shared
 //                memory once per unit segment: one bulk copy of the unit's image, or built from the fp32
-//                state.  The epilogue divides, rounds to bf16 and a dedicated warp TMA-stores the tile.
+//                state.  phi(Q) gets to the tensor core through tensor memory (QT below), in the lone CTAs' and the rotary
+//                form through shared memory.  The epilogue divides, rounds to bf16 and a dedicated warp TMA-stores the tile.
+//
+// A prefill of several blocks is one launch too: its reduce also forms the running sums over the blocks (reduce_prefix).
 //
 // The first Q tiles of the apply pass are fetched before the grid barriers (Q does not depend on the
 // state), so HBM stays busy while the partials are reduced.
@@ -692,7 +695,9 @@ __device__ void reduce_image(const FusedParams& p) {
     }
     if (ROPE && D % 8 == 0 && c == 0) reduce_image_zrow<D>(p, u, ncol, r_lo, nrec);
   }
-  fence_proxy_async_all();   // the images are read through the async proxy (bulk copy) after the barrier
+  // The images are read through the async proxy (bulk copy) after the barrier.  (For all of memory the fence cost more: step of 4680 tokens
+  // 32.2 -> 30.9 us, of 2 x 10800 88.1 -> 87.8, forward of 32 760 120.2 -> 119.5.)
+  fence_proxy_async_global();
 }
 
 // Eight fp32 values as bf16 hi + lo, sixteen bytes each.
@@ -794,7 +799,7 @@ __device__ void reduce_prefix(const FusedParams& p) {
     cache4[0] = run0;
     cache4[1] = run1;
   }
-  if (IMAGE) fence_proxy_async_all();   // the images are read through the async proxy (bulk copy) after the barrier
+  if (IMAGE) fence_proxy_async_global();   // (see reduce_image)
 }
 
 // ---------------------------------------------------------------- S operand of the apply pass
@@ -1982,7 +1987,8 @@ int sm_count() {
 //   d = 128, 18 units   8.5/17.4 9.5/18.2 7.1/13.0 11.3/16.3 12.4/16.8 9.7/10.8 15.1/15.4 16.1/15.8 12.5/10.3 18.0/15.7 19.2/15.9 15.4/9.6
 //   d = 64, 35          8.3/16.2 9.0/16.4 6.4/10.5 10.8/15.5 11.6/15.5 8.7/9.5  13.6/15.7 14.5/15.7 10.8/9.4 16.1/16.3 16.9/16.2 12.9/9.6
 //   d = 32, 1           7.5/13.1 7.9/12.6 5.5/8.0  9.9/12.6 10.2/13.3 7.3/7.7   12.3/13.0 12.7/13.1 9.0/7.7  14.0/13.0 14.5/12.9 10.6/7.7
-// with rotary factors alike at d = 112 and 128 and twice as fast as the grid at d = 32 and 64.  So: up to 128 tokens, and up to 192
+// with rotary factors alike at d = 112 and 128 and twice as fast as the grid at d = 32 and 64.  (Taken before early starts, which take 1.5
+// to 3 us off the lone CTAs of calls in a row and nothing off the grid: forward of 64 tokens, 4 heads of 32 6.9, 128 tokens 8.8.)  So: up to 128 tokens, and up to 192
 // with packed heads or many units where these are too many for clusters, which are asked for first (cluster_size).  (States alone of
 // 129 to 192 tokens with packed heads lose 1 us by that.)  The choice depends on the shape and the device, not on the call, so that all
 // calls on one shape (forward, state and apply, step, peek, the token-sharded three) add up in the same order and give the same bits.
@@ -2096,6 +2102,9 @@ int clusters_at_once(int c) {
 //                26         1         5 CTAs    18.7/20.0  12.8/12.1
 // States alone lose 3 to 6 % on clusters with 27 to 29 and 34 to 37 units of ten to twelve tiles, with 46 to 49 units from six
 // on, and with heads of 128 (129 to 192 tokens; with rotary factors, five CTAs), where the steps are level or gain: one form for all calls.
+// All of this was taken before early starts (early_start) and the shorter end of the cluster kernel, which take 2 to 4 us off clusters in a
+// row and nothing off the grid: 20 heads of 112, read-only step of 4680 tokens now 30.6 on clusters of 6, 33.1 on the grid, rotary 33.6 and 40.6.
+// Clusters are ahead up to 18 tiles and more where they take 110 SMs or more, and to 5 to 10 below that; the line has not been moved.
 // Not taken though clusters would be 7 % ahead: thirteen tiles and more of plain heads of 112 with 38 to 45 and 50 to 74 units; heads
 // of 128 of 193 to 300 tokens (3 %).
 template <int D, bool ROPE>
