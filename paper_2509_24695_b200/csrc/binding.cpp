@@ -45,13 +45,15 @@ const at::Tensor* plain(PyObject* o) {
 
 int dtype_of(const at::Tensor& t) { return t.scalar_type() == at::kBFloat16 ? LINATTN_BF16 : t.scalar_type() == at::kFloat ? LINATTN_F32 : -1; }
 
+bool fits(int64_t n) { return n <= INT32_MAX; }   // (a descriptor's numbers; of an expanded tensor they may not)
+
 bool same(const at::Tensor& a, const at::Tensor& b) {
   return a.sizes() == b.sizes() && a.strides() == b.strides() && a.scalar_type() == b.scalar_type() && a.get_device() == b.get_device();
 }
 
 // [B, N, H, d] tensors of one layout: the descriptor.
 bool describe(const at::Tensor& t, linattn_desc* d) {
-  if (t.dim() != 4 || t.stride(3) != 1 || dtype_of(t) < 0) return false;
+  if (t.dim() != 4 || t.stride(3) != 1 || dtype_of(t) < 0 || !fits(t.size(0)) || !fits(t.size(2)) || !fits(t.size(3))) return false;
   d->B = (int32_t)t.size(0); d->H = (int32_t)t.size(2); d->d = (int32_t)t.size(3); d->dtype = dtype_of(t);
   d->stride_b = t.stride(0); d->stride_n = t.stride(1); d->stride_h = t.stride(2);
   return true;
@@ -148,7 +150,9 @@ PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (n != 5 || !p_tconv_forward || watched()) return general();
   const at::Tensor *x = plain(a[0]), *w = plain(a[1]), *frame = a[3] == Py_None ? nullptr : plain(a[3]);
   at::Tensor y;
-  if (!x || !w || (a[3] != Py_None && !frame) || x->dim() != 4 || dtype_of(*x) < 0 || !x->is_contiguous()) return general();
+  if (!x || !w || (a[3] != Py_None && !frame) || x->dim() != 4 || dtype_of(*x) < 0 || !x->is_contiguous() || !fits(x->size(0)) ||
+      !fits(x->size(2)) || !fits(x->size(3)))
+    return general();
   if (w->scalar_type() != at::kFloat || w->dim() != 2 || w->size(0) != 3 || w->size(1) != x->size(3) || !w->is_contiguous()) return general();
   if (frame && (frame->dim() != 3 || frame->size(0) != x->size(0) || frame->size(1) != x->size(2) || frame->size(2) != x->size(3) ||
                 frame->scalar_type() != x->scalar_type() || !frame->is_contiguous()))

@@ -33,7 +33,7 @@ static_assert(sizeof(WorkspaceCtrl) <= LINATTN_WORKSPACE_CTRL_BYTES, "control bl
 
 // A kernel launched with this may be set up while the one before it in the stream is still running (programmatic dependent
 // launch); nothing that it does to memory stands before its wait_for_prior_grids().  That takes the launch, and what a kernel
-// does before its first load (barriers, tensor memory, zeros), off the time of calls in a row: back to back, forward of 192
+// does before its first load (barriers, zeros), off the time of calls in a row: back to back, forward of 192
 // tokens, 4 heads of 32 12.3 -> 10.0 us, rotary read-only step of 4680 tokens 38.8 -> 35.6, temporal convolution of three 480p
 // frames 14.3 -> 11.6, bf16 read-only step of 114 tokens, 56 heads of 40 (two kernels) 18.4 -> 13.1.  Cooperative kernels, which
 // fill the chip, do not gain by it; fma_state_reduce neither (see there).
@@ -52,6 +52,9 @@ cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 #ifdef __CUDACC__
+// Tensor memory is allocated between the two calls below: behind the wait, since a CTA of the grid before that is on the same SM and has
+// yet to allocate its own would wait for this one, which waits for it; and before the next grid may start, for the same reason.
+//
 // All grids before this one in the stream are complete and what they wrote is seen.  (Loads that the compiler takes for free to
 // move, __ldg and through __restrict__, want a pointer from behind_wait.)
 __device__ __forceinline__ void wait_for_prior_grids() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -326,9 +326,8 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   }
   // padded features are never written and must read as zero
   for (int i = tid; i < 2 * S::STAGE / 16; i += kBlock) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-  if (warp == 0) { tmem_alloc(tmem_holder, S::COLS); tmem_relinquish(); }
-  let_next_grid_start();
   wait_for_prior_grids();
+  if (warp == 0) { tmem_alloc(tmem_holder, S::COLS); tmem_relinquish(); }
 
   // preparing: this thread's row of every tile, and its pieces of it, features feature(0), feature(1), ...
   const int row = (tid % kPrepare) / S::LANES, l = tid % S::LANES;
@@ -400,6 +399,7 @@ split_state_kernel(const T* __restrict__ k, const T* __restrict__ v, Problem p, 
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
+  let_next_grid_start();
   const uint32_t tmem = *tmem_holder;
 
   // draining: accumulator lane = key feature; each of the two warps of a lane quarter takes half of the value features
@@ -635,7 +635,6 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   const int tiles = (int)((blockIdx.x + 1) * all / gridDim.x - first);
   // (Waited for here and not behind the barriers' and tensor memory's set-up: the first pieces were asked for later then, and with more
   // registers spilled in the loops the pass took 168 us and not 159; at the start of the kernel without an early start, 161.)
-  let_next_grid_start();
   wait_for_prior_grids();
   const float* W = behind_wait(state) + (long long)u * p.state_elems();
   const long long base = (long long)(u / p.H) * p.sb + (long long)(u % p.H) * p.sh;
@@ -697,6 +696,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
+  let_next_grid_start();
   const uint32_t tmem = *tmem_holder;
 
   if (preparing) {

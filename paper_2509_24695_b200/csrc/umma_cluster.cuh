@@ -135,12 +135,12 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     prefetch_tensormap(&map_k);
     prefetch_tensormap(&map_v);
   }
-  if (warp == 1) { tmem_alloc(tmem_holder, kTmemCols); tmem_relinquish(); }
-  let_next_grid_start();
   wait_for_prior_grids();
+  if (warp == 1) { tmem_alloc(tmem_holder, kTmemCols); tmem_relinquish(); }
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
+  let_next_grid_start();
   const uint32_t tmem_base = *tmem_holder;
   cluster_arrive();   // the peers' barriers are set up: waited for before the first access to a peer
 

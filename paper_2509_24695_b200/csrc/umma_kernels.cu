@@ -1272,11 +1272,12 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     }
     fence_proxy_async_smem();
   }
+  if (SOLO) wait_for_prior_grids();
   if (warp == 1) { tmem_alloc(tmem_holder, kTmemCols); tmem_relinquish(); }
-  if (SOLO) { let_next_grid_start(); wait_for_prior_grids(); }
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
+  if (SOLO) let_next_grid_start();
   const uint32_t tmem_base = *tmem_holder;
 
   // apply-pass producer state lives across the grid barriers (the first tiles are fetched before them)
