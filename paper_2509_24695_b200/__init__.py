@@ -131,7 +131,7 @@ def load_library(path: str | None = None):
 
 
 # The short way (csrc/binding.cpp): the calls of one layer, on plain tensors.  Each function answers NotImplemented for what it
-# does not take, and the general way below goes on.
+# does not take, before it calls the library, and the general way below goes on.
 _fast = None
 _FAST_CALLS = ("linattn_forward", "linattn_forward_rope", "blocklin_step", "blocklin_peek", "blocklin_step_rope", "blocklin_peek_rope",
                "tconv_forward", "tconv_block_step")
@@ -156,7 +156,7 @@ def _bind(lib):
     except ImportError:
         _fast = _NoBinding
     else:
-        _binding.bind(*(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _FAST_CALLS))
+        _binding.bind(_check, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _FAST_CALLS))
         _fast = _binding
     return _fast
 

@@ -2,8 +2,8 @@
 //
 // With few tokens a call's time is the time its arguments take: in Python, tensor by tensor and through ctypes, 9.4 us a call, of which the
 // launch is 2.6.  Here the same checks read the tensors' fields.  Only the plain case is taken: exact torch.Tensor arguments, dense memory
-// on a CUDA device, no mode or transform that wants to see torch functions.  Anything else, and anything the library
-// refuses, answers NotImplemented, and the caller goes the general way, which says what is wrong.  Time to issue a call, before and after, us:
+// on a CUDA device, no mode or transform that wants to see torch functions.  Anything else answers NotImplemented before the library is called,
+// and the caller goes the general way, which says what is wrong.  Time to issue a call, before and after, us:
 // forward of 192 tokens 9.4 -> 5.1, cached step 9.7 -> 5.9, rotary read-only step 10.3 -> 5.4, temporal convolution step 9.0 -> 4.6 (which is then
 // all that one of a few hundred positions takes: 9.0 -> 4.3).
 #include <torch/csrc/Exceptions.h>
@@ -27,6 +27,7 @@ decltype(&blocklin_step_rope) p_step_rope;
 decltype(&blocklin_peek_rope) p_peek_rope;
 decltype(&tconv_forward) p_tconv_forward;
 decltype(&tconv_block_step) p_tconv_step;
+PyObject* p_failed;   // failed(status, where): raises what the library's status means
 
 PyObject* general() { Py_RETURN_NOTIMPLEMENTED; }
 
@@ -78,8 +79,15 @@ bool output(PyObject* out, const at::Tensor& like, at::Tensor* o) {
   return true;
 }
 
-PyObject* answer(int status, PyObject* out, at::Tensor&& o) {
-  if (status != LINATTN_OK) return general();
+// What the library answered.  It has been called, and is not called again: a call that commits a block and takes several launches may
+// have done so before it failed.
+PyObject* answer(int status, const char* where, PyObject* out, at::Tensor&& o) {
+  if (status != LINATTN_OK) {
+    PyObject* none = PyObject_CallFunction(p_failed, "is", status, where);
+    if (!none) return nullptr;
+    Py_DECREF(none);
+    return PyErr_Format(PyExc_SystemError, "%s: status %d", where, status);
+  }
   if (out != Py_None) { Py_INCREF(out); return out; }
   return THPVariable_Wrap(std::move(o));
 }
@@ -97,7 +105,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   Py_BEGIN_ALLOW_THREADS
   st = p_forward(&d, q->size(1), q->data_ptr(), k->data_ptr(), v->data_ptr(), o.data_ptr(), eps, ws->data_ptr(), (size_t)ws->numel(), stream_of(*q));
   Py_END_ALLOW_THREADS
-  return answer(st, a[4], std::move(o));
+  return answer(st, "linattn_forward", a[4], std::move(o));
   END_HANDLE_TH_ERRORS
 }
 
@@ -117,7 +125,7 @@ PyObject* forward_rope(PyObject*, PyObject* const* a, Py_ssize_t n) {
   st = p_forward_rope(&d, q->size(1), q->data_ptr(), k->data_ptr(), v->data_ptr(), o.data_ptr(), eps, table->data_ptr(), ws->data_ptr(), (size_t)ws->numel(),
                       stream_of(*q));
   Py_END_ALLOW_THREADS
-  return answer(st, a[5], std::move(o));
+  return answer(st, "linattn_forward_rope", a[5], std::move(o));
   END_HANDLE_TH_ERRORS
 }
 
@@ -140,7 +148,7 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (table) st = (commit ? p_step_rope : p_peek_rope)(cache, T, pq, pk, pv, o.data_ptr(), table->data_ptr(), stream_of(*k));
   else st = (commit ? p_step : p_peek)(cache, T, pq, pk, pv, o.data_ptr(), stream_of(*k));
   Py_END_ALLOW_THREADS
-  return answer(st, a[10], std::move(o));
+  return answer(st, table ? (commit ? "blocklin_step_rope" : "blocklin_peek_rope") : commit ? "blocklin_step" : "blocklin_peek", a[10], std::move(o));
   END_HANDLE_TH_ERRORS
 }
 
@@ -166,16 +174,18 @@ PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (frame) st = p_tconv_step(&d, T, x->data_ptr(), w->data_ptr<float>(), frame->data_ptr(), y.data_ptr(), commit, stream_of(*x));
   else st = p_tconv_forward(&d, T, x->data_ptr(), w->data_ptr<float>(), y.data_ptr(), stream_of(*x));
   Py_END_ALLOW_THREADS
-  return answer(st, a[2], std::move(y));
+  return answer(st, frame ? "tconv_block_step" : "tconv_forward", a[2], std::move(y));
   END_HANDLE_TH_ERRORS
 }
 
-// bind(addresses of forward, forward_rope, step, peek, step_rope, peek_rope, tconv_forward, tconv_block_step)
+// bind(failed, addresses of forward, forward_rope, step, peek, step_rope, peek_rope, tconv_forward, tconv_block_step)
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  if (n != 8) return PyErr_Format(PyExc_TypeError, "eight addresses");
+  if (n != 9 || !PyCallable_Check(a[0])) return PyErr_Format(PyExc_TypeError, "what raises an error, and eight addresses");
   void* p[8];
   for (int i = 0; i < 8; ++i)
-    if (!(p[i] = PyLong_AsVoidPtr(a[i]))) return PyErr_Occurred() ? nullptr : PyErr_Format(PyExc_ValueError, "an address is null");
+    if (!(p[i] = PyLong_AsVoidPtr(a[1 + i]))) return PyErr_Occurred() ? nullptr : PyErr_Format(PyExc_ValueError, "an address is null");
+  Py_INCREF(a[0]);
+  Py_XSETREF(p_failed, a[0]);
   p_forward = reinterpret_cast<decltype(p_forward)>(p[0]);
   p_forward_rope = reinterpret_cast<decltype(p_forward_rope)>(p[1]);
   p_step = reinterpret_cast<decltype(p_step)>(p[2]);

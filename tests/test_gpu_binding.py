@@ -1,5 +1,8 @@
 """The short way from torch tensors to the library (csrc/binding.cpp) against the general one: the same results, and whatever it does
 not take ends where the general way ends."""
+import ctypes
+import types
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -116,3 +119,40 @@ def test_modes_see_the_allocation():
         with mode():
             la.linattn_forward(q, k, v, workspace=ws)
         assert any("empty_like" in str(f) for f in seen)
+
+
+@pytest.mark.parametrize("name", la._FAST_CALLS)
+def test_a_failed_call_is_not_made_again(name, monkeypatch):
+    """A call that commits a block may have done so before it failed (its second launch, say): one call to the library, one error.
+    Stand-ins for the library's functions fail the first time only, so a second try would pass unseen; nothing is launched."""
+    lib, made = la.load_library(), []
+
+    def fails_once(*args):
+        made.append(name)
+        return -5 if len(made) == 1 else 0
+
+    callback = ctypes.CFUNCTYPE(ctypes.c_int, *(t if isinstance(t, type) and issubclass(t, ctypes._SimpleCData) else ctypes.c_void_p
+                                                for t in getattr(lib, name).argtypes))(fails_once)
+    stand_in = types.SimpleNamespace(**{n: callback if n == name else getattr(lib, n) for n in la._FAST_CALLS})
+    q, k, v = qkv(1, 40, 2, 64)
+    tab = torch.zeros(40, 32, 2, dtype=torch.float16, device="cuda")
+    x, w = q.view(1, 4, 10, 128), torch.zeros(3, 128, device="cuda")
+    cache = la.BlockLinCache(1, 2, 64, torch.bfloat16, "cuda", max_T_b=40)
+    conv = la.TConvCache(1, 10, 128, torch.bfloat16, "cuda")
+    ws, rope_ws = la.new_workspace(q), la.new_rope_workspace(q)
+    call = {"linattn_forward": lambda: la.linattn_forward(q, k, v, workspace=ws),
+            "linattn_forward_rope": lambda: la.linattn_forward_rope(q, k, v, tab, workspace=rope_ws),
+            "blocklin_step": lambda: cache.step(q, k, v), "blocklin_peek": lambda: cache.peek(q, k, v),
+            "blocklin_step_rope": lambda: cache.step_rope(q, k, v, tab), "blocklin_peek_rope": lambda: cache.peek_rope(q, k, v, tab),
+            "tconv_forward": lambda: la.tconv_forward(x, w), "tconv_block_step": lambda: conv.step(x, w)}[name]
+    monkeypatch.setattr(lib, name, fails_once)   # (for the general way)
+    try:
+        la._bind(stand_in)
+        assert la._fast is not la._NoBinding, "the binding is not built"
+        with pytest.raises(la.LinAttnError, match=f"^{name}: .*status -5"):
+            call()
+        assert made == [name]
+        assert call() is not None and made == [name, name]   # (and the next call is a call like any other)
+    finally:
+        monkeypatch.undo()
+        la._bind(lib)
