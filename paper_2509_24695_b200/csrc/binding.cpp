@@ -92,6 +92,9 @@ PyObject* answer(int status, const char* where, PyObject* out, at::Tensor&& o) {
   return THPVariable_Wrap(std::move(o));
 }
 
+// In the calls below pointers and streams are taken before the interpreter's lock is let go: taking them may throw, and what is thrown becomes a
+// Python error.
+
 // forward(q, k, v, eps, out, workspace)
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
@@ -101,9 +104,13 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
   at::Tensor o;
   if (!q || !k || !v || !ws || !describe(*q, &d) || !same(*k, *q) || !same(*v, *q) || ws->scalar_type() != at::kByte || !output(a[4], *q, &o)) return general();
   const float eps = (float)PyFloat_AS_DOUBLE(a[3]);
+  const int64_t N = q->size(1);
+  const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr();
+  void *po = o.data_ptr(), *pw = ws->data_ptr(), *stream = stream_of(*q);
+  const size_t room = (size_t)ws->numel();
   int st;
   Py_BEGIN_ALLOW_THREADS
-  st = p_forward(&d, q->size(1), q->data_ptr(), k->data_ptr(), v->data_ptr(), o.data_ptr(), eps, ws->data_ptr(), (size_t)ws->numel(), stream_of(*q));
+  st = p_forward(&d, N, pq, pk, pv, po, eps, pw, room, stream);
   Py_END_ALLOW_THREADS
   return answer(st, "linattn_forward", a[4], std::move(o));
   END_HANDLE_TH_ERRORS
@@ -120,10 +127,13 @@ PyObject* forward_rope(PyObject*, PyObject* const* a, Py_ssize_t n) {
       ws->scalar_type() != at::kByte || !output(a[5], *q, &o))
     return general();
   const float eps = (float)PyFloat_AS_DOUBLE(a[4]);
+  const int64_t N = q->size(1);
+  const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr(), *pt = table->data_ptr();
+  void *po = o.data_ptr(), *pw = ws->data_ptr(), *stream = stream_of(*q);
+  const size_t room = (size_t)ws->numel();
   int st;
   Py_BEGIN_ALLOW_THREADS
-  st = p_forward_rope(&d, q->size(1), q->data_ptr(), k->data_ptr(), v->data_ptr(), o.data_ptr(), eps, table->data_ptr(), ws->data_ptr(), (size_t)ws->numel(),
-                      stream_of(*q));
+  st = p_forward_rope(&d, N, pq, pk, pv, po, eps, pt, pw, room, stream);
   Py_END_ALLOW_THREADS
   return answer(st, "linattn_forward_rope", a[5], std::move(o));
   END_HANDLE_TH_ERRORS
@@ -142,11 +152,12 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   auto* cache = static_cast<blocklin_cache*>(PyLong_AsVoidPtr(a[1]));
   const bool commit = a[0] == Py_True;
   const int64_t T = k->size(1);
-  const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr();
+  const void *pq = q->data_ptr(), *pk = k->data_ptr(), *pv = v->data_ptr(), *pt = table ? table->data_ptr() : nullptr;
+  void *po = o.data_ptr(), *stream = stream_of(*k);
   int st;
   Py_BEGIN_ALLOW_THREADS
-  if (table) st = (commit ? p_step_rope : p_peek_rope)(cache, T, pq, pk, pv, o.data_ptr(), table->data_ptr(), stream_of(*k));
-  else st = (commit ? p_step : p_peek)(cache, T, pq, pk, pv, o.data_ptr(), stream_of(*k));
+  if (table) st = (commit ? p_step_rope : p_peek_rope)(cache, T, pq, pk, pv, po, pt, stream);
+  else st = (commit ? p_step : p_peek)(cache, T, pq, pk, pv, po, stream);
   Py_END_ALLOW_THREADS
   return answer(st, table ? (commit ? "blocklin_step_rope" : "blocklin_peek_rope") : commit ? "blocklin_step" : "blocklin_peek", a[10], std::move(o));
   END_HANDLE_TH_ERRORS
@@ -169,10 +180,13 @@ PyObject* conv(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const tconv_desc d{(int32_t)x->size(0), (int32_t)x->size(2), (int32_t)x->size(3), dtype_of(*x), 0, 0};
   const int commit = a[4] == Py_True;
   const int64_t T = x->size(1);
+  const void* px = x->data_ptr();
+  const float* taps = w->data_ptr<float>();
+  void *pf = frame ? frame->data_ptr() : nullptr, *py = y.data_ptr(), *stream = stream_of(*x);
   int st;
   Py_BEGIN_ALLOW_THREADS
-  if (frame) st = p_tconv_step(&d, T, x->data_ptr(), w->data_ptr<float>(), frame->data_ptr(), y.data_ptr(), commit, stream_of(*x));
-  else st = p_tconv_forward(&d, T, x->data_ptr(), w->data_ptr<float>(), y.data_ptr(), stream_of(*x));
+  if (frame) st = p_tconv_step(&d, T, px, taps, pf, py, commit, stream);
+  else st = p_tconv_forward(&d, T, px, taps, py, stream);
   Py_END_ALLOW_THREADS
   return answer(st, frame ? "tconv_block_step" : "tconv_forward", a[2], std::move(y));
   END_HANDLE_TH_ERRORS

@@ -156,3 +156,28 @@ def test_a_failed_call_is_not_made_again(name, monkeypatch):
     finally:
         monkeypatch.undo()
         la._bind(lib)
+
+
+@pytest.mark.parametrize("which", ["q", "k", "v", "out", "table", "ws", "x", "w", "frame"])
+def test_a_pointer_that_cannot_be_had_is_an_error(which):
+    """Memory that throws when it is asked for (here because it is told to) ends in Python's error, as the general way."""
+    q, k, v = qkv(1, 40, 2, 64)
+    t = {"q": q, "k": k, "v": v, "out": torch.empty_like(q), "table": torch.zeros(40, 32, 2, dtype=torch.float16, device="cuda"),
+         "ws": la.new_rope_workspace(q), "x": q.clone().view(1, 4, 10, 128), "w": torch.zeros(3, 128, device="cuda")}
+    conv = la.TConvCache(1, 10, 128, torch.bfloat16, "cuda")
+    cache = la.BlockLinCache(1, 2, 64, torch.bfloat16, "cuda", max_T_b=40)
+    t["frame"] = conv.frame
+    calls = {"attention": [lambda: la.linattn_forward(t["q"], t["k"], t["v"], out=t["out"], workspace=t["ws"]),
+                           lambda: la.linattn_forward_rope(t["q"], t["k"], t["v"], t["table"], out=t["out"], workspace=t["ws"]),
+                           lambda: cache.step(t["q"], t["k"], t["v"], out=t["out"]),
+                           lambda: cache.peek_rope(t["q"], t["k"], t["v"], t["table"], out=t["out"])],
+             "conv": [lambda: la.tconv_forward(t["x"], t["w"]), lambda: conv.step(t["x"], t["w"])]}
+    takes = {"table": [1, 3], "ws": [0, 1], "frame": [1]}.get(which, range(4))
+    torch._C._set_throw_on_mutable_data_ptr(t[which])
+    for i, call in enumerate(calls["conv" if which in ("x", "w", "frame") else "attention"]):
+        if i in takes:
+            with pytest.raises(RuntimeError, match="data pointer"):
+                call()
+        else:
+            call()
+    torch.cuda.synchronize()
