@@ -2267,22 +2267,40 @@ int cluster_ctas(const Problem& p) {
   return cluster_size<D, ROPE>(p, p.B * ((p.H + Cfg<D>::G - 1) / Cfg<D>::G), (p.N + kTileState - 1) / kTileState, sms);
 }
 
-// One launch for all blocks, or a state launch, prefix_states and an apply launch?  A thread of reduce_prefix walks the records of all blocks
-// of its piece, CTAs / head groups of them, eight at a time; from some 70 on that is longer than what it saves.  One launch / three, us:
-//                       tokens a block    64         128        192        300        600        1200       2400
-//   d = 112, 20 groups, 2 blocks          18.6/22.6  18.6/26.7  16.5/25.1  17.1/26.7  18.6/26.9  20.6/28.5  24.0/31.1
-//             2                           18.5/22.6  17.3/26.3  16.5/24.7  16.5/24.9  18.6/24.8  20.6/25.0  22.7/25.7
-//            20         7                 18.6/28.8  18.6/30.8  20.6/32.9  22.8/35.4  31.0/45.3  45.4/59.7  68.7/84.5
-//             2         7                 16.5/24.7  16.9/28.8  18.6/26.8  20.6/28.4  26.8/28.8  27.3/28.3  29.4/31.2   (74 records from 1200)
-//             1         7                 16.1/23.7  16.5/27.7  18.6/26.7  20.6/27.9  26.6/27.8  36.4/27.8  37.0/27.9   (35, 70, 133, 148 from 300)
-//   d = 64,  18         2                 18.6/22.7  16.5/24.7  16.5/24.7  18.5/24.7  20.3/24.7  21.5/28.8  24.7/30.9
-//             2         7                 17.1/22.9  18.5/25.2  18.6/26.8  22.4/26.7  27.0/26.7  28.8/29.3  30.9/28.5
-//   d = 32,   2         7                 16.5/22.6  16.5/24.7  18.6/22.7  20.6/22.6  26.7/23.9  26.8/25.6  28.9/26.8
-//   d = 128, 20         7                 18.6/28.8  20.5/30.9  20.7/37.0  24.8/39.1  35.1/51.7  50.0/66.4  78.4/95.0
+// One launch for all blocks, or a state launch, prefix_states and an apply launch?
+//
+// One launch where the grid takes the blocks' state anyway.  Lone CTAs and clusters keep their chains of the tensor core's additions at one and two, in
+// the grid they are as long as a CTA has tiles: blocks that the former take would get sums further from 64 bits, and others than the
+// same call without queries gives.  S, relative, one launch / three: 2 blocks of 2304 tokens, 20 heads of 112 1.20e-7 / 8.8e-8, 4 of 900, 35 heads of 64
+// 1.10e-7 / 8.0e-8, 7 of 128, 70 heads of 32 7.1e-8 / 6.8e-8; never the other way round.  (One launch would be the faster one there: 18.6 / 28.8 us
+// for 7 blocks of 64 tokens, 20 heads of 112.)
+//
+// And not for few heads: a thread of reduce_prefix walks the records of all blocks of its piece, CTAs / head groups of them, eight at a
+// time.  The line is at 64 for every head dim; at 70 to 74 heads of 112 still gain, packed heads lose.  One launch / three, us:
+//                       tokens a block    300        600        1200       2400
+//   d = 112, 20 groups, 7 blocks          22.8/35.4  31.0/45.3  45.4/59.7  68.7/84.5
+//             2         2                 16.5/24.9  18.6/24.8  20.6/25.0  22.7/25.7   (74 records at 2400)
+//             2         7                 20.6/28.4  26.8/28.8  27.3/28.3  29.4/31.2   (35, 70, 74, 74)
+//             1         7                 20.6/27.9  26.6/27.8  36.4/27.8  37.0/27.9   (35, 70, 133, 148)
+//   d = 64,   2         7                 22.4/26.7  27.0/26.7  28.8/29.3  30.9/28.5   (35, 70, 74, 74)
+//   d = 32,   2         7                 20.6/22.6  26.7/23.9  26.8/25.6  28.9/26.8   (35, 70, 74, 74)
+//   d = 128, 20         7                 24.8/39.1  35.1/51.7  50.0/66.4  78.4/95.0
+template <int D>
+bool joins_prefill(const Problem& p, int blocks) {
+  const int sms = sm_count(), hg = (p.H + Cfg<D>::G - 1) / Cfg<D>::G;
+  if (!sms || cluster_ctas<D, false>(p) || solo_pays(p, p.B * hg, sms)) return false;   // (an error here is the state launch's to report)
+  const long long groups = (long long)(p.B / blocks) * hg, tiles = groups * blocks * ((p.N + kTileState - 1) / kTileState);
+  return (tiles < sms ? tiles : sms) <= 64 * groups;
+}
+
 bool umma_joins_prefill(const Problem& p, int blocks) {
-  const int sms = sm_count(), G = groups_of(p.d);
-  const long long groups = (long long)(p.B / blocks) * ((p.H + G - 1) / G), tiles = groups * blocks * ((p.N + kTileState - 1) / kTileState);
-  return sms && (tiles < sms ? tiles : sms) <= 64 * groups;
+  switch (p.d) {
+    case 32: return joins_prefill<32>(p, blocks);
+    case 64: return joins_prefill<64>(p, blocks);
+    case 112: return joins_prefill<112>(p, blocks);
+    case 128: return joins_prefill<128>(p, blocks);
+  }
+  return false;
 }
 
 int umma_cluster_ctas(const Problem& p, bool rope) {

@@ -43,13 +43,15 @@ def test_prefill_is_its_parts(B, M, T, H, d):
 
 
 @pytest.mark.parametrize("B,M,T,H,d,launches", [
-    (1, 7, 64, 20, 112, 1),     # blocks that lone CTAs would take
-    (1, 3, 130, 1, 32, 1),
-    (2, 5, 700, 4, 112, 1),     # ... and clusters
-    (1, 2, 33, 3, 128, 1),
-    (1, 9, 1, 2, 64, 1),        # blocks of one token
+    (1, 7, 64, 20, 112, 3),     # blocks that lone CTAs take
+    (1, 3, 130, 1, 32, 3),
+    (2, 5, 700, 4, 112, 3),     # ... and clusters
+    (1, 2, 33, 3, 128, 3),
+    (1, 9, 1, 2, 64, 3),        # blocks of one token
     (1, 7, 600, 1, 112, 3),     # 70 records to a piece
     (1, 7, 1500, 2, 64, 3),
+    (1, 7, 300, 20, 112, 1),    # blocks that the grid takes
+    (1, 7, 257, 70, 32, 1),
 ])
 def test_prefill_of_small_blocks(B, M, T, H, d, launches):
     """Against the steps, block by block: other forms, so to rounding (both sums of S within 1e-6 of 64 bits, outputs bf16)."""
@@ -67,3 +69,22 @@ def test_prefill_of_small_blocks(B, M, T, H, d, launches):
     assert (got.float() - want.float()).abs().max() <= 2 ** -7 * want.float().abs().max()
     assert (got.float() - want.float()).norm() <= 1e-3 * want.float().norm()
     assert one.status() == 0
+
+
+@pytest.mark.parametrize("B,M,T,H,d", [(1, 7, 64, 20, 112), (1, 7, 128, 70, 32), (2, 3, 132, 20, 112), (1, 2, 192, 35, 64), (1, 3, 107, 6, 128),   # lone CTAs
+                                       (2, 5, 700, 4, 112), (1, 2, 2304, 20, 112), (1, 4, 900, 35, 64), (2, 7, 709, 9, 32),                    # clusters
+                                       (1, 7, 300, 20, 112), (1, 3, 1500, 18, 128)])                                                        # the grid
+def test_state_is_the_blocks_own(B, M, T, H, d):
+    """Whatever takes a block's state in the other calls on its shape takes it here: with queries and without the cache is what the states of
+    the blocks add up to, bit for bit, and as near to 64 bits."""
+    gen = torch.Generator(device="cuda").manual_seed(T + d)
+    q, k, v = (torch.randn(B, M * T, H, d, device="cuda", generator=gen).bfloat16() for _ in range(3))
+    own = la.linattn_state(k.view(B * M, T, H, d), v.view(B * M, T, H, d)).view(B, M, H, d + 1, d)
+    want = torch.zeros_like(own[:, 0])
+    for m in range(M):
+        want = want + own[:, m]
+    for queries in (q, None):
+        cache = la.BlockLinCache(B, H, d, torch.bfloat16, "cuda", max_T_b=T, prefill_blocks=M)
+        cache.reset()
+        cache.prefill(queries, k, v, M)
+        assert torch.equal(cache.state, want)
