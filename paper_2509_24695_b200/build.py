@@ -1,5 +1,6 @@
-"""Builds the C-ABI shared library (``liblinattn.so``) in-tree with nvcc for sm_100a, and ``_binding.so``, the short way of the
-Python calls to it, with g++ against the installed torch.
+"""Builds the C-ABI shared library (``liblinattn.so``) in-tree with nvcc for sm_100a, and ``_binding``, the short way of the
+Python calls to it, with g++ against the installed torch.  The library needs no torch: where the binding cannot be built (no torch, one
+without CUDA, no headers) a warning says so, and the calls go the general way.
 
     python -m paper_2509_24695_b200.build [--force] [--verbose]
 
@@ -24,6 +25,7 @@ LIB = os.path.join(PKG, "liblinattn.so")
 STAMP = os.path.join(PKG, "_build", "stamp")
 BINDING_SRC = os.path.join(CSRC, "binding.cpp")
 BINDING = os.path.join(PKG, "_binding.so")
+WITHOUT_BINDING = " without binding"   # in the stamp of a build whose binding failed
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -66,10 +68,38 @@ def _fingerprint() -> str:
     return h.hexdigest()
 
 
+def _start_binding(out: str):
+    """(the compiler at work on the binding, or why there is none; the command; its output file)."""
+    cmd = _binding_command(out)
+    if cmd is None:
+        return "no torch is installed", [], out
+    try:
+        return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True), cmd, out
+    except OSError as e:
+        return str(e), cmd, out
+
+
+def _finish_binding(compiler, cmd, out, verbose) -> bool:
+    """Puts the binding in place; False where it could not be built (an older one, of other sources or another torch, then goes too)."""
+    text = compiler if isinstance(compiler, str) else compiler.communicate()[0]
+    ok = not isinstance(compiler, str) and compiler.returncode == 0
+    if cmd and (verbose or not ok):
+        sys.stderr.write(" ".join(cmd) + "\n" + text + "\n")
+    if ok:
+        os.replace(out, BINDING)
+        return True
+    sys.stderr.write("warning: the short way from torch tensors to the library is not built; calls take the general way\n")
+    for stale in (out, BINDING):
+        if os.path.exists(stale):
+            os.remove(stale)
+    return False
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu under csrc/ into liblinattn.so (skipped when sources are unchanged)."""
     fp = _fingerprint()
-    if not force and os.path.exists(LIB) and (os.path.exists(BINDING) or _torch_dir() is None) and os.path.exists(STAMP) and open(STAMP).read() == fp:
+    built = fp if os.path.exists(BINDING) else fp + WITHOUT_BINDING
+    if not force and os.path.exists(LIB) and os.path.exists(STAMP) and open(STAMP).read() == built:
         return LIB
     os.makedirs(os.path.dirname(STAMP), exist_ok=True)
     objs = []
@@ -82,10 +112,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(2, "-v")
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
-    binding_tmp = BINDING + f".tmp{os.getpid()}"
-    binding_cmd = _binding_command(binding_tmp)
-    if binding_cmd:
-        procs.append((binding_cmd, subprocess.Popen(binding_cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    binding = _start_binding(BINDING + f".tmp{os.getpid()}")
     failed = False
     for cmd, p in procs:
         out, _ = p.communicate()
@@ -98,10 +125,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call(["nvcc", "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs,
                            "-Xlinker", "--exclude-libs=ALL"])
     os.replace(tmp, LIB)
-    if binding_cmd:
-        os.replace(binding_tmp, BINDING)
+    built = fp if _finish_binding(*binding, verbose) else fp + WITHOUT_BINDING
     with open(STAMP, "w") as f:
-        f.write(fp)
+        f.write(built)
     return LIB
 
 
