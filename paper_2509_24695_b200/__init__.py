@@ -138,7 +138,7 @@ _FAST_CALLS = ("linattn_forward", "linattn_forward_rope", "blocklin_step", "bloc
 
 
 class _NoBinding:
-    """In the place of the binding where it is not built (another torch than the one it was built against)."""
+    """In the place of the binding where there is none for this torch and this Python."""
 
     @staticmethod
     def forward(*args):
@@ -148,12 +148,14 @@ class _NoBinding:
 
 
 def _bind(lib):
-    """The short way to `lib`."""
+    """The short way to `lib`.  The binding reads torch's structures where the torch that it was built against has them."""
     global _fast
-    _torch()
+    torch = _torch()
     try:
         from . import _binding
     except ImportError:
+        _binding = None
+    if getattr(_binding, "built_against", None) != str(torch.__version__):
         _fast = _NoBinding
     else:
         _binding.bind(_check, *(ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _FAST_CALLS))

@@ -14,6 +14,7 @@ import glob
 import hashlib
 import importlib.util
 import os
+import runpy
 import subprocess
 import sys
 import sysconfig
@@ -24,7 +25,7 @@ CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "liblinattn.so")
 STAMP = os.path.join(PKG, "_build", "stamp")
 BINDING_SRC = os.path.join(CSRC, "binding.cpp")
-BINDING = os.path.join(PKG, "_binding.so")
+BINDING = os.path.join(PKG, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))   # (another Python does not see it)
 WITHOUT_BINDING = " without binding"   # in the stamp of a build whose binding failed
 
 NVCC_FLAGS = [
@@ -45,25 +46,30 @@ def _torch_dir() -> str | None:
     return os.path.dirname(spec.origin) if spec and spec.origin else None
 
 
+def _torch_version() -> str | None:
+    """``torch.__version__`` of the torch that is installed, not imported."""
+    path = os.path.join(_torch_dir() or "", "version.py")
+    return runpy.run_path(path)["__version__"] if os.path.exists(path) else None
+
+
 def _binding_command(out: str) -> list[str] | None:
-    torch = _torch_dir()
-    if torch is None:
+    torch, version = _torch_dir(), _torch_version()
+    if version is None:
         return None
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     include = [os.path.join(ROOT, "include"), os.path.join(torch, "include"), os.path.join(torch, "include", "torch", "csrc", "api", "include"),
                sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
-    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", *(f"-I{i}" for i in include), BINDING_SRC, "-o", out,
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", f'-DBUILT_AGAINST="{version}"', *(f"-I{i}" for i in include), BINDING_SRC, "-o", out,
             f"-L{os.path.join(torch, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
 def _fingerprint() -> str:
     h = hashlib.sha256()
     files = sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + sorted(glob.glob(os.path.join(ROOT, "include", "*.h"))) + [BINDING_SRC]
-    if _torch_dir():
-        files.append(os.path.join(_torch_dir(), "version.py"))
     for f in files:
         h.update(f.encode())
         h.update(open(f, "rb").read())
+    h.update(f"{_torch_version()} {sys.version_info[:2]}".encode())
     h.update(" ".join(NVCC_FLAGS).encode())
     return h.hexdigest()
 

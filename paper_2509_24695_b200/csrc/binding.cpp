@@ -217,4 +217,11 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding() { return PyModule_Create(&module); }
+#ifndef BUILT_AGAINST
+#error "the version of the torch that this is built against"
+#endif
+PyMODINIT_FUNC PyInit__binding() {
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "built_against", BUILT_AGAINST) < 0) Py_CLEAR(m);
+  return m;
+}

@@ -1,9 +1,11 @@
-"""The build where the binding cannot be had."""
+"""The build where the binding cannot be had, and a binding that was built against another torch."""
 import subprocess
 import sys
+import types
 
 import pytest
 
+import paper_2509_24695_b200 as la
 from paper_2509_24695_b200 import build
 
 
@@ -40,3 +42,15 @@ def test_the_library_is_built_without_the_binding(tree, command, monkeypatch, ca
     assert build.build() and len(links) == 2
     (folder / "binding.so").unlink()                               # lost: built again
     assert build.build() and (folder / "binding.so").exists() and len(links) == 3
+
+
+@pytest.mark.parametrize("other", [{}, {"built_against": "1.0.0"}], ids=str)
+def test_a_binding_of_another_torch_is_left_alone(other, monkeypatch):
+    def bind(*args):
+        raise AssertionError("bound")
+
+    module = types.SimpleNamespace(bind=bind, **other)
+    monkeypatch.setitem(sys.modules, la.__name__ + "._binding", module)
+    monkeypatch.setattr(la, "_binding", module, raising=False)
+    monkeypatch.setattr(la, "_fast", None)
+    assert la._bind(None) is la._NoBinding
