@@ -55,8 +55,8 @@ cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 // Tensor memory is allocated between the two calls below: behind the wait, since a CTA of the grid before that is on the same SM and has
 // yet to allocate its own would wait for this one, which waits for it; and before the next grid may start, for the same reason.
 //
-// All grids before this one in the stream are complete and what they wrote is seen.  (Loads that the compiler takes for free to
-// move, __ldg and through __restrict__, want a pointer from behind_wait.)
+// All grids before this one in the stream are complete and what they wrote is seen.  (Loads that the compiler may take for free to
+// move, __ldg, __ldcg and __ldcs, want a pointer from behind_wait; copies, bulk copies and what functions that are not inlined load stay where they are.)
 __device__ __forceinline__ void wait_for_prior_grids() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename T>
 __device__ __forceinline__ T* behind_wait(T* p) {

@@ -702,6 +702,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
   if (preparing) {
     // denominators from z_max 2^-50 to z_max 2^35: rows of queries from 2^-57 to 2^35, products with S from 2^-132 to 2^125
     float z_max = 0.f;
+    const __half2* const turns = behind_wait(tab);
     for (int i = lane; i < d; i += 32) z_max = fmaxf(z_max, fabsf(zs[i]));
 #pragma unroll
     for (int st = 1; st < 32; st *= 2) z_max = fmaxf(z_max, __shfl_xor_sync(0xffffffffu, z_max, st));
@@ -714,7 +715,7 @@ split_apply_kernel(const T* __restrict__ q, const float* __restrict__ state, T* 
         const long long n = (first + t) * A::TOK + row;
 #pragma unroll
         for (int i = 0; i < PIECES; ++i)
-          if (feature(i) < d) tb[i] = __ldg(reinterpret_cast<const Tab*>(tab + (n < p.N ? n : 0) * (d / 2) + feature(i) / 2));
+          if (feature(i) < d) tb[i] = __ldg(reinterpret_cast<const Tab*>(turns + (n < p.N ? n : 0) * (d / 2) + feature(i) / 2));
       }
       copy_wait<A::RAW_STAGES - 1>();
 #pragma unroll

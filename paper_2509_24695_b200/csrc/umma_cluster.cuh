@@ -240,15 +240,16 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     for (int e = 0; e < 8; ++e) zacc[e] = make_float2(0.f, 0.f);
     // rotary variant: this role takes box 0 and half the rows of box 1, the epilogue the other half; rotations one tile ahead
     uint4 tab0[kTileState / 32], tab1;
+    const uint4* const rope = ROPE ? behind_wait(p.rope) : nullptr;
     auto fetch_rot = [&](int tile, int i) {
       const long long m = (long long)tile * kTileState + row0 + 32 * i;
       tab0[i] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
       if (i == 0) tab1 = tab0[i];
       if (m < p.N) {
-        tab0[i] = __ldg(p.rope + m * (D / 8) + C::tab_chunk(0, lc));
+        tab0[i] = __ldg(rope + m * (D / 8) + C::tab_chunk(0, lc));
         if (i == 0) {
           if (C::SAME_TAB) tab1 = tab0[0];
-          else if (box1_live) tab1 = __ldg(p.rope + m * (D / 8) + C::tab_chunk(1, lc));
+          else if (box1_live) tab1 = __ldg(rope + m * (D / 8) + C::tab_chunk(1, lc));
         }
       }
     };
@@ -303,7 +304,8 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         fence_proxy_async_smem();
       }
     }
-    const float z_old = z_owned && p.accumulate ? __ldcg(p.state_base + z_at()) : 0.f;
+    const float* const base = behind_wait(p.state_base);
+    const float z_old = z_owned && p.accumulate ? __ldcg(base + z_at()) : 0.f;
     if (!L::Z_LANE && ok) {
       leave_z(z_slots, zacc, tr, lc, box1_live);
       mbar_arrive(z_left);
@@ -330,10 +332,11 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 #pragma unroll
       for (int e = 0; e < 4; ++e) zh[e] = make_float2(0.f, 0.f);
       uint4 tabh[2];
+      const uint4* const rope = ROPE ? behind_wait(p.rope) : nullptr;
       auto fetch_roth = [&](int tile, int i) {
         const long long m = (long long)tile * kTileState + 32 + row0h + 16 * i;
         tabh[i] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
-        if (h_live && m < p.N) tabh[i] = __ldg(p.rope + m * (D / 8) + C::tab_chunk(1, lch));
+        if (h_live && m < p.N) tabh[i] = __ldg(rope + m * (D / 8) + C::tab_chunk(1, lch));
       };
       if (!TAB) {
         fetch_roth(t0, 0);
@@ -491,6 +494,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     float4 acc[ITEMS][2];
     int j_of[ITEMS], q_of[ITEMS];
     size_t at_of[ITEMS];
+    const float* const base = behind_wait(p.state_base);
     bool live[ITEMS], held[ITEMS];   // held: a head there is, not padding of the group
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {   // the old state is asked for before the wait
@@ -502,8 +506,8 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
       at_of[k] = ((size_t)(b * p.H + h) * (D + 1) + il) * D + q * 8;
       acc[k][0] = acc[k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (p.accumulate && held[k]) {
-        acc[k][0] = __ldcg(reinterpret_cast<const float4*>(p.state_base + at_of[k]));
-        acc[k][1] = __ldcg(reinterpret_cast<const float4*>(p.state_base + at_of[k]) + 1);
+        acc[k][0] = __ldcg(reinterpret_cast<const float4*>(base + at_of[k]));
+        acc[k][1] = __ldcg(reinterpret_cast<const float4*>(base + at_of[k]) + 1);
       }
     }
 

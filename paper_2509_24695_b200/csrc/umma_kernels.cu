@@ -1373,15 +1373,16 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     // Of the second K box these warps take the first 32 token rows of a stage; the epilogue warps, idle until the
     // segment's accumulators are complete, take the other 32 (this role is what the pass waits for).
     uint4 tab0[kTileState / 32], tab1[1];
+    const uint4* const rope = SOLO && ROPE ? behind_wait(p.rope) : p.rope;
     auto fetch_rot = [&](int tile, int i) {
       const long long n = (long long)tile * kTileState + row0 + 32 * i;
       tab0[i] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
       if (i == 0) tab1[0] = tab0[i];
       if (n < p.N) {
-        tab0[i] = __ldg(p.rope + n * (D / 8) + C::tab_chunk(0, lc));
+        tab0[i] = __ldg(rope + n * (D / 8) + C::tab_chunk(0, lc));
         if (i == 0) {
           if (C::SAME_TAB) tab1[0] = tab0[0];
-          else if (box1_live) tab1[0] = __ldg(p.rope + n * (D / 8) + C::tab_chunk(1, lc));
+          else if (box1_live) tab1[0] = __ldg(rope + n * (D / 8) + C::tab_chunk(1, lc));
         }
       }
     };
@@ -1505,10 +1506,11 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 #pragma unroll
     for (int e = 0; e < 4; ++e) zh[e] = make_float2(0.f, 0.f);
     uint4 tabh[2];
+    const uint4* const rope = SOLO && ROPE ? behind_wait(p.rope) : p.rope;
     auto fetch_roth = [&](int tile, int j) {
       const long long n = (long long)tile * kTileState + 32 + row0h + 16 * j;
       tabh[j] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
-      if (h_live && n < p.N) tabh[j] = __ldg(p.rope + n * (D / 8) + C::tab_chunk(1, lch));
+      if (h_live && n < p.N) tabh[j] = __ldg(rope + n * (D / 8) + C::tab_chunk(1, lch));
     };
     if (ROPE && SOLO) {
       TileWalk t0(wa);
