@@ -304,8 +304,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         fence_proxy_async_smem();
       }
     }
-    const float* const base = behind_wait(p.state_base);
-    const float z_old = z_owned && p.accumulate ? __ldcg(base + z_at()) : 0.f;
+    const float z_old = z_owned && p.accumulate ? __ldcg(behind_wait(p.state_base) + z_at()) : 0.f;
     if (!L::Z_LANE && ok) {
       leave_z(z_slots, zacc, tr, lc, box1_live);
       mbar_arrive(z_left);
