@@ -240,7 +240,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     for (int e = 0; e < 8; ++e) zacc[e] = make_float2(0.f, 0.f);
     // rotary variant: this role takes box 0 and half the rows of box 1, the epilogue the other half; rotations one tile ahead
     uint4 tab0[kTileState / 32], tab1;
-    const uint4* const rope = ROPE ? behind_wait(p.rope) : nullptr;
+    const uint4* const rope = ROPE && !TAB ? behind_wait(p.rope) : nullptr;
     auto fetch_rot = [&](int tile, int i) {
       const long long m = (long long)tile * kTileState + row0 + 32 * i;
       tab0[i] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
@@ -331,7 +331,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 #pragma unroll
       for (int e = 0; e < 4; ++e) zh[e] = make_float2(0.f, 0.f);
       uint4 tabh[2];
-      const uint4* const rope = ROPE ? behind_wait(p.rope) : nullptr;
+      const uint4* const rope = ROPE && !TAB ? behind_wait(p.rope) : nullptr;
       auto fetch_roth = [&](int tile, int i) {
         const long long m = (long long)tile * kTileState + 32 + row0h + 16 * i;
         tabh[i] = make_uint4(kRopeIdentity, kRopeIdentity, kRopeIdentity, kRopeIdentity);
@@ -472,19 +472,7 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     cluster_wait();
   }
 
-  // Plain: the Q tiles that have come are clamped while the peers' sums are on their way, not behind the operand: 900 cycles of the
-  // 18 000 that a forward of 192 tokens, 4 heads of 32 takes.
-  int q_done = 0;   // of this warp of the ReLU role
-  if (!ROPE && warp >= 2 && warp < R::EPI_WARP0) {
-    const int most = n_apply < NSC ? n_apply : NSC;
-    for (int spin = 0; spin < 4096 && q_done < most && !__all_sync(0xffffffffu, mbar_test(x_full, 0)); ++spin) {
-      if (!__all_sync(0xffffffffu, mbar_test(&c_full[q_done], 0))) continue;
-      relu_pass<C::FEAT, kTileApply>(slots + q_done * SLOT, slots + q_done * SLOT + HALF, tr);
-      fence_proxy_async_smem();
-      mbar_arrive(&c_ready[q_done]);
-      ++q_done;
-    }
-  }
+  int q_done = 0;   // Q tiles that this warp of the ReLU role has clamped before the apply pass
 
   // ==================================================================== the rows this CTA owns: sum, state, apply operand
   if (warp >= 2 && warp < R::STORE_WARP) {
@@ -494,10 +482,12 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     int j_of[ITEMS], q_of[ITEMS];
     size_t at_of[ITEMS];
     const float* const base = behind_wait(p.state_base);
+    const int recip = ((1 << 20) + rows_here - 1) / rows_here;
+    static_assert(ITEMS * OWN_THREADS * 64 < 1 << 20, "recip");
     bool live[ITEMS], held[ITEMS];   // held: a head there is, not padding of the group
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {   // the old state is asked for before the wait
-      const int idx = ot + k * OWN_THREADS, q = idx / rows_here, j = rank * rows + (idx - q * rows_here);
+      const int idx = ot + k * OWN_THREADS, q = (idx * recip) >> 20, j = rank * rows + (idx - q * rows_here);   // (idx / rows_here)
       live[k] = q < L::CPR;
       const int g = C::G == 1 ? 0 : j / D, il = j - g * D, h = hg * C::G + g;
       held[k] = live[k] && h < p.H;
@@ -507,6 +497,21 @@ umma_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
       if (p.accumulate && held[k]) {
         acc[k][0] = __ldcg(reinterpret_cast<const float4*>(base + at_of[k]));
         acc[k][1] = __ldcg(reinterpret_cast<const float4*>(base + at_of[k]) + 1);
+      }
+    }
+
+    // Plain: the Q tiles that have come are clamped while the peers' sums and the old state are on their way, not behind the operand: 900 cycles
+    // of the 18 000 that a forward of 192 tokens, 4 heads of 32 takes.  (The old state is asked for first.  Behind the clamping its way began when
+    // the sums had come, and the operand waited for it.  Steps, us, behind / first: 500 tokens, 56 heads of 112 18.9 / 16.5, 2300 tokens,
+    // 40 heads 29.0 / 27.2, 300 tokens, 4 heads 11.9 / 11.6, 150 tokens, 18 heads of 128 14.5 / 14.2; but 700 tokens, 20 heads 14.2 / 14.4.)
+    if (!ROPE && warp < R::EPI_WARP0) {
+      const int most = n_apply < NSC ? n_apply : NSC;
+      for (int spin = 0; spin < 4096 && q_done < most && !__all_sync(0xffffffffu, mbar_test(x_full, 0)); ++spin) {
+        if (!__all_sync(0xffffffffu, mbar_test(&c_full[q_done], 0))) continue;
+        relu_pass<C::FEAT, kTileApply>(slots + q_done * SLOT, slots + q_done * SLOT + HALF, tr);
+        fence_proxy_async_smem();
+        mbar_arrive(&c_ready[q_done]);
+        ++q_done;
       }
     }
 

@@ -57,3 +57,11 @@ def test_many_commits_see_what_the_read_only_step_saw(rope, shape):
     assert differ.item() == 0 and cache.status() == 0
     z = k.float().clamp_min(0).double().sum(1) + k0.float().clamp_min(0).double().sum(1)
     assert np.abs((new[:, :, d].double() - z).cpu().numpy()).max() <= 1e-6 * z.max().item()
+
+
+def test_old_state_is_asked_for_before_queries_are_clamped():
+    """The loads of the old state are on their way while the clamping goes on, and are used behind the sums' arrival."""
+    body = open(os.path.join(CSRC, "umma_cluster.cuh")).read()
+    asked = [m.start() for m in re.finditer(r"= __ldcg\(reinterpret_cast<const float4\*>\(base", body)]
+    clamped, used = body.index("mbar_test(x_full"), body.index("mbar_wait_cluster(x_full")
+    assert asked and max(asked) < clamped < used
