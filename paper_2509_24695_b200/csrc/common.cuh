@@ -43,6 +43,27 @@ inline cudaLaunchAttribute early_start() {
   at.val.programmaticStreamSerializationAllowed = 1;
   return at;
 }
+// May a grid of `units` clusters of c CTAs start early?  `at_once`, `wider`: clusters of c and of c + 1 that the device holds; share: tiles of a CTA.
+//
+// Not where clusters of three or five take nearly all the room that there is for them: those that are placed while the grid before is
+// still leaving lie so that the last ones find no place before others are done.  (Even numbers of CTAs do not show it, and seven take
+// the room of eight.)  Without early starts, with them in a row, with them behind a temporal convolution of 1560 positions; time of the read-only
+// rotary step, heads of 112 (a unit each), relative to the first, by units and 64-token tiles a CTA:
+//   clusters of 3 (45 at once)  45 units    1 tile .95 1.25   4 .95 1.34   12 1.26 1.49
+//                               44                 .92 1.13     .90 1.18      1.09 1.34
+//                               43                 .92 1.00     .90 1.02       .97 1.11
+//                               42                 .92  .92     .90  .93       .92 1.00
+//   clusters of 5 (26 at once)  26                 .92 1.18    1.05 1.22      1.24 1.32
+//                               25                 .89  .99     .94 1.01      1.00 1.12
+//                               24                 .86  .92     .93  .91       .96  .96
+//   of 2, 4, 6, 8, all that fit                    .84 to .90   .89 to .93     .91 to .95
+// fp32 steps of 600 and 1200 tokens (18 and 37 tiles of 32, behind the apply pass of the one before) 45 units 1.40, 44 1.35, 43 1.15, 42 1.02,
+// 41 .95.  (Where the two columns disagree, few tiles a CTA, they cancel out: those start early.)
+inline bool clusters_start_early(int c, long long units, int at_once, int wider, long long share) {
+  if (c < 3 || c % 2 == 0 || units <= wider) return true;
+  const long long spare = ((units + at_once - 1) / at_once * at_once - units) * c;   // SMs, in the last wave
+  return spare > 6 || share <= spare;
+}
 template <typename... P, typename... A>
 cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
   cudaLaunchAttribute at[1] = {early_start()};

@@ -960,6 +960,10 @@ cudaError_t launch_state(const Problem& p, const void* k, const void* v, const f
     const double now = (double)((p.units() + at_once - 1) / at_once) * ((double)((tiles + c - 1) / c) + 6.0);
     if (now < cost) { together = c; cost = now; }
   }
+  bool early = true;
+  if (together > 1 && together < 8)
+    early = clusters_start_early(together, p.units(), clusters_at_once(kernel, S::SMEM, together, fits), clusters_at_once(kernel, S::SMEM, together + 1, fits),
+                                 (p.N + 32ll * together - 1) / (32ll * together));
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim = {(unsigned)(together ? together : 1), 1, 1};
@@ -967,7 +971,7 @@ cudaError_t launch_state(const Problem& p, const void* k, const void* v, const f
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(together ? together : *P, p.units());
   cfg.blockDim = dim3(kBlock); cfg.dynamicSmemBytes = S::SMEM; cfg.stream = stream;
-  cfg.attrs = at; cfg.numAttrs = 2;
+  cfg.attrs = at; cfg.numAttrs = early ? 2 : 1;
   const cudaError_t st = cudaLaunchKernelEx(&cfg, kernel, (const T*)k, (const T*)v, p, together ? together : *P, partials, base,
                                             together ? state : (float*)nullptr, tab, ctrl);
   if (st != cudaSuccess) { cudaGetLastError(); return st; }
