@@ -79,3 +79,55 @@ def test_calls_in_a_row(shape):
 def test_calls_in_a_row_captured(shape):
     for got, ref in zip(chain(*shape, wait=False, capture=True), chain(*shape, wait=True)):
         assert torch.equal(got, ref)
+
+
+@pytest.mark.parametrize("shape", [SHAPES[1], SHAPES[2], SHAPES[6]], ids=str)
+def test_calls_behind_memsets_copies_and_joins(shape):
+    """What stands before a call is not always a kernel of its stream: a memset, a copy, the join of two streams; eager and captured."""
+    N, H, d, dtype, rope = shape
+    dt = {"bf16": torch.bfloat16, "f32": torch.float32}[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(N + d)
+    x0, x1 = (torch.randn(1, N, H, d, device="cuda", generator=gen).to(dt) for _ in range(2))
+    w = torch.randn(3, H * d, device="cuda", generator=gen) * 0.25
+    x, o, p, z = (torch.zeros_like(x0) for _ in range(4))
+    cache, conv = la.BlockLinCache(1, H, d, dt, "cuda", max_T_b=N), la.TConvCache(1, N, H * d, dt, "cuda")
+    ws = la.new_workspace(x)
+    side = torch.cuda.Stream()
+
+    def once(done=lambda: None):
+        main = torch.cuda.current_stream()
+        cache.reset()                                        # a memset
+        cache.step(x1, x1, x0, out=o)
+        done()
+        x.copy_(o)                                           # a copy
+        cache.peek(x, x1, x0, out=p)
+        done()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            conv.reset()
+            conv.step(p.view(1, 1, N, H * d), w, out=z.view(1, 1, N, H * d))
+        done()
+        cache.step(p, x, x1, out=o)
+        main.wait_stream(side)
+        done()
+        la.linattn_forward(z, o, x0, out=x, workspace=ws)    # behind both streams
+        done()
+
+    once(torch.cuda.synchronize)
+    want = [t.clone() for t in (x, o, p, z, cache.state, conv.frame)]
+    got = []
+    once()
+    torch.cuda.synchronize()
+    got.append([t.clone() for t in (x, o, p, z, cache.state, conv.frame)])
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        once()
+    for t in (x, o, p, z):
+        t.zero_()
+    for _ in range(2):
+        g.replay()
+        torch.cuda.synchronize()
+        got.append([t.clone() for t in (x, o, p, z, cache.state, conv.frame)])
+    for run in got:
+        for a, b in zip(run, want):
+            assert b.isfinite().all() and torch.equal(a, b)
