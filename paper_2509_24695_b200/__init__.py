@@ -236,12 +236,21 @@ def workspace_bytes(B: int, H: int, d: int, N: int, dtype_code: int = LINATTN_BF
     return out.value
 
 
+def _workspace_for(need, like, N, where) -> int:
+    """Bytes for tensors shaped like `like`, dense or with its strides: heads of 32 that are not side by side take other kernels."""
+    B, _, H, d = like.shape
+    dense, own = ctypes.c_size_t(), ctypes.c_size_t()
+    _check(need(ctypes.byref(_Desc(B, H, d, _dtype_code(like), 0, 0, 0)), N, ctypes.byref(dense)), where)
+    if not like.is_contiguous():   # (strides that no call takes leave it at 0)
+        need(ctypes.byref(_Desc(B, H, d, _dtype_code(like), *like.stride()[:3])), N, ctypes.byref(own))
+    return max(dense.value, own.value)
+
+
 def new_workspace(like, N: int | None = None):
     """Allocate (with torch) and initialise a workspace fit for tensors shaped like `like`."""
     torch = _torch()
     lib = load_library()
-    B, n, H, d = like.shape
-    nbytes = workspace_bytes(B, H, d, n if N is None else N, _dtype_code(like))
+    nbytes = _workspace_for(lib.linattn_workspace_bytes, like, like.shape[1] if N is None else N, "linattn_workspace_bytes")
     ws = torch.empty(nbytes, dtype=torch.uint8, device=like.device)
     _check(lib.linattn_workspace_init(_ptr(ws), nbytes, _stream(like)), "linattn_workspace_init")
     return ws
@@ -288,12 +297,9 @@ def new_rope_workspace(like):
     """Allocate (with torch) and initialise a workspace for ``linattn_forward_rope`` on tensors shaped like `like`."""
     torch = _torch()
     lib = load_library()
-    B, N, H, d = like.shape
-    nb = ctypes.c_size_t()
-    _check(lib.linattn_rope_workspace_bytes(ctypes.byref(_Desc(B, H, d, _dtype_code(like), 0, 0, 0)), N, ctypes.byref(nb)),
-           "linattn_rope_workspace_bytes")
-    ws = torch.empty(nb.value, dtype=torch.uint8, device=like.device)
-    _check(lib.linattn_workspace_init(_ptr(ws), nb.value, _stream(like)), "linattn_workspace_init")
+    nbytes = _workspace_for(lib.linattn_rope_workspace_bytes, like, like.shape[1], "linattn_rope_workspace_bytes")
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=like.device)
+    _check(lib.linattn_workspace_init(_ptr(ws), nbytes, _stream(like)), "linattn_workspace_init")
     return ws
 
 
