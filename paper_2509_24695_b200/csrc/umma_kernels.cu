@@ -695,8 +695,8 @@ __device__ void reduce_image(const FusedParams& p) {
     }
     if (ROPE && D % 8 == 0 && c == 0) reduce_image_zrow<D>(p, u, ncol, r_lo, nrec);
   }
-  // The images are read through the async proxy (bulk copy) after the barrier.  (For all of memory the fence cost more: step of 4680 tokens
-  // 32.2 -> 30.9 us, of 2 x 10800 88.1 -> 87.8, forward of 32 760 120.2 -> 119.5.)
+  // The images are read through the async proxy (bulk copy) after the barrier.  (A fence for all of memory, in turn with this: step of 4680 tokens
+  // 31.1 and 30.8 us, of 2 x 10800 90.5 and 89.9, forwards level.)
   fence_proxy_async_global();
 }
 
@@ -718,8 +718,8 @@ __device__ __forceinline__ void split_hi_lo(const float (&x)[8], uint4& hi, uint
 // their fixed order, adds that to what it has, and leaves the result as the block's operand image (IMAGE) or state.  The records of all
 // blocks make one list, of which NR are in flight together (about 148 / heads of them, however they fall on the blocks).  Same sums in
 // the same order as a state launch, prefix_states and an apply launch, without the gaps between three launches and with the operands made
-// once instead of by every CTA from the states.  Before and after, us: 7 blocks of 4680 tokens, 20 heads of 112 134.9 -> 123.5, of 10800 280 -> 241, of 300
-// 36.9 -> 22.6 (more beside umma_joins_prefill); 2 entries of 6 blocks of 3040, 35 heads of 64 157 -> 142; 7 blocks of 300, 18 heads of 128 39.0 -> 24.7.
+// once instead of by every CTA from the states.  Three launches and one, in turn, us: 7 blocks of 4680 tokens, 20 heads of 112 138 and 122, of 10800 298 and 264,
+// of 300 34.9 and 22.6 (more beside joins_prefill); 2 entries of 6 blocks of 3040, 35 heads of 64 157 and 144; 7 blocks of 300, 18 heads of 128 39.0 and 22.6.
 template <int D, bool IMAGE>
 __device__ __forceinline__ void prefix_slice(const FusedParams& p, int& i0, int& i1) {   // this CTA's share of the cache's 32-byte chunks
   const long long tot = (long long)(p.B / p.blocks) * p.H * ((D + 1) * D / 8);
@@ -1183,8 +1183,9 @@ umma_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
   constexpr bool TAB = ROPE && !SOLO;
   // QT: phi(Q) is an operand in tensor memory, beside the accumulator of its tile.  Of the 260 KB that a tile of 128 rows moves through shared
   // memory that takes out 84 (the clamped rows back, and both MMAs' reads of them): time where a tile is waited for, power where the
-  // chip is at its cap (1000 W, 1.5 to 1.6 GHz: forwards of 32 760 tokens and more).  Before and after, us: step of 4680 tokens 31.6 -> 30.9, of
-  // 2 x 10800 90.0 -> 89.2, 720p, 35 heads of 64 249.5 -> 246.7, 480p 123.3 -> 122.2; same bits.  (Lone CTAs: their accumulators take
+  // chip is at its cap (1000 W, 1.5 to 1.6 GHz: forwards of 32 760 tokens and more).  Without and with, in turn, us: step of 4680 tokens 31.1 and 30.8, of
+  // 2 x 10800 90.7 and 89.9, forward of 75 600 tokens, 35 heads of 64 252.7 and 249.4; 20 heads of 112 level (32 760 tokens 124.8 and 124.2, 75 600 266 and
+  // 267, runs of one side differ by 1 to 2 %); same bits.  (Lone CTAs: their accumulators take
   // all columns up to the first Q tile.  Rotary: the rotated rows come eight lanes to a row.)
   constexpr bool QT = !ROPE && !SOLO;
   constexpr uint32_t QT_COL = 160;         // behind the accumulator's columns
@@ -1977,23 +1978,22 @@ int sm_count() {
   return cached[dev];
 }
 
-// One CTA per unit instead of all CTAs on all units?  A lone CTA takes about 6 us and 1.6 (packed heads) to 3 us for every 64
-// tokens of its unit; the grid takes 13 to 15 us (two grid barriers, the partial records, the reduce and the operand images
-// between the passes; 8 to 10 without an apply pass) and a time that grows with all units' tokens together.  Measured, launches
+// One CTA per unit instead of all CTAs on all units?  A lone CTA takes about 4 us and 2 (packed heads) to 3 us for every 64
+// tokens of its unit; the grid takes 14 to 18 us (two grid barriers, the partial records, the reduce and the operand images
+// between the passes; 10 to 14 without an apply pass) and a time that grows with all units' tokens together.  Measured, launches
 // back to back, lone CTAs against the grid, in us:
 //                       64 tokens                  128                        192                        256
 //                       forward  step  state       forward  step  state       forward  step  state       forward  step  state
-//   d = 112, 1 unit     7.9/16.1 8.5/17.4 6.5/11.4 10.6/14.8 11.6/15.1 9.0/9.8  14.2/14.0 15.2/14.4 11.7/9.2 17.0/13.9 18.0/14.1 14.3/9.0
-//            20         8.1/17.3 8.9/18.2 6.7/12.1 11.0/16.4 11.7/16.9 9.3/10.7 14.4/15.2 15.3/15.6 12.0/9.8 17.3/15.3 18.1/15.6 14.4/9.6
-//            60         8.4/17.4 9.1/18.3 6.8/12.2 11.0/17.5 12.0/17.9 9.3/11.0 14.6/18.3 15.6/18.7 12.1/11.3 17.4/18.5 18.4/19.1 14.5/11.4
-//            148        10.5/19.4 11.1/19.4 7.5/12.5 12.9/20.2 13.9/20.4 9.8/13.1 15.8/21.6 17.1/21.6 12.5/13.6 18.6/22.5 19.6/22.5 15.1/14.1
-//   d = 128, 18 units   8.5/17.4 9.5/18.2 7.1/13.0 11.3/16.3 12.4/16.8 9.7/10.8 15.1/15.4 16.1/15.8 12.5/10.3 18.0/15.7 19.2/15.9 15.4/9.6
-//   d = 64, 35          8.3/16.2 9.0/16.4 6.4/10.5 10.8/15.5 11.6/15.5 8.7/9.5  13.6/15.7 14.5/15.7 10.8/9.4 16.1/16.3 16.9/16.2 12.9/9.6
-//   d = 32, 1           7.5/13.1 7.9/12.6 5.5/8.0  9.9/12.6 10.2/13.3 7.3/7.7   12.3/13.0 12.7/13.1 9.0/7.7  14.0/13.0 14.5/12.9 10.6/7.7
-// with rotary factors alike at d = 112 and 128 and twice as fast as the grid at d = 32 and 64.  (Taken before early starts, which take 1.5
-// to 3 us off the lone CTAs of calls in a row and nothing off the grid: forward of 64 tokens, 4 heads of 32 6.9, 128 tokens 8.8.)  So: up to 128 tokens, and up to 192
-// with packed heads or many units where these are too many for clusters, which are asked for first (cluster_size).  (States alone of
-// 129 to 192 tokens with packed heads lose 1 us by that.)  The choice depends on the shape and the device, not on the call, so that all
+//   d = 112, 1 unit     7.2/16.4 7.8/16.4 6.0/12.4 10.1/14.6 10.9/16.4 8.3/10.3 13.7/14.4 14.6/14.4 11.1/10.3 16.6/14.4 17.5/14.4 13.8/10.3
+//            20         7.6/17.9 8.1/18.5 5.9/14.4 10.4/16.4 11.1/18.4 8.5/12.3 14.0/16.4 14.8/16.4 11.3/11.5 16.9/16.4 17.7/16.4 14.0/11.7
+//            60         8.1/18.5 8.6/18.5 6.1/14.4 10.8/17.6 11.5/18.5 8.6/12.4 14.2/18.5 15.0/18.5 11.3/12.4 17.2/18.5 17.9/18.6 14.0/12.4
+//            148        10.0/20.5 10.6/20.6 6.9/14.4 12.5/22.5 13.4/22.6 9.2/14.4 15.5/22.6 16.6/22.6 11.9/14.7 18.4/24.6 19.3/24.6 14.7/16.4
+//   d = 128, 18 units   7.7/18.5 8.6/18.5 6.3/15.2 10.6/16.4 11.8/18.4 8.8/12.4 14.4/16.4 15.6/16.4 11.8/12.3 17.4/16.4 18.7/16.4 14.7/11.8
+//   d = 64, 35          7.9/18.5 8.5/18.5 5.9/12.3 10.2/16.8 11.0/16.5 7.8/10.9 13.0/17.9 13.8/18.2 10.0/10.3 15.5/18.5 16.3/18.5 12.2/11.2
+//   d = 32, 1           7.1/14.4 7.4/14.4 5.8/10.3 9.1/14.4 9.4/14.4 6.6/10.3 11.5/14.4 11.8/14.4 8.2/10.3 13.2/14.4 13.6/14.4 9.7/9.9
+// with rotary factors alike at d = 112 and 128 and twice as fast as the grid at d = 32 and 64.  (The grid's calls in a row come out at multiples of
+// 2.05 us.)  So: up to 128 tokens, and up to 192
+// with packed heads or many units where these are too many for clusters, which are asked for first (cluster_size).  The choice depends on the shape and the device, not on the call, so that all
 // calls on one shape (forward, state and apply, step, peek, the token-sharded three) add up in the same order and give the same bits.
 inline bool solo_pays(const Problem& p, int U, int sms) {
   return U <= sms && (p.N <= 128 || (p.N <= 192 && (p.d <= 64 || 3 * U >= 2 * sms)));
@@ -2063,19 +2063,19 @@ int clusters_at_once(int c) {
 // sums and operand leave two Q slots, lose early.  Read-only step, back to back, clusters against the grid (lone CTAs where
 // they would be taken), us:
 //                        192 tokens   300          600          1200         2400         4680
-//   d = 112,  4 heads    14.8/16.8    14.8/16.8    14.9/16.9    16.9/17.0    19.0/17.2    25.1/19.0
-//            20          14.9/16.9    14.9/17.0    17.0/17.1    19.0/19.2    24.0/23.1    31.7/31.3
-//            40          15.2/18.8    16.9/18.9    19.0/21.1    23.0/25.5    31.3/33.7    49.8/49.8
-//            60          16.4/19.7    18.9/21.0    21.0/24.7    27.2/31.2    41.5/45.0    66.3/64.4
-//   d = 64,  35          14.7/16.8    14.8/17.1    16.9/18.9    19.0/21.0    23.9/23.0    33.3/31.2
-//   d = 128, 18          16.0/17.0    17.2/17.6    19.2/18.8    23.0/19.9    29.6/23.3    41.8/33.2
-//   rotary, 112,  4      16.9/19.0    17.0/19.0    18.1/20.1    20.0/25.2    23.2/26.8    29.3/31.3
-//                20      17.2/19.0    17.7/19.4    19.0/21.1    22.3/24.3    27.5/29.1    38.0/39.6
-//                40      18.9/20.9    19.1/21.2    21.2/25.1    27.2/31.3    39.7/41.5    60.3/58.8
-//                60      18.9/21.2    21.0/23.9    24.9/27.3    33.4/35.7    51.8/51.8    82.5/75.2
-//   rotary, 64,  35      15.8/19.0    17.1/19.4    19.1/21.1    21.1/25.1    27.2/27.9    37.1/39.0
-//   rotary, 128, 18      17.0/20.3    18.9/20.9    21.0/21.2    23.1/25.2    30.3/29.3    43.8/39.6
-// Up to 128 tokens lone CTAs are as fast or faster (14.3 against 14.6, 12.9 against 14.9).  S is as far from 64 bits as the
+//   d = 112,  4 heads    10.9/16.4    11.4/16.3    11.8/16.4    13.8/16.4    16.1/16.4    21.9/18.5
+//            20          11.4/16.4    13.3/16.4    13.8/16.4    16.5/18.5    19.9/22.0    27.9/28.7
+//            40          12.7/16.7    13.7/18.5    16.0/20.5    19.2/24.6    27.8/31.8    47.8/48.0
+//            60          13.2/18.5    15.2/20.5    17.4/22.6    23.1/28.7    38.1/43.1    63.5/63.6
+//   d = 64,  35          13.4/13.7    14.0/18.5    14.9/20.5    19.0/22.6    28.0/27.6    46.8/46.7
+//   d = 128, 18          13.3/16.4    15.4/16.5    16.4/17.5    19.6/18.6    25.6/22.0    38.9/28.7
+//   rotary, 112,  4      13.1/18.5    13.4/18.5    14.1/20.2    16.1/24.6    18.6/26.3    25.3/30.9
+//                20      13.6/18.9    15.5/18.6    15.7/20.5    18.2/22.8    22.6/26.7    32.8/37.0
+//                40      15.1/20.5    15.7/20.5    17.7/24.6    21.9/28.9    33.3/40.2    58.1/58.1
+//                60      15.5/20.5    17.0/22.6    19.7/26.7    27.5/34.8    46.4/51.3    76.5/76.7
+//   rotary, 64,  35      14.6/16.4    14.5/20.5    16.3/22.6    20.4/26.7    31.2/34.9    55.6/55.4
+//   rotary, 128, 18      14.1/20.5    16.7/20.5    16.8/20.5    19.3/24.6    25.0/27.5    37.1/36.9
+// Up to 128 tokens lone CTAs are as fast or faster (steps of 20 heads of 112 11.2 against 11.8, of 18 of 128 11.9 against 14.3; states alone 8.7 and 8.3).  S is as far from 64 bits as the
 // grid's or closer (4680 tokens, 20 heads: 9.0e-8 against 1.20e-7; rotary: see the kernel's MMA issuer).  The choice depends on the shape and on the device (how its SMs
 // are spread over GPCs), as the grid's split depends on its SM count: all calls on one shape give the same bits on one GPU.
 //
@@ -2084,32 +2084,30 @@ int clusters_at_once(int c) {
 // adds up the records of 148 / units CTAs.  Packed heads, whose grid form is slower, lose at thirteen tiles with 3 to 9 units and
 // rotary factors, and at twelve without and below two thirds.  Read-only step and state alone, from CUDA graphs, clusters against the
 // grid, us:
-//   rotary, 112,  4 units, 12 tiles of 8 CTAs   31.9/32.2  18.5/21.7   13 tiles   34.0/32.9  19.2/21.8
-//                 6        10                   29.3/30.0  17.3/19.7   11         31.3/30.4  18.0/20.5
-//                 8         8                   26.3/26.3  16.0/17.2    9         28.7/27.1  16.7/17.7    13  34.6/30.2  19.6/19.0
-//                12         8                   27.5/28.2  16.8/17.6    9         29.8/28.8  17.4/17.9    12  33.9/32.6  19.6/19.2
-//                16         8         6 CTAs    27.6/27.6  17.1/17.1    9         29.9/28.2  17.7/17.3    13  36.0/34.9  20.2/19.4
-//                18        12         6 CTAs    34.4/34.5  19.9/19.4   13         37.1/35.6  20.7/20.1
-//                26        13         5 CTAs    37.9/39.7  21.0/22.7
-//                33        13         4 CTAs    39.0/40.9  21.5/21.3
-//                35        12         3 CTAs    34.1/33.8  19.7/18.6   13         36.2/34.3  20.6/19.2
-//                46         8         2 CTAs    27.3/27.3  17.7/16.7    9         29.7/27.8  18.4/16.9    12  34.1/31.9  20.5/18.3
-//                50        12         2 CTAs    34.9/38.6  20.8/21.7
-//   d = 112,     46         8         2 CTAs    22.5/22.8  14.8/14.3    9         24.2/23.4  15.5/14.3    12  27.5/26.6  17.5/15.5
-//   rotary, 64,   8        12         8 CTAs    31.0/30.8  15.9/18.5   13         33.4/31.1  16.5/18.8
-//   d = 64,      46        11         2 CTAs    27.3/27.6  16.0/15.0   12         28.8/28.2  16.5/15.1
-//   d = 32,      33         4         4 CTAs    18.3/20.9  10.4/11.9
-//   rotary, 32,  22        13         6 CTAs    36.2/42.4  16.7/21.2
-//   d = 128,     18         1         3 CTAs    13.8/15.7  10.8/10.7
-//   rotary, 128, 18         4         6 CTAs    22.9/25.4  15.6/16.0
-//                26         1         5 CTAs    18.7/20.0  12.8/12.1
-// States alone lose 3 to 6 % on clusters with 27 to 29 and 34 to 37 units of ten to twelve tiles, with 46 to 49 units from six
-// on, and with heads of 128 (129 to 192 tokens; with rotary factors, five CTAs), where the steps are level or gain: one form for all calls.
-// All of this was taken before early starts (early_start) and the shorter end of the cluster kernel, which take 2 to 4 us off clusters in a
-// row and nothing off the grid: 20 heads of 112, read-only step of 4680 tokens now 30.6 on clusters of 6, 33.1 on the grid, rotary 33.6 and 40.6.
-// Clusters are ahead up to 18 tiles and more where they take 110 SMs or more, and to 5 to 10 below that; the line has not been moved.
-// Not taken though clusters would be 7 % ahead: thirteen tiles and more of plain heads of 112 with 38 to 45 and 50 to 74 units; heads
-// of 128 of 193 to 300 tokens (3 %).
+//   rotary, 112,  4 units, 12 tiles of 8 CTAs   28.3/30.3  15.6/20.0   13 tiles   30.0/31.0  16.2/20.3
+//                 6        10                   25.9/28.4  14.5/18.3   11         27.5/28.7  15.1/18.8
+//                 8         8                   23.8/24.4  13.9/15.8    9         25.9/24.9  14.5/16.1    13  31.1/27.9  16.9/17.5
+//                12         8                   24.0/26.1  14.2/16.2    9         26.1/26.4  14.8/16.5    12  30.0/30.1  16.6/17.6
+//                16         8         6 CTAs    24.2/25.7  14.3/15.7    9         26.3/26.0  14.9/15.8    13  32.5/32.2  17.3/17.8
+//                18        12         6 CTAs    30.3/32.3  16.9/17.9   13         33.0/33.2  17.4/18.5
+//                26        13         5 CTAs    36.0/39.2  18.8/20.0
+//                33        13         4 CTAs    34.8/39.7  17.9/19.8
+//                35        12         3 CTAs    30.2/31.2  16.8/17.1   13         32.8/32.3  17.5/17.8
+//                46         8         2 CTAs    23.7/25.5  15.1/15.5    9         25.7/25.5  15.7/15.5    12  30.4/29.1  17.6/16.8
+//                50        12         2 CTAs    31.3/37.3  17.6/20.4
+//   d = 112,     46         8         2 CTAs    20.1/20.8  12.5/12.3    9         21.6/20.8  13.2/12.4    12  25.2/23.5  15.1/13.4
+//   rotary, 64,   8        12         8 CTAs    27.7/27.7  13.7/17.0   13         29.5/27.8  14.2/17.2
+//   d = 64,      46        11         2 CTAs    24.5/22.8  13.4/12.8   12         25.5/23.4  14.0/12.8
+//   d = 32,      33         4         4 CTAs    14.9/17.6   8.0/10.2
+//   rotary, 32,  22        13         6 CTAs    34.3/42.1  13.6/18.7
+//   d = 128,     18         1         3 CTAs    13.0/15.2   9.7/10.6
+//   rotary, 128, 18         4         6 CTAs    19.1/23.1  12.8/14.1
+//                26         1         5 CTAs    17.7/18.8  12.4/11.7
+// One form for all calls: states alone lose up to 9 % on clusters with 46 to 49 units from six tiles on.
+// Not taken though clusters would be ahead (the line was drawn before early starts, which shorten clusters and not the grid): plain heads of 112 from
+// three tiles to a CTA on in clusters of four and more (20 units 15.5/17.0 at three tiles, 26.2/27.2 at twelve, level at thirteen; 33 units 15.5/17.6 at
+// three), and from thirteen on with 38 to 45 and 50 to 74 units (40 units 27.6/30.5, 60 27.5/32.2).  Taken though the grid would be: packed heads
+// without rotary factors, 46 to 49 units of eleven tiles.
 template <int D, bool ROPE>
 int cluster_size(const Problem& p, int U, long long tiles, int sms) {
   if (p.N <= 128) return 0;
@@ -2281,15 +2279,19 @@ int cluster_ctas(const Problem& p) {
 // for 7 blocks of 64 tokens, 20 heads of 112.)
 //
 // And not for few heads: a thread of reduce_prefix walks the records of all blocks of its piece, CTAs / head groups of them, eight at a
-// time.  The line is at 64 for every head dim; at 70 to 74 heads of 112 still gain, packed heads lose.  One launch / three, us:
-//                       tokens a block    300        600        1200       2400
-//   d = 112, 20 groups, 7 blocks          22.8/35.4  31.0/45.3  45.4/59.7  68.7/84.5
-//             2         2                 16.5/24.9  18.6/24.8  20.6/25.0  22.7/25.7   (74 records at 2400)
-//             2         7                 20.6/28.4  26.8/28.8  27.3/28.3  29.4/31.2   (35, 70, 74, 74)
-//             1         7                 20.6/27.9  26.6/27.8  36.4/27.8  37.0/27.9   (35, 70, 133, 148)
-//   d = 64,   2         7                 22.4/26.7  27.0/26.7  28.8/29.3  30.9/28.5   (35, 70, 74, 74)
-//   d = 32,   2         7                 20.6/22.6  26.7/23.9  26.8/25.6  28.9/26.8   (35, 70, 74, 74)
-//   d = 128, 20         7                 24.8/39.1  35.1/51.7  50.0/66.4  78.4/95.0
+// time: 49 with three groups, 74 with two, 148 with one.  The line is at 64 for every head dim and any number of blocks.  At 74 heads of 112 and
+// 128 would still gain a little, packed heads lose, at 148 all lose.  One launch / three, us (-: lone CTAs or clusters take the blocks):
+//                       tokens a block    300        600        1200       2400       4680
+//   d = 112, 20 groups, 7 blocks          22.6/34.9  28.7/40.2  45.2/59.8  68.6/84.2  122/138
+//             3         7                 -          -          25.8/28.6  28.8/32.8  37.0/40.5
+//             2         7                 -          -          26.7/28.1  28.8/28.3  33.2/34.1
+//             2         2                 -          -          20.6/24.7  22.6/24.7  27.4/28.8   (38, 74, 74 records)
+//             1         7                 -          -          34.9/26.7  36.5/27.3  38.4/29.5
+//   d = 64,   2         7                 -          -          -          30.8/28.5  34.9/34.9
+//   d = 32,   2         7                 -          -          -          28.8/26.7  34.3/32.9
+//   d = 128, 20         7                 22.6/39.0  32.9/49.3  49.4/65.9  76.7/94.5
+//             2         7                 20.6/27.7  26.7/28.7  27.4/28.5  29.0/31.9  34.5/36.8   (35, 70, 74, 74, 74)
+//             1         7                 20.6/26.6  26.7/28.0  36.7/28.1  36.9/27.7  39.0/32.1   (35, 70, 133, 148, 148)
 template <int D>
 bool joins_prefill(const Problem& p, int blocks) {
   const int sms = sm_count(), hg = (p.H + Cfg<D>::G - 1) / Cfg<D>::G;
