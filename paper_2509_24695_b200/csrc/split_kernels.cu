@@ -961,7 +961,7 @@ cudaError_t launch_state(const Problem& p, const void* k, const void* v, const f
     if (now < cost) { together = c; cost = now; }
   }
   bool early = true;
-  if (together > 1 && together < 8)
+  if (together > 2 && together % 2)
     early = clusters_start_early(together, p.units(), clusters_at_once(kernel, S::SMEM, together, fits), clusters_at_once(kernel, S::SMEM, together + 1, fits),
                                  (p.N + 32ll * together - 1) / (32ll * together));
   cudaLaunchAttribute at[2];

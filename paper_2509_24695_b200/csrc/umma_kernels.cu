@@ -2154,9 +2154,12 @@ int launch_cluster(const Problem& p, const UmmaCall& c, int size, int U, void* w
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim = {(unsigned)size, 1, 1};
   at[1] = early_start();
-  const int at_once = clusters_at_once<D, ROPE>(size), wider = size < 8 ? clusters_at_once<D, ROPE>(size + 1) : U;
-  if (at_once <= 0 || wider < 0) return LINATTN_ERR_CUDA;
-  const bool early = clusters_start_early(size, U, at_once, wider, (cp.tiles + size - 1) / size);
+  bool early = true;
+  if (size > 2 && size % 2) {
+    const int at_once = clusters_at_once<D, ROPE>(size), wider = clusters_at_once<D, ROPE>(size + 1);
+    if (at_once <= 0 || wider < 0) return LINATTN_ERR_CUDA;
+    early = clusters_start_early(size, U, at_once, wider, (cp.tiles + size - 1) / size);
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(size * U); cfg.blockDim = dim3(Roles<ROPE>::THREADS); cfg.dynamicSmemBytes = L::SMEM; cfg.stream = stream;
   cfg.attrs = at; cfg.numAttrs = early ? 2 : 1;
